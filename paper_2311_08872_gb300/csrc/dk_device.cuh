@@ -34,6 +34,23 @@ __device__ __forceinline__ uint4 philox10(uint4 c, uint32_t k0, uint32_t k1) {
     return c;
 }
 
+// Rounds FROM .. TO - 1 of two counters at once (none unless ON).
+template <int FROM, int TO, bool ON = true>
+__device__ __forceinline__ void philox_rounds(uint4& c, uint4& d, uint32_t k0, uint32_t k1) {
+#pragma unroll
+    for (int r = FROM; ON && r < TO; ++r) {
+        const uint32_t ka = k0 + static_cast<uint32_t>(r) * kPhiloxW0, kb = k1 + static_cast<uint32_t>(r) * kPhiloxW1;
+        const unsigned long long p0 = static_cast<unsigned long long>(c.x) * kPhiloxM0;
+        const unsigned long long p1 = static_cast<unsigned long long>(c.z) * kPhiloxM1;
+        const unsigned long long q0 = static_cast<unsigned long long>(d.x) * kPhiloxM0;
+        const unsigned long long q1 = static_cast<unsigned long long>(d.z) * kPhiloxM1;
+        c = make_uint4(static_cast<uint32_t>(p1 >> 32) ^ c.y ^ ka, static_cast<uint32_t>(p1),
+                       static_cast<uint32_t>(p0 >> 32) ^ c.w ^ kb, static_cast<uint32_t>(p0));
+        d = make_uint4(static_cast<uint32_t>(q1 >> 32) ^ d.y ^ ka, static_cast<uint32_t>(q1),
+                       static_cast<uint32_t>(q0 >> 32) ^ d.w ^ kb, static_cast<uint32_t>(q0));
+    }
+}
+
 __device__ __forceinline__ float sqrt_approx(float x) {
     float y;
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -60,6 +77,75 @@ __device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, float& z1, fl
     z2 = r * s;
 }
 
+// Two FP32 values in a 64-bit register pair.  The packed multiply and FMA round
+// each half exactly as the scalar instructions do, in one issue slot.
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+
+__device__ __forceinline__ float lo2(f32x2 v) { return __uint_as_float(static_cast<uint32_t>(v)); }
+__device__ __forceinline__ float hi2(f32x2 v) { return __uint_as_float(static_cast<uint32_t>(v >> 32)); }
+
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// The hardware logarithm, sine and cosine on arguments that are never
+// subnormal (u >= 2^-32, |theta| >= pi 2^-32), where the flush-to-zero forms
+// return what __log2f, __sinf and __cosf do without their subnormal branches.
+__device__ __forceinline__ float lg2_normal(float x) {
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ float sin_normal(float x) {
+    float y;
+    asm("sin.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ float cos_normal(float x) {
+    float y;
+    asm("cos.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Box--Muller in polar form for one word pair of each of two counters, in its
+// parts: -2 ln u from the first words, theta from the second (the arithmetic of
+// box_muller_polar on both halves).
+__device__ __forceinline__ f32x2 bm_lnu2(uint32_t a0, uint32_t a1) {
+    const f32x2 k = pack2(2.3283064365386963e-10f, 2.3283064365386963e-10f);
+    const f32x2 u = fma2(pack2(static_cast<float>(a0), static_cast<float>(a1)), k, k);
+    return mul2(pack2(-1.3862943611198906f, -1.3862943611198906f), pack2(lg2_normal(lo2(u)), lg2_normal(hi2(u))));
+}
+
+__device__ __forceinline__ f32x2 bm_angle2(uint32_t b0, uint32_t b1) {
+    return fma2(pack2(static_cast<float>(static_cast<int32_t>(b0)), static_cast<float>(static_cast<int32_t>(b1))),
+                pack2(1.4629180792671596e-09f, 1.4629180792671596e-09f),
+                pack2(7.314590396335798e-10f, 7.314590396335798e-10f));
+}
+
+__device__ __forceinline__ void box_muller_polar2(uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1, f32x2& r,
+                                                  f32x2& c, f32x2& s) {
+    const f32x2 l = bm_lnu2(a0, a1), th = bm_angle2(b0, b1);
+    r = pack2(sqrt_approx(lo2(l)), sqrt_approx(hi2(l)));
+    c = pack2(cos_normal(lo2(th)), cos_normal(hi2(th)));
+    s = pack2(sin_normal(lo2(th)), sin_normal(hi2(th)));
+}
+
 // Progress counters shared between CTAs of one launch: an acquire load, a
 // release increment (after the CTA's or warp's writes), a volatile read.
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
@@ -81,10 +167,21 @@ __device__ __forceinline__ float noise_amp(int32_t q, float g) {
     return g * sqrt_approx(__int2float_rn(max(q, 0)));
 }
 
+// noise_amp of two cells.
+__device__ __forceinline__ f32x2 noise_amp2(int32_t q0, int32_t q1, f32x2 g) {
+    return mul2(g, pack2(sqrt_approx(__int2float_rn(max(q0, 0))), sqrt_approx(__int2float_rn(max(q1, 0)))));
+}
+
 // The same for a fluctuation state dq = (rho - rho-bar) 2^S: the transfer is
 // g sqrt([rho-bar + dq 2^-S]^+) z with g = c 2^S, rho-bar the noise-free path.
 __device__ __forceinline__ float noise_amp_fluct(int32_t dq, float rbar, float inv_scale, float g) {
     return g * sqrt_approx(fmaxf(fmaf(__int2float_rn(dq), inv_scale, rbar), 0.f));
+}
+
+__device__ __forceinline__ f32x2 noise_amp_fluct2(int32_t d0, int32_t d1, float rbar0, float rbar1, float inv_scale,
+                                                  f32x2 g) {
+    const f32x2 x = fma2(pack2(__int2float_rn(d0), __int2float_rn(d1)), pack2(inv_scale, inv_scale), pack2(rbar0, rbar1));
+    return mul2(g, pack2(sqrt_approx(fmaxf(lo2(x), 0.f)), sqrt_approx(fmaxf(hi2(x), 0.f))));
 }
 
 // Diffusion flux across one edge: round(a * (q_far - q_near)) with a given as

@@ -31,6 +31,17 @@
 // exactly, so sum_x q is invariant bit for bit (the divergence form of the
 // scheme) and every rounding error enters in divergence form.  Observables
 // and moments are accumulated in FP64.
+//
+// What bounds it: instruction pipes, not memory.  A fine cell-step needs 7 XU
+// operations (log, sine, cosine, two square roots, two conversions: 56 cycles of
+// the sub-partition per warp), about 11 wide multiplies (half a Philox4x32-10
+// call and the fluxes: 55 cycles of the FMA pipe) and some 50 instructions in
+// all.  Hence two cell pairs at a time in packed FP32 (half the FP32
+// instructions, the same roundings) and, where the registers allow, the next
+// pairs' Philox rounds interleaved with the current pairs' functions (PIPE).
+// Per warp of fine cells, 64^2 coupled: 107 cycles before, 89 now (9.47 ms for
+// 1151 samples x 832 steps, 11.07 before); 256^2, 59 x 1536: 19.7 ms, 22.8
+// before; 32^2 fine only, 1000 x 103: 0.280 ms, 0.316 before.
 #include <cooperative_groups.h>
 
 #include <atomic>
@@ -63,7 +74,42 @@ struct Shape {
     static constexpr int SPW = WARP ? 32 / LPS : 1;
     static constexpr int THREADS = WARP ? 128 : LPS / CL;
     static constexpr int BPC = WARP ? 1 : NB / CL;   // bands per CTA
+    // How a step is laid out in the instruction stream (the arithmetic is the
+    // same), by block size and registers per thread; measured, ms at the sizes
+    // given (coupled unless said otherwise):
+    //   PIPE   the Philox rounds of the next two cell pairs run between the
+    //          Box--Muller stages of the current two (FMA and ALU pipes under the
+    //          XU pipe), and a row is updated as soon as its transfers are known.
+    //          It wants the registers of 8 to 12 warps per SM: one-CTA samples of
+    //          several warps (64^2, 1151 samples x 832 steps: 9.6, without 10.5,
+    //          scalar FP32 before 11.1; 32^2, 4630 x 208: 2.31, 2.52, 2.57) and
+    //          blocks of 32 cells (256^2, 59 x 1536: 19.8, 23.5, 22.8).  At 128
+    //          registers it spills and loses (128^2, 304 x 1664: 25.0, without 23.7).
+    //   REDRAW the sample's Philox counter word is opaque to the compiler, which
+    //          then does not keep the step-independent parts of the first rounds in
+    //          registers, where those would spill (128^2: 22.7 with, 23.7 without,
+    //          25.1 before; 256^2: 19.8 with, 23.0 without).
+    //   The fluctuation state needs its mean-field rows in registers as well and
+    //   is fastest with neither (128^2, 311 x 1024: 18.6, before 20.2; 64^2, 997 x
+    //   256: 2.89, with PIPE 3.28, before 3.13; loading the next step's rows
+    //   early: 20.3 at 128^2).
+    static constexpr bool PIPE = !FLUCT && (CL == 1 ? !WARP : FR * FC >= 32);
+    static constexpr bool REDRAW = !FLUCT && CL > 1;
+    // Resident warps per SM asked for (a bound on the registers per thread).
+    // 32^2 fine-only, 1000 x 103: 8 warps 0.288 ms, 12 warps 0.282; 16^2 in one
+    // warp, 9250 x 52: 16 warps 0.316, 24 warps 0.306 (before 0.337).
+    static constexpr int WARPS_MIN = FLUCT ? 16 : FR * FC >= 32 ? 8 : PIPE ? (COUPLED && FR * FC >= 16 ? 8 : 12)
+                                   : FR * FC >= 16 || FR * FC < 8 ? 16 : 24;
+    static constexpr int MINB = WARPS_MIN * 32 / THREADS > 0 ? WARPS_MIN * 32 / THREADS : 1;
     static constexpr int SLOTS_PER_CTA = WARP ? (THREADS / 32) * SPW : 1;
+    // Two cell pairs (Philox calls) are worked on together, packed: neighbours
+    // along a row (C even), or the same pair of two coarse rows (C = 1, R = 2),
+    // or the two rows of a single coarse cell (C = R = 1).
+    static constexpr int DPC = C >= 2 ? 1 : 0;                 // offset of the second pair: columns,
+    static constexpr int DR = C >= 2 ? 0 : (R >= 2 ? 2 : 1);   // fine rows
+    static constexpr bool ZPACK = C >= 2 || R >= 2;            // their coupled sums are two coarse cells'
+    static constexpr int NZ = (R * C + 1) / 2;                 // packed coupled sums per component
+    static_assert(C % 2 == 0 || (C == 1 && R <= 2), "cell pairs are worked on two at a time");
     static_assert(LPB <= 32 && (LPB & (LPB - 1)) == 0, "a band must be a power-of-two warp segment");
     static_assert(NC % C == 0 && NC % R == 0, "lane blocks must tile the coarse grid");
     static_assert(WARP || (THREADS % 32 == 0 && THREADS <= 1024 && NB % CL == 0), "bad CTA shape");
@@ -140,12 +186,43 @@ __device__ __forceinline__ void get_edge(const int2* row, int lib, int32_t (&qv)
     }
 }
 
+// Index of the cell pair `pc` of a lane's block row at column col0.
 template <class S>
-__device__ __forceinline__ void block_or_cluster_sync() {
-    if constexpr (S::CL > 1) {
-        cg::this_cluster().sync();
-    } else {
-        __syncthreads();
+__device__ __forceinline__ uint32_t pair_index(int row, int col0, int pc) {
+    return static_cast<uint32_t>((row * S::NF + col0 + 2 * pc) >> 1);
+}
+
+// Row r's part of the update, with its transfers known and its state (and the
+// row above's) old: the horizontal fluxes and transfers, halo columns by
+// shuffles from the adjacent lanes, and the vertical flux between rows r - 1
+// and r, which completes row r - 1 (all but the first row, which waits for the
+// row above the block).  Row by row, only one row's pending change and transfers
+// are live at a time.
+template <class S>
+__device__ __forceinline__ void row_update(int r, int32_t (&q)[S::FR][S::FC], const int32_t (&G1)[S::FR][S::FC],
+                                           const int32_t (&G2)[S::FR][S::FC], int32_t (&pend)[2][S::FC],
+                                           int32_t (&pend0)[S::FC], int left, int right, int32_t A) {
+    constexpr int FC = S::FC;
+    const int32_t qL = __shfl_sync(kFull, q[r][FC - 1], left, S::LPB), gL = __shfl_sync(kFull, G2[r][FC - 1], left, S::LPB);
+    const int32_t qR = __shfl_sync(kFull, q[r][0], right, S::LPB), gR = __shfl_sync(kFull, G2[r][0], right, S::LPB);
+    int32_t (&cur)[FC] = pend[r & 1];
+    int32_t h = edge_flux(A, q[r][0] - qL);
+#pragma unroll
+    for (int c = 0; c < FC; ++c) {
+        const int32_t hn = c + 1 < FC ? edge_flux(A, q[r][c + 1] - q[r][c]) : edge_flux(A, qR - q[r][FC - 1]);
+        const int32_t g2r = c + 1 < FC ? G2[r][c + 1] : gR, g2l = c > 0 ? G2[r][c - 1] : gL;
+        cur[c] = (hn - h) + (g2r - g2l);
+        h = hn;
+    }
+    if (r > 0) {
+#pragma unroll
+        for (int c = 0; c < FC; ++c) {
+            const int32_t v = edge_flux(A, q[r][c] - q[r - 1][c]);
+            cur[c] -= v + G1[r - 1][c];
+            const int32_t u = pend[(r - 1) & 1][c] + v + G1[r][c];
+            if (r == 1) pend0[c] = u;
+            else q[r - 1][c] += u;
+        }
     }
 }
 
@@ -233,7 +310,7 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
 
 template <class S>
-__global__ void __launch_bounds__(S::THREADS) level_kernel(const KArgs a) {
+__global__ void __launch_bounds__(S::THREADS, S::MINB) level_kernel(const KArgs a) {
     constexpr int NF = S::NF, NC = S::NC, FR = S::FR, FC = S::FC, R = S::R, C = S::C;
     constexpr int LPB = S::LPB, LPS = S::LPS, CL = S::CL, BPC = S::BPC;
     constexpr bool CPL = S::COUPLED;
@@ -293,22 +370,25 @@ __global__ void __launch_bounds__(S::THREADS) level_kernel(const KArgs a) {
         const long long idx = slot + it * n_slots;
         const bool active = idx < a.count;
         const long long sid = a.first + (active ? idx : 0);
-        const uint32_t c2 = static_cast<uint32_t>(sid);
+        uint32_t c2 = static_cast<uint32_t>(sid);
         const uint32_t c3 = a.tag | ((static_cast<uint32_t>(static_cast<unsigned long long>(sid) >> 32) & 0xffffu) << 16);
 
         int32_t q[FR][FC];
 #pragma unroll
         for (int r = 0; r < FR; ++r) load_row<FC>(q[r], a.q0f + (size_t)(row0 + r) * NF + col0);
         int32_t qc[R][C];
-        float zt[R][C][2];
+        f32x2 zt[S::NZ][2];                 // coupled normal sums, two coarse cells each
         if constexpr (CPL) {
 #pragma unroll
             for (int i = 0; i < R; ++i) load_row<C>(qc[i], a.q0c + (size_t)(crow0 + i) * NC + ccol0);
 #pragma unroll
-            for (int i = 0; i < R; ++i)
-#pragma unroll
-                for (int j = 0; j < C; ++j) zt[i][j][0] = zt[i][j][1] = 0.f;
+            for (int z = 0; z < S::NZ; ++z) zt[z][0] = zt[z][1] = 0ull;
         }
+
+        // Philox words of the two cell pairs drawn next
+        uint4 w0 = make_uint4(pair_index<S>(row0, col0, 0), 0u, c2, c3);
+        uint4 w1 = make_uint4(pair_index<S>(row0 + S::DR, col0, S::DPC), 0u, c2, c3);
+        philox_rounds<0, 10>(w0, w1, a.key0, a.key1);
 
         for (int m = 0; m < a.M; ++m) {
             // fluctuation state: the noise-free path rho-bar^m of this lane's cells
@@ -318,37 +398,98 @@ __global__ void __launch_bounds__(S::THREADS) level_kernel(const KArgs a) {
                 for (int r = 0; r < FR; ++r)
                     load_row_f<FC>(rb[r], a.rbf + (size_t)m * NF * NF + (size_t)(row0 + r) * NF + col0);
             }
-            // ---- noise: Philox4x32-10 per horizontal cell pair, Box--Muller, transfers
+            if constexpr (S::REDRAW) asm volatile("" : "+r"(c2));
+            // ---- rows of the block in order: noise, transfers, and the row's part of the update
+            const bool cstep = CPL && ((m & 3) == 3);
+            const int par = m & 1;
+            const f32x2 gf2 = pack2(a.gf, a.gf);
             int32_t G1[FR][FC], G2[FR][FC];
+            int32_t pend[2][FC];      // change of the row in hand still to be added (parity of the row)
+            int32_t pend0[FC];        // the same for the first row, which waits for the row above it
 #pragma unroll
             for (int r = 0; r < FR; ++r) {
+                if (S::DR == 0 || !(r & S::DR)) {   // with DR, row r + DR's noise is drawn with row r's
 #pragma unroll
-                for (int pc = 0; pc < C; ++pc) {
-                    const uint32_t p = static_cast<uint32_t>(((row0 + r) * NF + col0 + 2 * pc) >> 1);
-                    const uint4 x = philox10(make_uint4(p, static_cast<uint32_t>(m), c2, c3), a.key0, a.key1);
-                    // normals (ra ca, ra sa) and (rb cb, rb sb); the amplitude scales the radius
-                    float ra, ca, sa, rb_, cb, sb;
-                    box_muller_polar(x.x, x.y, ra, ca, sa);
-                    box_muller_polar(x.z, x.w, rb_, cb, sb);
-                    float ta, tb;
-                    if constexpr (S::FLUCT) {
-                        ta = noise_amp_fluct(q[r][2 * pc], rb[r][2 * pc], a.isf, a.gf) * ra;
-                        tb = noise_amp_fluct(q[r][2 * pc + 1], rb[r][2 * pc + 1], a.isf, a.gf) * rb_;
-                    } else {
-                        ta = noise_amp(q[r][2 * pc], a.gf) * ra;
-                        tb = noise_amp(q[r][2 * pc + 1], a.gf) * rb_;
-                    }
-                    G1[r][2 * pc] = __float2int_rn(ta * ca);
-                    G2[r][2 * pc] = __float2int_rn(ta * sa);
-                    G1[r][2 * pc + 1] = __float2int_rn(tb * cb);
-                    G2[r][2 * pc + 1] = __float2int_rn(tb * sb);
-                    if constexpr (CPL) {
-                        zt[r >> 1][pc][0] = fmaf(rb_, cb, fmaf(ra, ca, zt[r >> 1][pc][0]));
-                        zt[r >> 1][pc][1] = fmaf(rb_, sb, fmaf(ra, sa, zt[r >> 1][pc][1]));
+                    for (int pa = 0; pa < C; pa += 1 + S::DPC) {
+                        const int r2 = r + S::DR, p2 = pa + S::DPC;
+                        const auto draw = [&](int row, int pair, int step) {
+                            w0 = make_uint4(pair_index<S>(row0 + row, col0, pair), static_cast<uint32_t>(step), c2, c3);
+                            w1 = make_uint4(pair_index<S>(row0 + row + S::DR, col0, pair + S::DPC),
+                                            static_cast<uint32_t>(step), c2, c3);
+                        };
+                        if constexpr (!S::PIPE) {
+                            draw(r, pa, m);
+                            philox_rounds<0, 10>(w0, w1, a.key0, a.key1);
+                        }
+                        const uint4 x0 = w0, x1 = w1;
+                        if constexpr (S::PIPE) {
+                            // the two pairs after these (the next step's first after the last)
+                            const bool row_end = pa + 1 + S::DPC >= C;
+                            int nr = row_end ? r + 1 : r;
+                            if (S::DR && (nr & S::DR)) nr += S::DR;
+                            const bool last = nr >= FR;
+                            draw(last ? 0 : nr, row_end ? 0 : pa + 1 + S::DPC, last ? m + 1 : m);
+                        }
+                        philox_rounds<0, 3, S::PIPE>(w0, w1, a.key0, a.key1);
+                        const f32x2 la = bm_lnu2(x0.x, x1.x), lb = bm_lnu2(x0.z, x1.z);
+                        philox_rounds<3, 4, S::PIPE>(w0, w1, a.key0, a.key1);
+                        const f32x2 ha = bm_angle2(x0.y, x1.y), hb = bm_angle2(x0.w, x1.w);
+                        const f32x2 ca = pack2(cos_normal(lo2(ha)), cos_normal(hi2(ha)));
+                        const f32x2 cb = pack2(cos_normal(lo2(hb)), cos_normal(hi2(hb)));
+                        philox_rounds<4, 5, S::PIPE>(w0, w1, a.key0, a.key1);
+                        const f32x2 ra = pack2(sqrt_approx(lo2(la)), sqrt_approx(hi2(la)));
+                        const f32x2 rbb = pack2(sqrt_approx(lo2(lb)), sqrt_approx(hi2(lb)));
+                        philox_rounds<5, 6, S::PIPE>(w0, w1, a.key0, a.key1);
+                        const f32x2 sa = pack2(sin_normal(lo2(ha)), sin_normal(hi2(ha)));
+                        const f32x2 sb = pack2(sin_normal(lo2(hb)), sin_normal(hi2(hb)));
+                        philox_rounds<6, 7, S::PIPE>(w0, w1, a.key0, a.key1);
+                        f32x2 ta, tb;
+                        if constexpr (S::FLUCT) {
+                            ta = noise_amp_fluct2(q[r][2 * pa], q[r2][2 * p2], rb[r][2 * pa], rb[r2][2 * p2], a.isf, gf2);
+                            tb = noise_amp_fluct2(q[r][2 * pa + 1], q[r2][2 * p2 + 1], rb[r][2 * pa + 1],
+                                                  rb[r2][2 * p2 + 1], a.isf, gf2);
+                        } else {
+                            ta = noise_amp2(q[r][2 * pa], q[r2][2 * p2], gf2);
+                            tb = noise_amp2(q[r][2 * pa + 1], q[r2][2 * p2 + 1], gf2);
+                        }
+                        ta = mul2(ta, ra);
+                        tb = mul2(tb, rbb);
+                        philox_rounds<7, 8, S::PIPE>(w0, w1, a.key0, a.key1);
+                        const f32x2 a1 = mul2(ta, ca), a2 = mul2(ta, sa), b1 = mul2(tb, cb), b2 = mul2(tb, sb);
+                        G1[r][2 * pa] = __float2int_rn(lo2(a1));
+                        G2[r][2 * pa] = __float2int_rn(lo2(a2));
+                        G1[r2][2 * p2] = __float2int_rn(hi2(a1));
+                        G2[r2][2 * p2] = __float2int_rn(hi2(a2));
+                        philox_rounds<8, 9, S::PIPE>(w0, w1, a.key0, a.key1);
+                        G1[r][2 * pa + 1] = __float2int_rn(lo2(b1));
+                        G2[r][2 * pa + 1] = __float2int_rn(lo2(b2));
+                        G1[r2][2 * p2 + 1] = __float2int_rn(hi2(b1));
+                        G2[r2][2 * p2 + 1] = __float2int_rn(hi2(b2));
+                        if constexpr (CPL) {
+                            if constexpr (S::ZPACK) {
+                                const int z = S::DPC ? ((r >> 1) * C + pa) / 2 : 0;
+                                zt[z][0] = fma2(rbb, cb, fma2(ra, ca, zt[z][0]));
+                                zt[z][1] = fma2(rbb, sb, fma2(ra, sa, zt[z][1]));
+                            } else {
+                                // one coarse cell: the sum runs over row 0, then row 1
+                                float z1 = lo2(zt[0][0]), z2 = lo2(zt[0][1]);
+                                z1 = fmaf(lo2(rbb), lo2(cb), fmaf(lo2(ra), lo2(ca), z1));
+                                z2 = fmaf(lo2(rbb), lo2(sb), fmaf(lo2(ra), lo2(sa), z2));
+                                z1 = fmaf(hi2(rbb), hi2(cb), fmaf(hi2(ra), hi2(ca), z1));
+                                z2 = fmaf(hi2(rbb), hi2(sb), fmaf(hi2(ra), hi2(sa), z2));
+                                zt[0][0] = pack2(z1, 0.f);
+                                zt[0][1] = pack2(z2, 0.f);
+                            }
+                        }
+                        philox_rounds<9, 10, S::PIPE>(w0, w1, a.key0, a.key1);
                     }
                 }
+                if constexpr (!S::WARP) {
+                    if (r == 0) put_edge<FC, LPB>(fx + ((par * 2 + 0) * BPC + bl) * NF, lib, q[0], G1[0]);
+                    if (r == FR - 1) put_edge<FC, LPB>(fx + ((par * 2 + 1) * BPC + bl) * NF, lib, q[FR - 1], G1[FR - 1]);
+                }
+                if constexpr (S::PIPE) row_update<S>(r, q, G1, G2, pend, pend0, left, right, a.Af);
             }
-            const bool cstep = CPL && ((m & 3) == 3);
             int32_t Gc1[R][C], Gc2[R][C];
             if constexpr (CPL) {
                 if (cstep) {
@@ -365,34 +506,32 @@ __global__ void __launch_bounds__(S::THREADS) level_kernel(const KArgs a) {
                             float s;
                             if constexpr (S::FLUCT) s = noise_amp_fluct(qc[i][j], rbc[i][j], a.isc, a.gc);
                             else s = noise_amp(qc[i][j], a.gc);
-                            Gc1[i][j] = __float2int_rn(s * zt[i][j][0]);
-                            Gc2[i][j] = __float2int_rn(s * zt[i][j][1]);
-                            zt[i][j][0] = zt[i][j][1] = 0.f;
+                            const int z = (i * C + j) / 2;
+                            const bool hi = (i * C + j) & 1;
+                            Gc1[i][j] = __float2int_rn(s * (hi ? hi2(zt[z][0]) : lo2(zt[z][0])));
+                            Gc2[i][j] = __float2int_rn(s * (hi ? hi2(zt[z][1]) : lo2(zt[z][1])));
                         }
-                }
-            }
-
-            if constexpr (SPLIT) {
-                const int par = m & 1;
-                put_edge<FC, LPB>(fx + ((par * 2 + 0) * BPC + bl) * NF, lib, q[0], G1[0]);
-                put_edge<FC, LPB>(fx + ((par * 2 + 1) * BPC + bl) * NF, lib, q[FR - 1], G1[FR - 1]);
-                if constexpr (CPL) {
-                    if (cstep) {
+#pragma unroll
+                    for (int z = 0; z < S::NZ; ++z) zt[z][0] = zt[z][1] = 0ull;
+                    if constexpr (!S::WARP) {
                         put_edge<C, LPB>(cx + bl * NC, lib, qc[0], Gc1[0]);
                         put_edge<C, LPB>(cx + (BPC + bl) * NC, lib, qc[R - 1], Gc1[R - 1]);
                     }
                 }
-                cluster_arrive();
             }
+            if constexpr (SPLIT) cluster_arrive();
+            else if constexpr (!S::WARP) __syncthreads();
 
             // ---- horizontal halo by shuffles within the band segment
             int32_t qL[FR], gL[FR], qR[FR], gR[FR];
+            if constexpr (!S::PIPE) {
 #pragma unroll
-            for (int r = 0; r < FR; ++r) {
-                qL[r] = __shfl_sync(kFull, q[r][FC - 1], left, LPB);
-                gL[r] = __shfl_sync(kFull, G2[r][FC - 1], left, LPB);
-                qR[r] = __shfl_sync(kFull, q[r][0], right, LPB);
-                gR[r] = __shfl_sync(kFull, G2[r][0], right, LPB);
+                for (int r = 0; r < FR; ++r) {
+                    qL[r] = __shfl_sync(kFull, q[r][FC - 1], left, LPB);
+                    gL[r] = __shfl_sync(kFull, G2[r][FC - 1], left, LPB);
+                    qR[r] = __shfl_sync(kFull, q[r][0], right, LPB);
+                    gR[r] = __shfl_sync(kFull, G2[r][0], right, LPB);
+                }
             }
             int32_t cqL[R], cgL[R], cqR[R], cgR[R];
             if constexpr (CPL) {
@@ -409,7 +548,7 @@ __global__ void __launch_bounds__(S::THREADS) level_kernel(const KArgs a) {
 
             // ---- vertical halo
             int32_t qU[FC], gU[FC], qD[FC], gD[FC];
-            int32_t keep1[FC], keep2[FC];   // old rows 1 and FR-2 (split barrier only)
+            [[maybe_unused]] int32_t keep1[FC], keep2[FC];
             int32_t cqU[C], cgU[C], cqD[C], cgD[C];
             if constexpr (S::WARP) {
 #pragma unroll
@@ -431,24 +570,13 @@ __global__ void __launch_bounds__(S::THREADS) level_kernel(const KArgs a) {
                     }
                 }
             } else {
-                const int par = m & 1;
                 int2* const ftop = fx + ((par * 2 + 0) * BPC) * NF;
                 int2* const fbot = fx + ((par * 2 + 1) * BPC) * NF;
                 int2* const ctop = cx;
                 int2* const cbot = cx + BPC * NC;
                 if constexpr (SPLIT) {
-                    flux_update_interior<FR, FC>(q, G1, G2, qL, gL, qR, gR, a.Af, keep1, keep2);
+                    if constexpr (!S::PIPE) flux_update_interior<FR, FC>(q, G1, G2, qL, gL, qR, gR, a.Af, keep1, keep2);
                     cluster_wait();
-                } else {
-                    put_edge<FC, LPB>(ftop + bl * NF, lib, q[0], G1[0]);
-                    put_edge<FC, LPB>(fbot + bl * NF, lib, q[FR - 1], G1[FR - 1]);
-                    if constexpr (CPL) {
-                        if (cstep) {
-                            put_edge<C, LPB>(ctop + bl * NC, lib, qc[0], Gc1[0]);
-                            put_edge<C, LPB>(cbot + bl * NC, lib, qc[R - 1], Gc1[R - 1]);
-                        }
-                    }
-                    block_or_cluster_sync<S>();
                 }
                 const int2* above = (bl > 0) ? fbot + (bl - 1) * NF
                                              : peer<S>(fbot + (BPC - 1) * NF, (rank + CL - 1) % CL);
@@ -466,8 +594,16 @@ __global__ void __launch_bounds__(S::THREADS) level_kernel(const KArgs a) {
                 }
             }
 
-            // ---- updates
-            if constexpr (SPLIT) {
+            // ---- first and last row, coarse step
+            if constexpr (S::PIPE) {
+#pragma unroll
+                for (int c = 0; c < FC; ++c) {
+                    const int32_t v0 = edge_flux(a.Af, q[0][c] - qU[c]);
+                    const int32_t v1 = edge_flux(a.Af, qD[c] - q[FR - 1][c]);
+                    q[0][c] += pend0[c] - v0 - gU[c];
+                    q[FR - 1][c] += pend[(FR - 1) & 1][c] + v1 + gD[c];
+                }
+            } else if constexpr (SPLIT) {
                 flux_update_boundary<FR, FC>(q, G1, G2, qU, gU, qD, gD, qL, gL, qR, gR, a.Af, keep1, keep2);
             } else {
                 flux_update<FR, FC>(q, G1, G2, qU, gU, qD, gD, qL, gL, qR, gR, a.Af);
