@@ -444,11 +444,11 @@ def level_launches(d, count, coupled):
     if d.band:                                   # zero + per wave (kernel + finish) + reduce
         return 2 + 2 * (-(-count // d.in_flight))
     if d.streamed:                               # zero + per wave (init, steps, observe, finish) + reduce
-        steps = 1 if d.persistent else d.M + (d.M // 4 if coupled else 0)
+        steps = 1 if d.persistent else d.M + (1 if coupled else 0)   # coarse steps share the fine launches, but the last
         return 2 + (-(-count // d.in_flight)) * (3 + steps)
     n = 2                                        # level kernel + reduce
     if d.batch_streamed > 0:                     # the split share: one launch per step, then the merge
-        n += 2 + (-(-d.batch_streamed // d.in_flight)) * (3 + d.M + d.M // 4) + 1
+        n += 2 + (-(-d.batch_streamed // d.in_flight)) * (3 + d.M + 1) + 1
     return n
 
 

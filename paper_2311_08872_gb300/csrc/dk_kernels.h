@@ -93,7 +93,7 @@ struct SArgs {
     long long sid0;              // sample id of the wave's first sample
     int32_t* q[2];               // [S][n][n] fine state, double buffered
     int32_t* qc[2];              // [S][n/2][n/2] coarse state, double buffered
-    float2* zt;                  // [S][n/2][n/2] coupled normal sums of the current coarse step
+    float2* zt[2];               // [S][n/2][n/2] coupled normal sums, buffer (m / 4) & 1 for fine step m
     double* tile_part;           // [S][tiles][2 kMaxObs + 2] per-tile observables
     const int32_t* q0f; const int32_t* qbf; const float* phif;
     const int32_t* q0c; const int32_t* qbc; const float* phic;

@@ -13,16 +13,27 @@
 // draws the normals of step m for the tile and for the halo cells (one extra
 // Philox call per halo cell pair, so the transfers G^m never go to memory),
 // and writes q^{m+1} and, for coupled samples, the running coarse sums zt.
-// After the fourth fine step of a coarse step, a coarse launch forms the
-// coarse transfers from qc and zt (tile and halo) and updates qc.  Kernel
-// boundaries order all reads and writes; in the default build the fine steps
-// are programmatic dependent launches that draw their noise before waiting
-// for the previous kernel.
+// After the fourth fine step of a coarse step the coarse transfers are formed
+// from qc and zt (tile and halo) and qc is updated, by extra CTAs of the next
+// fine step's launch (zt is double buffered by coarse step) or, after the last
+// fine step, by a launch of its own.  Kernel boundaries order all reads and
+// writes; in the default build the fine steps are programmatic dependent
+// launches that draw their noise before waiting for the previous kernel.
 //
 // Fine-step CTAs: 16 x 16 threads on a 32 x 64 tile, each thread a 2 x 4 block
 // of fine cells (two coarse cells); two builds, for 4 or 5 resident CTAs per
 // SM (at most 64 or 48 registers per thread), picked by the autotuner.
+// Neighbouring blocks exchange the state and transfer of their edge cells:
+// columns by shuffles, rows and the halo's cells through shared memory.
 // The coarse step and the observables use 32 x 32 tiles.
+//
+// What bounds it: the same XU and FMA pipes as the register kernels, plus the
+// halo's noise (128 extra pairs per 1024) and the tile's loads and stores.  The
+// state of the samples in flight stays in L2.  The coarse step had a launch of
+// its own every fourth step, which waited for the fine step's last wave and was
+// waited for: 512^2, 7 samples x 2048 steps 17.8 ms, now 15.6; 1024^2, 5 x 1024:
+// 21.1 ms, now 19.6 (packed FP32 noise, one component drawn in the halo and
+// only edge rows in shared memory, 17.9 KB instead of 29.4, included).
 #include <cstdint>
 
 #include "dk_device.cuh"
@@ -35,59 +46,65 @@ namespace {
 constexpr int kTile = 32;            // fine cells per tile side
 constexpr int kTc = kTile / 2;       // coarse cells per tile side (= threads per side)
 constexpr int kThreads = kTc * kTc;  // 256
-// fine-step tiles: FR x kFC fine cells with a one-cell halo in shared memory,
-// row lr = r - R0 + 1 (0 .. FR+1), column lc = c - C0 + 4 (3 .. kFC+4), so
-// that each thread's own four cells sit on a 16-byte boundary
+// fine-step tiles: FR x kFC fine cells, thread rows of two fine rows
 constexpr int kFC = 64;
-constexpr int kFW = kFC + 8;
 constexpr int kFR = 32;
 constexpr int kStreamVariants = 6;
 __host__ __device__ constexpr int fine_threads(int fr) { return 8 * fr; }
-__host__ __device__ constexpr int fine_smem(int fr) { return 3 * (fr + 2) * kFW * (int)sizeof(int32_t); }
+// words of shared memory of a fine tile: state and transfer of the first and
+// the last row of every thread row (FR/2 + 1 each: with the row below and the
+// row above the tile), and of the columns left and right of the tile
+__host__ __device__ constexpr int fine_words(int fr) { return 4 * (fr / 2 + 1) * kFC + 4 * fr; }
+// the same for a coarse tile, one cell row per thread row
+constexpr int kCoarseWords = 4 * (kTile + 1) * kTile + 4 * kTile;
+__host__ __device__ constexpr int fine_smem(int fr) {
+    return (int)sizeof(int32_t) * (fine_words(fr) > kCoarseWords ? fine_words(fr) : kCoarseWords);
+}
 
 __device__ __forceinline__ int wrapi(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
-
-// Transfers of the horizontal cell pair p (cells 2p, 2p+1 of the row-major
-// grid) at fine step m, from the pair's state qa, qb; the normals of the pair
-// are also added to the running coarse sums (z1, z2) in the register kernels'
-// order (cell 2p first).
-struct PairNoise {
-    int32_t g1a, g2a, g1b, g2b;
-};
 
 __device__ __forceinline__ uint4 pair_words(const SArgs& a, uint32_t p, int m, uint32_t c2, uint32_t c3) {
     return philox10(make_uint4(p, static_cast<uint32_t>(m), c2, c3), a.key0, a.key1);
 }
 
-// Box--Muller radii and directions of the pair's two cells.
-struct PairNormals {
-    float ra, ca, sa, rb, cb, sb;
+// Box--Muller radii and directions of four cells of a row (two cell pairs):
+// packed cells 0 and 2 (a) and cells 1 and 3 (b).
+struct RowNormals {
+    f32x2 ra, ca, sa, rb, cb, sb;
 };
 
-__device__ __forceinline__ PairNormals pair_normals(uint4 x) {
-    PairNormals z;
-    box_muller_polar(x.x, x.y, z.ra, z.ca, z.sa);
-    box_muller_polar(x.z, x.w, z.rb, z.cb, z.sb);
+__device__ __forceinline__ RowNormals row_normals(uint4 x, uint4 y) {
+    RowNormals z;
+    box_muller_polar2(x.x, x.y, y.x, y.y, z.ra, z.ca, z.sa);
+    box_muller_polar2(x.z, x.w, y.z, y.w, z.rb, z.cb, z.sb);
     return z;
+}
+
+// A halo pair's normals of one component: radius and cosine (rows) or sine
+// (columns) of its first and second cell.
+struct HaloNormals {
+    float ra, da, rb, db;
+};
+
+__device__ __forceinline__ HaloNormals halo_normals(uint4 x, bool rows) {
+    HaloNormals h;
+    float ca, sa, cb, sb;
+    box_muller_polar(x.x, x.y, h.ra, ca, sa);
+    box_muller_polar(x.z, x.w, h.rb, cb, sb);
+    h.da = rows ? ca : sa;
+    h.db = rows ? cb : sb;
+    return h;
 }
 
 // Makes the normals exist at this point of the program (an empty asm
 // statement that reads and writes them): the compiler keeps their arithmetic
 // before a later volatile asm statement such as the grid dependency wait.
-__device__ __forceinline__ void pin(PairNormals& z) {
-    asm volatile("" : "+f"(z.ra), "+f"(z.ca), "+f"(z.sa), "+f"(z.rb), "+f"(z.cb), "+f"(z.sb));
+__device__ __forceinline__ void pin(RowNormals& z) {
+    asm volatile("" : "+l"(z.ra), "+l"(z.ca), "+l"(z.sa), "+l"(z.rb), "+l"(z.cb), "+l"(z.sb));
 }
-
-// The transfers from the pair's normals (drawn earlier).
-__device__ __forceinline__ PairNoise pair_noise_n(const SArgs& a, const PairNormals& z, int32_t qa, int32_t qb,
-                                                  float& z1, float& z2) {
-    const float ta = noise_amp(qa, a.gf) * z.ra, tb = noise_amp(qb, a.gf) * z.rb;
-    z1 = fmaf(z.rb, z.cb, fmaf(z.ra, z.ca, z1));
-    z2 = fmaf(z.rb, z.sb, fmaf(z.ra, z.sa, z2));
-    return {__float2int_rn(ta * z.ca), __float2int_rn(ta * z.sa), __float2int_rn(tb * z.cb),
-            __float2int_rn(tb * z.sb)};
+__device__ __forceinline__ void pin(HaloNormals& z) {
+    asm volatile("" : "+f"(z.ra), "+f"(z.da), "+f"(z.rb), "+f"(z.db));
 }
-
 
 // Programmatic dependent launch: let the next kernel in the stream start its
 // CTAs once every CTA of this one has started, and wait until the previous
@@ -129,6 +146,12 @@ __device__ __forceinline__ T ldg(const T* p) {
     else return *p;
 }
 
+// Four words of shared memory.
+__device__ __forceinline__ void ld4(int32_t (&v)[4], const int32_t* p) {
+    const int4 x = *reinterpret_cast<const int4*>(p);
+    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+}
+
 // Fine step m of the FR x 64 tile at (R0, C0) of sample s: noise of step m on
 // the tile and its halo, then q^{m+1}.  Thread (tx, ty) of the 16 x FR/2
 // threads owns the 2 x 4 fine block at (R0 + 2 ty, C0 + 4 tx) = 2 coarse cells.
@@ -136,14 +159,15 @@ __device__ __forceinline__ T ldg(const T* p) {
 // persistent kernel, whether any warp's wait timed out (`stop`): then no thread
 // stores and the function returns true.
 // With PDL (one launch per step, launched as a programmatic dependent of the
-// previous kernel in the stream) the Philox words of the tile and its halo,
-// which depend on no state, are drawn before the wait for the previous step:
-// CTAs that start while the previous step's last wave still runs do that part
-// of their work in its shadow.
+// previous kernel in the stream) the normals of the tile and its halo, which
+// depend on no state, are drawn before the wait for the previous step: CTAs
+// that start while the previous step's last wave still runs do that part of
+// their work in its shadow.
 template <int FR, bool PERSIST, bool PDL = false>
 __device__ __forceinline__ bool fine_tile(const SArgs& a, int s, int R0, int C0, int m, int32_t* smem, int stop) {
     constexpr int kHaloPairs = 64 + 2 * FR;   // 2 x 32 pairs in the halo rows, one per row in the halo columns
     static_assert(!(PDL && PERSIST), "the persistent launch has no previous grid to wait for");
+    static_assert(kHaloPairs <= fine_threads(FR), "one halo pair per thread");
     const int n = a.n;
     const int t = threadIdx.x;
     const int tx = t % 16, ty = t / 16;
@@ -153,10 +177,12 @@ __device__ __forceinline__ bool fine_tile(const SArgs& a, int s, int R0, int C0,
     int32_t* qout = a.q[(m + 1) & 1] + base;
     uint32_t c2, c3;
     sample_counter(a, s, c2, c3);
-    // halo cell pair of this thread (t < kHaloPairs): row halo (t < 64) or column halo
+    // halo cell pair of this thread (t < kHaloPairs): row halo (t < 64, whole
+    // warps) or column halo
+    const bool has_halo = t < kHaloPairs, row_halo = t < 64;
     int hr = 0, hc = 0;
-    auto halo_cell = [&]() {
-        if (t < 64) {
+    if (has_halo) {
+        if (row_halo) {
             hr = wrapi((t >> 5) ? R0 + FR : R0 - 1, n);
             hc = C0 + 2 * (t & 31);
         } else {
@@ -164,157 +190,126 @@ __device__ __forceinline__ bool fine_tile(const SArgs& a, int s, int R0, int C0,
             hr = R0 + u % FR;
             hc = wrapi(u / FR ? C0 + kFC : C0 - 2, n);
         }
-    };
-    PairNormals w[2][2], hw{};
+    }
+    const uint32_t hp = static_cast<uint32_t>((hr * n + hc) >> 1);
+    RowNormals w[2];
+    HaloNormals hw{};
     if constexpr (PDL) {
-        if (t < kHaloPairs) halo_cell();
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const uint32_t p = static_cast<uint32_t>(((r0 + i) * n + c0) >> 1);
-            w[i][0] = pair_normals(pair_words(a, p, m, c2, c3));
-            w[i][1] = pair_normals(pair_words(a, p + 1, m, c2, c3));
+            w[i] = row_normals(pair_words(a, p, m, c2, c3), pair_words(a, p + 1, m, c2, c3));
         }
-        if (t < kHaloPairs) hw = pair_normals(pair_words(a, static_cast<uint32_t>((hr * n + hc) >> 1), m, c2, c3));
+        if (has_halo) hw = halo_normals(pair_words(a, hp, m, c2, c3), row_halo);
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            pin(w[i][0]);
-            pin(w[i][1]);
-        }
+        for (int i = 0; i < 2; ++i) pin(w[i]);
         pin(hw);
         wait_previous_grid();
     }
 
-    int32_t (*sq)[kFW] = reinterpret_cast<int32_t (*)[kFW]>(smem);
-    int32_t (*s1)[kFW] = reinterpret_cast<int32_t (*)[kFW]>(smem + (FR + 2) * kFW);
-    int32_t (*s2)[kFW] = reinterpret_cast<int32_t (*)[kFW]>(smem + 2 * (FR + 2) * kFW);
+    // first rows (q, G1; row FR/2: the row below the tile), last rows (row 0: the
+    // row above it), columns left and right of it (q, G2)
+    int32_t (*tq)[kFC] = reinterpret_cast<int32_t (*)[kFC]>(smem);
+    int32_t (*tg)[kFC] = tq + FR / 2 + 1;
+    int32_t (*bq)[kFC] = tg + FR / 2 + 1;
+    int32_t (*bg)[kFC] = bq + FR / 2 + 1;
+    int2* const sl = reinterpret_cast<int2*>(bg + FR / 2 + 1);   // [FR]
+    int2* const sr = sl + FR;                                    // [FR]
 
     // own 2x4 block: state, normals of step m, transfers; coupled sums of its
     // two coarse cells in the register kernels' order
-    const int lr0 = 2 * ty + 1, lc0 = 4 * tx + 4;
     int32_t q[2][4], G1[2][4], G2[2][4];
-    float4* const zp = reinterpret_cast<float4*>(a.zt + (size_t)s * a.nc * a.nc + (size_t)(r0 >> 1) * a.nc + (c0 >> 1));
-    float z[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+    float4* const zp = reinterpret_cast<float4*>(a.zt[(m >> 2) & 1] + (size_t)s * a.nc * a.nc +
+                                                 (size_t)(r0 >> 1) * a.nc + (c0 >> 1));
+    f32x2 z1 = 0ull, z2 = 0ull;
     if (a.coupled && (m & 3) != 0) {
         const float4 v = ldg<PERSIST>(zp);
-        z[0][0] = v.x; z[0][1] = v.y; z[1][0] = v.z; z[1][1] = v.w;
+        z1 = pack2(v.x, v.z);
+        z2 = pack2(v.y, v.w);
     }
+    const f32x2 gf2 = pack2(a.gf, a.gf);
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
         const int4 v = ldg<PERSIST>(reinterpret_cast<const int4*>(qin + (size_t)(r0 + i) * n + c0));
         q[i][0] = v.x; q[i][1] = v.y; q[i][2] = v.z; q[i][3] = v.w;
-        const uint32_t p = static_cast<uint32_t>(((r0 + i) * n + c0) >> 1);
         if constexpr (!PDL) {
-            w[i][0] = pair_normals(pair_words(a, p, m, c2, c3));
-            w[i][1] = pair_normals(pair_words(a, p + 1, m, c2, c3));
+            const uint32_t p = static_cast<uint32_t>(((r0 + i) * n + c0) >> 1);
+            w[i] = row_normals(pair_words(a, p, m, c2, c3), pair_words(a, p + 1, m, c2, c3));
         }
-        const PairNoise g = pair_noise_n(a, w[i][0], v.x, v.y, z[0][0], z[0][1]);
-        const PairNoise h = pair_noise_n(a, w[i][1], v.z, v.w, z[1][0], z[1][1]);
-        G1[i][0] = g.g1a; G2[i][0] = g.g2a; G1[i][1] = g.g1b; G2[i][1] = g.g2b;
-        G1[i][2] = h.g1a; G2[i][2] = h.g2a; G1[i][3] = h.g1b; G2[i][3] = h.g2b;
-        if constexpr (!PERSIST) {
-            *reinterpret_cast<int4*>(&sq[lr0 + i][lc0]) = v;
-            *reinterpret_cast<int4*>(&s1[lr0 + i][lc0]) = make_int4(g.g1a, g.g1b, h.g1a, h.g1b);
-            *reinterpret_cast<int4*>(&s2[lr0 + i][lc0]) = make_int4(g.g2a, g.g2b, h.g2a, h.g2b);
+        const f32x2 ta = mul2(noise_amp2(v.x, v.z, gf2), w[i].ra), tb = mul2(noise_amp2(v.y, v.w, gf2), w[i].rb);
+        const f32x2 a1 = mul2(ta, w[i].ca), a2 = mul2(ta, w[i].sa), b1 = mul2(tb, w[i].cb), b2 = mul2(tb, w[i].sb);
+        G1[i][0] = __float2int_rn(lo2(a1)); G1[i][1] = __float2int_rn(lo2(b1));
+        G1[i][2] = __float2int_rn(hi2(a1)); G1[i][3] = __float2int_rn(hi2(b1));
+        G2[i][0] = __float2int_rn(lo2(a2)); G2[i][1] = __float2int_rn(lo2(b2));
+        G2[i][2] = __float2int_rn(hi2(a2)); G2[i][3] = __float2int_rn(hi2(b2));
+        z1 = fma2(w[i].rb, w[i].cb, fma2(w[i].ra, w[i].ca, z1));
+        z2 = fma2(w[i].rb, w[i].sb, fma2(w[i].ra, w[i].sa, z2));
+    }
+    // halo: rows R0-1 and R0+FR (32 pairs each, both cells, component 1) and
+    // columns C0-1 and C0+kFC (one pair per row, the cell next to the tile,
+    // component 2)
+    int2 hv = make_int2(0, 0), hg = make_int2(0, 0);
+    if (has_halo) {
+        hv = ldg<PERSIST>(reinterpret_cast<const int2*>(qin + (size_t)hr * n + hc));
+        if constexpr (!PDL) hw = halo_normals(pair_words(a, hp, m, c2, c3), row_halo);
+        hg.x = __float2int_rn(noise_amp(hv.x, a.gf) * hw.ra * hw.da);
+        hg.y = __float2int_rn(noise_amp(hv.y, a.gf) * hw.rb * hw.db);
+    }
+    // in the persistent kernel shared memory is free once every warp has finished the previous item
+    if constexpr (PERSIST) __syncthreads();
+    *reinterpret_cast<int4*>(&tq[ty][4 * tx]) = make_int4(q[0][0], q[0][1], q[0][2], q[0][3]);
+    *reinterpret_cast<int4*>(&tg[ty][4 * tx]) = make_int4(G1[0][0], G1[0][1], G1[0][2], G1[0][3]);
+    *reinterpret_cast<int4*>(&bq[ty + 1][4 * tx]) = make_int4(q[1][0], q[1][1], q[1][2], q[1][3]);
+    *reinterpret_cast<int4*>(&bg[ty + 1][4 * tx]) = make_int4(G1[1][0], G1[1][1], G1[1][2], G1[1][3]);
+    if (has_halo) {
+        if (row_halo) {
+            const bool above = t < 32;
+            *reinterpret_cast<int2*>((above ? bq[0] : tq[FR / 2]) + 2 * (t & 31)) = hv;
+            *reinterpret_cast<int2*>((above ? bg[0] : tg[FR / 2]) + 2 * (t & 31)) = hg;
+        } else {
+            const int u = t - 64;
+            if (u < FR) sl[u] = make_int2(hv.y, hg.y);
+            else sr[u - FR] = make_int2(hv.x, hg.x);
         }
     }
-    // halo: rows R0-1 and R0+FR (32 pairs each: state and G1), columns C0-1
-    // and C0+kFC (one pair per row: state and G2 of the cell next to the tile);
-    // (hq, hg): the state and transfer a halo thread stores
-    int32_t* hq = nullptr;
-    int32_t* hg = nullptr;
-    int2 hqv = make_int2(0, 0), hgv = make_int2(0, 0);
-    bool hpair = false;
-    if (t < kHaloPairs) {
-        float d1 = 0.f, d2 = 0.f;   // halo normals do not enter this tile's coarse sums
-        if (t < 64) {
-            const int side = t >> 5, k = t & 31;
-            const int r = PDL ? hr : wrapi(side ? R0 + FR : R0 - 1, n), c = PDL ? hc : C0 + 2 * k;
-            const int2 v = ldg<PERSIST>(reinterpret_cast<const int2*>(qin + (size_t)r * n + c));
-            const PairNormals x = PDL ? hw : pair_normals(pair_words(a, static_cast<uint32_t>((r * n + c) >> 1), m, c2, c3));
-            const PairNoise g = pair_noise_n(a, x, v.x, v.y, d1, d2);
-            const int lr = side ? FR + 1 : 0;
-            if constexpr (PERSIST) {
-                hq = &sq[lr][4 + 2 * k];
-                hg = &s1[lr][4 + 2 * k];
-                hqv = v;
-                hgv = make_int2(g.g1a, g.g1b);
-                hpair = true;
-            } else {
-                *reinterpret_cast<int2*>(&sq[lr][4 + 2 * k]) = v;
-                *reinterpret_cast<int2*>(&s1[lr][4 + 2 * k]) = make_int2(g.g1a, g.g1b);
-            }
-        } else {
-            const int u = t - 64, side = u / FR, rr = u % FR;
-            const int r = PDL ? hr : R0 + rr, c = PDL ? hc : wrapi(side ? C0 + kFC : C0 - 2, n);
-            const int2 v = ldg<PERSIST>(reinterpret_cast<const int2*>(qin + (size_t)r * n + c));
-            const PairNormals x = PDL ? hw : pair_normals(pair_words(a, static_cast<uint32_t>((r * n + c) >> 1), m, c2, c3));
-            const PairNoise g = pair_noise_n(a, x, v.x, v.y, d1, d2);
-            if constexpr (PERSIST) {
-                hq = side ? &sq[rr + 1][kFC + 4] : &sq[rr + 1][3];
-                hg = side ? &s2[rr + 1][kFC + 4] : &s2[rr + 1][3];
-                hqv.x = side ? v.x : v.y;
-                hgv.x = side ? g.g2a : g.g2b;
-            } else if (side) {
-                sq[rr + 1][kFC + 4] = v.x;
-                s2[rr + 1][kFC + 4] = g.g2a;
-            } else {
-                sq[rr + 1][3] = v.y;
-                s2[rr + 1][3] = g.g2b;
-            }
-        }
+    // columns: the neighbouring lanes of the 16-lane thread row
+    int32_t ql[2], qr[2], gl[2], gr[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        ql[i] = __shfl_up_sync(0xffffffffu, q[i][3], 1, 16);
+        gl[i] = __shfl_up_sync(0xffffffffu, G2[i][3], 1, 16);
+        qr[i] = __shfl_down_sync(0xffffffffu, q[i][0], 1, 16);
+        gr[i] = __shfl_down_sync(0xffffffffu, G2[i][0], 1, 16);
     }
     if constexpr (PERSIST) {
-        // shared memory is free once every warp has finished the previous item
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            *reinterpret_cast<int4*>(&sq[lr0 + i][lc0]) = make_int4(q[i][0], q[i][1], q[i][2], q[i][3]);
-            *reinterpret_cast<int4*>(&s1[lr0 + i][lc0]) = make_int4(G1[i][0], G1[i][1], G1[i][2], G1[i][3]);
-            *reinterpret_cast<int4*>(&s2[lr0 + i][lc0]) = make_int4(G2[i][0], G2[i][1], G2[i][2], G2[i][3]);
-        }
-        if (t < kHaloPairs) {
-            if (hpair) {
-                *reinterpret_cast<int2*>(hq) = hqv;
-                *reinterpret_cast<int2*>(hg) = hgv;
-            } else {
-                *hq = hqv.x;
-                *hg = hgv.x;
-            }
-        }
         if (__syncthreads_or(stop)) return true;
     } else {
         __syncthreads();
     }
 
-    unsigned bad = 0;
+    if (tx == 0) {
+        const int4 v = *reinterpret_cast<const int4*>(sl + 2 * ty);
+        ql[0] = v.x; gl[0] = v.y; ql[1] = v.z; gl[1] = v.w;
+    }
+    if (tx == 15) {
+        const int4 v = *reinterpret_cast<const int4*>(sr + 2 * ty);
+        qr[0] = v.x; gr[0] = v.y; qr[1] = v.z; gr[1] = v.w;
+    }
     int32_t up[4], dn[4], gu[4], gd[4];
-    {
-        const int4 a0 = *reinterpret_cast<const int4*>(&sq[lr0 - 1][lc0]);
-        const int4 a1 = *reinterpret_cast<const int4*>(&sq[lr0 + 2][lc0]);
-        const int4 b0 = *reinterpret_cast<const int4*>(&s1[lr0 - 1][lc0]);
-        const int4 b1 = *reinterpret_cast<const int4*>(&s1[lr0 + 2][lc0]);
-        up[0] = a0.x; up[1] = a0.y; up[2] = a0.z; up[3] = a0.w;
-        dn[0] = a1.x; dn[1] = a1.y; dn[2] = a1.z; dn[3] = a1.w;
-        gu[0] = b0.x; gu[1] = b0.y; gu[2] = b0.z; gu[3] = b0.w;
-        gd[0] = b1.x; gd[1] = b1.y; gd[2] = b1.z; gd[3] = b1.w;
-    }
-    int32_t ql[2], qr[2], gl[2], gr[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        ql[i] = sq[lr0 + i][lc0 - 1];
-        qr[i] = sq[lr0 + i][lc0 + 4];
-        gl[i] = s2[lr0 + i][lc0 - 1];
-        gr[i] = s2[lr0 + i][lc0 + 4];
-    }
+    ld4(up, &bq[ty][4 * tx]);
+    ld4(gu, &bg[ty][4 * tx]);
+    ld4(dn, &tq[ty + 1][4 * tx]);
+    ld4(gd, &tg[ty + 1][4 * tx]);
     // each edge flux once per block, as in the register kernels
     flux_update<2, 4>(q, G1, G2, up, gu, dn, gd, ql, gl, qr, gr, a.Af);
+    unsigned bad = 0;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) bad |= (static_cast<uint32_t>(q[i][j]) + 0x40000000u) >> 31;
         *reinterpret_cast<int4*>(qout + (size_t)(r0 + i) * n + c0) = make_int4(q[i][0], q[i][1], q[i][2], q[i][3]);
     }
-    if (a.coupled) *zp = make_float4(z[0][0], z[0][1], z[1][0], z[1][1]);
+    if (a.coupled) *zp = make_float4(lo2(z1), lo2(z2), hi2(z1), hi2(z2));
     if (bad) atomicOr(a.err, kErrRange);
     return false;
 }
@@ -322,61 +317,108 @@ __device__ __forceinline__ bool fine_tile(const SArgs& a, int s, int R0, int C0,
 // Coarse step cn (after fine step 4 cn + 3) of the 32 x 32 coarse tile
 // (T1, T2) of sample s: transfers from qc^cn and the coupled sums on the tile
 // and its halo (no corners: the stencil does not use them), then qc^{cn+1}.
+// Thread (tx, ty) of the 8 x 32 threads owns four cells of row ty; the 128 halo
+// cells belong to the first 128 threads.
 template <bool PERSIST>
 __device__ __forceinline__ void coarse_tile(const SArgs& a, int s, int T1, int T2, int cn, int32_t* smem) {
+    static_assert(kThreads == 8 * kTile && 4 * kTile <= kThreads, "8 x 32 threads, one halo cell each");
     const int nc = a.nc;
     const size_t base = (size_t)s * nc * nc;
     const int32_t* qin = a.qc[cn & 1] + base;
     int32_t* qout = a.qc[(cn + 1) & 1] + base;
-    const float2* zt = a.zt + base;
-    int32_t (*sq)[kTile + 2] = reinterpret_cast<int32_t (*)[kTile + 2]>(smem);
-    int2 (*sg)[kTile + 2] = reinterpret_cast<int2 (*)[kTile + 2]>(smem + (kTile + 2) * (kTile + 2));
+    const float2* zt = a.zt[cn & 1] + base;
+    int32_t (*tq)[kTile] = reinterpret_cast<int32_t (*)[kTile]>(smem);
+    int32_t (*tg)[kTile] = tq + kTile + 1;
+    int32_t (*bq)[kTile] = tg + kTile + 1;
+    int32_t (*bg)[kTile] = bq + kTile + 1;
+    int2* const sl = reinterpret_cast<int2*>(bg + kTile + 1);
+    int2* const sr = sl + kTile;
+    const int t = threadIdx.x, tx = t % 8, ty = t / 8;
     const int R0 = T1 * kTile, C0 = T2 * kTile;
-    for (int k = threadIdx.x; k < (kTile + 2) * (kTile + 2); k += kThreads) {
-        const int lr = k / (kTile + 2), lc = k % (kTile + 2);
-        if ((lr == 0 || lr == kTile + 1) && (lc == 0 || lc == kTile + 1)) continue;
-        const int gr = wrapi(R0 + lr - 1, nc), gcol = wrapi(C0 + lc - 1, nc);
-        const int32_t qv = ldg<PERSIST>(qin + (size_t)gr * nc + gcol);
-        const float2 z = ldg<PERSIST>(zt + (size_t)gr * nc + gcol);
-        const float amp = noise_amp(qv, a.gc);
-        sq[lr][lc] = qv;
-        sg[lr][lc] = make_int2(__float2int_rn(amp * z.x), __float2int_rn(amp * z.y));
+    const size_t x = (size_t)(R0 + ty) * nc + C0 + 4 * tx;
+    const int4 qv = ldg<PERSIST>(reinterpret_cast<const int4*>(qin + x));
+    const float4 za = ldg<PERSIST>(reinterpret_cast<const float4*>(zt + x));
+    const float4 zb = ldg<PERSIST>(reinterpret_cast<const float4*>(zt + x) + 1);
+    int32_t q[1][4] = {{qv.x, qv.y, qv.z, qv.w}}, G1[1][4], G2[1][4];
+    const float w1[4] = {za.x, za.z, zb.x, zb.z}, w2[4] = {za.y, za.w, zb.y, zb.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float amp = noise_amp(q[0][j], a.gc);
+        G1[0][j] = __float2int_rn(amp * w1[j]);
+        G2[0][j] = __float2int_rn(amp * w2[j]);
     }
+    // one row: first and last row of the block are the same words
+    const int4 g1v = make_int4(G1[0][0], G1[0][1], G1[0][2], G1[0][3]);
+    *reinterpret_cast<int4*>(&tq[ty][4 * tx]) = qv;
+    *reinterpret_cast<int4*>(&tg[ty][4 * tx]) = g1v;
+    *reinterpret_cast<int4*>(&bq[ty + 1][4 * tx]) = qv;
+    *reinterpret_cast<int4*>(&bg[ty + 1][4 * tx]) = g1v;
+    if (t < 4 * kTile) {
+        const int side = t / kTile, k = t % kTile;   // rows above, below; columns left, right
+        const int r = side < 2 ? wrapi(side ? R0 + kTile : R0 - 1, nc) : R0 + k;
+        const int c = side < 2 ? C0 + k : wrapi(side == 3 ? C0 + kTile : C0 - 1, nc);
+        const int32_t v = ldg<PERSIST>(qin + (size_t)r * nc + c);
+        const float2 z = ldg<PERSIST>(zt + (size_t)r * nc + c);
+        const int32_t g = __float2int_rn(noise_amp(v, a.gc) * (side < 2 ? z.x : z.y));
+        if (side == 0) {
+            bq[0][k] = v;
+            bg[0][k] = g;
+        } else if (side == 1) {
+            tq[kTile][k] = v;
+            tg[kTile][k] = g;
+        } else {
+            (side == 2 ? sl : sr)[k] = make_int2(v, g);
+        }
+    }
+    int32_t ql[1] = {__shfl_up_sync(0xffffffffu, q[0][3], 1, 8)}, gl[1] = {__shfl_up_sync(0xffffffffu, G2[0][3], 1, 8)};
+    int32_t qr[1] = {__shfl_down_sync(0xffffffffu, q[0][0], 1, 8)}, gr[1] = {__shfl_down_sync(0xffffffffu, G2[0][0], 1, 8)};
     __syncthreads();
-    unsigned bad = 0;
-    for (int k = threadIdx.x; k < kTile * kTile; k += kThreads) {
-        const int lr = k / kTile + 1, lc = k % kTile + 1;
-        const int32_t x = sq[lr][lc];
-        const int32_t d = edge_flux(a.Ac, sq[lr + 1][lc] - x) - edge_flux(a.Ac, x - sq[lr - 1][lc]) +
-                          edge_flux(a.Ac, sq[lr][lc + 1] - x) - edge_flux(a.Ac, x - sq[lr][lc - 1]);
-        const int32_t v = x + d + (sg[lr + 1][lc].x - sg[lr - 1][lc].x) + (sg[lr][lc + 1].y - sg[lr][lc - 1].y);
-        qout[(size_t)(R0 + lr - 1) * nc + (C0 + lc - 1)] = v;
-        bad |= (static_cast<uint32_t>(v) + 0x40000000u) >> 31;
+    if (tx == 0) {
+        ql[0] = sl[ty].x;
+        gl[0] = sl[ty].y;
     }
+    if (tx == 7) {
+        qr[0] = sr[ty].x;
+        gr[0] = sr[ty].y;
+    }
+    int32_t up[4], dn[4], gu[4], gd[4];
+    ld4(up, &bq[ty][4 * tx]);
+    ld4(gu, &bg[ty][4 * tx]);
+    ld4(dn, &tq[ty + 1][4 * tx]);
+    ld4(gd, &tg[ty + 1][4 * tx]);
+    flux_update<1, 4>(q, G1, G2, up, gu, dn, gd, ql, gl, qr, gr, a.Ac);
+    *reinterpret_cast<int4*>(qout + x) = make_int4(q[0][0], q[0][1], q[0][2], q[0][3]);
+    unsigned bad = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) bad |= (static_cast<uint32_t>(q[0][j]) + 0x40000000u) >> 31;
     if (bad) atomicOr(a.err, kErrRange);
 }
 
 // One launch per fine step m (PDL: launched as a programmatic dependent of the
-// previous kernel, which it waits for after drawing its Philox words).
+// previous kernel, which it waits for after drawing its normals).  The CTAs
+// past the samples' (blockIdx.z >= count, launched for the first fine step of a
+// coarse step but the first) do the coarse step that ended with the previous
+// fine step: its state and sums are other buffers than the fine step's, so the
+// two share the launch instead of following one another.
 template <int FR, int MINB, bool PDL>
 __global__ void __launch_bounds__(fine_threads(FR), MINB) stream_fine_kernel(const SArgs a, int m) {
     if constexpr (PDL) launch_dependents();
-    const int s = blockIdx.z;
-    if (s >= a.count) return;
     extern __shared__ __align__(16) int32_t smem_fine[];
-    fine_tile<FR, false, PDL>(a, s, blockIdx.y * FR, blockIdx.x * kFC, m, smem_fine, 0);
+    if (blockIdx.z >= a.count) {
+        if constexpr (PDL) wait_previous_grid();
+        const int k = ((blockIdx.z - a.count) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+        const int tpr = a.nc / kTile, s = k / (tpr * tpr), r = k - s * tpr * tpr;
+        if (s < a.count) coarse_tile<false>(a, s, r / tpr, r % tpr, (m >> 2) - 1, smem_fine);
+        return;
+    }
+    fine_tile<FR, false, PDL>(a, blockIdx.z, blockIdx.y * FR, blockIdx.x * kFC, m, smem_fine, 0);
 }
 
-// One launch per coarse step cn (after fine step 4 cn + 3).  It lets the next
-// fine step's CTAs start early; launched as a dependent launch itself (with the
-// dependent fine steps), its CTAs are placed while the fine step's last wave
-// runs and wait there for it to finish.
+// The last coarse step, after the last fine step.
 __global__ void __launch_bounds__(kThreads) stream_coarse_kernel(const SArgs a, int cn) {
-    launch_dependents();
-    wait_previous_grid();
     const int s = blockIdx.y;
     if (s >= a.count) return;
-    __shared__ __align__(16) int32_t smem_coarse[(kTile + 2) * (kTile + 2) * 3];
+    __shared__ __align__(16) int32_t smem_coarse[kCoarseWords];
     const int tpr = a.nc / kTile;
     coarse_tile<false>(a, s, blockIdx.x / tpr, blockIdx.x % tpr, cn, smem_coarse);
 }
@@ -679,9 +721,17 @@ static size_t counter_bytes(int n, int S) {
     return (((size_t)S * (ft + ct) * sizeof(unsigned) + 15) & ~(size_t)15) + 16;
 }
 
+// Bytes that the steps of one sample work on: of the two buffers of coupled
+// sums, one at a time.
+static size_t sample_working_set(int n) {
+    const size_t nc = n / 2, tiles = (size_t)(n / kTile) * (n / kTile);
+    return (size_t)n * n * 2 * sizeof(int32_t) + nc * nc * (2 * sizeof(int32_t) + sizeof(float2)) +
+           tiles * (2 * kMaxObs + 2) * sizeof(double) + counter_bytes(n, 1);
+}
+
 size_t stream_bytes(int n, int S) {
     const size_t nc = n / 2, tiles = (size_t)(n / kTile) * (n / kTile);
-    return (size_t)S * ((size_t)n * n * 2 * sizeof(int32_t) + nc * nc * (2 * sizeof(int32_t) + sizeof(float2)) +
+    return (size_t)S * ((size_t)n * n * 2 * sizeof(int32_t) + nc * nc * 2 * (sizeof(int32_t) + sizeof(float2)) +
                         tiles * (2 * kMaxObs + 2) * sizeof(double)) +
            counter_bytes(n, S);
 }
@@ -742,7 +792,7 @@ cudaError_t stream_variant_info(int n, int variant, VariantInfo* out) {
 int stream_inflight(int n, size_t budget, int variant) {
     // the largest count that fits the budget, lowered while a smaller count
     // fills the last wave of fine-step CTAs clearly better
-    const int s_max = (int)std::max<size_t>(1, budget / stream_bytes(n, 1));
+    const int s_max = (int)std::max<size_t>(1, budget / sample_working_set(n));
     VariantInfo vi{};
     if (stream_variant_info(n, variant, &vi) != cudaSuccess || !vi.supported) return s_max;
     const long long resident = vi.max_ctas, ctas = (long long)(n / kFC) * (n / vi.tile_rows);
@@ -767,7 +817,8 @@ void stream_carve(SArgs* a, void* buf, int n, int S) {
     a->q[1] = reinterpret_cast<int32_t*>(p); p += cf * sizeof(int32_t);
     a->qc[0] = reinterpret_cast<int32_t*>(p); p += cc * sizeof(int32_t);
     a->qc[1] = reinterpret_cast<int32_t*>(p); p += cc * sizeof(int32_t);
-    a->zt = reinterpret_cast<float2*>(p); p += cc * sizeof(float2);
+    a->zt[0] = reinterpret_cast<float2*>(p); p += cc * sizeof(float2);
+    a->zt[1] = reinterpret_cast<float2*>(p); p += cc * sizeof(float2);
     a->tile_part = reinterpret_cast<double*>(p);
     p += (size_t)S * (n / kTile) * (n / kTile) * (2 * kMaxObs + 2) * sizeof(double);
     a->counters = p;
@@ -800,7 +851,14 @@ cudaError_t stream_run(const KArgs& k, SArgs a, int S, int variant, cudaStream_t
     for (long long done = 0; done < k.count; done += S) {
         a.sid0 = k.first + done;
         a.count = (int)std::min<long long>(S, k.count - done);
-        const dim3 grid(tiles, a.count), cgrid(ctiles, a.count), fgrid(n / kFC, n / fr, a.count);
+        const dim3 grid(tiles, a.count), cgrid(ctiles, a.count);
+        // CTAs of fine step m: the samples' fine tiles, and after them the coarse
+        // tiles of the coarse step that ended before it
+        const int ftiles = (n / kFC) * (n / fr);
+        auto step_grid = [&](int m) {
+            const int extra = a.coupled && m > 0 && (m & 3) == 0 ? (int)((a.count * (long long)ctiles + ftiles - 1) / ftiles) : 0;
+            return dim3(n / kFC, n / fr, a.count + extra);
+        };
         stream_init_kernel<<<grid, kThreads, 0, st>>>(a);
         if (persistent_variant(variant)) {
             // one grid of resident CTAs (at most one per item) takes the items in order
@@ -817,32 +875,27 @@ cudaError_t stream_run(const KArgs& k, SArgs a, int S, int variant, cudaStream_t
             attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
             attr[0].val.programmaticStreamSerializationAllowed = 1;
             cudaLaunchConfig_t cfg{};
-            cfg.gridDim = fgrid;
             cfg.blockDim = dim3(fine_threads(kFR));
             cfg.dynamicSmemBytes = fine_smem(kFR);
             cfg.stream = st;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            cudaLaunchConfig_t ccfg = cfg;
-            ccfg.gridDim = cgrid;
-            ccfg.blockDim = dim3(kThreads);
-            ccfg.dynamicSmemBytes = 0;
             for (int m = 0; m < a.M; ++m) {
+                cfg.gridDim = step_grid(m);
                 e = variant == 4 ? cudaLaunchKernelEx(&cfg, stream_fine_kernel<kFR, 4, true>, a, m)
                                  : cudaLaunchKernelEx(&cfg, stream_fine_kernel<kFR, 5, true>, a, m);
-                if (e == cudaSuccess && a.coupled && (m & 3) == 3)
-                    e = cudaLaunchKernelEx(&ccfg, stream_coarse_kernel, a, m >> 2);
                 if (e != cudaSuccess) return e;
             }
         } else {
             for (int m = 0; m < a.M; ++m) {
                 if (variant == 0)
-                    stream_fine_kernel<kFR, 4, false><<<fgrid, fine_threads(kFR), fine_smem(kFR), st>>>(a, m);
+                    stream_fine_kernel<kFR, 4, false><<<step_grid(m), fine_threads(kFR), fine_smem(kFR), st>>>(a, m);
                 else
-                    stream_fine_kernel<kFR, 5, false><<<fgrid, fine_threads(kFR), fine_smem(kFR), st>>>(a, m);
-                if (a.coupled && (m & 3) == 3) stream_coarse_kernel<<<cgrid, kThreads, 0, st>>>(a, m >> 2);
+                    stream_fine_kernel<kFR, 5, false><<<step_grid(m), fine_threads(kFR), fine_smem(kFR), st>>>(a, m);
             }
         }
+        if (a.coupled && !persistent_variant(variant))
+            stream_coarse_kernel<<<cgrid, kThreads, 0, st>>>(a, (a.M >> 2) - 1);
         stream_observe_kernel<<<grid, kThreads, 0, st>>>(a);
         stream_finish_kernel<<<(a.count + 63) / 64, 64, 0, st>>>(a, k, tiles, S);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
