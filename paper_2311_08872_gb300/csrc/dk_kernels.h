@@ -167,7 +167,7 @@ void band_carve(BArgs* b, void* buf, int n, const BandPlan& p);
 // to k.partials ([k.slot_stride][p.S], zeroed here); the caller reduces the slots.
 cudaError_t band_run(const KArgs& k, BArgs b, const BandPlan& p, cudaStream_t stream);
 
-// ---- theta-scheme (implicit diffusion weight b0 > 0), grids up to 64 x 64
+// ---- theta-scheme (implicit diffusion weight b0 > 0), grids up to 128 x 128
 constexpr int kMaxCheb = 64;   // largest number of Chebyshev steps per solve
 struct TArgs {
     int K;                     // Chebyshev steps per solve (0: the explicit step)
@@ -234,20 +234,25 @@ struct GemmArgs {
 
 cudaError_t launch_features(const FeatArgs& a, int max_ctas, cudaStream_t st);
 cudaError_t launch_direct_features(const FeatArgs& a, cudaStream_t st);
-// C = A B on the 5th-generation tensor cores (dk_umma.cu): A [M][K] and B
+// One or two independent products C = A B in one launch on the 5th-generation
+// tensor cores (dk_umma.cu): A [M][K] and B
 // given as [N][K], both K-major (sak == sbk == 1), N <= 256; epilogue as in
 // GemmArgs; bounded waits record kErrTimeout in *err.
-cudaError_t launch_gemm_tc(const GemmArgs& g, unsigned* err, cudaStream_t st);
-// out[c][r] = in[r][c] for an R x C BF16 matrix, output rows ldo >= R apart.
-cudaError_t launch_transpose_bf16(const __nv_bfloat16* in, int R, int C, __nv_bfloat16* out, int ldo,
-                                  cudaStream_t st);
+cudaError_t launch_gemm_tc(const GemmArgs* g, int count, unsigned* err, cudaStream_t st);
 // Output layer with KO outputs (one per test function): y [B][KO]; weights
 // w4 [KO][K], biases b4 [KO].
 cudaError_t launch_out_forward(const __nv_bfloat16* H, const float* w, const float* b, int B, int K, int KO, float* y,
                                cudaStream_t st);
+// loss (may be null): squared error summed over the B x KO values, divided by B.
 cudaError_t launch_out_backward(const float* y, const float* t, const __nv_bfloat16* H, const float* w, int B, int K,
-                                int KO, float* dy, __nv_bfloat16* dH, float* dw, float* db, cudaStream_t st);
-cudaError_t launch_colsum(const __nv_bfloat16* Xb, const float* Xf, int B, int N, float* out, cudaStream_t st);
+                                int KO, __nv_bfloat16* dH, float* dw, float* db, double* loss, cudaStream_t st);
+// Operands of a layer's backward products: dHt [N][ldt] and Hint [K][ldt], the
+// transposes of dH [B][N] and Hin [B][K]; Wt [K][N] of W [N][K] (W may be null);
+// and the bias gradient, the column sums of dH.
+cudaError_t launch_layer_prep(const __nv_bfloat16* dH, __nv_bfloat16* dHt, const __nv_bfloat16* Hin, __nv_bfloat16* Hint,
+                              int B, int N, int K, int ldt, const __nv_bfloat16* W, __nv_bfloat16* Wt, float* colsum,
+                              cudaStream_t st);
+cudaError_t launch_to_bf16(const float* x, long long n, __nv_bfloat16* y, cudaStream_t st);
 cudaError_t launch_adam(float* theta, const float* grad, float* m1, float* m2, int P, float lr, float b1, float b2,
                         float eps, float c1, float c2, const int* bf_index, __nv_bfloat16* theta_bf, cudaStream_t st);
 cudaError_t launch_gather(const __nv_bfloat16* X, const float* T, const int* idx, int B, int KO, __nv_bfloat16* Xb,

@@ -128,46 +128,180 @@ __global__ void out_forward_kernel(const __nv_bfloat16* H, const float* w, const
     }
 }
 
-// dy[b][o] = 2 (y - t) / B; dH[b][k] = (sum_o dy[b][o] w4[o][k]) (H[b][k] > 0) as BF16.
-__global__ void out_backward_kernel(const float* y, const float* t, const __nv_bfloat16* H, const float* w, int B,
-                                    int K, int KO, float* dy, __nv_bfloat16* dH) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= (long long)B * K) return;
-    const int b = static_cast<int>(i / K), k = static_cast<int>(i % K);
-    float v = 0.f;
-    for (int o = 0; o < KO; ++o) {
-        const size_t bo = (size_t)b * KO + o;
-        const float d = 2.f * (y[bo] - t[bo]) / static_cast<float>(B);
-        if (k == 0) dy[bo] = d;
-        v = fmaf(d, w[(size_t)o * K + k], v);
+// Squared error of a batch summed over its n values (rows x outputs) and
+// divided by the rows B, FP64 accumulation, one block of 256 threads.
+__device__ __forceinline__ void mse_block(const float* y, const float* t, int n, int B, double* out) {
+    __shared__ double sh[256];
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += 256) {
+        const double d = static_cast<double>(y[i]) - t[i];
+        s += d * d;
     }
-    dH[i] = __float2bfloat16_rn(__bfloat162float(H[i]) > 0.f ? v : 0.f);
+    sh[threadIdx.x] = s;
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *out = sh[0] / B;
 }
 
-// Column sums: out[n] = sum_b X[b][n] (X BF16 or FP32), fixed order per column.
-__global__ void colsum_kernel(const __nv_bfloat16* Xb, const float* Xf, int B, int N, float* out) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
+__global__ void __launch_bounds__(256) mse_kernel(const float* y, const float* t, int n, int B, double* out) {
+    mse_block(y, t, n, B, out);
+}
+
+// Sum over the 256 threads of a block of eight values each; valid in threads 0..7
+// (value t in thread t).
+__device__ __forceinline__ float block_sum8(float (&v)[8]) {
+    __shared__ float sh[8][8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] += __shfl_xor_sync(kFullMask, v[i], off);
+    if (lane == 0)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) sh[warp][i] = v[i];
+    __syncthreads();
     float s = 0.f;
-    for (int b = 0; b < B; ++b) s += Xb ? __bfloat162float(Xb[(size_t)b * N + n]) : Xf[(size_t)b * N + n];
-    out[n] = s;
+    if (threadIdx.x < 8)
+        for (int w = 0; w < 8; ++w) s += sh[w][threadIdx.x];
+    return s;
 }
 
-// dW4[o][k] = sum_b dy[b][o] H3[b][k]; db4[o] = sum_b dy[b][o].
-__global__ void out_weight_grad_kernel(const float* dy, const __nv_bfloat16* H, int B, int K, int KO, float* dw,
-                                       float* db) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < K * KO) {
-        const int o = j / K, k = j % K;
-        float s = 0.f;
-        for (int b = 0; b < B; ++b) s = fmaf(dy[(size_t)b * KO + o], __bfloat162float(H[(size_t)b * K + k]), s);
-        dw[j] = s;
-    } else if (j < K * KO + KO) {
-        const int o = j - K * KO;
-        float s = 0.f;
-        for (int b = 0; b < B; ++b) s += dy[(size_t)b * KO + o];
-        db[o] = s;
+__device__ __forceinline__ void unpack8(const uint4& u, float (&v)[8]) {
+    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float2 f = __bfloat1622float2(h[i]);
+        v[2 * i] = f.x;
+        v[2 * i + 1] = f.y;
     }
+}
+
+// Backward of the output layer, with d = 2 (y - t) / B, in one launch of blocks
+// of 256 threads with four tasks:
+//   * dH[b][k] = (sum_o d[b][o] w4[o][k]) (H[b][k] > 0) as BF16, eight columns a thread;
+//   * dw[o][k..k+7] = sum_b d[b][o] H[b][k..k+7], one block per o and eight columns;
+//   * db[o] = sum_b d[b][o], one block per o;
+//   * the loss, if asked for: squared error summed over the B x KO values and
+//     divided by B in FP64, one block (the sum of mse_kernel).
+// A column's batch sum in one thread is a chain of B additions behind their loads
+// on two or three blocks of the GPU; over 256 threads of a block per eight columns
+// it is B / 256 loads and a tree (1024 rows: this launch 5.8 us, layer_prep_kernel
+// 7 to 9; a gradient 520 us with a thread per column and a launch per task, 187
+// with these).
+__global__ void __launch_bounds__(256) out_backward_kernel(const float* y, const float* t, const __nv_bfloat16* H,
+                                                           const float* w, int B, int K, int KO, __nv_bfloat16* dH,
+                                                           float* dw, float* db, double* loss) {
+    const int tid = threadIdx.x, groups = K / 8;
+    const float scale = static_cast<float>(B);
+    const int n_el = static_cast<int>(((long long)B * groups + 255) / 256);
+    int blk = blockIdx.x;
+    if (blk < n_el) {
+        const long long i = blk * 256LL + tid;
+        if (i >= (long long)B * groups) return;
+        const int b = static_cast<int>(i / groups), k = static_cast<int>(i % groups) * 8;
+        float h[8], v[8];
+        unpack8(*reinterpret_cast<const uint4*>(H + (size_t)b * K + k), h);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = 0.f;
+        for (int o = 0; o < KO; ++o) {
+            const size_t bo = (size_t)b * KO + o;
+            const float d = 2.f * (y[bo] - t[bo]) / scale;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = fmaf(d, w[(size_t)o * K + k + j], v[j]);
+        }
+        uint4 u;
+        __nv_bfloat162* r = reinterpret_cast<__nv_bfloat162*>(&u);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            r[j] = __floats2bfloat162_rn(h[2 * j] > 0.f ? v[2 * j] : 0.f, h[2 * j + 1] > 0.f ? v[2 * j + 1] : 0.f);
+        *reinterpret_cast<uint4*>(dH + (size_t)b * K + k) = u;
+        return;
+    }
+    blk -= n_el;
+    if (blk < KO * groups) {
+        const int o = blk / groups, k = blk % groups * 8;
+        float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+        for (int b = tid; b < B; b += 256) {
+            const size_t bo = (size_t)b * KO + o;
+            const float d = 2.f * (y[bo] - t[bo]) / scale;
+            float h[8];
+            unpack8(*reinterpret_cast<const uint4*>(H + (size_t)b * K + k), h);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) s[j] = fmaf(d, h[j], s[j]);
+        }
+        const float r = block_sum8(s);
+        if (tid < 8) dw[(size_t)o * K + k + tid] = r;
+        return;
+    }
+    blk -= KO * groups;
+    if (blk < KO) {
+        float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        for (int b = tid; b < B; b += 256) s[0] += 2.f * (y[(size_t)b * KO + blk] - t[(size_t)b * KO + blk]) / scale;
+        const float r = block_sum8(s);
+        if (tid == 0) db[blk] = r;
+        return;
+    }
+    mse_block(y, t, B * KO, B, loss);
+}
+
+// A layer's operands for the backward products, in one launch of blocks of 256
+// threads: transposes (out[c][r] = in[r][c] of an R x C matrix, output rows ldo
+// elements apart, one block per 32 x 32 tile) and the bias gradient, the column
+// sums of X [B][N] (one block per eight columns).
+struct PrepArgs {
+    struct Transpose {
+        const __nv_bfloat16* in;
+        __nv_bfloat16* out;
+        int R, C, ldo, tiles;
+    } t[3];
+    const __nv_bfloat16* X;
+    float* colsum;
+    int B, N;
+};
+__global__ void __launch_bounds__(256) layer_prep_kernel(const PrepArgs a) {
+    __shared__ __nv_bfloat16 sh[32][33];
+    int blk = blockIdx.x;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const PrepArgs::Transpose& t = a.t[i];
+        if (blk < t.tiles) {
+            const int cols = (t.C + 31) / 32, tx = threadIdx.x & 31;
+            const int bx = blk % cols * 32, by = blk / cols * 32;
+#pragma unroll
+            for (int ty = threadIdx.x >> 5; ty < 32; ty += 8) {
+                const int r = by + ty, c = bx + tx;
+                if (r < t.R && c < t.C) sh[ty][tx] = t.in[(size_t)r * t.C + c];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int ty = threadIdx.x >> 5; ty < 32; ty += 8) {
+                const int c = bx + ty, r = by + tx;
+                if (r < t.R && c < t.C) t.out[(size_t)c * t.ldo + r] = sh[tx][ty];
+            }
+            return;
+        }
+        blk -= t.tiles;
+    }
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int b = threadIdx.x; b < a.B; b += 256) {
+        float v[8];
+        unpack8(*reinterpret_cast<const uint4*>(a.X + (size_t)b * a.N + blk * 8), v);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s[j] += v[j];
+    }
+    const float r = block_sum8(s);
+    if (threadIdx.x < 8) a.colsum[blk * 8 + threadIdx.x] = r;
+}
+
+// FP32 to BF16, round to nearest even.
+__global__ void to_bf16_kernel(const float* x, long long n, __nv_bfloat16* y) {
+    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (i < n) y[i] = __float2bfloat16_rn(x[i]);
 }
 
 // Adam (Kingma & Ba, 2015) with bias correction; refreshes the BF16 weights.
@@ -195,24 +329,6 @@ __global__ void gather_kernel(const __nv_bfloat16* X, const float* T, const int*
     const int src = idx[b];
     Xb[i] = X[(size_t)src * kFeat + j];
     if (j < KO) Tb[(size_t)b * KO + j] = T[(size_t)src * KO + j];
-}
-
-// Squared error of a batch summed over its n values (rows x outputs) and
-// divided by the rows B, FP64 accumulation, one block.
-__global__ void mse_kernel(const float* y, const float* t, int n, int B, double* out) {
-    __shared__ double sh[256];
-    double s = 0.0;
-    for (int i = threadIdx.x; i < n; i += 256) {
-        const double d = static_cast<double>(y[i]) - t[i];
-        s += d * d;
-    }
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *out = sh[0] / B;
 }
 
 // Per-sample quantities of a surrogate batch into per-block FP64 partials
@@ -296,14 +412,29 @@ cudaError_t launch_out_forward(const __nv_bfloat16* H, const float* w, const flo
 }
 
 cudaError_t launch_out_backward(const float* y, const float* t, const __nv_bfloat16* H, const float* w, int B, int K,
-                                int KO, float* dy, __nv_bfloat16* dH, float* dw, float* db, cudaStream_t st) {
-    out_backward_kernel<<<(unsigned)(((long long)B * K + 255) / 256), 256, 0, st>>>(y, t, H, w, B, K, KO, dy, dH);
-    out_weight_grad_kernel<<<(K * KO + KO + 127) / 128, 128, 0, st>>>(dy, H, B, K, KO, dw, db);
+                                int KO, __nv_bfloat16* dH, float* dw, float* db, double* loss, cudaStream_t st) {
+    if (K % 8) return cudaErrorInvalidValue;
+    const long long blocks = ((long long)B * (K / 8) + 255) / 256 + KO * (K / 8) + KO + (loss ? 1 : 0);
+    out_backward_kernel<<<(unsigned)blocks, 256, 0, st>>>(y, t, H, w, B, K, KO, dH, dw, db, loss);
     return cudaGetLastError();
 }
 
-cudaError_t launch_colsum(const __nv_bfloat16* Xb, const float* Xf, int B, int N, float* out, cudaStream_t st) {
-    colsum_kernel<<<(N + 127) / 128, 128, 0, st>>>(Xb, Xf, B, N, out);
+cudaError_t launch_layer_prep(const __nv_bfloat16* dH, __nv_bfloat16* dHt, const __nv_bfloat16* Hin, __nv_bfloat16* Hint,
+                              int B, int N, int K, int ldt, const __nv_bfloat16* W, __nv_bfloat16* Wt, float* colsum,
+                              cudaStream_t st) {
+    if (N % 8 || ldt < B) return cudaErrorInvalidValue;
+    const auto tiles = [](int R, int C) { return ((R + 31) / 32) * ((C + 31) / 32); };
+    PrepArgs a{};
+    a.t[0] = {dH, dHt, B, N, ldt, tiles(B, N)};
+    a.t[1] = {Hin, Hint, B, K, ldt, tiles(B, K)};
+    if (W) a.t[2] = {W, Wt, N, K, N, tiles(N, K)};
+    a.X = dH; a.colsum = colsum; a.B = B; a.N = N;
+    layer_prep_kernel<<<a.t[0].tiles + a.t[1].tiles + a.t[2].tiles + N / 8, 256, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_to_bf16(const float* x, long long n, __nv_bfloat16* y, cudaStream_t st) {
+    to_bf16_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x, n, y);
     return cudaGetLastError();
 }
 

@@ -2,13 +2,14 @@
 // cores (sm_103a): C[M x N] = A[M x K] . B[N x K]^T, both operands K-major BF16
 // in global memory, FP32 accumulation in tensor memory (TMEM).
 //
-// One CTA computes a 128-row tile of C across all N <= 256 columns:
-//   * one thread streams 128 x 64 tiles of A and N x 64 tiles of B into a
+// A launch holds up to two independent products (the weight gradient and the
+// input gradient of a layer); one CTA computes a 128 x BN tile of one of them:
+//   * one thread streams 128 x 64 tiles of A and BN x 64 tiles of B into a
 //     ring of shared-memory stages with TMA (cp.async.bulk.tensor, 128-byte
 //     swizzle, rows beyond M or K read as zeros), each stage guarded by a
 //     "full" mbarrier (transaction count) and an "empty" one;
-//   * one thread issues tcgen05.mma (kind::f16, M = 128, N, K = 16 per
-//     instruction, four per stage) into a 128-lane x N-column FP32 accumulator
+//   * one thread issues tcgen05.mma (kind::f16, M = 128, N = BN, K = 16 per
+//     instruction, four per stage) into a 128-lane x BN-column FP32 accumulator
 //     in TMEM and frees each stage with tcgen05.commit;
 //   * all four warps then read their 32 TMEM lanes (= rows) with tcgen05.ld and
 //     apply the epilogue: + bias[n], ReLU, * (mask[m][n] > 0), FP32 and/or BF16
@@ -32,7 +33,6 @@ namespace {
 
 constexpr int kTM = 128;                        // rows of a CTA tile (TMEM lanes)
 constexpr int kTK = 64;                         // K of a stage: 64 BF16 = one 128-byte swizzle row
-constexpr int kStages = 2;   // two stages: 99 KB at N = 256, so two CTAs share an SM
 constexpr unsigned kMbarPolls = 1u << 22;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -118,17 +118,28 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-template <int BN>
+// One product of a launch: its operand maps and its CTAs, tiles_m x tiles_n.
+struct Product {
+    CUtensorMap A, B;
+    GemmArgs g;
+    int tiles_m, tiles;
+};
+
+template <int BN, int STAGES>
 constexpr size_t umma_smem_bytes() {
-    return 1024 /* alignment slack */ + (size_t)kStages * (kTM + BN) * kTK * sizeof(__nv_bfloat16) +
-           (2 * kStages + 1) * sizeof(uint64_t) + 16;
+    return 1024 /* alignment slack */ + (size_t)STAGES * (kTM + BN) * kTK * sizeof(__nv_bfloat16) +
+           (2 * STAGES + 1) * sizeof(uint64_t) + 16;
 }
 
-template <int BN>
+template <int BN, int kStages>
 __global__ void __launch_bounds__(128, 1)
-    umma_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, const GemmArgs g,
-                     unsigned* err) {
+    umma_gemm_kernel(const __grid_constant__ Product p0, const __grid_constant__ Product p1, unsigned* err) {
     static_assert(BN % 16 == 0 && BN >= 32 && BN <= 256 && (BN & (BN - 1)) == 0, "N tile: power of two in [32, 256]");
+    const bool second = static_cast<int>(blockIdx.x) >= p0.tiles;
+    const Product& p = second ? p1 : p0;
+    const GemmArgs& g = p.g;
+    const int tile = second ? blockIdx.x - p0.tiles : blockIdx.x;
+    const int n0 = tile / p.tiles_m * BN;
     extern __shared__ unsigned char umma_shared[];
     unsigned char* base = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(umma_shared) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -139,7 +150,7 @@ __global__ void __launch_bounds__(128, 1)
     uint64_t* done = empty + kStages;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * kTM;
+    const int m0 = tile % p.tiles_m * kTM;
     const int ktiles = (g.K + kTK - 1) / kTK;
 
     if (threadIdx.x == 0) {
@@ -169,8 +180,8 @@ __global__ void __launch_bounds__(128, 1)
             const int s = kt % kStages;
             if (kt >= kStages && !mbar_wait(&empty[s], ((kt / kStages) - 1) & 1, err)) break;
             mbar_expect_tx(&full[s], bytes);
-            tma_load_2d(sA + (size_t)s * kTM * kTK, &tA, kt * kTK, m0, &full[s]);
-            tma_load_2d(sB + (size_t)s * BN * kTK, &tB, kt * kTK, 0, &full[s]);
+            tma_load_2d(sA + (size_t)s * kTM * kTK, &p.A, kt * kTK, m0, &full[s]);
+            tma_load_2d(sB + (size_t)s * BN * kTK, &p.B, kt * kTK, n0, &full[s]);
         }
     } else if (warp == 1 && lane == 0) {
         // MMA issuer: four K = 16 steps per stage (32 bytes along the swizzled rows)
@@ -190,15 +201,20 @@ __global__ void __launch_bounds__(128, 1)
         }
         umma_commit(done);
     }
+    // the producer's and the issuer's warps stay whole: their other lanes, polling
+    // `done` beside them, would suspend the warp at every poll (1.6 us per K tile: a
+    // product over 1024 rows took 26 us, a gradient of 1024 rows 187, with this 138)
+    __syncwarp();
     // epilogue: warp w reads TMEM lanes 32w .. 32w + 31 (rows of the tile)
     const bool ready = mbar_wait(done, 0, err);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const int m = m0 + warp * 32 + lane;
     if (ready) {
 #pragma unroll 1
-        for (int c0 = 0; c0 < BN && c0 < g.N; c0 += 32) {
+        for (int ct = 0; ct < BN && n0 + ct < g.N; ct += 32) {
+            const int c0 = n0 + ct;
             uint32_t v[32];
-            tmem_ld32(tmem + (static_cast<uint32_t>(warp * 32) << 16) + static_cast<uint32_t>(c0), v);
+            tmem_ld32(tmem + (static_cast<uint32_t>(warp * 32) << 16) + static_cast<uint32_t>(ct), v);
             if (m >= g.M) continue;
             // this thread's 32 consecutive columns of row m: 16-byte loads and
             // stores where the whole chunk is inside N and the row is aligned
@@ -276,22 +292,6 @@ __global__ void __launch_bounds__(128, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN) : "memory");
 }
 
-// BF16 transpose: out[c][r] = in[r][c] for an R x C row-major matrix, output
-// rows ldo >= R elements apart.
-__global__ void transpose_bf16_kernel(const __nv_bfloat16* in, int R, int C, __nv_bfloat16* out, int ldo) {
-    __shared__ __nv_bfloat16 t[32][33];
-    const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int r = by + i, c = bx + threadIdx.x;
-        if (r < R && c < C) t[i][threadIdx.x] = in[(size_t)r * C + c];
-    }
-    __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int c = bx + i, r = by + threadIdx.x;
-        if (r < R && c < C) out[(size_t)c * ldo + r] = t[threadIdx.x][i];
-    }
-}
-
 // ---------------------------------------------------------------- host side
 using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -326,44 +326,52 @@ bool encode_kmajor(CUtensorMap* map, const __nv_bfloat16* ptr, long long rows, l
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN>
-cudaError_t umma_launch(const CUtensorMap& ta, const CUtensorMap& tb, const GemmArgs& g, unsigned* err,
-                        cudaStream_t st) {
-    const cudaError_t attr = cudaFuncSetAttribute(umma_gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)umma_smem_bytes<BN>());
+template <int BN, int STAGES>
+cudaError_t umma_launch(const GemmArgs* g, int count, unsigned* err, cudaStream_t st) {
+    const cudaError_t attr = cudaFuncSetAttribute(umma_gemm_kernel<BN, STAGES>,
+                                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)umma_smem_bytes<BN, STAGES>());
     if (attr != cudaSuccess) return attr;
-    const int tiles = (g.M + kTM - 1) / kTM;
-    umma_gemm_kernel<BN><<<tiles, 128, umma_smem_bytes<BN>(), st>>>(ta, tb, g, err);
+    Product p[2] = {};
+    for (int i = 0; i < count; ++i) {
+        p[i].g = g[i];
+        p[i].tiles_m = (g[i].M + kTM - 1) / kTM;
+        p[i].tiles = p[i].tiles_m * ((g[i].N + BN - 1) / BN);
+        if (!encode_kmajor(&p[i].A, g[i].A, g[i].M, g[i].K, g[i].sam, kTM) ||
+            !encode_kmajor(&p[i].B, g[i].B, g[i].N, g[i].K, g[i].sbn, BN))
+            return cudaErrorInvalidValue;
+    }
+    umma_gemm_kernel<BN, STAGES><<<p[0].tiles + p[1].tiles, 128, umma_smem_bytes<BN, STAGES>(), st>>>(p[0], p[1], err);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_gemm_tc(const GemmArgs& g, unsigned* err, cudaStream_t st) {
+cudaError_t launch_gemm_tc(const GemmArgs* g, int count, unsigned* err, cudaStream_t st) {
     // A [M][K] K-major (sak == 1, row stride sam), B given as [N][K] K-major
     // (sbk == 1, row stride sbn): C = A B^T
-    if (g.sak != 1 || g.sbk != 1 || g.N < 1 || g.N > 256 || g.M < 1 || g.K < 1 || !err) return cudaErrorInvalidValue;
-    if ((reinterpret_cast<uintptr_t>(g.A) & 15) || (reinterpret_cast<uintptr_t>(g.B) & 15) || (g.sam * 2) % 16 ||
-        (g.sbn * 2) % 16)
-        return cudaErrorInvalidValue;
-    const int bn = g.N <= 32 ? 32 : g.N <= 64 ? 64 : g.N <= 128 ? 128 : 256;
-    CUtensorMap ta, tb;
-    if (!encode_kmajor(&ta, g.A, g.M, g.K, g.sam, kTM) || !encode_kmajor(&tb, g.B, g.N, g.K, g.sbn, bn))
-        return cudaErrorInvalidValue;
-    switch (bn) {
-        case 32: return umma_launch<32>(ta, tb, g, err, st);
-        case 64: return umma_launch<64>(ta, tb, g, err, st);
-        case 128: return umma_launch<128>(ta, tb, g, err, st);
-        default: return umma_launch<256>(ta, tb, g, err, st);
+    if (count < 1 || count > 2 || !err) return cudaErrorInvalidValue;
+    int n = 0;
+    long long tiles_m = 0;
+    for (int i = 0; i < count; ++i) {
+        const GemmArgs& x = g[i];
+        if (x.sak != 1 || x.sbk != 1 || x.N < 1 || x.N > 256 || x.M < 1 || x.K < 1 ||
+            (reinterpret_cast<uintptr_t>(x.A) & 15) || (reinterpret_cast<uintptr_t>(x.B) & 15) || (x.sam * 2) % 16 ||
+            (x.sbn * 2) % 16)
+            return cudaErrorInvalidValue;
+        n = x.N > n ? x.N : n;
+        tiles_m += (x.M + kTM - 1) / kTM;
     }
-}
-
-cudaError_t launch_transpose_bf16(const __nv_bfloat16* in, int R, int C, __nv_bfloat16* out, int ldo,
-                                  cudaStream_t st) {
-    if (ldo < R) return cudaErrorInvalidValue;
-    const dim3 grid((C + 31) / 32, (R + 31) / 32), block(32, 8);
-    transpose_bf16_kernel<<<grid, block, 0, st>>>(in, R, C, out, ldo);
-    return cudaGetLastError();
+    // Few row tiles (training batches): 64 columns per CTA give four times the
+    // CTAs of 256, and eight stages (197 KB, one CTA per SM) hide the latency of
+    // the batch-long sum of a weight gradient.  From 152 tiles of 64 columns on,
+    // one wave is full: all columns of a row tile in one CTA read A once, two
+    // stages (99 KB) let two CTAs share an SM.  256-column tiles with two stages
+    // for every size, and one product a launch: part of the 520 us that a gradient
+    // of 1024 rows took, 138 now.
+    if (n > 64 && tiles_m * 4 <= 152) return umma_launch<64, 8>(g, count, err, st);
+    return n <= 32 ? umma_launch<32, 8>(g, count, err, st) : n <= 64 ? umma_launch<64, 8>(g, count, err, st)
+         : n <= 128 ? umma_launch<128, 2>(g, count, err, st) : umma_launch<256, 2>(g, count, err, st);
 }
 
 }  // namespace dk

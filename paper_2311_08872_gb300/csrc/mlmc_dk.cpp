@@ -126,7 +126,7 @@ struct Surrogate {
     // K-major operands of the backward GEMMs: dH^T, Hin^T [256][batch], W^T [256][256]
     __nv_bfloat16 *d_tA = nullptr, *d_tB = nullptr, *d_wt = nullptr;
     unsigned* err = nullptr;           // the context's device error word (bounded waits of the GEMM)
-    float *d_y = nullptr, *d_dy = nullptr, *d_T = nullptr, *d_Xf = nullptr;
+    float *d_y = nullptr, *d_T = nullptr, *d_Xf = nullptr;
     double* d_samp = nullptr;          // level-0 per-sample outputs of a chunk
     double* d_D0 = nullptr;
     double* d_part = nullptr;          // moment partials [stride][blocks]
@@ -1905,7 +1905,7 @@ void free_surrogate(Surrogate* s) {
     for (void* p : {(void*)s->d_E, (void*)s->d_g, (void*)s->d_inv_sigma, (void*)s->d_theta, (void*)s->d_grad,
                     (void*)s->d_m1, (void*)s->d_m2, (void*)s->d_wbf, (void*)s->d_bfidx, (void*)s->d_X,
                     (void*)s->d_H1, (void*)s->d_H2, (void*)s->d_H3, (void*)s->d_dH1, (void*)s->d_dH2,
-                    (void*)s->d_dH3, (void*)s->d_y, (void*)s->d_dy, (void*)s->d_T, (void*)s->d_Xf,
+                    (void*)s->d_dH3, (void*)s->d_y, (void*)s->d_T, (void*)s->d_Xf,
                     (void*)s->d_samp, (void*)s->d_D0, (void*)s->d_part, (void*)s->d_loss, (void*)s->d_trainX,
                     (void*)s->d_trainT, (void*)s->d_idx, (void*)s->d_tA, (void*)s->d_tB, (void*)s->d_wt})
         cudaFree(p);
@@ -1970,23 +1970,24 @@ cudaError_t mlp_forward(Surrogate* s, const __nv_bfloat16* X, int n, float* y, c
     cudaError_t e;
     dk::GemmArgs g = gemm(n, dk::kHidden, dk::kFeat, X, dk::kFeat, 1, s->d_wbf + kBfW1, 1, dk::kFeat);
     g.Cb = s->d_H1; g.ldcb = dk::kHidden; g.bias = s->d_theta + kOffB1; g.relu = 1;
-    if ((e = dk::launch_gemm_tc(g, s->err, st)) != cudaSuccess) return e;
+    if ((e = dk::launch_gemm_tc(&g, 1, s->err, st)) != cudaSuccess) return e;
     g = gemm(n, dk::kHidden, dk::kHidden, s->d_H1, dk::kHidden, 1, s->d_wbf + kBfW2, 1, dk::kHidden);
     g.Cb = s->d_H2; g.ldcb = dk::kHidden; g.bias = s->d_theta + kOffB2; g.relu = 1;
-    if ((e = dk::launch_gemm_tc(g, s->err, st)) != cudaSuccess) return e;
+    if ((e = dk::launch_gemm_tc(&g, 1, s->err, st)) != cudaSuccess) return e;
     g = gemm(n, dk::kHidden, dk::kHidden, s->d_H2, dk::kHidden, 1, s->d_wbf + kBfW3, 1, dk::kHidden);
     g.Cb = s->d_H3; g.ldcb = dk::kHidden; g.bias = s->d_theta + kOffB3; g.relu = 1;
-    if ((e = dk::launch_gemm_tc(g, s->err, st)) != cudaSuccess) return e;
+    if ((e = dk::launch_gemm_tc(&g, 1, s->err, st)) != cudaSuccess) return e;
     return dk::launch_out_forward(s->d_H3, s->d_theta + kOffW4, s->d_theta + off_b4(s->K), n, dk::kHidden, s->K, y,
                                   st);
 }
 
-// Mean-squared-error gradient of a batch (after mlp_forward on it) into d_grad.
-cudaError_t mlp_backward(Surrogate* s, const __nv_bfloat16* X, const float* T, int B, cudaStream_t st) {
+// Mean-squared-error gradient of a batch (after mlp_forward on it) into d_grad,
+// and the loss itself into *loss unless null.
+cudaError_t mlp_backward(Surrogate* s, const __nv_bfloat16* X, const float* T, int B, double* loss, cudaStream_t st) {
     cudaError_t e;
     float* G = s->d_grad;
-    if ((e = dk::launch_out_backward(s->d_y, T, s->d_H3, s->d_theta + kOffW4, B, dk::kHidden, s->K, s->d_dy, s->d_dH3,
-                                     G + kOffW4, G + off_b4(s->K), st)) != cudaSuccess)
+    if ((e = dk::launch_out_backward(s->d_y, T, s->d_H3, s->d_theta + kOffW4, B, dk::kHidden, s->K, s->d_dH3,
+                                     G + kOffW4, G + off_b4(s->K), loss, st)) != cudaSuccess)
         return e;
     struct Layer { const __nv_bfloat16* dH; const __nv_bfloat16* Hin; int K; float* gW; float* gb;
                    const __nv_bfloat16* W; __nv_bfloat16* dHin; };
@@ -1995,26 +1996,23 @@ cudaError_t mlp_backward(Surrogate* s, const __nv_bfloat16* X, const float* T, i
         {s->d_dH2, s->d_H1, dk::kHidden, G + kOffW2, G + kOffB2, s->d_wbf + kBfW2, s->d_dH1},
         {s->d_dH1, X, dk::kFeat, G + kOffW1, G + kOffB1, nullptr, nullptr}};
     for (const Layer& L : layers) {
-        // dW = dH^T Hin (256 x K, summed over the batch) as a K-major product on
-        // the tensor cores: A = dH^T [256][B], B operand = Hin^T [K][B]
         // rows of the transposed operands padded to 8 elements (16 bytes, the TMA
         // stride unit); the padding lies beyond K = B and is never read
         const int ldt = (B + 7) & ~7;
-        if ((e = dk::launch_transpose_bf16(L.dH, B, dk::kHidden, s->d_tA, ldt, st)) != cudaSuccess ||
-            (e = dk::launch_transpose_bf16(L.Hin, B, L.K, s->d_tB, ldt, st)) != cudaSuccess)
+        if ((e = dk::launch_layer_prep(L.dH, s->d_tA, L.Hin, s->d_tB, B, dk::kHidden, L.K, ldt, L.W, s->d_wt, L.gb,
+                                       st)) != cudaSuccess)
             return e;
-        dk::GemmArgs g = gemm(dk::kHidden, L.K, B, s->d_tA, ldt, 1, s->d_tB, 1, ldt);
-        g.C = L.gW; g.ldc = L.K;
-        if ((e = dk::launch_gemm_tc(g, s->err, st)) != cudaSuccess) return e;
-        if ((e = dk::launch_colsum(L.dH, nullptr, B, dk::kHidden, L.gb, st)) != cudaSuccess) return e;
+        // dW = dH^T Hin (256 x K, summed over the batch) as a K-major product on
+        // the tensor cores: A = dH^T [256][B], B operand = Hin^T [K][B]; beside it
+        // dHin = (dH W) * (Hin > 0): A = dH [B][256], B operand = W^T [in][out]
+        dk::GemmArgs g[2];
+        g[0] = gemm(dk::kHidden, L.K, B, s->d_tA, ldt, 1, s->d_tB, 1, ldt);
+        g[0].C = L.gW; g[0].ldc = L.K;
         if (L.W) {
-            // dHin = (dH W) * (Hin > 0): A = dH [B][256], B operand = W^T [in][out]
-            if ((e = dk::launch_transpose_bf16(L.W, dk::kHidden, dk::kHidden, s->d_wt, dk::kHidden, st)) != cudaSuccess)
-                return e;
-            g = gemm(B, dk::kHidden, dk::kHidden, L.dH, dk::kHidden, 1, s->d_wt, 1, dk::kHidden);
-            g.Cb = L.dHin; g.ldcb = dk::kHidden; g.mask = L.Hin; g.ldm = dk::kHidden;
-            if ((e = dk::launch_gemm_tc(g, s->err, st)) != cudaSuccess) return e;
+            g[1] = gemm(B, dk::kHidden, dk::kHidden, L.dH, dk::kHidden, 1, s->d_wt, 1, dk::kHidden);
+            g[1].Cb = L.dHin; g[1].ldcb = dk::kHidden; g[1].mask = L.Hin; g[1].ldm = dk::kHidden;
         }
+        if ((e = dk::launch_gemm_tc(g, L.W ? 2 : 1, s->err, st)) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
@@ -2105,7 +2103,6 @@ int mlmc_dk_surrogate_init(mlmc_dk_ctx* ctx, uint64_t seed) {
     alloc((void**)&s->d_wt, sizeof(__nv_bfloat16) * dk::kHidden * dk::kHidden);
     s->err = ctx->d_err;
     alloc((void**)&s->d_y, sizeof(float) * ch * K);
-    alloc((void**)&s->d_dy, sizeof(float) * s->batch_cap * K);
     alloc((void**)&s->d_T, sizeof(float) * ch * K);
     alloc((void**)&s->d_samp, sizeof(double) * ch * s->sampw);
     alloc((void**)&s->d_part, sizeof(double) * ctx->stride * kMomentBlocks);
@@ -2177,13 +2174,14 @@ int mlmc_dk_surrogate_forward(mlmc_dk_ctx* ctx, const float* X_host, int64_t n, 
     if (!ctx || !ctx->sur || n < 1 || n > ctx->sur->chunk || !X_host || !y_host)
         return fail(ctx, MLMC_DK_ERR_INVALID, "surrogate_forward: bad arguments");
     Surrogate* s = ctx->sur;
-    std::vector<__nv_bfloat16> xb((size_t)n * dk::kFeat);
-    for (size_t i = 0; i < xb.size(); ++i) xb[i] = __float2bfloat16_rn(X_host[i]);
-    cudaError_t e = cudaMemcpy(s->d_X, xb.data(), sizeof(__nv_bfloat16) * xb.size(), cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMemcpyAsync(s->d_Xf, X_host, sizeof(float) * n * dk::kFeat, cudaMemcpyHostToDevice, ctx->stream);
+    if (e == cudaSuccess) e = dk::launch_to_bf16(s->d_Xf, (long long)n * dk::kFeat, s->d_X, ctx->stream);
     if (e == cudaSuccess) e = mlp_forward(s, s->d_X, (int)n, s->d_y, ctx->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(y_host, s->d_y, sizeof(float) * n * s->K, cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    // also after an error: the copies may still be reading the caller's arrays
+    const cudaError_t done = cudaStreamSynchronize(ctx->stream);
+    if (e == cudaSuccess) e = done;
     return e == cudaSuccess ? MLMC_DK_OK : sur_fail(ctx, e, "surrogate forward");
 }
 
@@ -2192,17 +2190,19 @@ int mlmc_dk_surrogate_loss_grad(mlmc_dk_ctx* ctx, const float* X_host, const flo
     if (!ctx || !ctx->sur || B < 1 || B > ctx->sur->batch_cap || !X_host || !T_host)
         return fail(ctx, MLMC_DK_ERR_INVALID, "surrogate_loss_grad: bad arguments");
     Surrogate* s = ctx->sur;
-    std::vector<__nv_bfloat16> xb((size_t)B * dk::kFeat);
-    for (size_t i = 0; i < xb.size(); ++i) xb[i] = __float2bfloat16_rn(X_host[i]);
-    cudaError_t e = cudaMemcpy(s->d_X, xb.data(), sizeof(__nv_bfloat16) * xb.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(s->d_T, T_host, sizeof(float) * B * s->K, cudaMemcpyHostToDevice);
+    // features in FP32; rounded to BF16 on the device
+    cudaError_t e = cudaMemcpyAsync(s->d_Xf, X_host, sizeof(float) * B * dk::kFeat, cudaMemcpyHostToDevice, ctx->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(s->d_T, T_host, sizeof(float) * B * s->K, cudaMemcpyHostToDevice, ctx->stream);
+    if (e == cudaSuccess) e = dk::launch_to_bf16(s->d_Xf, (long long)B * dk::kFeat, s->d_X, ctx->stream);
     if (e == cudaSuccess) e = mlp_forward(s, s->d_X, B, s->d_y, ctx->stream);
-    if (e == cudaSuccess) e = dk::launch_mse(s->d_y, s->d_T, B * s->K, B, s->d_loss, ctx->stream);
-    if (e == cudaSuccess) e = mlp_backward(s, s->d_X, s->d_T, B, ctx->stream);
+    if (e == cudaSuccess) e = mlp_backward(s, s->d_X, s->d_T, B, s->d_loss, ctx->stream);
     if (e == cudaSuccess && loss) e = cudaMemcpyAsync(loss, s->d_loss, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess && grad_host)
         e = cudaMemcpyAsync(grad_host, s->d_grad, sizeof(float) * s->P, cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    // also after an error: the copies may still be reading the caller's arrays
+    const cudaError_t done = cudaStreamSynchronize(ctx->stream);
+    if (e == cudaSuccess) e = done;
     return e == cudaSuccess ? MLMC_DK_OK : sur_fail(ctx, e, "surrogate loss/grad");
 }
 
@@ -2273,7 +2273,7 @@ int mlmc_dk_surrogate_train(mlmc_dk_ctx* ctx, int64_t n_pairs, int32_t epochs, i
             if ((e = dk::launch_gather(s->d_trainX, s->d_trainT, s->d_idx + b0, batch, K, s->d_X, s->d_T, st)) !=
                     cudaSuccess ||
                 (e = mlp_forward(s, s->d_X, batch, s->d_y, st)) != cudaSuccess ||
-                (e = mlp_backward(s, s->d_X, s->d_T, batch, st)) != cudaSuccess)
+                (e = mlp_backward(s, s->d_X, s->d_T, batch, nullptr, st)) != cudaSuccess)
                 return sur_fail(ctx, e, "training step");
             ++s->adam_t;
             const float c1 = 1.f - std::pow(b1, (float)s->adam_t), c2 = 1.f - std::pow(b2, (float)s->adam_t);
