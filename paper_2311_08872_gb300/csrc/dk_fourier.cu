@@ -25,13 +25,19 @@
 // about the noise-free path and the amplitudes read rho-bar^m from the
 // per-step tables (fine: step m; coarse: coarse step m / 9).
 //
-// Work decomposition.  One CTA per sample.  A thread holds a segment of 6
-// consecutive fine cells of one row (3 Philox cell pairs) in registers, with
-// its row's periodic neighbours fixed once, so a fine step needs no index
-// arithmetic; the state and transfers are published in shared memory for the
-// rows above and below and the segment ends.  The coarse grid and the
-// restriction loop over cells with the CTA's stride.  Two barriers per fine
-// step, two more at a coarse step.
+// Work decomposition.  One CTA per sample.  A thread holds a block of 2 x 6
+// fine cells (two rows of 3 Philox cell pairs), their transfers and their
+// summed normals in registers; its two rows of state and G1 and the end columns
+// of G2 pass through shared memory, double buffered by the step's parity, so a
+// fine step has one barrier.  Every 9 steps the summed normals go to shared
+// memory and are restricted by register tiles: a thread forms 2 x 2 points of
+// S P1^T, both components packed, then two points of the coarse field.
+//
+// Bound by instruction issue and its latencies (issue slots 47% busy with 16 warps;
+// fixed-latency waits, the special functions and shared memory lead).  54^2, 607
+// samples x 648 steps: 4.25 ms; 5.20 with a 1 x 6 segment of cells per thread, whose
+// shared-memory traffic (12 words a cell, here 5, with the summed normals there as
+// well) and one-point restriction (two loads per FMA) were half of the time.
 #include "dk_device.cuh"
 #include "dk_kernels.h"
 
@@ -44,16 +50,18 @@ constexpr int kRedF = 2 * kMaxObs + 2;
 template <int N_>
 struct FShape {
     static constexpr int N = N_, NC = N / 3;
-    static constexpr int SEG = 6;                       // fine cells per thread: one row segment (3 Philox pairs)
-    static constexpr int SEGS = N / SEG;                // segments per row
-    static constexpr int FT = N * SEGS;                 // threads that hold fine cells
-    static constexpr int THREADS = FT > 256 ? 512 : (FT > 32 ? 64 : 32);
-    static_assert(N % SEG == 0 && FT <= THREADS, "fine row segments must cover the grid");
-    static constexpr int MINB = THREADS >= 512 ? 2 : 1;   // two samples per SM at 54^2 (64 registers)
+    static constexpr int R = 2, C = 6;                  // fine cells per thread
+    static constexpr int BRW = N / R, BCL = N / C;      // rows / columns of blocks
+    static constexpr int FT = BRW * BCL;                // threads that hold fine cells
+    static constexpr int THREADS = (FT + 31) / 32 * 32;
+    static_assert(N % R == 0 && N % C == 0 && NC == 2 * BCL && NC % 2 == 0, "blocks must cover the grid");
+    static constexpr int MINB = 512 / THREADS;          // 16 warps of 128 registers on an SM (two samples at 54^2)
     static constexpr int WARPS = THREADS / 32;
-    // words: q (2 buffers), G1, G2, summed normals (2), coarse q (2 buffers),
-    // coarse G1, G2, the row-restricted sums T (N x NC x 2), P1 (NC x N)
-    static constexpr int WORDS = 2 * N * N + 2 * N * N + 2 * N * N + 2 * NC * NC + 2 * NC * NC + 2 * N * NC + NC * N;
+    // words: two exchange buffers (q and G1 of every cell, the end columns of G2),
+    // summed normals (2), coarse q (2 buffers), coarse G1, G2, the row-restricted
+    // sums T (N x NC x 2), P1 (NC x N)
+    static constexpr int XBUF = 2 * N * N + 2 * N * BCL;
+    static constexpr int WORDS = 2 * XBUF + 2 * N * N + 2 * NC * NC + 2 * NC * NC + 2 * N * NC + NC * N;
     static size_t smem(int slot_stride) {
         return sizeof(int32_t) * (size_t)((WORDS + 1) / 2 * 2) + sizeof(double) * WARPS * kRedF +
                sizeof(double) * slot_stride;
@@ -85,32 +93,27 @@ __global__ void __launch_bounds__(FShape<N>::THREADS, FShape<N>::MINB) fourier_k
     constexpr int NC = S::NC, THREADS = S::THREADS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tid = threadIdx.x;
-    int32_t* const qA = reinterpret_cast<int32_t*>(smem_raw);   // fine state, double buffered
-    int32_t* const qB = qA + N * N;
-    int32_t* G1 = qB + N * N;
-    int32_t* G2 = G1 + N * N;
-    float* Zs = reinterpret_cast<float*>(G2 + N * N);      // [N*N][2] summed fine normals
-    int32_t* const qcA = reinterpret_cast<int32_t*>(Zs + 2 * N * N);   // coarse state, double buffered
+    int32_t* const xbuf = reinterpret_cast<int32_t*>(smem_raw);     // exchange buffers
+    f32x2* const Zs = reinterpret_cast<f32x2*>(xbuf + 2 * S::XBUF); // [N*N] summed fine normals, both components
+    f32x2* const Tm = Zs + N * N;                                   // [N][NC]
+    float* const P1 = reinterpret_cast<float*>(Tm + N * NC);        // [NC][N]
+    int32_t* const qcA = reinterpret_cast<int32_t*>(P1 + NC * N);   // coarse state, double buffered
     int32_t* const qcB = qcA + NC * NC;
-    int32_t* Gc1 = qcB + NC * NC;
-    int32_t* Gc2 = Gc1 + NC * NC;
-    float* Tm = reinterpret_cast<float*>(Gc2 + NC * NC);    // [2][N][NC]
-    float* P1 = Tm + 2 * N * NC;                            // [NC][N]
+    int32_t* const Gc1 = qcB + NC * NC;
+    int32_t* const Gc2 = Gc1 + NC * NC;
     double* red = reinterpret_cast<double*>(smem_raw + sizeof(int32_t) * (size_t)((S::WORDS + 1) / 2 * 2));
     double* acc = red + S::WARPS * kRedF;
     for (int i = tid; i < a.slot_stride; i += THREADS) acc[i] = 0.0;
     if constexpr (CPL)
         for (int i = tid; i < NC * N; i += THREADS) P1[i] = f.P1[i];
 
-    constexpr int SEG = S::SEG, SEGS = S::SEGS;
+    constexpr int R = S::R, C = S::C, BRW = S::BRW, BCL = S::BCL;
     const bool fine_thread = tid < S::FT;
-    const int frow = fine_thread ? tid / SEGS : 0;
-    const int fc0 = fine_thread ? (tid % SEGS) * SEG : 0;
-    const int fx0 = frow * N + fc0;                                  // first cell of the segment
-    const int upo = frow == 0 ? N * (N - 1) : -N;                    // offsets to the rows above / below
-    const int dno = frow == N - 1 ? -N * (N - 1) : N;
-    const int lfx = fc0 == 0 ? fx0 + N - 1 : fx0 - 1;                // left of the first cell
-    const int rtx = fc0 + SEG == N ? fx0 + SEG - N : fx0 + SEG;      // right of the last cell
+    const int br = fine_thread ? tid / BCL : 0, bc = fine_thread ? tid % BCL : 0;
+    const int fx0 = br * R * N + bc * C;                             // first cell of the block
+    const int xup = (br == 0 ? N - 1 : br * R - 1) * N + bc * C;     // cells of the rows above / below
+    const int xdn = (br == BRW - 1 ? 0 : (br + 1) * R) * N + bc * C;
+    const int lb = (bc + BCL - 1) % BCL, rb = (bc + 1) % BCL;        // blocks left / right
 
     unsigned bad = 0;
     const long long slot = blockIdx.x, n_slots = gridDim.x;
@@ -122,138 +125,175 @@ __global__ void __launch_bounds__(FShape<N>::THREADS, FShape<N>::MINB) fourier_k
         const long long sid = a.first + idx;
         const uint32_t c2 = static_cast<uint32_t>(sid);
         const uint32_t c3 = a.tag | ((static_cast<uint32_t>(static_cast<unsigned long long>(sid) >> 32) & 0xffffu) << 16);
-        int cur = 0, ccur = 0;
-        int32_t qr[SEG];
-        if (fine_thread) {
+        int ccur = 0;
+        int32_t q[R][C];
+        f32x2 Z[R][C];   // summed normals of the coarse step, both components
 #pragma unroll
-            for (int j = 0; j < SEG; ++j) {
-                qr[j] = a.q0f[fx0 + j];
-                qA[fx0 + j] = qr[j];
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                q[r][c] = a.q0f[fx0 + r * N + c];
+                Z[r][c] = pack2(0.f, 0.f);
             }
-        }
         if constexpr (CPL)
             for (int y = tid; y < NC * NC; y += THREADS) qcA[y] = a.q0c[y];
         __syncthreads();
 
-        for (int m = 0; m < a.M; ++m) {
-            const int32_t* q = cur ? qB : qA;
-            const bool first_of_coarse = CPL && (m % 9) == 0;
-            // ---- noise of the segment: Philox4x32-10 per horizontal cell pair, Box--Muller, transfers
-            int32_t g1[SEG], g2[SEG];
+        for (int m = 0, m9 = 0; m < a.M; ++m) {
+            int32_t* const xq = xbuf + (m & 1) * S::XBUF;   // [N*N] state
+            int32_t* const xg = xq + N * N;                 // [N*N] G1
+            int32_t* const xl = xg + N * N;                 // [N][BCL] G2 of the blocks' first column
+            int32_t* const xr = xl + N * BCL;               // [N][BCL] ... last column
+            int32_t G1[R][C], G2[R][C];
+            // ---- noise of the block: Philox4x32-10 per horizontal cell pair, Box--Muller, transfers
             if (fine_thread) {
+                const f32x2 g2v = pack2(a.gf, a.gf);
 #pragma unroll
-                for (int j = 0; j < SEG / 2; ++j) {
-                    const int p = (fx0 >> 1) + j;
-                    const uint4 x = philox10(make_uint4(static_cast<uint32_t>(p), static_cast<uint32_t>(m), c2, c3),
-                                             a.key0, a.key1);
-                    float ra, ca, sa, rb, cb, sb;
-                    box_muller_polar(x.x, x.y, ra, ca, sa);
-                    box_muller_polar(x.z, x.w, rb, cb, sb);
-                    float ta, tb;
-                    if constexpr (FL) {
-                        const float2 rbar = reinterpret_cast<const float2*>(a.rbf + (size_t)m * N * N)[p];
-                        ta = noise_amp_fluct(qr[2 * j], rbar.x, a.isf, a.gf) * ra;
-                        tb = noise_amp_fluct(qr[2 * j + 1], rbar.y, a.isf, a.gf) * rb;
-                    } else {
-                        ta = noise_amp(qr[2 * j], a.gf) * ra;
-                        tb = noise_amp(qr[2 * j + 1], a.gf) * rb;
+                for (int r = 0; r < R; ++r) {
+#pragma unroll
+                    for (int j = 0; j < C / 2; ++j) {
+                        const int p = ((fx0 + r * N) >> 1) + j;
+                        const uint4 x = philox10(make_uint4(static_cast<uint32_t>(p), static_cast<uint32_t>(m), c2, c3),
+                                                 a.key0, a.key1);
+                        f32x2 rad, co, si;
+                        box_muller_polar2(x.x, x.y, x.z, x.w, rad, co, si);
+                        f32x2 t;
+                        if constexpr (FL) {
+                            const float2 rbar = reinterpret_cast<const float2*>(a.rbf + (size_t)m * N * N)[p];
+                            t = noise_amp_fluct2(q[r][2 * j], q[r][2 * j + 1], rbar.x, rbar.y, a.isf, g2v);
+                        } else {
+                            t = noise_amp2(q[r][2 * j], q[r][2 * j + 1], g2v);
+                        }
+                        t = mul2(t, rad);
+                        const f32x2 t1 = mul2(t, co), t2 = mul2(t, si);
+                        G1[r][2 * j] = __float2int_rn(lo2(t1));
+                        G1[r][2 * j + 1] = __float2int_rn(hi2(t1));
+                        G2[r][2 * j] = __float2int_rn(lo2(t2));
+                        G2[r][2 * j + 1] = __float2int_rn(hi2(t2));
+                        reinterpret_cast<int2*>(xq)[p] = make_int2(q[r][2 * j], q[r][2 * j + 1]);
+                        reinterpret_cast<int2*>(xg)[p] = make_int2(G1[r][2 * j], G1[r][2 * j + 1]);
+                        if constexpr (CPL) {
+                            const float ra = lo2(rad), rb2 = hi2(rad);
+                            Z[r][2 * j] = fma2(pack2(ra, ra), pack2(lo2(co), lo2(si)), Z[r][2 * j]);
+                            Z[r][2 * j + 1] = fma2(pack2(rb2, rb2), pack2(hi2(co), hi2(si)), Z[r][2 * j + 1]);
+                        }
                     }
-                    g1[2 * j] = __float2int_rn(ta * ca);
-                    g2[2 * j] = __float2int_rn(ta * sa);
-                    g1[2 * j + 1] = __float2int_rn(tb * cb);
-                    g2[2 * j + 1] = __float2int_rn(tb * sb);
-                    reinterpret_cast<int2*>(G1)[p] = make_int2(g1[2 * j], g1[2 * j + 1]);
-                    reinterpret_cast<int2*>(G2)[p] = make_int2(g2[2 * j], g2[2 * j + 1]);
-                    if constexpr (CPL) {
-                        float4 z = first_of_coarse ? make_float4(0.f, 0.f, 0.f, 0.f)
-                                                   : reinterpret_cast<float4*>(Zs)[p];
-                        z.x += ra * ca;
-                        z.y += ra * sa;
-                        z.z += rb * cb;
-                        z.w += rb * sb;
-                        reinterpret_cast<float4*>(Zs)[p] = z;
+                    xl[(br * R + r) * BCL + bc] = G2[r][0];
+                    xr[(br * R + r) * BCL + bc] = G2[r][C - 1];
+                }
+                if constexpr (CPL) {
+                    if (m9 == 8) {
+#pragma unroll
+                        for (int r = 0; r < R; ++r)
+#pragma unroll
+                            for (int c = 0; c < C; c += 2) {
+                                reinterpret_cast<ulonglong2*>(Zs)[(fx0 + r * N + c) / 2] =
+                                    make_ulonglong2(Z[r][c], Z[r][c + 1]);
+                                Z[r][c] = Z[r][c + 1] = pack2(0.f, 0.f);
+                            }
                     }
                 }
             }
             __syncthreads();
-            // ---- explicit step of the segment in flux form (every edge flux computed
+            // ---- explicit step of the block in flux form (every edge flux computed
             // from the same two states by both of its cells)
             if (fine_thread) {
-                int32_t* qn = cur ? qA : qB;
-                // the rows above and below, 8-byte loads (segments start at even cells)
-                int32_t qu[SEG], qd[SEG], gu[SEG], gd[SEG];
+                int32_t qu[C], qd[C], gu[C], gd[C], ql[R], qr[R], gl[R], gr[R];
 #pragma unroll
-                for (int j = 0; j < SEG; j += 2) {
-                    const int2 a0 = *reinterpret_cast<const int2*>(q + fx0 + upo + j);
-                    const int2 a1 = *reinterpret_cast<const int2*>(q + fx0 + dno + j);
-                    const int2 b0 = *reinterpret_cast<const int2*>(G1 + fx0 + upo + j);
-                    const int2 b1 = *reinterpret_cast<const int2*>(G1 + fx0 + dno + j);
+                for (int j = 0; j < C; j += 2) {
+                    const int2 a0 = *reinterpret_cast<const int2*>(xq + xup + j);
+                    const int2 a1 = *reinterpret_cast<const int2*>(xq + xdn + j);
+                    const int2 b0 = *reinterpret_cast<const int2*>(xg + xup + j);
+                    const int2 b1 = *reinterpret_cast<const int2*>(xg + xdn + j);
                     qu[j] = a0.x; qu[j + 1] = a0.y; qd[j] = a1.x; qd[j + 1] = a1.y;
                     gu[j] = b0.x; gu[j + 1] = b0.y; gd[j] = b1.x; gd[j + 1] = b1.y;
                 }
-                const int32_t qlf = q[lfx], qrt = q[rtx], g2lf = G2[lfx], g2rt = G2[rtx];
-                int32_t nq[SEG];
 #pragma unroll
-                for (int j = 0; j < SEG; ++j) {
-                    const int32_t c = qr[j];
-                    const int32_t lf = j == 0 ? qlf : qr[j - 1];
-                    const int32_t rt = j == SEG - 1 ? qrt : qr[j + 1];
-                    const int32_t g2l = j == 0 ? g2lf : g2[j - 1];
-                    const int32_t g2r = j == SEG - 1 ? g2rt : g2[j + 1];
-                    nq[j] = c + (edge_flux(a.Af, qd[j] - c) - edge_flux(a.Af, c - qu[j])) +
-                            (edge_flux(a.Af, rt - c) - edge_flux(a.Af, c - lf)) + (gd[j] - gu[j]) + (g2r - g2l);
-                    bad |= (static_cast<uint32_t>(nq[j]) + 0x40000000u) >> 31;
+                for (int r = 0; r < R; ++r) {
+                    const int row = br * R + r;
+                    ql[r] = xq[row * N + lb * C + C - 1];
+                    qr[r] = xq[row * N + rb * C];
+                    gl[r] = xr[row * BCL + lb];
+                    gr[r] = xl[row * BCL + rb];
                 }
+                flux_update<R, C>(q, G1, G2, qu, gu, qd, gd, ql, gl, qr, gr, a.Af);
 #pragma unroll
-                for (int j = 0; j < SEG; j += 2) {
-                    qr[j] = nq[j];
-                    qr[j + 1] = nq[j + 1];
-                    *reinterpret_cast<int2*>(qn + fx0 + j) = make_int2(nq[j], nq[j + 1]);
-                }
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int c = 0; c < C; ++c) bad |= (static_cast<uint32_t>(q[r][c]) + 0x40000000u) >> 31;
             }
-            cur ^= 1;
             if constexpr (CPL) {
-                if ((m % 9) == 8) {
-                    // ---- coarse noise: P1 S P1^T per component (S = summed fine normals)
-                    for (int o = tid; o < 2 * N * NC; o += THREADS) {
-                        const int r = o / (N * NC), x1 = (o / NC) % N, y2 = o % NC;
-                        float s = 0.f;
-                        for (int x2 = 0; x2 < N; ++x2) s = fmaf(Zs[2 * (x1 * N + x2) + r], P1[y2 * N + x2], s);
-                        Tm[o] = s;
+                if (m9 == 8) {
+                    // ---- coarse noise P1 S P1^T (S = summed fine normals, published by the barrier above):
+                    // T = S P1^T, a thread the rows 2 br, 2 br + 1 and the coarse columns 2 bc, 2 bc + 1
+                    if (fine_thread) {
+                        const ulonglong2* const z0 = reinterpret_cast<const ulonglong2*>(Zs + 2 * br * N);
+                        const ulonglong2* const z1 = reinterpret_cast<const ulonglong2*>(Zs + (2 * br + 1) * N);
+                        const float2* const w0 = reinterpret_cast<const float2*>(P1 + 2 * bc * N);
+                        const float2* const w1 = reinterpret_cast<const float2*>(P1 + (2 * bc + 1) * N);
+                        f32x2 s00 = pack2(0.f, 0.f), s01 = s00, s10 = s00, s11 = s00;
+#pragma unroll 3
+                        for (int x = 0; x < N / 2; ++x) {
+                            const ulonglong2 u = z0[x], v = z1[x];
+                            const float2 p = w0[x], w = w1[x];
+                            const f32x2 px = pack2(p.x, p.x), py = pack2(p.y, p.y), wx = pack2(w.x, w.x), wy = pack2(w.y, w.y);
+                            s00 = fma2(u.y, py, fma2(u.x, px, s00));
+                            s01 = fma2(u.y, wy, fma2(u.x, wx, s01));
+                            s10 = fma2(v.y, py, fma2(v.x, px, s10));
+                            s11 = fma2(v.y, wy, fma2(v.x, wx, s11));
+                        }
+                        reinterpret_cast<ulonglong2*>(Tm)[br * NC + bc] = make_ulonglong2(s00, s01);
+                        reinterpret_cast<ulonglong2*>(Tm)[br * NC + NC / 2 + bc] = make_ulonglong2(s10, s11);
                     }
                     __syncthreads();
                     const int32_t* qc = ccur ? qcB : qcA;
-                    for (int o = tid; o < NC * NC; o += THREADS) {
-                        const int y1 = o / NC, y2 = o % NC;
-                        float s1 = 0.f, s2 = 0.f;
-                        for (int x1 = 0; x1 < N; ++x1) {
-                            const float w = P1[y1 * N + x1];
-                            s1 = fmaf(w, Tm[x1 * NC + y2], s1);
-                            s2 = fmaf(w, Tm[N * NC + x1 * NC + y2], s2);
+                    // two coarse points (y1, y2), (y1 + 1, y2) a thread
+                    for (int o = tid; o < NC * NC / 2; o += THREADS) {
+                        const int y1 = o / NC * 2, y2 = o % NC;
+                        const float2* const w0 = reinterpret_cast<const float2*>(P1 + y1 * N);
+                        const float2* const w1 = reinterpret_cast<const float2*>(P1 + (y1 + 1) * N);
+                        f32x2 s[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
+#pragma unroll 3
+                        for (int x = 0; x < N / 2; ++x) {
+                            const f32x2 t0 = Tm[2 * x * NC + y2], t1 = Tm[(2 * x + 1) * NC + y2];
+                            const float2 p = w0[x], w = w1[x];
+                            s[0] = fma2(pack2(p.y, p.y), t1, fma2(pack2(p.x, p.x), t0, s[0]));
+                            s[1] = fma2(pack2(w.y, w.y), t1, fma2(pack2(w.x, w.x), t0, s[1]));
                         }
-                        // gc includes the 1/3 of the 9-step sum
-                        const float amp = FL ? noise_amp_fluct(qc[o], a.rbc[(size_t)(m / 9) * NC * NC + o], a.isc, a.gc)
-                                             : noise_amp(qc[o], a.gc);
-                        Gc1[o] = __float2int_rn(amp * s1);
-                        Gc2[o] = __float2int_rn(amp * s2);
+#pragma unroll
+                        for (int v = 0; v < 2; ++v) {
+                            const int y = (y1 + v) * NC + y2;
+                            // gc includes the 1/3 of the 9-step sum
+                            const float amp = FL ? noise_amp_fluct(qc[y], a.rbc[(size_t)(m / 9) * NC * NC + y], a.isc, a.gc)
+                                                 : noise_amp(qc[y], a.gc);
+                            Gc1[y] = __float2int_rn(amp * lo2(s[v]));
+                            Gc2[y] = __float2int_rn(amp * hi2(s[v]));
+                        }
                     }
                     __syncthreads();
                     explicit_update<NC, THREADS>(qc, Gc1, Gc2, ccur ? qcA : qcB, a.Ac, bad);
                     ccur ^= 1;
+                    m9 = -1;   // the next barriers order the coarse state for its next step, 9 fine steps on
                 }
+                ++m9;
             }
-            __syncthreads();
         }
+        __syncthreads();
 
         // ---- observables against FP64 test functions, mass; CTA reduction
         double v[kRedF];
 #pragma unroll
         for (int i = 0; i < kRedF; ++i) v[i] = 0.0;
-        const int32_t* q = cur ? qB : qA;
-        for (int x = tid; x < N * N; x += THREADS) {
-            v[2 * kMaxObs] += static_cast<double>(q[x]);
-            const double d = static_cast<double>(q[x] - a.qbf[x]);
-            for (int k = 0; k < a.n_obs; ++k) v[k] += d * f.phif64[(size_t)k * N * N + x];
+        if (fine_thread) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    const int x = fx0 + r * N + c;
+                    v[2 * kMaxObs] += static_cast<double>(q[r][c]);
+                    const double d = static_cast<double>(q[r][c] - a.qbf[x]);
+                    for (int k = 0; k < a.n_obs; ++k) v[k] += d * f.phif64[(size_t)k * N * N + x];
+                }
         }
         if constexpr (CPL) {
             const int32_t* qc = ccur ? qcB : qcA;
