@@ -11,11 +11,17 @@
 // Work decomposition.  A sample's 162^2 fine cells (and their transfers and
 // summed normals) need about 630 KB, so a thread-block cluster of CL = 6 CTAs
 // carries one sample: CTA `rank` holds the band of fine rows 27 rank ..
-// 27 rank + 26 and the coarse rows 9 rank .. 9 rank + 8.  A thread owns a
-// segment of 6 consecutive fine cells of one row in registers (3 Philox cell
-// pairs) and publishes its state and transfers in shared memory; the rows just
-// above and below a band come from the neighbouring CTAs' shared memory
-// (distributed shared memory, periodic over the cluster).
+// 27 rank + 26 and the coarse rows 9 rank .. 9 rank + 8.  A thread owns a block
+// of 3 x 6 fine cells, their transfers and summed normals in registers (three
+// rows of 3 Philox cell pairs) and publishes the block's edges in shared memory
+// (q and G1 of its first and last row, q and G2 of its first and last column);
+// the rows just above and below a band come from the neighbouring CTAs' shared
+// memory (distributed shared memory, periodic over the cluster).
+//
+// Bound by instruction issue and latency with 8 warps of 246 registers on an SM.
+// 45 samples x 1458 steps: 9.03 ms; 11.65 with a 1 x 6 segment of cells per thread,
+// its summed normals in shared memory and 23 warps, whose exchange moved 12 words a
+// cell (here 4) and whose restriction loaded two operands per two FMAs.
 //
 // Exchanges.  State and transfers are double-buffered by the step's parity,
 // so a fine step needs one cluster barrier, split: a thread arrives (release)
@@ -44,21 +50,26 @@ struct XShape {
     static constexpr int N = N_, NC = N / 3, CL = CL_;
     static constexpr int BR = N / CL;               // fine rows per CTA
     static constexpr int CBR = NC / CL;             // coarse rows per CTA
-    static constexpr int SEG = 6;                   // fine cells per thread: one row segment (3 Philox pairs)
-    static constexpr int SEGS = N / SEG;            // segments per row
-    static constexpr int FT = BR * SEGS;            // threads that hold fine cells
+    static constexpr int R = 3, C = 6;              // fine cells per thread
+    static constexpr int BRW = BR / R, BCL = N / C; // rows / columns of blocks per CTA
+    static constexpr int FT = BRW * BCL;            // threads that hold fine cells
     static constexpr int THREADS = (FT + 31) / 32 * 32;
     static constexpr int WARPS = THREADS / 32;
     static constexpr int BAND = BR * N;             // fine cells per CTA
     static constexpr int CBAND = CBR * NC;          // coarse cells per CTA
     static constexpr int HY = NC / 2;               // coarse column pairs
-    static_assert(N % CL == 0 && NC % CL == 0 && N % SEG == 0 && NC % 2 == 0 && BR >= 2 && CBR >= 2,
+    static constexpr int WY = 6;                    // coarse rows of a thread's tile of the partial product
+    static_assert(N % CL == 0 && NC % CL == 0 && N % C == 0 && BR % R == 0 && NC == 2 * BCL && NC % WY == 0 &&
+                      BRW >= 2 && CBR >= 2,
                   "band shape");
-    static_assert(BR * HY <= THREADS && CBAND <= THREADS && THREADS <= 1024, "one task per thread");
-    // words: fine q, G1, G2 (two buffers each) of the band; for a coupled level
-    // the summed normals (2 per cell), P1 transposed (N x NC), T (BR x NC x 2),
-    // the partial product (NC x NC x 2), coarse q (two buffers), Gc1, Gc2
-    static constexpr int WORDS_F = 6 * BAND;
+    static_assert(NC / WY * HY <= THREADS && THREADS <= 1024, "one task per thread");
+    // words: two exchange buffers of edges (q and G1 of the blocks' first and last
+    // rows, q and G2 of their first and last columns); for a coupled level the summed
+    // normals (2 per cell), P1 (NC x N), T (BR x NC x 2), the partial product (NC x
+    // NC x 2), coarse q (two buffers), Gc1, Gc2
+    static constexpr int ROWS = BRW * N, COLS = BR * BCL;
+    static constexpr int XBUF = 4 * ROWS + 4 * COLS;
+    static constexpr int WORDS_F = 2 * XBUF;
     static constexpr int WORDS_C = 2 * BAND + N * NC + 2 * BR * NC + 2 * NC * NC + 4 * CBAND;
     __host__ __device__ static constexpr int words(bool cpl) { return WORDS_F + (cpl ? WORDS_C : 0); }
     static size_t smem(bool cpl, int slot_stride) {
@@ -74,12 +85,10 @@ struct XPhase {
     bool edge;
     bool pend = false;
     __device__ __forceinline__ explicit XPhase(bool edge_) : edge(edge_) {}
-    __device__ __forceinline__ static void arrive() {
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    }
-    __device__ __forceinline__ static void wait() {
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    }
+    // the built-in forms (release / acquire), which the compiler keeps convergent: the
+    // CTA's last warp holds fine cells in part of its lanes only
+    __device__ __forceinline__ static void arrive() { __cluster_barrier_arrive(); }
+    __device__ __forceinline__ static void wait() { __cluster_barrier_wait(); }
     __device__ __forceinline__ void settle() {
         if (pend) {
             wait();
@@ -104,53 +113,41 @@ template <int N, int CL, bool CPL>
 __global__ void __launch_bounds__(XShape<N, CL>::THREADS, 1)
     fourier_cluster_kernel(const KArgs a, const FArgs f) {
     using S = XShape<N, CL>;
-    constexpr int NC = S::NC, BR = S::BR, CBR = S::CBR, SEG = S::SEG, SEGS = S::SEGS, THREADS = S::THREADS;
-    constexpr int BAND = S::BAND, CBAND = S::CBAND, HY = S::HY;
+    constexpr int NC = S::NC, BR = S::BR, CBR = S::CBR, R = S::R, C = S::C, BRW = S::BRW, BCL = S::BCL;
+    constexpr int BAND = S::BAND, CBAND = S::CBAND, HY = S::HY, ROWS = S::ROWS, COLS = S::COLS, THREADS = S::THREADS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cg::cluster_group cluster = cg::this_cluster();
     const int tid = threadIdx.x;
     const int rank = static_cast<int>(cluster.block_rank());
     int32_t* const words = reinterpret_cast<int32_t*>(smem_raw);
-    // fine planes: q buffers at 0, BAND; G1 buffers at 2 BAND, 3 BAND; G2 buffers at 4 BAND, 5 BAND
-    float* const Zs = reinterpret_cast<float*>(words + S::WORDS_F);        // [BAND][2] summed normals
-    float* const P1t = Zs + 2 * BAND;                                      // [N][NC]
-    float* const Tm = P1t + N * NC;                                        // [BR][NC][2]
-    float* const Wp = Tm + 2 * BR * NC;                                    // [NC][NC][2] partial product
-    int32_t* const qc0 = reinterpret_cast<int32_t*>(Wp + 2 * NC * NC);     // coarse q buffers at qc0, qc0 + CBAND
+    f32x2* const Zs = reinterpret_cast<f32x2*>(words + S::WORDS_F);        // [BAND] summed normals, both components
+    f32x2* const Tm = Zs + BAND;                                           // [BR][NC]
+    f32x2* const Wp = Tm + BR * NC;                                        // [NC][NC] partial product
+    float* const P1 = reinterpret_cast<float*>(Wp + NC * NC);              // [NC][N]
+    int32_t* const qc0 = reinterpret_cast<int32_t*>(P1 + NC * N);        // coarse q buffers at qc0, qc0 + CBAND
     int32_t* const Gc1 = qc0 + 2 * CBAND;
     int32_t* const Gc2 = Gc1 + CBAND;
     double* const red = reinterpret_cast<double*>(smem_raw + sizeof(int32_t) * (size_t)((S::words(CPL) + 1) / 2 * 2));
     double* const tot = red + S::WARPS * kRedX;      // this CTA's band totals
     double* const acc = tot + kRedX;                 // the slot's moment sums (rank 0)
     for (int i = tid; i < a.slot_stride; i += THREADS) acc[i] = 0.0;
-    if constexpr (CPL)
-        for (int i = tid; i < N * NC; i += THREADS) {
-            const int x = i / NC, y = i % NC;
-            P1t[i] = f.P1[(size_t)y * N + x];
-        }
+    if constexpr (CPL) {
+        for (int i = tid; i < N * NC; i += THREADS) P1[i] = f.P1[i];
+    }
 
-    // ---- the thread's fine segment and its neighbours
+    // ---- the thread's fine block and its neighbours
     const bool fine_thread = tid < S::FT;
-    const int lr = fine_thread ? tid / SEGS : 0;
-    const int c0 = fine_thread ? (tid % SEGS) * SEG : 0;
-    const int x0 = lr * N + c0;                                   // first cell of the segment in the band
-    const int gx0 = rank * BAND + x0;                             // ... on the whole grid
-    const int ra = lr > 0 ? rank : (rank + CL - 1) % CL;          // CTA of the row above / below
-    const int rb = lr < BR - 1 ? rank : (rank + 1) % CL;
-    const int ia = lr > 0 ? x0 - N : (BR - 1) * N + c0;           // its first cell there
-    const int ib = lr < BR - 1 ? x0 + N : c0;
-    const int32_t* const up = ra == rank ? words : cluster.map_shared_rank(words, ra);
-    const int32_t* const dn = rb == rank ? words : cluster.map_shared_rank(words, rb);
-    const int lfx = c0 == 0 ? x0 + N - 1 : x0 - 1;                // left of the first cell
-    const int rtx = c0 + SEG == N ? x0 + SEG - N : x0 + SEG;      // right of the last cell
-    // the warps holding a cell of the band's first or last row read other CTAs
-    // (rows are not warp-aligned, so the test is per warp: the cluster wait is .aligned)
+    const int br = fine_thread ? tid / BCL : 0, bc = fine_thread ? tid % BCL : 0;
+    const int gx0 = (rank * BR + br * R) * N + bc * C;            // first cell on the whole grid
+    const int lb = (bc + BCL - 1) % BCL, rb = (bc + 1) % BCL;     // blocks left / right
+    // the block rows above / below: row of blocks and CTA
+    const int rup = br > 0 ? br - 1 : BRW - 1, rdn = br < BRW - 1 ? br + 1 : 0;
+    const int32_t* const up = br > 0 ? words : cluster.map_shared_rank(words, (rank + CL - 1) % CL);
+    const int32_t* const dn = br < BRW - 1 ? words : cluster.map_shared_rank(words, (rank + 1) % CL);
+    // the warps holding a block of the band's first or last block row read other CTAs
+    // (block rows are not warp-aligned, so the test is per warp: the cluster wait is .aligned)
     const int wf = tid & ~31, wl = min(wf + 31, S::FT - 1);
-    XPhase ph(wf < S::FT && (wf / SEGS == 0 || wl / SEGS >= BR - 1));
-
-    // ---- the thread's coarse cell (coupled levels): local index tid, global index
-    // (rank CBR + tid / NC) NC + tid % NC = rank CBAND + tid
-    const bool coarse_thread = CPL && tid < CBAND;
+    XPhase ph(wf < S::FT && (wf / BCL == 0 || wl / BCL == BRW - 1));
 
     const long long n_slots = (long long)gridDim.x / CL;
     const long long slot = (long long)blockIdx.x / CL;
@@ -163,157 +160,183 @@ __global__ void __launch_bounds__(XShape<N, CL>::THREADS, 1)
         const long long sid = a.first + idx;
         const uint32_t c2 = static_cast<uint32_t>(sid);
         const uint32_t c3 = a.tag | ((static_cast<uint32_t>(static_cast<unsigned long long>(sid) >> 32) & 0xffffu) << 16);
-        int32_t qr[SEG];
-        if (fine_thread) {
+        int32_t q[R][C];
+        f32x2 Z[R][C];   // summed normals of the coarse step, both components
 #pragma unroll
-            for (int j = 0; j < SEG; j += 2) {
-                qr[j] = a.q0f[gx0 + j];
-                qr[j + 1] = a.q0f[gx0 + j + 1];
-                *reinterpret_cast<int2*>(words + x0 + j) = make_int2(qr[j], qr[j + 1]);
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                q[r][c] = a.q0f[gx0 + r * N + c];
+                Z[r][c] = pack2(0.f, 0.f);
             }
-        }
         int cb = 0;
-        if (coarse_thread) qc0[tid] = a.q0c[rank * CBAND + tid];
+        if constexpr (CPL) {
+            for (int y = tid; y < CBAND; y += THREADS) qc0[y] = a.q0c[rank * CBAND + y];
+        }
         ph.full();
 
-        for (int m = 0; m < a.M; ++m) {
-            const int b = m & 1;
-            const bool first_of_coarse = CPL && (m % 9) == 0;
-            int32_t g1[SEG], g2[SEG];
-            // ---- noise of the segment: Philox4x32-10 per horizontal cell pair, Box--Muller, transfers
+        for (int m = 0, m9 = 0; m < a.M; ++m) {
+            // the step's exchange buffer: rows [BRW][N] of q top, q bottom, G1 top, G1
+            // bottom; columns [BR][BCL] of q first, q last, G2 first, G2 last
+            const int xo = (m & 1) * S::XBUF, xc = xo + 4 * ROWS;
+            int32_t G1[R][C], G2[R][C];
+            // ---- noise of the block: Philox4x32-10 per horizontal cell pair, Box--Muller, transfers
             if (fine_thread) {
-                int2* const G1w = reinterpret_cast<int2*>(words + (2 + b) * BAND);
-                int2* const G2w = reinterpret_cast<int2*>(words + (4 + b) * BAND);
+                const f32x2 g2v = pack2(a.gf, a.gf);
 #pragma unroll
-                for (int j = 0; j < SEG / 2; ++j) {
-                    const int p = (gx0 >> 1) + j, lp = (x0 >> 1) + j;
-                    const uint4 x = philox10(make_uint4(static_cast<uint32_t>(p), static_cast<uint32_t>(m), c2, c3),
-                                             a.key0, a.key1);
-                    float ra_, ca, sa, rb_, cbn, sb;
-                    box_muller_polar(x.x, x.y, ra_, ca, sa);
-                    box_muller_polar(x.z, x.w, rb_, cbn, sb);
-                    const float ta = noise_amp(qr[2 * j], a.gf) * ra_;
-                    const float tb = noise_amp(qr[2 * j + 1], a.gf) * rb_;
-                    g1[2 * j] = __float2int_rn(ta * ca);
-                    g2[2 * j] = __float2int_rn(ta * sa);
-                    g1[2 * j + 1] = __float2int_rn(tb * cbn);
-                    g2[2 * j + 1] = __float2int_rn(tb * sb);
-                    G1w[lp] = make_int2(g1[2 * j], g1[2 * j + 1]);
-                    G2w[lp] = make_int2(g2[2 * j], g2[2 * j + 1]);
-                    if constexpr (CPL) {
-                        float4 z = first_of_coarse ? make_float4(0.f, 0.f, 0.f, 0.f)
-                                                   : reinterpret_cast<float4*>(Zs)[lp];
-                        z.x += ra_ * ca;
-                        z.y += ra_ * sa;
-                        z.z += rb_ * cbn;
-                        z.w += rb_ * sb;
-                        reinterpret_cast<float4*>(Zs)[lp] = z;
+                for (int r = 0; r < R; ++r) {
+#pragma unroll
+                    for (int j = 0; j < C / 2; ++j) {
+                        const int p = ((gx0 + r * N) >> 1) + j;
+                        const uint4 x = philox10(make_uint4(static_cast<uint32_t>(p), static_cast<uint32_t>(m), c2, c3),
+                                                 a.key0, a.key1);
+                        f32x2 rad, co, si;
+                        box_muller_polar2(x.x, x.y, x.z, x.w, rad, co, si);
+                        const f32x2 t = mul2(noise_amp2(q[r][2 * j], q[r][2 * j + 1], g2v), rad);
+                        const f32x2 t1 = mul2(t, co), t2 = mul2(t, si);
+                        G1[r][2 * j] = __float2int_rn(lo2(t1));
+                        G1[r][2 * j + 1] = __float2int_rn(hi2(t1));
+                        G2[r][2 * j] = __float2int_rn(lo2(t2));
+                        G2[r][2 * j + 1] = __float2int_rn(hi2(t2));
+                        if (r == 0 || r == R - 1) {
+                            int32_t* const row = words + xo + (r == 0 ? 0 : ROWS) + br * N + bc * C + 2 * j;
+                            *reinterpret_cast<int2*>(row) = make_int2(q[r][2 * j], q[r][2 * j + 1]);
+                            *reinterpret_cast<int2*>(row + 2 * ROWS) = make_int2(G1[r][2 * j], G1[r][2 * j + 1]);
+                        }
+                        if constexpr (CPL) {
+                            const float za = lo2(rad), zb = hi2(rad);
+                            Z[r][2 * j] = fma2(pack2(za, za), pack2(lo2(co), lo2(si)), Z[r][2 * j]);
+                            Z[r][2 * j + 1] = fma2(pack2(zb, zb), pack2(hi2(co), hi2(si)), Z[r][2 * j + 1]);
+                        }
+                    }
+                    int32_t* const col = words + xc + (br * R + r) * BCL + bc;
+                    col[0] = q[r][0];
+                    col[COLS] = q[r][C - 1];
+                    col[2 * COLS] = G2[r][0];
+                    col[3 * COLS] = G2[r][C - 1];
+                }
+                if constexpr (CPL) {
+                    if (m9 == 8) {
+#pragma unroll
+                        for (int r = 0; r < R; ++r)
+#pragma unroll
+                            for (int c = 0; c < C; c += 2) {
+                                reinterpret_cast<ulonglong2*>(Zs)[((br * R + r) * N + bc * C + c) / 2] =
+                                    make_ulonglong2(Z[r][c], Z[r][c + 1]);
+                                Z[r][c] = Z[r][c + 1] = pack2(0.f, 0.f);
+                            }
                     }
                 }
             }
             ph.publish();
-            // ---- explicit step of the segment in flux form (every edge flux computed
+            // ---- explicit step of the block in flux form (every edge flux computed
             // from the same two states by both of its cells)
             if (fine_thread) {
-                const int32_t* const q = words + b * BAND;
-                const int32_t* const G2 = words + (4 + b) * BAND;
-                int32_t qu[SEG], qd[SEG], gu[SEG], gd[SEG];
+                int32_t qu[C], qd[C], gu[C], gd[C], ql[R], qr[R], gl[R], gr[R];
+                const int32_t* const ru = up + xo + ROWS + rup * N + bc * C;
+                const int32_t* const rd = dn + xo + rdn * N + bc * C;
 #pragma unroll
-                for (int j = 0; j < SEG; j += 2) {
-                    const int2 a0 = *reinterpret_cast<const int2*>(up + b * BAND + ia + j);
-                    const int2 a1 = *reinterpret_cast<const int2*>(dn + b * BAND + ib + j);
-                    const int2 b0 = *reinterpret_cast<const int2*>(up + (2 + b) * BAND + ia + j);
-                    const int2 b1 = *reinterpret_cast<const int2*>(dn + (2 + b) * BAND + ib + j);
+                for (int j = 0; j < C; j += 2) {
+                    const int2 a0 = *reinterpret_cast<const int2*>(ru + j);
+                    const int2 a1 = *reinterpret_cast<const int2*>(rd + j);
+                    const int2 b0 = *reinterpret_cast<const int2*>(ru + 2 * ROWS + j);
+                    const int2 b1 = *reinterpret_cast<const int2*>(rd + 2 * ROWS + j);
                     qu[j] = a0.x; qu[j + 1] = a0.y; qd[j] = a1.x; qd[j + 1] = a1.y;
                     gu[j] = b0.x; gu[j + 1] = b0.y; gd[j] = b1.x; gd[j + 1] = b1.y;
                 }
-                const int32_t qlf = q[lfx], qrt = q[rtx], g2lf = G2[lfx], g2rt = G2[rtx];
-                int32_t nq[SEG];
 #pragma unroll
-                for (int j = 0; j < SEG; ++j) {
-                    const int32_t c = qr[j];
-                    const int32_t lf = j == 0 ? qlf : qr[j - 1];
-                    const int32_t rt = j == SEG - 1 ? qrt : qr[j + 1];
-                    const int32_t g2l = j == 0 ? g2lf : g2[j - 1];
-                    const int32_t g2r = j == SEG - 1 ? g2rt : g2[j + 1];
-                    nq[j] = c + (edge_flux(a.Af, qd[j] - c) - edge_flux(a.Af, c - qu[j])) +
-                            (edge_flux(a.Af, rt - c) - edge_flux(a.Af, c - lf)) + (gd[j] - gu[j]) + (g2r - g2l);
-                    bad |= (static_cast<uint32_t>(nq[j]) + 0x40000000u) >> 31;
+                for (int r = 0; r < R; ++r) {
+                    const int32_t* const col = words + xc + (br * R + r) * BCL;
+                    ql[r] = col[COLS + lb];
+                    qr[r] = col[rb];
+                    gl[r] = col[3 * COLS + lb];
+                    gr[r] = col[2 * COLS + rb];
                 }
-                int32_t* const qn = words + (b ^ 1) * BAND;
+                flux_update<R, C>(q, G1, G2, qu, gu, qd, gd, ql, gl, qr, gr, a.Af);
 #pragma unroll
-                for (int j = 0; j < SEG; j += 2) {
-                    qr[j] = nq[j];
-                    qr[j + 1] = nq[j + 1];
-                    *reinterpret_cast<int2*>(qn + x0 + j) = make_int2(nq[j], nq[j + 1]);
-                }
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int c = 0; c < C; ++c) bad |= (static_cast<uint32_t>(q[r][c]) + 0x40000000u) >> 31;
             }
             if constexpr (CPL) {
-                if ((m % 9) == 8) {
+                if (m9 == 8) {
                     ph.settle();
-                    // ---- T = S_band P1^T: row x1 of the band, coarse columns 2 yy and 2 yy + 1, both components
-                    if (tid < BR * HY) {
-                        const int lx1 = tid / HY, yy = tid % HY;
-                        const float2* const zrow = reinterpret_cast<const float2*>(Zs) + lx1 * N;
-                        const float2* const pcol = reinterpret_cast<const float2*>(P1t) + yy;
-                        float s00 = 0.f, s01 = 0.f, s10 = 0.f, s11 = 0.f;
-#pragma unroll 6
-                        for (int x2 = 0; x2 < N; ++x2) {
-                            const float2 z = zrow[x2], w = pcol[x2 * HY];
-                            s00 = fmaf(z.x, w.x, s00);
-                            s01 = fmaf(z.y, w.x, s01);
-                            s10 = fmaf(z.x, w.y, s10);
-                            s11 = fmaf(z.y, w.y, s11);
+                    // ---- T = S_band P1^T (S published by the barrier above): the block's rows,
+                    // coarse columns 2 bc and 2 bc + 1, both components packed
+                    if (fine_thread) {
+                        const float2* const w0 = reinterpret_cast<const float2*>(P1 + 2 * bc * N);
+                        const float2* const w1 = reinterpret_cast<const float2*>(P1 + (2 * bc + 1) * N);
+                        const ulonglong2* const z = reinterpret_cast<const ulonglong2*>(Zs + br * R * N);
+                        f32x2 s0[R], s1[R];
+#pragma unroll
+                        for (int r = 0; r < R; ++r) s0[r] = s1[r] = pack2(0.f, 0.f);
+#pragma unroll 3
+                        for (int x = 0; x < N / 2; ++x) {
+                            const float2 p = w0[x], w = w1[x];
+                            const f32x2 px = pack2(p.x, p.x), py = pack2(p.y, p.y), wx = pack2(w.x, w.x), wy = pack2(w.y, w.y);
+#pragma unroll
+                            for (int r = 0; r < R; ++r) {
+                                const ulonglong2 u = z[r * (N / 2) + x];
+                                s0[r] = fma2(u.y, py, fma2(u.x, px, s0[r]));
+                                s1[r] = fma2(u.y, wy, fma2(u.x, wx, s1[r]));
+                            }
                         }
-                        reinterpret_cast<float4*>(Tm)[lx1 * HY + yy] = make_float4(s00, s01, s10, s11);
+#pragma unroll
+                        for (int r = 0; r < R; ++r)
+                            reinterpret_cast<ulonglong2*>(Tm)[(br * R + r) * HY + bc] = make_ulonglong2(s0[r], s1[r]);
                     }
                     __syncthreads();
-                    // ---- the band's part of P1 S P1^T: every coarse point (y1, 2 yy + v)
-                    for (int o = tid; o < NC * HY; o += THREADS) {
-                        const int y1 = o / HY, yy = o % HY;
-                        float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 9
-                        for (int lx1 = 0; lx1 < BR; ++lx1) {
-                            const float p = P1t[(rank * BR + lx1) * NC + y1];
-                            const float4 t = reinterpret_cast<const float4*>(Tm)[lx1 * HY + yy];
-                            w.x = fmaf(p, t.x, w.x);
-                            w.y = fmaf(p, t.y, w.y);
-                            w.z = fmaf(p, t.z, w.z);
-                            w.w = fmaf(p, t.w, w.w);
+                    // ---- the band's part of P1 S P1^T: WY coarse rows of the columns 2 yy, 2 yy + 1
+                    if (tid < NC / S::WY * HY) {
+                        const int y0 = tid / HY * S::WY, yy = tid % HY;
+                        f32x2 w0[S::WY], w1[S::WY];
+#pragma unroll
+                        for (int v = 0; v < S::WY; ++v) w0[v] = w1[v] = pack2(0.f, 0.f);
+#pragma unroll 3
+                        for (int x = 0; x < BR; ++x) {
+                            const ulonglong2 t = reinterpret_cast<const ulonglong2*>(Tm)[x * HY + yy];
+#pragma unroll
+                            for (int v = 0; v < S::WY; ++v) {
+                                const float p = P1[(y0 + v) * N + rank * BR + x];
+                                w0[v] = fma2(pack2(p, p), t.x, w0[v]);
+                                w1[v] = fma2(pack2(p, p), t.y, w1[v]);
+                            }
                         }
-                        reinterpret_cast<float4*>(Wp)[o] = w;
+#pragma unroll
+                        for (int v = 0; v < S::WY; ++v)
+                            reinterpret_cast<ulonglong2*>(Wp)[(y0 + v) * HY + yy] = make_ulonglong2(w0[v], w1[v]);
                     }
                     ph.full();
                     // ---- coarse transfers of the CTA's coarse rows: the partials summed in rank order
                     int32_t* const qc = qc0 + cb * CBAND;
-                    if (coarse_thread) {
-                        const int o = rank * CBAND + tid;   // coarse point (y1, y2), y1 = rank CBR + tid / NC
+                    for (int y = tid; y < CBAND; y += THREADS) {
+                        const int o = rank * CBAND + y;   // coarse point (y1, y2), y1 = rank CBR + y / NC
                         float w0 = 0.f, w1 = 0.f;
 #pragma unroll
                         for (int r = 0; r < CL; ++r) {
-                            const float* const src = r == rank ? Wp : cluster.map_shared_rank(Wp, r);
-                            const float2 v = reinterpret_cast<const float2*>(src)[o];
-                            w0 += v.x;
-                            w1 += v.y;
+                            const f32x2* const src = r == rank ? Wp : cluster.map_shared_rank(Wp, r);
+                            const f32x2 v = src[o];
+                            w0 += lo2(v);
+                            w1 += hi2(v);
                         }
-                        const float amp = noise_amp(qc[tid], a.gc);   // gc includes the 1/3 of the 9-step sum
-                        Gc1[tid] = __float2int_rn(amp * w0);
-                        Gc2[tid] = __float2int_rn(amp * w1);
+                        const float amp = noise_amp(qc[y], a.gc);   // gc includes the 1/3 of the 9-step sum
+                        Gc1[y] = __float2int_rn(amp * w0);
+                        Gc2[y] = __float2int_rn(amp * w1);
                     }
                     ph.full();
                     // ---- explicit coarse step of the CTA's coarse rows
-                    if (coarse_thread) {
+                    for (int y = tid; y < CBAND; y += THREADS) {
                         // neighbours of the coarse cell: above / below in the neighbouring CTA for
                         // the band's first / last coarse row (periodic over the cluster)
-                        const int cl1 = tid / NC, cy2 = tid % NC;
+                        const int cl1 = y / NC, cy2 = y % NC;
                         const int cra = cl1 > 0 ? rank : (rank + CL - 1) % CL;
                         const int crb = cl1 < CBR - 1 ? rank : (rank + 1) % CL;
-                        const int cia = cl1 > 0 ? tid - NC : (CBR - 1) * NC + cy2;
-                        const int cib = cl1 < CBR - 1 ? tid + NC : cy2;
+                        const int cia = cl1 > 0 ? y - NC : (CBR - 1) * NC + cy2;
+                        const int cib = cl1 < CBR - 1 ? y + NC : cy2;
                         const int clf = cl1 * NC + (cy2 + NC - 1) % NC, crt = cl1 * NC + (cy2 + 1) % NC;
                         const int32_t* const cup = cra == rank ? qc0 : cluster.map_shared_rank(qc0, cra);
                         const int32_t* const cdn = crb == rank ? qc0 : cluster.map_shared_rank(qc0, crb);
-                        const int32_t c = qc[tid];
+                        const int32_t c = qc[y];
                         const int32_t* const gu_p = cra == rank ? Gc1 : cluster.map_shared_rank(Gc1, cra);
                         const int32_t* const gd_p = crb == rank ? Gc1 : cluster.map_shared_rank(Gc1, crb);
                         const int32_t qu = cup[cb * CBAND + cia], qd = cdn[cb * CBAND + cib];
@@ -321,10 +344,12 @@ __global__ void __launch_bounds__(XShape<N, CL>::THREADS, 1)
                                           (edge_flux(a.Ac, qc[crt] - c) - edge_flux(a.Ac, c - qc[clf])) +
                                           (gd_p[cib] - gu_p[cia]) + (Gc2[crt] - Gc2[clf]);
                         bad |= (static_cast<uint32_t>(v) + 0x40000000u) >> 31;
-                        qc0[(cb ^ 1) * CBAND + tid] = v;
+                        qc0[(cb ^ 1) * CBAND + y] = v;
                     }
                     cb ^= 1;
+                    m9 = -1;
                 }
+                ++m9;
             }
         }
 
@@ -336,27 +361,35 @@ __global__ void __launch_bounds__(XShape<N, CL>::THREADS, 1)
         if (fine_thread) {
             long long mf = 0;
 #pragma unroll
-            for (int j = 0; j < SEG; ++j) mf += qr[j];
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < C; ++c) mf += q[r][c];
             v[2 * kMaxObs] = static_cast<double>(mf);
 #pragma unroll
             for (int k = 0; k < kMaxObs; ++k) {
                 if (k < a.n_obs) {
                     double s = 0.0;
 #pragma unroll
-                    for (int j = 0; j < SEG; ++j)
-                        s += static_cast<double>(qr[j] - a.qbf[gx0 + j]) * f.phif64[(size_t)k * N * N + gx0 + j];
+                    for (int r = 0; r < R; ++r)
+#pragma unroll
+                        for (int c = 0; c < C; ++c) {
+                            const int x = gx0 + r * N + c;
+                            s += static_cast<double>(q[r][c] - a.qbf[x]) * f.phif64[(size_t)k * N * N + x];
+                        }
                     v[k] = s;
                 }
             }
         }
-        if (coarse_thread) {
-            const int cg1 = rank * CBAND + tid;
-            const int32_t qv = qc0[cb * CBAND + tid];
-            v[2 * kMaxObs + 1] = static_cast<double>(qv);
-            const double d = static_cast<double>(qv - a.qbc[cg1]);
+        if constexpr (CPL) {
+            for (int y = tid; y < CBAND; y += THREADS) {
+                const int cg1 = rank * CBAND + y;
+                const int32_t qv = qc0[cb * CBAND + y];
+                v[2 * kMaxObs + 1] += static_cast<double>(qv);
+                const double d = static_cast<double>(qv - a.qbc[cg1]);
 #pragma unroll
-            for (int k = 0; k < kMaxObs; ++k)
-                if (k < a.n_obs) v[kMaxObs + k] = d * f.phic64[(size_t)k * NC * NC + cg1];
+                for (int k = 0; k < kMaxObs; ++k)
+                    if (k < a.n_obs) v[kMaxObs + k] += d * f.phic64[(size_t)k * NC * NC + cg1];
+            }
         }
 #pragma unroll
         for (int off = 16; off >= 1; off >>= 1)
