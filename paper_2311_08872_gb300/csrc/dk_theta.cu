@@ -1,7 +1,7 @@
 // Theta-scheme sample kernel for sm_103a: Eq. (FullyDiscreteDK) with an
 // implicit diffusion weight b0 > 0 (b1 = 1 - b0; Definition 2.1, the operator
 // A_h of Appendix C), for the NN-coupled pair of Section 3.2 on grids up to
-// 64 x 64.
+// 128 x 128.
 //
 // Step.  Subtracting (I - b0 tau/2 Delta_h) rho^(m-1) from both sides of the
 // scheme gives the increment
@@ -20,18 +20,43 @@
 // keeps sum_x q invariant bit for bit, as in the explicit kernels.  K = 0
 // (b0 = 0) is exactly the explicit step.
 //
-// Work decomposition.  One CTA holds SPB samples; each sample uses (n/2)^2
-// threads, thread t owning coarse cell t and the 2 x 2 block of fine cells to
-// its right-most side (the coupling block of Section 3.2), so the coupled
-// coarse increment is summed in the thread's registers.  The fine state and
-// every Chebyshev operand stay in registers: a coarse row of blocks is a
-// segment of n/2 consecutive lanes, so left / right neighbours come by warp
-// shuffles (the segment wrap is the periodic wrap) and only the top and
-// bottom rows of each block pass through shared memory for the blocks above
-// and below (contiguous 8- and 16-byte accesses), one barrier per Chebyshev
-// step.  The coarse step (1/16 of the work) keeps its state and operands in
-// shared memory.
+// Work decomposition.  A thread owns an R x C block of fine cells (and the
+// (R/2) x (C/2) coarse cells they couple to, so the coupled increments are
+// summed in registers); the state, the face fluxes and the Chebyshev operands
+// stay in registers, the two components of a cell packed in one FP32 pair, so
+// an iteration is 9 packed operations per cell.  A row of blocks is a segment
+// of N/C <= 32 consecutive lanes: left / right neighbours come by warp shuffles
+// (the segment wrap is the periodic wrap) and only the blocks' top and bottom
+// rows pass through shared memory, one CTA barrier per iteration (two buffers
+// in turn).  An exchange costs 4 R shuffles and 8 C shared-memory words per
+// block against R C cells of arithmetic: 4 x 4 blocks balance the two (2 x 2
+// blocks spent more on the exchange than on the cells) and fit in 255
+// registers with 8 warps on an SM.  A sample of up to 16 x 16 cells fits one
+// warp (no CTA barrier).
+//
+// 128 x 128 takes a cluster of 4 CTAs, each a band of 8 block rows (one warp
+// each).  A warp of the band's first or last block row sends its edge row to
+// the neighbouring CTA's shared memory with asynchronous stores that complete
+// on an mbarrier there, and waits on its own: an exchange is one message each
+// way between two warps, where a cluster barrier held all 4 CTAs at every
+// iteration.  Four message slots in turn need no other handshake: slot n % 4 is
+// written again by exchange n + 4, after the sender has received the neighbour's
+// message n + 3, which that warp sent after the CTA barriers of its exchanges
+// n + 1 and n + 2, before which it read message n.  (Two slots are not enough:
+// message n + 1 need not depend on message n, as between the coarse and the next
+// fine step, and nothing else orders that read before it.)  Every wait is bounded: after kMbarPolls polls it records kErrTimeout, and the CTA waits no
+// more.
+//
+// Bound by instruction issue and latency: 9 packed operations per cell and iteration
+// take two cycles each on the FP32 pipe, and an iteration ends in a barrier.
+// Crank--Nicolson (14 iterations), ms, in brackets with 2 x 2 blocks per thread and a
+// cluster barrier per iteration: 128^2, 75 samples x 384 steps, 14.2 (29.7), 36
+// samples 4.95 (9.90); 64^2, 1000 x 96, 6.15 (8.98), 152 samples 1.03 (1.29); 32^2,
+// 20000 x 24, 7.14 (10.4).  With the inner rows of a block after the barrier instead
+// of before it, 64^2 took 1.11 (152 samples) and 6.61 (1000).
 #include <cooperative_groups.h>
+
+#include <type_traits>
 
 #include "dk_device.cuh"
 #include "dk_kernels.h"
@@ -39,19 +64,39 @@
 namespace dk {
 namespace {
 
+namespace cg = cooperative_groups;
+
 constexpr unsigned kFullMask = 0xffffffffu;
 constexpr int kRed = 2 * kMaxObs + 2;   // reduced values per sample
 
-template <int N_>
+// Shapes: fine block R x C per thread, CL CTAs per sample.
+template <int N_, bool DENSE_>
 struct TShape {
     static constexpr int N = N_, NC = N / 2;
-    static constexpr int TPS = NC * NC;                    // threads per sample
-    static constexpr int THREADS = TPS >= 128 ? TPS : 128;
+    static constexpr bool DENSE = DENSE_;
+    static constexpr bool SMALL = N < 32 || (N == 32 && !DENSE);
+    static constexpr int R = SMALL ? 2 : 4, C = N >= 16 && !(N == 32 && !DENSE) ? 4 : 2;
+    static constexpr int CL = N >= 128 ? 4 : 1;
+    static constexpr int LPR = N / C;                      // lanes per row of blocks
+    static constexpr int NBR = N / R / CL;                 // block rows per CTA and sample
+    static constexpr int TPS = NBR * LPR;                  // threads per sample and CTA
+    static constexpr int THREADS = TPS >= 64 ? TPS : 128;
     static constexpr int SPB = THREADS / TPS;              // samples per CTA
-    // per sample: four planes of n^2 words, coarse state
-    static constexpr size_t SAMPLE_BYTES = sizeof(int32_t) * (N * N * 4 + NC * NC);
+    // Registers per thread: up to 255 (8 warps on an SM), 128 for the 2 x 2 blocks at
+    // 32^2 and where DENSE (16 warps; the fluxes and the coarse state of 4 x 4 blocks
+    // then spill outside the iteration).  16^2 wants the first: 256 samples 34.0 us
+    // with 155 registers, 40.0 with 128.
+    static constexpr int MIN_CTAS = (DENSE || N == 32 ? 512 : 256) / THREADS;
+    static_assert(LPR <= 32 && (SPB == 1 || TPS <= 32) && (CL == 1 || LPR == 32), "block layout");
+    // per sample: two buffers of the blocks' top and bottom rows, two words a cell;
+    // in a cluster also four message slots for the rows above and below the band,
+    // and their mbarriers
+    static constexpr int BUF = 4 * N * NBR;                // words of one buffer
+    static constexpr int SLOT = 4 * N;                     // words of one message slot (both sides)
+    static constexpr int WORDS = 2 * BUF + (CL > 1 ? 4 * SLOT : 0);
+    static constexpr size_t SAMPLE_BYTES = sizeof(int32_t) * WORDS + (CL > 1 ? 8 * sizeof(uint64_t) : 0);
     static size_t smem(int slot_stride) {
-        return SAMPLE_BYTES * SPB + sizeof(double) * ((THREADS + 31) / 32) * kRed +
+        return SAMPLE_BYTES * SPB + sizeof(double) * ((THREADS + 31) / 32) * kRed + sizeof(double) * kRed +
                sizeof(double) * SPB * slot_stride;
     }
 };
@@ -63,293 +108,344 @@ __device__ __forceinline__ int32_t edge_flux64(long long A, int32_t d) {
 __device__ __forceinline__ float as_f(int32_t v) { return __int_as_float(v); }
 __device__ __forceinline__ int32_t as_i(float v) { return __float_as_int(v); }
 
-// One step of the theta-scheme on an NN x NN periodic grid for the NCELL cells
-// (row[i], col[i]) of this thread.  On entry sq holds the state of every cell
-// and P0 / P2 the noise transfers G_1 / G_2 of every cell (as integers),
-// published by a barrier.  On exit q and sq hold the new state, published by a
-// barrier.  P0..P3 are NN x NN scratch planes.
-template <int NN, int NCELL>
-__device__ __forceinline__ void theta_step(int32_t (&q)[NCELL], const int (&row)[NCELL], const int (&col)[NCELL],
-                                           int32_t* sq, float* P0, float* P1, float* P2, float* P3, long long A,
-                                           const TArgs& t, unsigned& bad) {
-    int idx[NCELL], dn[NCELL], rt[NCELL], up[NCELL], lf[NCELL];
-#pragma unroll
-    for (int i = 0; i < NCELL; ++i) {
-        idx[i] = row[i] * NN + col[i];
-        dn[i] = ((row[i] + 1) % NN) * NN + col[i];
-        up[i] = ((row[i] + NN - 1) % NN) * NN + col[i];
-        rt[i] = row[i] * NN + (col[i] + 1) % NN;
-        lf[i] = row[i] * NN + (col[i] + NN - 1) % NN;
-    }
-    // face fluxes across x -> x + e_1 (down) and x -> x + e_2 (right), exact
-    long long F1[NCELL], F2[NCELL];
-#pragma unroll
-    for (int i = 0; i < NCELL; ++i) {
-        const int32_t g1 = as_i(P0[idx[i]]), g2 = as_i(P2[idx[i]]);
-        F1[i] = (long long)edge_flux64(A, sq[dn[i]] - q[i]) + g1 + as_i(P0[dn[i]]);
-        F2[i] = (long long)edge_flux64(A, sq[rt[i]] - q[i]) + g2 + as_i(P2[rt[i]]);
-    }
-    float u1[NCELL], u2[NCELL];
-#pragma unroll
-    for (int i = 0; i < NCELL; ++i) u1[i] = u2[i] = 0.f;
-    float* out1 = P1;   // plane that receives the corrected fluxes
-    float* out2 = P3;
-    if (t.K > 0) {
-        // right-hand side -alpha L F and the first Chebyshev direction (the
-        // barrier after the F planes also orders every read of the G planes
-        // before the direction overwrites them)
-#pragma unroll
-        for (int i = 0; i < NCELL; ++i) {
-            P1[idx[i]] = static_cast<float>(F1[i]);
-            P3[idx[i]] = static_cast<float>(F2[i]);
-        }
-        __syncthreads();
-        float r1[NCELL], r2[NCELL], d1[NCELL], d2[NCELL];
-#pragma unroll
-        for (int i = 0; i < NCELL; ++i) {
-            const float f1 = P1[idx[i]], f2 = P3[idx[i]];
-            const float l1 = 4.f * f1 - P1[up[i]] - P1[dn[i]] - P1[lf[i]] - P1[rt[i]];
-            const float l2 = 4.f * f2 - P3[up[i]] - P3[dn[i]] - P3[lf[i]] - P3[rt[i]];
-            r1[i] = -t.alpha * l1;
-            r2[i] = -t.alpha * l2;
-            d1[i] = r1[i] * t.inv_theta;
-            d2[i] = r2[i] * t.inv_theta;
-            P0[idx[i]] = d1[i];
-            P2[idx[i]] = d2[i];
-        }
-        __syncthreads();
-        float *c1p = P0, *c2p = P2, *n1p = P1, *n2p = P3;   // current / next direction planes
-        const float diag = 1.f + 4.f * t.alpha;
-        for (int k = 0; k < t.K; ++k) {
-#pragma unroll
-            for (int i = 0; i < NCELL; ++i) {
-                const float a1 = diag * d1[i] - t.alpha * (c1p[up[i]] + c1p[dn[i]] + c1p[lf[i]] + c1p[rt[i]]);
-                const float a2 = diag * d2[i] - t.alpha * (c2p[up[i]] + c2p[dn[i]] + c2p[lf[i]] + c2p[rt[i]]);
-                u1[i] += d1[i];
-                u2[i] += d2[i];
-                r1[i] -= a1;
-                r2[i] -= a2;
-            }
-            if (k + 1 < t.K) {
-                const float ca = t.c1[k], cb = t.c2[k];
-#pragma unroll
-                for (int i = 0; i < NCELL; ++i) {
-                    d1[i] = ca * d1[i] + cb * r1[i];
-                    d2[i] = ca * d2[i] + cb * r2[i];
-                    n1p[idx[i]] = d1[i];
-                    n2p[idx[i]] = d2[i];
-                }
-                __syncthreads();
-                float* s1 = c1p; c1p = n1p; n1p = s1;
-                float* s2 = c2p; c2p = n2p; n2p = s2;
-            }
-        }
-        // the planes not read by the last Chebyshev step take the result
-        out1 = n1p;
-        out2 = n2p;
-    }
-    long long H1[NCELL], H2[NCELL];
-#pragma unroll
-    for (int i = 0; i < NCELL; ++i) {
-        H1[i] = F1[i] + __float2ll_rn(u1[i]);
-        H2[i] = F2[i] + __float2ll_rn(u2[i]);
-        bad |= (H1[i] != (long long)(int32_t)H1[i]) | (H2[i] != (long long)(int32_t)H2[i]);
-        out1[idx[i]] = as_f(static_cast<int32_t>(H1[i]));
-        out2[idx[i]] = as_f(static_cast<int32_t>(H2[i]));
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < NCELL; ++i) {
-        const long long v = (long long)q[i] + (H1[i] - as_i(out1[up[i]])) + (H2[i] - as_i(out2[lf[i]]));
-        bad |= (unsigned)((v >= (1LL << 30)) | (v <= -(1LL << 30)));
-        q[i] = static_cast<int32_t>(v);
-        sq[idx[i]] = q[i];
-    }
-    __syncthreads();
+__device__ __forceinline__ f32x2 pack2i(int32_t lo, int32_t hi) { return pack2(as_f(lo), as_f(hi)); }
+__device__ __forceinline__ int32_t lo2i(f32x2 v) { return as_i(lo2(v)); }
+__device__ __forceinline__ int32_t hi2i(f32x2 v) { return as_i(hi2(v)); }
+
+constexpr unsigned kMbarPolls = 1u << 22;
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) {
+    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// Left / right neighbour values along a coarse row of W blocks (W lanes).
-template <int W, class T>
-__device__ __forceinline__ T from_left(T v, int l) {
-    return __shfl_sync(kFullMask, v, (l + W - 1) % W, W);
-}
-template <int W, class T>
-__device__ __forceinline__ T from_right(T v, int l) {
-    return __shfl_sync(kFullMask, v, (l + 1) % W, W);
-}
-
-// A plane of a block field: the top rows of all blocks, then the bottom rows
-// ([NC^2] float2 each, block index I1 NC + I2).
-template <int NC>
-struct Plane {
-    float2* top;
-    float2* bot;
-    __device__ __forceinline__ explicit Plane(float* base) : top(reinterpret_cast<float2*>(base)), bot(top + NC * NC) {}
-    __device__ __forceinline__ void put(int qi, const float (&v)[4]) const {
-        top[qi] = make_float2(v[0], v[1]);
-        bot[qi] = make_float2(v[2], v[3]);
+// The exchange of the blocks' top and bottom rows, two words a cell: buffer
+// n % 2 of exchange n holds [top, bottom][row of blocks][C/2][lane] vectors of two
+// cells (16 bytes, conflict-free).  In a cluster, slot n % 4 takes the rows that the
+// CTAs above and below sent, guarded by mbarriers up[n % 4] and dn[n % 4].
+template <class S>
+struct Exchange {
+    float* buf;
+    uint64_t* bars = nullptr;              // [up, dn][4]
+    uint32_t rup = 0, rdn = 0;             // shared::cluster address of `buf` in the CTA above / below
+    unsigned* err;
+    int br, bc;
+    unsigned n = 0;
+    bool dead = false;
+    __device__ __forceinline__ Exchange(float* b, int br_, int bc_, int rank, unsigned* err_)
+        : buf(b), err(err_), br(br_), bc(bc_) {
+        if constexpr (S::CL > 1) {
+            bars = reinterpret_cast<uint64_t*>(b + S::WORDS);
+            rup = mapa(smem_u32(b), (rank + S::CL - 1) % S::CL);
+            rdn = mapa(smem_u32(b), (rank + 1) % S::CL);
+            if (threadIdx.x == 0) {
+                for (int i = 0; i < 8; ++i)
+                    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bars + i)) : "memory");
+                asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            }
+        }
     }
+    __device__ __forceinline__ static uint32_t mapa(uint32_t a, int r) {
+        uint32_t v;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(v) : "r"(a), "r"(r));
+        return v;
+    }
+    // word offset of vector h (of two cells, or of one cell where W = 1) of a row:
+    // side 0 top, 1 bottom; row NBR: the row from above (side 0) / below (side 1)
+    template <int W>
+    __device__ __forceinline__ int at(int side, int row, int h) const {
+        constexpr int V = W == 1 ? 2 : 4, H = W == 1 ? 1 : W / 2;
+        return (row < S::NBR ? static_cast<int>(n & 1) * S::BUF + ((side * S::NBR + row) * H + h) * (S::LPR * V)
+                             : 2 * S::BUF + static_cast<int>(n & 3) * S::SLOT + (side * H + h) * (S::LPR * V)) +
+               bc * V;
+    }
+    // Send this thread's part of row v to buffer row NBR, side `side`, of the CTA at `base`.
+    template <int W>
+    __device__ __forceinline__ void send(uint32_t base, int side, const f32x2 (&v)[W]) const {
+        const uint32_t bar = base + 4u * S::WORDS + 8u * (4 * side + (n & 3));
+#pragma unroll
+        for (int h = 0; h < (W + 1) / 2; ++h) {
+            const uint32_t dst = base + 4u * at<W>(side, S::NBR, h);
+            if constexpr (W == 1)
+                asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(dst),
+                             "l"(v[0]), "r"(bar)
+                             : "memory");
+            else
+                asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(dst),
+                             "l"(v[2 * h]), "l"(v[2 * h + 1]), "r"(bar)
+                             : "memory");
+        }
+    }
+    template <int W>
+    __device__ __forceinline__ void store(int side, const f32x2 (&v)[W]) const {
+#pragma unroll
+        for (int h = 0; h < (W + 1) / 2; ++h) {
+            float* o = buf + at<W>(side, br, h);
+            if constexpr (W == 1) *reinterpret_cast<f32x2*>(o) = v[0];
+            else *reinterpret_cast<ulonglong2*>(o) = make_ulonglong2(v[2 * h], v[2 * h + 1]);
+        }
+    }
+    template <int W>
+    __device__ __forceinline__ void load(int side, int row, f32x2 (&v)[W]) const {
+#pragma unroll
+        for (int h = 0; h < (W + 1) / 2; ++h) {
+            const float* o = buf + at<W>(side, row, h);
+            if constexpr (W == 1) v[0] = *reinterpret_cast<const f32x2*>(o);
+            else {
+                const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(o);
+                v[2 * h] = x.x;
+                v[2 * h + 1] = x.y;
+            }
+        }
+    }
+    // The message of this exchange on side `side` (all lanes of the warp).
+    template <int W>
+    __device__ __forceinline__ void receive(int side) {
+        const uint32_t bar = smem_u32(bars + 4 * side + (n & 3));
+        if (bc == 0)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(S::LPR * W * 8)
+                         : "memory");
+        const uint32_t parity = (n >> 2) & 1;
+        for (unsigned i = 0; i < kMbarPolls && !dead; ++i) {
+            uint32_t ok;
+            asm volatile(
+                "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                : "=r"(ok)
+                : "r"(bar), "r"(parity)
+                : "memory");
+            if (ok) return;
+        }
+        dead = true;
+        atomicOr(err, kErrTimeout);
+    }
+    // Hand out the block's first and last row ...
+    template <int W>
+    __device__ __forceinline__ void publish(const f32x2 (&top)[W], const f32x2 (&bot)[W]) const {
+        if (S::CL > 1 && br == 0) send<W>(rup, 1, top);
+        else store<W>(0, top);
+        if (S::CL > 1 && br == S::NBR - 1) send<W>(rdn, 0, bot);
+        else store<W>(1, bot);
+    }
+    // ... and take the rows above and below it.
+    template <int W>
+    __device__ __forceinline__ void collect(f32x2 (&up)[W], f32x2 (&dn)[W]) {
+        const bool first = br == 0, last = br == S::NBR - 1;
+        if constexpr (S::TPS <= 32) __syncwarp();
+        else __syncthreads();
+        if (!first) load<W>(1, br - 1, up);
+        else if constexpr (S::CL == 1) load<W>(1, S::NBR - 1, up);
+        if (!last) load<W>(0, br + 1, dn);
+        else if constexpr (S::CL == 1) load<W>(0, 0, dn);
+        if constexpr (S::CL > 1) {
+            if (first) {
+                receive<W>(0);
+                load<W>(0, S::NBR, up);
+            }
+            if (last) {
+                receive<W>(1);
+                load<W>(1, S::NBR, dn);
+            }
+        }
+        ++n;
+    }
+    __device__ __forceinline__ int32_t left(int32_t v) const {
+        return __shfl_sync(kFullMask, v, (bc + S::LPR - 1) % S::LPR, S::LPR);
+    }
+    __device__ __forceinline__ int32_t right(int32_t v) const {
+        return __shfl_sync(kFullMask, v, (bc + 1) % S::LPR, S::LPR);
+    }
+    __device__ __forceinline__ f32x2 left2(f32x2 v) const { return pack2i(left(lo2i(v)), left(hi2i(v))); }
+    __device__ __forceinline__ f32x2 right2(f32x2 v) const { return pack2i(right(lo2i(v)), right(hi2i(v))); }
 };
 
-// Sum of the four periodic neighbours of each cell of the 2 x 2 block v
-// (cells: 0 top-left, 1 top-right, 2 bottom-left, 3 bottom-right), the rows
-// above / below from the blocks qa / qb of plane P, the columns by shuffles.
-template <int NC>
-__device__ __forceinline__ void neighbour_sum(const float (&v)[4], const Plane<NC>& P, int qa, int qb, int l,
-                                              float (&s)[4]) {
-    const float2 ab = P.bot[qa], bl = P.top[qb];
-    const float l0 = from_left<NC>(v[1], l), l2 = from_left<NC>(v[3], l);
-    const float r1 = from_right<NC>(v[0], l), r3 = from_right<NC>(v[2], l);
-    s[0] = (ab.x + v[2]) + (l0 + v[1]);
-    s[1] = (ab.y + v[3]) + (v[0] + r1);
-    s[2] = (v[0] + bl.x) + (l2 + v[3]);
-    s[3] = (v[1] + bl.y) + (v[2] + r3);
+// Exchange of a block field a; f(r, c, up, down, left, right) for every cell, the
+// inner rows before the barrier and the neighbours' messages are waited for.
+template <int R, int C, class S, class F>
+__device__ __forceinline__ void neighbours(f32x2 (&a)[R][C], Exchange<S>& x, F&& f) {
+    x.template publish<C>(a[0], a[R - 1]);
+    f32x2 l[R], rt[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        l[r] = x.left2(a[r][C - 1]);
+        rt[r] = x.right2(a[r][0]);
+    }
+    const auto row = [&](int r, const f32x2 (&up)[C], const f32x2 (&dn)[C]) {
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+            f(r, c, up[c], dn[c], c > 0 ? a[r][c > 0 ? c - 1 : 0] : l[r], c + 1 < C ? a[r][c + 1 < C ? c + 1 : 0] : rt[r]);
+    };
+#pragma unroll
+    for (int r = 1; r + 1 < R; ++r) row(r, a[r - 1], a[r + 1]);
+    f32x2 up[C], dn[C];
+    x.template collect<C>(up, dn);
+    if constexpr (R == 1) {
+        row(0, up, dn);
+    } else {
+        row(0, up, a[1]);
+        row(R - 1, a[R - 2], dn);
+    }
 }
 
-// One fine theta step for this thread's 2 x 2 block (coarse cell (I1, I2),
-// lane l = I2 of its row segment); B[0..3] are four n^2-word planes.  Enters
-// and leaves with the planes free (a barrier at the end).
-template <int N>
-__device__ __forceinline__ void theta_fine_step(int32_t (&q)[4], const int32_t (&G1)[4], const int32_t (&G2)[4],
-                                                int I1, int I2, float* const (&B)[4], long long A, const TArgs& t,
-                                                unsigned& bad) {
-    constexpr int NC = N / 2;
-    const int qi = I1 * NC + I2;
-    const int qa = ((I1 + NC - 1) % NC) * NC + I2;   // block above
-    const int qb = ((I1 + 1) % NC) * NC + I2;        // block below
-    const int l = I2;
-    // ---- exact face fluxes: the row below from the block below, the column right by shuffles
-    int4* Q = reinterpret_cast<int4*>(B[0]);
-    Q[qi] = make_int4(q[0], q[1], G1[0], G1[1]);
-    __syncthreads();
-    const int4 bq = Q[qb];
-    const int32_t qr1 = from_right<NC>(q[0], l), qr3 = from_right<NC>(q[2], l);
-    const int32_t gr1 = from_right<NC>(G2[0], l), gr3 = from_right<NC>(G2[2], l);
-    const int32_t qdn[4] = {q[2], q[3], bq.x, bq.y}, gdn[4] = {G1[2], G1[3], bq.z, bq.w};
-    const int32_t qrt[4] = {q[1], qr1, q[3], qr3}, grt[4] = {G2[1], gr1, G2[3], gr3};
-    int32_t F1[4], F2[4];
+// One theta step of an R x C block of a periodic grid of LPR C columns (the
+// fine grid, or the coarse one with COARSE: the four neighbours are added in
+// another order there).
+template <int R, int C, bool COARSE, class S>
+__device__ __forceinline__ void theta_step(int32_t (&q)[R][C], const int32_t (&G1)[R][C], const int32_t (&G2)[R][C],
+                                           long long A, const TArgs& t, unsigned& bad, Exchange<S>& x) {
+    // ---- exact face fluxes across the lower and the right edge of every cell
+    int32_t F1[R][C], F2[R][C];
+    {
+        f32x2 top[C], bot[C], up[C], dn[C];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const long long f1 = (long long)edge_flux64(A, qdn[c] - q[c]) + G1[c] + gdn[c];
-        const long long f2 = (long long)edge_flux64(A, qrt[c] - q[c]) + G2[c] + grt[c];
-        bad |= (unsigned)((f1 != (long long)(int32_t)f1) | (f2 != (long long)(int32_t)f2));
-        F1[c] = static_cast<int32_t>(f1);
-        F2[c] = static_cast<int32_t>(f2);
+        for (int c = 0; c < C; ++c) {
+            top[c] = pack2i(q[0][c], G1[0][c]);
+            bot[c] = pack2i(q[R - 1][c], G1[R - 1][c]);
+        }
+        x.template publish<C>(top, bot);
+        x.template collect<C>(up, dn);
+        const auto face = [&](int32_t near, int32_t far, int32_t gn, int32_t gf) {
+            const long long f = (long long)edge_flux64(A, far - near) + gn + gf;
+            bad |= (unsigned)(f != (long long)(int32_t)f);
+            return static_cast<int32_t>(f);
+        };
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int32_t qr = x.right(q[r][0]), gr = x.right(G2[r][0]);
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                F1[r][c] = face(q[r][c], r + 1 < R ? q[r + 1 < R ? r + 1 : 0][c] : lo2i(dn[c]), G1[r][c],
+                                r + 1 < R ? G1[r + 1 < R ? r + 1 : 0][c] : hi2i(dn[c]));
+                F2[r][c] = face(q[r][c], c + 1 < C ? q[r][c + 1 < C ? c + 1 : 0] : qr, G2[r][c],
+                                c + 1 < C ? G2[r][c + 1 < C ? c + 1 : 0] : gr);
+            }
+        }
     }
-    float u1[4] = {0.f, 0.f, 0.f, 0.f}, u2[4] = {0.f, 0.f, 0.f, 0.f};
-    float* hplane = B[1];   // plane that carries the corrected fluxes of the bottom rows
+    f32x2 u[R][C];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < C; ++c) u[r][c] = pack2(0.f, 0.f);
     if (t.K > 0) {
         // ---- right-hand side -alpha L F and the first Chebyshev direction
-        float f1[4], f2[4];
+        const f32x2 minus1 = pack2(-1.f, -1.f), nalpha = pack2(-t.alpha, -t.alpha);
+        f32x2 res[R][C], d[R][C];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            f1[c] = static_cast<float>(F1[c]);
-            f2[c] = static_cast<float>(F2[c]);
-        }
-        const Plane<NC> PF1(B[1]), PF2(B[2]);
-        PF1.put(qi, f1);
-        PF2.put(qi, f2);
-        __syncthreads();   // also orders every read of B[0] before it is reused below
-        float s1[4], s2[4], r1[4], r2[4], d1[4], d2[4];
-        neighbour_sum<NC>(f1, PF1, qa, qb, l, s1);
-        neighbour_sum<NC>(f2, PF2, qa, qb, l, s2);
+        for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            r1[c] = -t.alpha * (4.f * f1[c] - s1[c]);
-            r2[c] = -t.alpha * (4.f * f2[c] - s2[c]);
-            d1[c] = r1[c] * t.inv_theta;
-            d2[c] = r2[c] * t.inv_theta;
-        }
-        float* cur1 = B[3];
-        float* cur2 = B[0];
-        float* nxt1 = B[1];
-        float* nxt2 = B[2];
-        Plane<NC>(cur1).put(qi, d1);
-        Plane<NC>(cur2).put(qi, d2);
-        __syncthreads();
-        const float diag = 1.f + 4.f * t.alpha;
-        for (int k = 0; k < t.K; ++k) {
-            neighbour_sum<NC>(d1, Plane<NC>(cur1), qa, qb, l, s1);
-            neighbour_sum<NC>(d2, Plane<NC>(cur2), qa, qb, l, s2);
+            for (int c = 0; c < C; ++c)
+                d[r][c] = pack2(static_cast<float>(F1[r][c]), static_cast<float>(F2[r][c]));
+        neighbours<R, C, S>(d, x, [&](int r, int c, f32x2 up, f32x2 dn, f32x2 l, f32x2 rt) {
+            f32x2 v = mul2(pack2(4.f, 4.f), d[r][c]);
+            if constexpr (COARSE) v = fma2(rt, minus1, fma2(l, minus1, fma2(dn, minus1, fma2(up, minus1, v))));
+            else v = fma2(add2(add2(up, dn), add2(l, rt)), minus1, v);
+            res[r][c] = mul2(nalpha, v);
+        });
+        const f32x2 inv = pack2(t.inv_theta, t.inv_theta);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                u1[c] += d1[c];
-                u2[c] += d2[c];
-                r1[c] -= diag * d1[c] - t.alpha * s1[c];
-                r2[c] -= diag * d2[c] - t.alpha * s2[c];
-            }
-            if (k + 1 < t.K) {
-                const float ca = t.c1[k], cb = t.c2[k];
+        for (int r = 0; r < R; ++r)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    d1[c] = ca * d1[c] + cb * r1[c];
-                    d2[c] = ca * d2[c] + cb * r2[c];
+            for (int c = 0; c < C; ++c) d[r][c] = mul2(res[r][c], inv);
+        // ---- K steps u += d, r -= (I + alpha L) d, d <- ca d + cb r; the last needs u only
+        const f32x2 diag = pack2(1.f + 4.f * t.alpha, 1.f + 4.f * t.alpha);
+#pragma unroll 1
+        for (int k = 0; k + 1 < t.K; ++k) {
+            neighbours<R, C, S>(d, x, [&](int r, int c, f32x2 up, f32x2 dn, f32x2 l, f32x2 rt) {
+                f32x2 s;
+                if constexpr (COARSE) s = add2(add2(add2(up, dn), l), rt);
+                else s = add2(add2(up, dn), add2(l, rt));
+                const f32x2 e = fma2(diag, d[r][c], mul2(nalpha, s));
+                res[r][c] = fma2(e, minus1, res[r][c]);
+            });
+            const f32x2 ca = pack2(t.c1[k], t.c1[k]), cb = pack2(t.c2[k], t.c2[k]);
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    u[r][c] = add2(u[r][c], d[r][c]);
+                    d[r][c] = fma2(ca, d[r][c], mul2(cb, res[r][c]));
                 }
-                Plane<NC>(nxt1).put(qi, d1);
-                Plane<NC>(nxt2).put(qi, d2);
-                __syncthreads();
-                float* x = cur1; cur1 = nxt1; nxt1 = x;
-                x = cur2; cur2 = nxt2; nxt2 = x;
-            }
         }
-        hplane = nxt1;   // not read by the last Chebyshev step
-    }
-    // ---- corrected fluxes, rounded once; the update adds integer face fluxes
-    int32_t H1[4], H2[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const long long h1 = (long long)F1[c] + __float2ll_rn(u1[c]);
-        const long long h2 = (long long)F2[c] + __float2ll_rn(u2[c]);
-        bad |= (unsigned)((h1 != (long long)(int32_t)h1) | (h2 != (long long)(int32_t)h2));
-        H1[c] = static_cast<int32_t>(h1);
-        H2[c] = static_cast<int32_t>(h2);
-    }
-    int2* Hb = reinterpret_cast<int2*>(hplane);
-    Hb[qi] = make_int2(H1[2], H1[3]);
-    __syncthreads();
-    const int2 ha = Hb[qa];
-    const int32_t hl0 = from_left<NC>(H2[1], l), hl2 = from_left<NC>(H2[3], l);
-    const int32_t h1up[4] = {ha.x, ha.y, H1[0], H1[1]}, h2lf[4] = {hl0, H2[0], hl2, H2[2]};
+        for (int r = 0; r < R; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const long long v = (long long)q[c] + ((long long)H1[c] - h1up[c]) + ((long long)H2[c] - h2lf[c]);
-        bad |= (unsigned)((v >= (1LL << 30)) | (v <= -(1LL << 30)));
-        q[c] = static_cast<int32_t>(v);
+            for (int c = 0; c < C; ++c) u[r][c] = add2(u[r][c], d[r][c]);
     }
-    __syncthreads();
+    // ---- corrected fluxes, rounded once; the update adds integer face fluxes.
+    // Corrections fit 32 bits in every sane state: the conversion to 64 bits, which
+    // runs on the FP64 pipe (two per cell were a seventh of the step), is kept for a
+    // block that has one beyond.
+    float big = 0.f;
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < C; ++c) big = fmaxf(big, fmaxf(fabsf(lo2(u[r][c])), fabsf(hi2(u[r][c]))));
+    const auto correct = [&](auto round) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const long long h1 = (long long)F1[r][c] + round(lo2(u[r][c]));
+                const long long h2 = (long long)F2[r][c] + round(hi2(u[r][c]));
+                bad |= (unsigned)((h1 != (long long)(int32_t)h1) | (h2 != (long long)(int32_t)h2));
+                F1[r][c] = static_cast<int32_t>(h1);
+                F2[r][c] = static_cast<int32_t>(h2);
+            }
+    };
+    if (big < 2147483648.f) correct([](float v) { return (long long)__float2int_rn(v); });
+    else correct([](float v) { return __float2ll_rn(v); });
+    f32x2 top[C], bot[C], up[C], dn[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        top[c] = pack2i(F1[0][c], 0);
+        bot[c] = pack2i(F1[R - 1][c], 0);
+    }
+    x.template publish<C>(top, bot);
+    x.template collect<C>(up, dn);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int32_t hl = x.left(F2[r][C - 1]);
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const int32_t ha = r > 0 ? F1[r > 0 ? r - 1 : 0][c] : lo2i(up[c]), hb = c > 0 ? F2[r][c > 0 ? c - 1 : 0] : hl;
+            const long long v = (long long)q[r][c] + ((long long)F1[r][c] - ha) + ((long long)F2[r][c] - hb);
+            bad |= (unsigned)((v >= (1LL << 30)) | (v <= -(1LL << 30)));
+            q[r][c] = static_cast<int32_t>(v);
+        }
+    }
 }
 
-template <int N, bool CPL>
-__global__ void __launch_bounds__(TShape<N>::THREADS) theta_kernel(const KArgs a, const TArgs t) {
-    using S = TShape<N>;
-    constexpr int NC = S::NC, TPS = S::TPS, SPB = S::SPB, THREADS = S::THREADS;
+// Barrier of all threads of a sample.
+template <class S>
+__device__ __forceinline__ void sample_barrier() {
+    if constexpr (S::CL > 1) cg::this_cluster().sync();
+    else __syncthreads();
+}
+
+template <int N, bool CPL, bool DENSE>
+__global__ void __launch_bounds__(TShape<N, DENSE>::THREADS, TShape<N, DENSE>::MIN_CTAS)
+    theta_kernel(const KArgs a, const TArgs t) {
+    using S = TShape<N, DENSE>;
+    constexpr int NC = S::NC, TPS = S::TPS, SPB = S::SPB, THREADS = S::THREADS, R = S::R, C = S::C, CL = S::CL;
+    constexpr int RC = R / 2, CC = C / 2;       // coarse block
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tid = threadIdx.x;
     const int sl = tid / TPS, lt = tid % TPS;   // sample slot in the CTA, thread within the sample
-    unsigned char* base = smem_raw + S::SAMPLE_BYTES * sl;
-    float* P0 = reinterpret_cast<float*>(base);
-    float* P1 = P0 + N * N;
-    float* P2 = P1 + N * N;
-    float* P3 = P2 + N * N;
-    int32_t* sqc = reinterpret_cast<int32_t*>(P3 + N * N);
+    int rank = 0;
+    if constexpr (CL > 1) rank = static_cast<int>(cg::this_cluster().block_rank());
     double* red = reinterpret_cast<double*>(smem_raw + S::SAMPLE_BYTES * SPB);
-    double* acc = red + ((THREADS + 31) / 32) * kRed;
+    double* tot = red + ((THREADS + 31) / 32) * kRed;   // this CTA's band total (clusters)
+    double* acc = tot + kRed;                           // moment sums of the CTA's slots (rank 0)
     for (int i = tid; i < SPB * a.slot_stride; i += THREADS) acc[i] = 0.0;
-    float* const planes[4] = {P0, P1, P2, P3};
 
-    const int I1 = lt / NC, I2 = lt % NC;   // coarse cell; fine block rows 2 I1 + v1, cols 2 I2 + v2
-    const int crow[1] = {I1}, ccol[1] = {I2};
-    const int f00 = (2 * I1) * N + 2 * I2;  // fine index of the block's top-left cell
-    const int fidx[4] = {f00, f00 + 1, f00 + N, f00 + N + 1};
-    const uint32_t p_top = static_cast<uint32_t>(f00 >> 1);
-    const uint32_t p_bot = static_cast<uint32_t>((f00 + N) >> 1);
+    const int br = lt / S::LPR, bc = lt % S::LPR;
+    const int i0 = (rank * S::NBR + br) * R, j0 = bc * C;   // the block's first fine cell
+    Exchange<S> x(reinterpret_cast<float*>(smem_raw + S::SAMPLE_BYTES * sl), br, bc, rank, a.err);
 
-    const long long n_slots = (long long)gridDim.x * SPB;
-    const long long slot = (long long)blockIdx.x * SPB + sl;
-    const long long cta_slot0 = (long long)blockIdx.x * SPB;
+    const long long n_slots = (long long)gridDim.x * SPB / CL;
+    const long long cta_slot0 = (long long)(blockIdx.x / CL) * SPB;
+    const long long slot = cta_slot0 + sl;
     const long long iters = a.count > cta_slot0 ? (a.count - cta_slot0 + n_slots - 1) / n_slots : 0;
     unsigned bad = 0;
-    __syncthreads();
+    sample_barrier<S>();
 
     for (long long it = 0; it < iters; ++it) {
         const long long idx = slot + it * n_slots;
@@ -358,47 +454,61 @@ __global__ void __launch_bounds__(TShape<N>::THREADS) theta_kernel(const KArgs a
         const uint32_t c2 = static_cast<uint32_t>(sid);
         const uint32_t c3 = a.tag | ((static_cast<uint32_t>(static_cast<unsigned long long>(sid) >> 32) & 0xffffu) << 16);
 
-        int32_t q[4], qc[1] = {0};
+        int32_t q[R][C], qc[RC][CC];
+        float zt0[RC][CC], zt1[RC][CC];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) q[i] = a.q0f[fidx[i]];
-        float zt0 = 0.f, zt1 = 0.f;
-        if constexpr (CPL) {
-            qc[0] = a.q0c[lt];
-            sqc[lt] = qc[0];
-        }
-        __syncthreads();
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) q[r][c] = a.q0f[(i0 + r) * N + j0 + c];
+#pragma unroll
+        for (int r = 0; r < RC; ++r)
+#pragma unroll
+            for (int c = 0; c < CC; ++c) {
+                zt0[r][c] = zt1[r][c] = 0.f;
+                qc[r][c] = CPL ? a.q0c[(i0 / 2 + r) * NC + j0 / 2 + c] : 0;
+            }
 
         for (int m = 0; m < a.M; ++m) {
-            // ---- noise of the fine block: Philox4x32-10 per horizontal cell pair, Box--Muller
-            int32_t G1[4], G2[4];
+            {
+                // ---- noise of the fine block: Philox4x32-10 per horizontal cell pair, Box--Muller
+                int32_t G1[R][C], G2[R][C];
+                const f32x2 g2 = pack2(a.gf, a.gf);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const uint4 x = philox10(make_uint4(h ? p_bot : p_top, static_cast<uint32_t>(m), c2, c3), a.key0, a.key1);
-                float ra, ca, sa, rb, cb, sb;
-                box_muller_polar(x.x, x.y, ra, ca, sa);
-                box_muller_polar(x.z, x.w, rb, cb, sb);
-                const float ta = noise_amp(q[2 * h], a.gf) * ra;
-                const float tb = noise_amp(q[2 * h + 1], a.gf) * rb;
-                G1[2 * h] = __float2int_rn(ta * ca);
-                G2[2 * h] = __float2int_rn(ta * sa);
-                G1[2 * h + 1] = __float2int_rn(tb * cb);
-                G2[2 * h + 1] = __float2int_rn(tb * sb);
-                if constexpr (CPL) {
-                    zt0 = fmaf(rb, cb, fmaf(ra, ca, zt0));
-                    zt1 = fmaf(rb, sb, fmaf(ra, sa, zt1));
-                }
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int p = 0; p < C / 2; ++p) {
+                        const uint32_t pair = static_cast<uint32_t>(((i0 + r) * N + j0) / 2 + p);
+                        const uint4 w = philox10(make_uint4(pair, static_cast<uint32_t>(m), c2, c3), a.key0, a.key1);
+                        f32x2 rad, co, si;
+                        box_muller_polar2(w.x, w.y, w.z, w.w, rad, co, si);
+                        const f32x2 ta = mul2(noise_amp2(q[r][2 * p], q[r][2 * p + 1], g2), rad);
+                        const f32x2 t1 = mul2(ta, co), t2 = mul2(ta, si);
+                        G1[r][2 * p] = __float2int_rn(lo2(t1));
+                        G1[r][2 * p + 1] = __float2int_rn(hi2(t1));
+                        G2[r][2 * p] = __float2int_rn(lo2(t2));
+                        G2[r][2 * p + 1] = __float2int_rn(hi2(t2));
+                        if constexpr (CPL) {
+                            float &z0 = zt0[r / 2][p], &z1 = zt1[r / 2][p];
+                            z0 = fmaf(hi2(rad), hi2(co), fmaf(lo2(rad), lo2(co), z0));
+                            z1 = fmaf(hi2(rad), hi2(si), fmaf(lo2(rad), lo2(si), z1));
+                        }
+                    }
+                theta_step<R, C, false, S>(q, G1, G2, t.Af64, t, bad, x);
             }
-            theta_fine_step<N>(q, G1, G2, I1, I2, planes, t.Af64, t, bad);
-
             if constexpr (CPL) {
                 if ((m & 3) == 3) {
                     // coupled coarse step: 1/4 of the 16 summed fine normals
-                    const float s = noise_amp(qc[0], a.gc);
-                    P0[lt] = as_f(__float2int_rn(s * zt0));
-                    P2[lt] = as_f(__float2int_rn(s * zt1));
-                    zt0 = zt1 = 0.f;
-                    __syncthreads();
-                    theta_step<NC, 1>(qc, crow, ccol, sqc, P0, P1, P2, P3, t.Ac64, t, bad);
+                    int32_t H1[RC][CC], H2[RC][CC];
+#pragma unroll
+                    for (int r = 0; r < RC; ++r)
+#pragma unroll
+                        for (int c = 0; c < CC; ++c) {
+                            const float s = noise_amp(qc[r][c], a.gc);
+                            H1[r][c] = __float2int_rn(s * zt0[r][c]);
+                            H2[r][c] = __float2int_rn(s * zt1[r][c]);
+                            zt0[r][c] = zt1[r][c] = 0.f;
+                        }
+                    theta_step<RC, CC, true, S>(qc, H1, H2, t.Ac64, t, bad, x);
                 }
             }
         }
@@ -406,45 +516,73 @@ __global__ void __launch_bounds__(TShape<N>::THREADS) theta_kernel(const KArgs a
         // ---- observables: fluctuation sums against the fixed-point mean field (FP64), mass
         double v[kRed];
         {
-            long long mf = 0;
+            long long mf = 0, mc = 0;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) mf += q[i];
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < C; ++c) mf += q[r][c];
+#pragma unroll
+            for (int r = 0; r < RC; ++r)
+#pragma unroll
+                for (int c = 0; c < CC; ++c) mc += qc[r][c];
             v[2 * kMaxObs] = static_cast<double>(mf);
-            v[2 * kMaxObs + 1] = CPL ? static_cast<double>(qc[0]) : 0.0;
+            v[2 * kMaxObs + 1] = CPL ? static_cast<double>(mc) : 0.0;
 #pragma unroll
             for (int k = 0; k < kMaxObs; ++k) {
                 double sf = 0.0, sc = 0.0;
                 if (k < a.n_obs) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        sf += static_cast<double>(q[i] - a.qbf[fidx[i]]) * t.phif64[(size_t)k * N * N + fidx[i]];
-                    if constexpr (CPL) sc = static_cast<double>(qc[0] - a.qbc[lt]) * t.phic64[(size_t)k * NC * NC + lt];
+                    for (int r = 0; r < R; ++r)
+#pragma unroll
+                        for (int c = 0; c < C; ++c) {
+                            const int f = (i0 + r) * N + j0 + c;
+                            sf += static_cast<double>(q[r][c] - a.qbf[f]) * t.phif64[(size_t)k * N * N + f];
+                        }
+                    if constexpr (CPL) {
+#pragma unroll
+                        for (int r = 0; r < RC; ++r)
+#pragma unroll
+                            for (int c = 0; c < CC; ++c) {
+                                const int g = (i0 / 2 + r) * NC + j0 / 2 + c;
+                                sc += static_cast<double>(qc[r][c] - a.qbc[g]) * t.phic64[(size_t)k * NC * NC + g];
+                            }
+                    }
                 }
                 v[k] = sf;
                 v[kMaxObs + k] = sc;
             }
         }
-        bool leader;
-        if constexpr (TPS < 32) {
+        constexpr int SEG = TPS < 32 ? TPS : 32;
 #pragma unroll
-            for (int off = TPS / 2; off >= 1; off >>= 1)
+        for (int off = SEG / 2; off >= 1; off >>= 1)
 #pragma unroll
-                for (int i = 0; i < kRed; ++i) v[i] += __shfl_xor_sync(kFullMask, v[i], off, TPS);
-            leader = lt == 0;
-        } else {
-#pragma unroll
-            for (int off = 16; off >= 1; off >>= 1)
-#pragma unroll
-                for (int i = 0; i < kRed; ++i) v[i] += __shfl_xor_sync(kFullMask, v[i], off);
+            for (int i = 0; i < kRed; ++i) v[i] += __shfl_xor_sync(kFullMask, v[i], off, SEG);
+        bool leader = lt == 0;
+        if constexpr (TPS > 32) {
             if ((tid & 31) == 0)
 #pragma unroll
                 for (int i = 0; i < kRed; ++i) red[(tid >> 5) * kRed + i] = v[i];
             __syncthreads();
-            leader = lt == 0;
-            if (leader) {
-                for (int w = 1; w < TPS / 32; ++w)
+            if constexpr (CL == 1) {
+                if (leader)
+                    for (int w = 1; w < TPS / 32; ++w)
 #pragma unroll
-                    for (int i = 0; i < kRed; ++i) v[i] += red[((tid >> 5) + w) * kRed + i];
+                        for (int i = 0; i < kRed; ++i) v[i] += red[w * kRed + i];
+            } else {
+                // the band totals, then their sum on rank 0 in rank order
+                if (tid < kRed) {
+                    double s = 0.0;
+                    for (int w = 0; w < THREADS / 32; ++w) s += red[w * kRed + tid];
+                    tot[tid] = s;
+                }
+                sample_barrier<S>();
+                leader = rank == 0 && tid == 0;
+                if (leader)
+                    for (int i = 0; i < kRed; ++i) {
+                        double s = 0.0;
+                        for (int r = 0; r < CL; ++r) s += cg::this_cluster().map_shared_rank(tot, r)[i];
+                        v[i] = s;
+                    }
             }
         }
 
@@ -484,727 +622,140 @@ __global__ void __launch_bounds__(TShape<N>::THREADS) theta_kernel(const KArgs a
                 o[2 * a.n_obs + 1] = CPL ? v[2 * kMaxObs + 1] * a.dscale_c : 0.0;
             }
         }
-        __syncthreads();   // the reduction scratch and the state planes are reused by the next sample
+        sample_barrier<S>();   // the reduction scratch is reused by the next sample
     }
     if (bad) atomicOr(a.err, kErrRange);
 
     // ---- per-slot partial sums to global scratch, entry-major [stride][n_slots]
     __syncthreads();
-    for (int i = tid; i < SPB * a.slot_stride; i += THREADS) {
-        const int s = i / a.slot_stride, e = i % a.slot_stride;
-        a.partials[(size_t)e * n_slots + cta_slot0 + s] = acc[i];
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Grids beyond one CTA (128 x 128): a thread-block cluster of CL CTAs per
-// sample, CTA `rank` holding the band of BR = NC/CL block rows (its threads
-// own those rows' 2 x 2 blocks as above).  The block fields live in the band's
-// shared memory with the same layout in every CTA; the rows just above and
-// below the band are read from the neighbouring CTAs' shared memory
-// (distributed shared memory), and every barrier that orders a plane's writes
-// before its reads is a cluster barrier.  The arithmetic is the one-CTA
-// kernel's, so both give the same integer paths.
-// ---------------------------------------------------------------------------
-namespace cg = cooperative_groups;
-
-template <int N, int CL, int NB>
-struct CShape {
-    static constexpr int NC = N / 2, BR = NC / CL;          // block rows per CTA
-    static constexpr int RT = NC / NB;                      // threads per block row (NB blocks each)
-    static constexpr int THREADS = BR * RT;
-    static constexpr int BAND = BR * NC;                    // blocks (= coarse cells) per CTA
-    static_assert(NC % CL == 0 && NC % NB == 0 && THREADS <= 1024 && RT % 32 == 0, "band shape");
-    // four block planes of BAND x 16 bytes (top and bottom rows, or an int4 per block),
-    // the coarse state of the band, reduction scratch
-    static size_t smem(int slot_stride) {
-        return 4 * sizeof(float) * 4 * BAND + sizeof(int32_t) * BAND + sizeof(double) * (THREADS / 32) * kRed +
-               sizeof(double) * kRed + sizeof(double) * slot_stride;
-    }
-};
-
-// Pointer into the shared memory of cluster rank r (this CTA's own when r == rank).
-template <class T>
-__device__ __forceinline__ T* band_at(T* local, int r, int rank) {
-    if (r == rank) return local;
-    return cg::this_cluster().map_shared_rank(local, r);
-}
-
-// Neighbours of block (or coarse cell) (lr, I2) of a band of BR rows x NC:
-// left / right in the same row (periodic), above / below in the row before /
-// after, in the neighbouring CTA for the band's first / last row (periodic
-// over the cluster).
-template <int NC, int BR>
-struct BandNbr {
-    int lq, il, ir, ia, ib, ra, rb, rank;
-    BandNbr() = default;
-    __device__ __forceinline__ BandNbr(int lr, int I2, int rank_, int cl) : rank(rank_) {
-        lq = lr * NC + I2;
-        il = lr * NC + (I2 + NC - 1) % NC;
-        ir = lr * NC + (I2 + 1) % NC;
-        if (lr > 0) { ia = lq - NC; ra = rank; } else { ia = (BR - 1) * NC + I2; ra = (rank + cl - 1) % cl; }
-        if (lr < BR - 1) { ib = lq + NC; rb = rank; } else { ib = I2; rb = (rank + 1) % cl; }
-    }
-    template <class T> __device__ __forceinline__ T above(T* p) const { return band_at(p, ra, rank)[ia]; }
-    template <class T> __device__ __forceinline__ T below(T* p) const { return band_at(p, rb, rank)[ib]; }
-    template <class T> __device__ __forceinline__ T left(const T* p) const { return p[il]; }
-    template <class T> __device__ __forceinline__ T right(const T* p) const { return p[ir]; }
-};
-
-// Split cluster barrier of a plane exchange.  After writing its part of a
-// plane a thread arrives (release); a CTA barrier then publishes the plane
-// inside the CTA.  The warps of the band's first and last block row, which
-// read the neighbouring CTAs' rows, wait (acquire) at once; the other warps
-// only read rows of their own CTA and defer the wait until just before they
-// next write a plane that other CTAs read, so the cluster barrier's latency
-// is spent on their arithmetic.  A thread always waits once between two
-// arrivals, so the barrier is never more than one phase ahead of it.
-struct ClPhase {
-    bool edge;
-    bool pend = false;
-    __device__ __forceinline__ explicit ClPhase(bool edge_) : edge(edge_) {}
-    __device__ __forceinline__ static void arrive() {
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    }
-    __device__ __forceinline__ static void wait() {
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    }
-    // before writing a plane that other CTAs read (or before a full barrier)
-    __device__ __forceinline__ void settle() {
-        if (pend) {
-            wait();
-            pend = false;
-        }
-    }
-    __device__ __forceinline__ void publish() {
-        arrive();
-        __syncthreads();
-        if (edge) wait();
-        else pend = true;
-    }
-    __device__ __forceinline__ void full() {
-        settle();
-        arrive();
-        wait();
-    }
-};
-
-// Sum of the four neighbours of each cell of block v = (top-left, top-right,
-// bottom-left, bottom-right), from the blocks above / below / left / right,
-// in the one-CTA kernel's order of additions.
-__device__ __forceinline__ void nsum4(const float (&v)[4], float4 A, float4 Bv, float4 L, float4 R, float (&s)[4]) {
-    s[0] = (A.z + v[2]) + (L.y + v[1]);
-    s[1] = (A.w + v[3]) + (v[0] + R.x);
-    s[2] = (v[0] + Bv.x) + (L.w + v[3]);
-    s[3] = (v[1] + Bv.y) + (v[2] + R.z);
-}
-
-template <int NC, int BR>
-__device__ __forceinline__ void nsum_band(const float (&v)[4], const float4* P, const BandNbr<NC, BR>& nb,
-                                          float (&s)[4]) {
-    nsum4(v, nb.above(P), nb.below(P), nb.left(P), nb.right(P), s);
-}
-
-// theta_fine_step for the NB blocks of a thread in a band (B: four planes of
-// one 16-byte word per block of the band; all neighbours through shared
-// memory).  Every plane write is preceded by ph.settle() and followed by
-// ph.publish(); the step ends with an arrival whose wait comes before the
-// next plane write.
-template <int NC, int BR, int NB>
-__device__ __forceinline__ void theta_fine_step_cl(int32_t (&q)[NB][4], const int32_t (&G1)[NB][4],
-                                                   const int32_t (&G2)[NB][4], const BandNbr<NC, BR> (&nb)[NB],
-                                                   float* const (&B)[4], long long A, const TArgs& t, unsigned& bad,
-                                                   ClPhase& ph) {
-    // ---- exact face fluxes: the top row of the block below, the left column of the block right
-    int4* Qd = reinterpret_cast<int4*>(B[0]);
-    int4* Qr = reinterpret_cast<int4*>(B[3]);
-    ph.settle();
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        Qd[nb[b].lq] = make_int4(q[b][0], q[b][1], G1[b][0], G1[b][1]);
-        Qr[nb[b].lq] = make_int4(q[b][0], q[b][2], G2[b][0], G2[b][2]);
-    }
-    ph.publish();
-    int32_t F1[NB][4], F2[NB][4];
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        const int4 bq = nb[b].below(Qd), rq = nb[b].right(Qr);
-        const int32_t qdn[4] = {q[b][2], q[b][3], bq.x, bq.y}, gdn[4] = {G1[b][2], G1[b][3], bq.z, bq.w};
-        const int32_t qrt[4] = {q[b][1], rq.x, q[b][3], rq.y}, grt[4] = {G2[b][1], rq.z, G2[b][3], rq.w};
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const long long f1 = (long long)edge_flux64(A, qdn[c] - q[b][c]) + G1[b][c] + gdn[c];
-            const long long f2 = (long long)edge_flux64(A, qrt[c] - q[b][c]) + G2[b][c] + grt[c];
-            bad |= (unsigned)((f1 != (long long)(int32_t)f1) | (f2 != (long long)(int32_t)f2));
-            F1[b][c] = static_cast<int32_t>(f1);
-            F2[b][c] = static_cast<int32_t>(f2);
-        }
-    }
-    float u1[NB][4], u2[NB][4];
-#pragma unroll
-    for (int b = 0; b < NB; ++b)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) u1[b][c] = u2[b][c] = 0.f;
-    float* hplane = B[1];
-    if (t.K > 0) {
-        float f1[NB][4], f2[NB][4];
-#pragma unroll
-        for (int b = 0; b < NB; ++b)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                f1[b][c] = static_cast<float>(F1[b][c]);
-                f2[b][c] = static_cast<float>(F2[b][c]);
-            }
-        float4* PF1 = reinterpret_cast<float4*>(B[1]);
-        float4* PF2 = reinterpret_cast<float4*>(B[2]);
-        ph.settle();
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            PF1[nb[b].lq] = make_float4(f1[b][0], f1[b][1], f1[b][2], f1[b][3]);
-            PF2[nb[b].lq] = make_float4(f2[b][0], f2[b][1], f2[b][2], f2[b][3]);
-        }
-        ph.publish();   // its wait also orders every read of B[0], B[3] before they are reused below
-        float r1[NB][4], r2[NB][4], d1[NB][4], d2[NB][4];
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            float s1[4], s2[4];
-            nsum_band(f1[b], PF1, nb[b], s1);
-            nsum_band(f2[b], PF2, nb[b], s2);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                r1[b][c] = -t.alpha * (4.f * f1[b][c] - s1[c]);
-                r2[b][c] = -t.alpha * (4.f * f2[b][c] - s2[c]);
-                d1[b][c] = r1[b][c] * t.inv_theta;
-                d2[b][c] = r2[b][c] * t.inv_theta;
-            }
-        }
-        float4* cur1 = reinterpret_cast<float4*>(B[3]);
-        float4* cur2 = reinterpret_cast<float4*>(B[0]);
-        float4* nxt1 = reinterpret_cast<float4*>(B[1]);
-        float4* nxt2 = reinterpret_cast<float4*>(B[2]);
-        ph.settle();
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            cur1[nb[b].lq] = make_float4(d1[b][0], d1[b][1], d1[b][2], d1[b][3]);
-            cur2[nb[b].lq] = make_float4(d2[b][0], d2[b][1], d2[b][2], d2[b][3]);
-        }
-        ph.publish();
-        const float diag = 1.f + 4.f * t.alpha;
-        for (int k = 0; k < t.K; ++k) {
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
-                float s1[4], s2[4];
-                nsum_band(d1[b], cur1, nb[b], s1);
-                nsum_band(d2[b], cur2, nb[b], s2);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    u1[b][c] += d1[b][c];
-                    u2[b][c] += d2[b][c];
-                    r1[b][c] -= diag * d1[b][c] - t.alpha * s1[c];
-                    r2[b][c] -= diag * d2[b][c] - t.alpha * s2[c];
-                }
-            }
-            if (k + 1 < t.K) {
-                const float ca = t.c1[k], cb = t.c2[k];
-#pragma unroll
-                for (int b = 0; b < NB; ++b)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        d1[b][c] = ca * d1[b][c] + cb * r1[b][c];
-                        d2[b][c] = ca * d2[b][c] + cb * r2[b][c];
-                    }
-                ph.settle();
-#pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                    nxt1[nb[b].lq] = make_float4(d1[b][0], d1[b][1], d1[b][2], d1[b][3]);
-                    nxt2[nb[b].lq] = make_float4(d2[b][0], d2[b][1], d2[b][2], d2[b][3]);
-                }
-                ph.publish();
-                float4* x = cur1; cur1 = nxt1; nxt1 = x;
-                x = cur2; cur2 = nxt2; nxt2 = x;
-            }
-        }
-        hplane = reinterpret_cast<float*>(nxt1);   // not read by the last Chebyshev step
-    }
-    int32_t H1[NB][4], H2[NB][4];
-#pragma unroll
-    for (int b = 0; b < NB; ++b)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const long long h1 = (long long)F1[b][c] + __float2ll_rn(u1[b][c]);
-            const long long h2 = (long long)F2[b][c] + __float2ll_rn(u2[b][c]);
-            bad |= (unsigned)((h1 != (long long)(int32_t)h1) | (h2 != (long long)(int32_t)h2));
-            H1[b][c] = static_cast<int32_t>(h1);
-            H2[b][c] = static_cast<int32_t>(h2);
-        }
-    int4* Hb = reinterpret_cast<int4*>(hplane);
-    ph.settle();
-#pragma unroll
-    for (int b = 0; b < NB; ++b) Hb[nb[b].lq] = make_int4(H1[b][2], H1[b][3], H2[b][1], H2[b][3]);
-    ph.publish();
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        const int4 ha = nb[b].above(Hb), hl = nb[b].left(Hb);
-        const int32_t h1up[4] = {ha.x, ha.y, H1[b][0], H1[b][1]}, h2lf[4] = {hl.z, H2[b][0], hl.w, H2[b][2]};
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const long long v = (long long)q[b][c] + ((long long)H1[b][c] - h1up[c]) + ((long long)H2[b][c] - h2lf[c]);
-            bad |= (unsigned)((v >= (1LL << 30)) | (v <= -(1LL << 30)));
-            q[b][c] = static_cast<int32_t>(v);
-        }
-    }
-    // every thread has read what it needs: arrive, wait before the next plane write
-    ph.settle();
-    ClPhase::arrive();
-    ph.pend = true;
-}
-
-// theta_step<NC, 1> for the NB coarse cells of a thread in a band: sq the
-// band's coarse state, P0 / P2 the coarse transfers G_1 / G_2 (as integers,
-// published by the caller), P0..P3 band planes of one float per cell.  The
-// one-CTA step's arithmetic and order of additions; plane exchanges as in the
-// fine step.
-template <int NC, int BR, int NB>
-__device__ __forceinline__ void theta_coarse_step_cl(int32_t (&q)[NB], const BandNbr<NC, BR> (&nb)[NB], int32_t* sq,
-                                                     float* P0, float* P1, float* P2, float* P3, long long A,
-                                                     const TArgs& t, unsigned& bad, ClPhase& ph) {
-    long long F1[NB], F2[NB];
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        const int idx = nb[b].lq;
-        const int32_t g1 = as_i(P0[idx]), g2 = as_i(P2[idx]);
-        F1[b] = (long long)edge_flux64(A, nb[b].below(sq) - q[b]) + g1 + as_i(nb[b].below(P0));
-        F2[b] = (long long)edge_flux64(A, nb[b].right(sq) - q[b]) + g2 + as_i(nb[b].right(P2));
-    }
-    float u1[NB], u2[NB];
-#pragma unroll
-    for (int b = 0; b < NB; ++b) u1[b] = u2[b] = 0.f;
-    float* out1 = P1;
-    float* out2 = P3;
-    if (t.K > 0) {
-        ph.settle();
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            P1[nb[b].lq] = static_cast<float>(F1[b]);
-            P3[nb[b].lq] = static_cast<float>(F2[b]);
-        }
-        ph.publish();   // its wait also orders every read of the G planes before they are overwritten
-        float r1[NB], r2[NB], d1[NB], d2[NB];
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            const BandNbr<NC, BR>& n = nb[b];
-            const float f1 = P1[n.lq], f2 = P3[n.lq];
-            const float l1 = 4.f * f1 - n.above(P1) - n.below(P1) - n.left(P1) - n.right(P1);
-            const float l2 = 4.f * f2 - n.above(P3) - n.below(P3) - n.left(P3) - n.right(P3);
-            r1[b] = -t.alpha * l1;
-            r2[b] = -t.alpha * l2;
-            d1[b] = r1[b] * t.inv_theta;
-            d2[b] = r2[b] * t.inv_theta;
-        }
-        ph.settle();
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            P0[nb[b].lq] = d1[b];
-            P2[nb[b].lq] = d2[b];
-        }
-        ph.publish();
-        float *c1p = P0, *c2p = P2, *n1p = P1, *n2p = P3;
-        const float diag = 1.f + 4.f * t.alpha;
-        for (int k = 0; k < t.K; ++k) {
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
-                const BandNbr<NC, BR>& n = nb[b];
-                const float a1 = diag * d1[b] - t.alpha * (n.above(c1p) + n.below(c1p) + n.left(c1p) + n.right(c1p));
-                const float a2 = diag * d2[b] - t.alpha * (n.above(c2p) + n.below(c2p) + n.left(c2p) + n.right(c2p));
-                u1[b] += d1[b];
-                u2[b] += d2[b];
-                r1[b] -= a1;
-                r2[b] -= a2;
-            }
-            if (k + 1 < t.K) {
-#pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                    d1[b] = t.c1[k] * d1[b] + t.c2[k] * r1[b];
-                    d2[b] = t.c1[k] * d2[b] + t.c2[k] * r2[b];
-                }
-                ph.settle();
-#pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                    n1p[nb[b].lq] = d1[b];
-                    n2p[nb[b].lq] = d2[b];
-                }
-                ph.publish();
-                float* x = c1p; c1p = n1p; n1p = x;
-                x = c2p; c2p = n2p; n2p = x;
-            }
-        }
-        out1 = n1p;
-        out2 = n2p;
-    }
-    long long H1[NB], H2[NB];
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        H1[b] = F1[b] + __float2ll_rn(u1[b]);
-        H2[b] = F2[b] + __float2ll_rn(u2[b]);
-        bad |= (unsigned)((H1[b] != (long long)(int32_t)H1[b]) | (H2[b] != (long long)(int32_t)H2[b]));
-    }
-    ph.settle();
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        out1[nb[b].lq] = as_f(static_cast<int32_t>(H1[b]));
-        out2[nb[b].lq] = as_f(static_cast<int32_t>(H2[b]));
-    }
-    ph.publish();
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        const long long v = (long long)q[b] + (H1[b] - as_i(nb[b].above(out1))) + (H2[b] - as_i(nb[b].left(out2)));
-        bad |= (unsigned)((v >= (1LL << 30)) | (v <= -(1LL << 30)));
-        q[b] = static_cast<int32_t>(v);
-    }
-    ph.settle();
-#pragma unroll
-    for (int b = 0; b < NB; ++b) sq[nb[b].lq] = q[b];
-    ClPhase::arrive();
-    ph.pend = true;
-}
-
-// The theta-scheme sample kernel for a cluster of CL CTAs per sample (see
-// above), NB blocks of a block row per thread; a cluster is one sample
-// slot of a persistent grid of clusters.
-template <int N, int CL, int NB, bool CPL>
-__global__ void __launch_bounds__(CShape<N, CL, NB>::THREADS, 1) theta_cluster_kernel(const KArgs a, const TArgs t) {
-    using S = CShape<N, CL, NB>;
-    constexpr int NC = S::NC, BR = S::BR, BAND = S::BAND, THREADS = S::THREADS, RT = S::RT;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int tid = threadIdx.x;
-    const int rank = static_cast<int>(cg::this_cluster().block_rank());
-    float* P0 = reinterpret_cast<float*>(smem_raw);
-    float* P1 = P0 + 4 * BAND;
-    float* P2 = P1 + 4 * BAND;
-    float* P3 = P2 + 4 * BAND;
-    int32_t* sqc = reinterpret_cast<int32_t*>(P3 + 4 * BAND);
-    double* red = reinterpret_cast<double*>(sqc + BAND);
-    double* tot = red + (THREADS / 32) * kRed;       // this CTA's band total
-    double* acc = tot + kRed;                        // the slot's moment sums (rank 0)
-    for (int i = tid; i < a.slot_stride; i += THREADS) acc[i] = 0.0;
-    float* const planes[4] = {P0, P1, P2, P3};
-
-    // block row within the band; the thread's blocks are columns j0, j0 + RT, ...
-    // (consecutive lanes on consecutive blocks: conflict-free 16-byte plane accesses)
-    const int lr = tid / RT, j0 = tid % RT;
-    const int I1 = rank * BR + lr;                    // coarse row; fine block rows 2 I1 + v1, cols 2 I2 + v2
-    BandNbr<NC, BR> nb[NB];
-#pragma unroll
-    for (int b = 0; b < NB; ++b) nb[b] = BandNbr<NC, BR>(lr, j0 + b * RT, rank, CL);
-    ClPhase ph(lr == 0 || lr == BR - 1);              // the band's first and last rows read other CTAs
-    int gc[NB], fidx[NB][4];
-    uint32_t p_top[NB], p_bot[NB];
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        const int I2 = j0 + b * RT;
-        gc[b] = I1 * NC + I2;                         // global coarse index
-        const int f00 = (2 * I1) * N + 2 * I2;
-        fidx[b][0] = f00; fidx[b][1] = f00 + 1; fidx[b][2] = f00 + N; fidx[b][3] = f00 + N + 1;
-        p_top[b] = static_cast<uint32_t>(f00 >> 1);
-        p_bot[b] = static_cast<uint32_t>((f00 + N) >> 1);
-    }
-
-    const long long n_slots = (long long)gridDim.x / CL;
-    const long long slot = (long long)blockIdx.x / CL;
-    const long long iters = a.count > slot ? (a.count - slot + n_slots - 1) / n_slots : 0;
-    unsigned bad = 0;
-    ph.full();
-
-    for (long long it = 0; it < iters; ++it) {
-        const long long idx = slot + it * n_slots;
-        const bool active = idx < a.count;
-        const long long sid = a.first + (active ? idx : 0);
-        const uint32_t c2 = static_cast<uint32_t>(sid);
-        const uint32_t c3 = a.tag | ((static_cast<uint32_t>(static_cast<unsigned long long>(sid) >> 32) & 0xffffu) << 16);
-
-        int32_t q[NB][4], qc[NB];
-        float zt0[NB], zt1[NB];
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) q[b][i] = a.q0f[fidx[b][i]];
-            zt0[b] = zt1[b] = 0.f;
-            qc[b] = 0;
-            if constexpr (CPL) {
-                qc[b] = a.q0c[gc[b]];
-                sqc[nb[b].lq] = qc[b];
-            }
-        }
-        ph.full();
-
-        for (int m = 0; m < a.M; ++m) {
-            int32_t G1[NB][4], G2[NB][4];
-#pragma unroll
-            for (int b = 0; b < NB; ++b)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const uint4 x = philox10(make_uint4(h ? p_bot[b] : p_top[b], static_cast<uint32_t>(m), c2, c3),
-                                             a.key0, a.key1);
-                    float ra, ca, sa, rb, cb, sb;
-                    box_muller_polar(x.x, x.y, ra, ca, sa);
-                    box_muller_polar(x.z, x.w, rb, cb, sb);
-                    const float ta = noise_amp(q[b][2 * h], a.gf) * ra;
-                    const float tb = noise_amp(q[b][2 * h + 1], a.gf) * rb;
-                    G1[b][2 * h] = __float2int_rn(ta * ca);
-                    G2[b][2 * h] = __float2int_rn(ta * sa);
-                    G1[b][2 * h + 1] = __float2int_rn(tb * cb);
-                    G2[b][2 * h + 1] = __float2int_rn(tb * sb);
-                    if constexpr (CPL) {
-                        zt0[b] = fmaf(rb, cb, fmaf(ra, ca, zt0[b]));
-                        zt1[b] = fmaf(rb, sb, fmaf(ra, sa, zt1[b]));
-                    }
-                }
-            theta_fine_step_cl<NC, BR, NB>(q, G1, G2, nb, planes, t.Af64, t, bad, ph);
-
-            if constexpr (CPL) {
-                if ((m & 3) == 3) {
-                    ph.settle();
-#pragma unroll
-                    for (int b = 0; b < NB; ++b) {
-                        const float sc = noise_amp(qc[b], a.gc);
-                        P0[nb[b].lq] = as_f(__float2int_rn(sc * zt0[b]));
-                        P2[nb[b].lq] = as_f(__float2int_rn(sc * zt1[b]));
-                        zt0[b] = zt1[b] = 0.f;
-                    }
-                    ph.publish();
-                    theta_coarse_step_cl<NC, BR, NB>(qc, nb, sqc, P0, P1, P2, P3, t.Ac64, t, bad, ph);
-                }
-            }
-        }
-
-        // ---- observables of the band, then the band totals summed on rank 0 in rank order
-        double v[kRed];
-        {
-            long long mf = 0, mc = 0;
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) mf += q[b][i];
-                mc += qc[b];
-            }
-            v[2 * kMaxObs] = static_cast<double>(mf);
-            v[2 * kMaxObs + 1] = CPL ? static_cast<double>(mc) : 0.0;
-#pragma unroll
-            for (int k = 0; k < kMaxObs; ++k) {
-                double sf = 0.0, sc = 0.0;
-                if (k < a.n_obs) {
-#pragma unroll
-                    for (int b = 0; b < NB; ++b) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            sf += static_cast<double>(q[b][i] - a.qbf[fidx[b][i]]) *
-                                  t.phif64[(size_t)k * N * N + fidx[b][i]];
-                        if constexpr (CPL)
-                            sc += static_cast<double>(qc[b] - a.qbc[gc[b]]) * t.phic64[(size_t)k * NC * NC + gc[b]];
-                    }
-                }
-                v[k] = sf;
-                v[kMaxObs + k] = sc;
-            }
-        }
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1)
-#pragma unroll
-            for (int i = 0; i < kRed; ++i) v[i] += __shfl_xor_sync(kFullMask, v[i], off);
-        if ((tid & 31) == 0)
-#pragma unroll
-            for (int i = 0; i < kRed; ++i) red[(tid >> 5) * kRed + i] = v[i];
-        __syncthreads();
-        if (tid < kRed) {
-            double x = 0.0;
-            for (int w = 0; w < THREADS / 32; ++w) x += red[w * kRed + tid];
-            tot[tid] = x;
-        }
-        ph.full();
-        if (rank == 0 && tid == 0 && active) {
-            for (int i = 0; i < kRed; ++i) {
-                double x = 0.0;
-                for (int r = 0; r < CL; ++r) x += band_at(tot, r, 0)[i];
-                v[i] = x;
-            }
-            double Df[kMaxObs], Dc[kMaxObs];
-#pragma unroll
-            for (int k = 0; k < kMaxObs; ++k) {
-                Df[k] = a.dscale_f * v[k] + a.delta_f[k];
-                Dc[k] = CPL ? a.dscale_c * v[kMaxObs + k] + a.delta_c[k] : 0.0;
-            }
-            acc[0] += 1.0;
-            double merr = fabs(v[2 * kMaxObs] - static_cast<double>(a.mass0_f)) * a.dscale_f;
-            if (CPL) merr = fmax(merr, fabs(v[2 * kMaxObs + 1] - static_cast<double>(a.mass0_c)) * a.dscale_c);
-            acc[1] = fmax(acc[1], merr);
-            int qi = 0;
-            for (int j = 0; j < a.n_obs; ++j) {
-                const int kend = a.products ? a.n_obs : j + 1;
-                for (int k = j; k < kend; ++k, ++qi) {
-                    const double pf = a.N * Df[j] * Df[k];
-                    const double pc = CPL ? a.N * Dc[j] * Dc[k] : 0.0;
-                    const double dp = pf - pc, dp2 = dp * dp;
-                    double* B = acc + 2 + kNSum * qi;
-                    B[0] += dp; B[1] += dp2; B[2] += dp2 * dp; B[3] += dp2 * dp2;
-                    B[4] += pf; B[5] += pf * pf; B[6] += pc; B[7] += pc * pc;
-                    B[8] += Df[j]; B[9] += Df[j] * Df[j]; B[10] += Dc[j]; B[11] += Dc[j] * Dc[j];
-                }
-            }
-            if (a.samples) {
-                double* o = a.samples + idx * (2 * a.n_obs + 2);
-                for (int k = 0; k < a.n_obs; ++k) {
-                    o[k] = Df[k];
-                    o[a.n_obs + k] = Dc[k];
-                }
-                o[2 * a.n_obs] = v[2 * kMaxObs] * a.dscale_f;
-                o[2 * a.n_obs + 1] = CPL ? v[2 * kMaxObs + 1] * a.dscale_c : 0.0;
-            }
-        }
-        ph.full();   // the band totals and the state planes are reused by the next sample
-    }
-    if (bad) atomicOr(a.err, kErrRange);
-
-    // ---- the slot's partial sums (rank 0), entry-major [stride][n_slots]
-    __syncthreads();
     if (rank == 0)
-        for (int i = tid; i < a.slot_stride; i += THREADS) a.partials[(size_t)i * n_slots + slot] = acc[i];
+        for (int i = tid; i < SPB * a.slot_stride; i += THREADS) {
+            const int s = i / a.slot_stride, e = i % a.slot_stride;
+            a.partials[(size_t)e * n_slots + cta_slot0 + s] = acc[i];
+        }
 }
+
+template <class S>
+void launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int n_ctas, int slot_stride,
+                   cudaStream_t st, int priority) {
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3(n_ctas);
+    cfg.blockDim = dim3(S::THREADS);
+    cfg.dynamicSmemBytes = S::smem(slot_stride);
+    cfg.stream = st;
+    int na = 0;
+    if constexpr (S::CL > 1) {
+        attr[na].id = cudaLaunchAttributeClusterDimension;
+        attr[na].val.clusterDim.x = S::CL;
+        attr[na].val.clusterDim.y = 1;
+        attr[na].val.clusterDim.z = 1;
+        ++na;
+    }
+    if (priority != 0) {
+        attr[na].id = cudaLaunchAttributePriority;
+        attr[na].val.priority = priority;
+        ++na;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = na;
+}
+
+// From 32 x 32 on there are two builds, chosen by the number of samples: one for
+// few, which is the faster one for a sample, and a DENSE one for the GPU's
+// throughput.  FEW is the number of samples that the first holds at once.
+// Measured, ms, first build / DENSE: 128^2 x 384 steps, 36 samples 5.1 / 6.7, 150
+// samples 25.3 / 22.6; 64^2 x 96, 152 samples 1.03 / 1.15, 304 2.2 / 1.8, 1000 7.7 /
+// 6.2; 32^2 x 24 (2 x 2 blocks / 4 x 4), 3 samples 0.10 / 0.22, 304 0.160 / 0.25.
+template <int N>
+constexpr long long kFew = N == 32 ? 304 : N == 64 ? 152 : N == 128 ? 36 : 0;
 
 template <int N, bool CPL>
 cudaError_t prepare(int slot_stride, VariantInfo* out) {
-    using S = TShape<N>;
+    using S = TShape<N, (N >= 32)>;
     const size_t smem = S::smem(slot_stride);
-    cudaError_t e = cudaFuncSetAttribute(theta_kernel<N, CPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const auto kernel = theta_kernel<N, CPL, (N >= 32)>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && N >= 32)
+        e = cudaFuncSetAttribute(theta_kernel<N, CPL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)TShape<N, false>::smem(slot_stride));
     if (e != cudaSuccess) return e;
-    int per_sm = 0, dev = 0, sms = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, theta_kernel<N, CPL>, S::THREADS, smem)) !=
-        cudaSuccess)
-        return e;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     *out = VariantInfo{};
-    out->supported = per_sm > 0;
     out->threads = S::THREADS;
-    out->cluster = 1;
-    out->slots_per_cta = S::SPB;
+    out->cluster = S::CL;
+    out->slots_per_cta = S::SPB;   // clusters: one sample slot per cluster
     out->smem = smem;
-    out->max_ctas = per_sm * sms;
+    if constexpr (S::CL > 1) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr[2];
+        launch_config<S>(cfg, attr, S::CL, slot_stride, nullptr, 0);
+        int clusters = 0;
+        if ((e = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg)) != cudaSuccess) return e;
+        out->max_ctas = clusters * S::CL;
+    } else {
+        int per_sm = 0, dev = 0, sms = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, S::THREADS, smem)) != cudaSuccess ||
+            (e = cudaGetDevice(&dev)) != cudaSuccess ||
+            (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+            return e;
+        out->max_ctas = per_sm * sms;
+    }
+    out->supported = out->max_ctas > 0;
     return cudaSuccess;
+}
+
+template <int N, bool CPL, bool DENSE>
+cudaError_t launch_build(const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t st, int priority) {
+    using S = TShape<N, DENSE>;
+    if (n_ctas % S::CL != 0) return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    launch_config<S>(cfg, attr, n_ctas, a.slot_stride, st, priority);
+    return cudaLaunchKernelEx(&cfg, theta_kernel<N, CPL, DENSE>, a, t);
 }
 
 template <int N, bool CPL>
 cudaError_t launch_n(const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t st, int priority) {
-    using S = TShape<N>;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(n_ctas);
-    cfg.blockDim = dim3(S::THREADS);
-    cfg.dynamicSmemBytes = S::smem(a.slot_stride);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    int na = 0;
-    if (priority != 0) {
-        attr[na].id = cudaLaunchAttributePriority;
-        attr[na].val.priority = priority;
-        ++na;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = na;
-    return cudaLaunchKernelEx(&cfg, theta_kernel<N, CPL>, a, t);
+    // (both builds have one sample slot per CTA or cluster from 32 x 32 on)
+    if constexpr (N >= 32)
+        if (a.count > kFew<N>) return launch_build<N, CPL, true>(a, t, n_ctas, st, priority);
+    return launch_build<N, CPL, false>(a, t, n_ctas, st, priority);
 }
 
-// Grids beyond one CTA: clusters of CL CTAs.
-constexpr int kThetaClusterN = 128, kThetaClusterCL = 4, kThetaClusterNB = 2;
-
-template <int N, int CL, int NB, bool CPL>
-cudaError_t prepare_cluster(int slot_stride, VariantInfo* out) {
-    using S = CShape<N, CL, NB>;
-    const size_t smem = S::smem(slot_stride);
-    cudaError_t e = cudaFuncSetAttribute(theta_cluster_kernel<N, CL, NB, CPL>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(CL);
-    cfg.blockDim = dim3(S::THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CL;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int clusters = 0;
-    if ((e = cudaOccupancyMaxActiveClusters(&clusters, theta_cluster_kernel<N, CL, NB, CPL>, &cfg)) != cudaSuccess)
-        return e;
-    *out = VariantInfo{};
-    out->supported = clusters > 0;
-    out->threads = S::THREADS;
-    out->cluster = CL;
-    out->slots_per_cta = 1;   // one sample slot per cluster
-    out->smem = smem;
-    out->max_ctas = clusters * CL;
-    return cudaSuccess;
-}
-
-template <int N, int CL, int NB, bool CPL>
-cudaError_t launch_cluster(const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t st, int priority) {
-    using S = CShape<N, CL, NB>;
-    if (n_ctas % CL != 0) return cudaErrorInvalidValue;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(n_ctas);
-    cfg.blockDim = dim3(S::THREADS);
-    cfg.dynamicSmemBytes = S::smem(a.slot_stride);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    int na = 0;
-    attr[na].id = cudaLaunchAttributeClusterDimension;
-    attr[na].val.clusterDim.x = CL;
-    attr[na].val.clusterDim.y = 1;
-    attr[na].val.clusterDim.z = 1;
-    ++na;
-    if (priority != 0) {
-        attr[na].id = cudaLaunchAttributePriority;
-        attr[na].val.priority = priority;
-        ++na;
+// f(std::integral_constant<int, N>) for the grid sizes with a kernel.
+template <class F>
+bool for_grid(int n, F&& f) {
+    switch (n) {
+        case 4: f(std::integral_constant<int, 4>{}); return true;
+        case 8: f(std::integral_constant<int, 8>{}); return true;
+        case 16: f(std::integral_constant<int, 16>{}); return true;
+        case 32: f(std::integral_constant<int, 32>{}); return true;
+        case 64: f(std::integral_constant<int, 64>{}); return true;
+        case 128: f(std::integral_constant<int, 128>{}); return true;
+        default: return false;
     }
-    cfg.attrs = attr;
-    cfg.numAttrs = na;
-    return cudaLaunchKernelEx(&cfg, theta_cluster_kernel<N, CL, NB, CPL>, a, t);
 }
 
 }  // namespace
 
-bool theta_supported(int n) { return n == 4 || n == 8 || n == 16 || n == 32 || n == 64 || n == kThetaClusterN; }
+bool theta_supported(int n) {
+    return for_grid(n, [](auto) {});
+}
 
 cudaError_t theta_variant_info(int n, bool coupled, int slot_stride, VariantInfo* out) {
-    *out = VariantInfo{};
-    switch (n) {
-        case 4: return coupled ? prepare<4, true>(slot_stride, out) : prepare<4, false>(slot_stride, out);
-        case 8: return coupled ? prepare<8, true>(slot_stride, out) : prepare<8, false>(slot_stride, out);
-        case 16: return coupled ? prepare<16, true>(slot_stride, out) : prepare<16, false>(slot_stride, out);
-        case 32: return coupled ? prepare<32, true>(slot_stride, out) : prepare<32, false>(slot_stride, out);
-        case 64: return coupled ? prepare<64, true>(slot_stride, out) : prepare<64, false>(slot_stride, out);
-        case kThetaClusterN:
-            return coupled ? prepare_cluster<kThetaClusterN, kThetaClusterCL, kThetaClusterNB, true>(slot_stride, out)
-                           : prepare_cluster<kThetaClusterN, kThetaClusterCL, kThetaClusterNB, false>(slot_stride, out);
-        default: return cudaSuccess;   // supported = 0
-    }
+    *out = VariantInfo{};   // supported = 0 for other grids
+    cudaError_t e = cudaSuccess;
+    for_grid(n, [&](auto N) { e = coupled ? prepare<N.value, true>(slot_stride, out) : prepare<N.value, false>(slot_stride, out); });
+    return e;
 }
 
 cudaError_t launch_theta(int n, bool coupled, const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t st,
                          int priority) {
     if (t.K < 0 || t.K > kMaxCheb) return cudaErrorInvalidValue;
-    switch (n) {
-        case 4: return coupled ? launch_n<4, true>(a, t, n_ctas, st, priority) : launch_n<4, false>(a, t, n_ctas, st, priority);
-        case 8: return coupled ? launch_n<8, true>(a, t, n_ctas, st, priority) : launch_n<8, false>(a, t, n_ctas, st, priority);
-        case 16: return coupled ? launch_n<16, true>(a, t, n_ctas, st, priority) : launch_n<16, false>(a, t, n_ctas, st, priority);
-        case 32: return coupled ? launch_n<32, true>(a, t, n_ctas, st, priority) : launch_n<32, false>(a, t, n_ctas, st, priority);
-        case 64: return coupled ? launch_n<64, true>(a, t, n_ctas, st, priority) : launch_n<64, false>(a, t, n_ctas, st, priority);
-        case kThetaClusterN:
-            return coupled ? launch_cluster<kThetaClusterN, kThetaClusterCL, kThetaClusterNB, true>(a, t, n_ctas, st, priority)
-                           : launch_cluster<kThetaClusterN, kThetaClusterCL, kThetaClusterNB, false>(a, t, n_ctas, st, priority);
-        default: return cudaErrorInvalidValue;
-    }
+    cudaError_t e = cudaErrorInvalidValue;
+    for_grid(n, [&](auto N) {
+        e = coupled ? launch_n<N.value, true>(a, t, n_ctas, st, priority) : launch_n<N.value, false>(a, t, n_ctas, st, priority);
+    });
+    return e;
 }
 
 }  // namespace dk
