@@ -58,13 +58,16 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kRedW = 2 * kMaxObs + 2;     // reduced values per sample
 constexpr int kMaxStride = 2 + kNSum * 10;  // largest slot stride (4 obs with products)
 
-template <int NF_, int C_, int R_, int CL_, bool COUPLED_, bool FLUCT_ = false>
+template <int NF_, int C_, int R_, int CL_, bool COUPLED_, bool FLUCT_ = false, int CHAIN_ = 1>
 struct Shape {
     static constexpr int NF = NF_, C = C_, R = R_, CL = CL_;
     static constexpr bool COUPLED = COUPLED_;
     // fluctuation state: q holds (rho - rho-bar^m) 2^S, rho-bar^m read from a
     // per-step mean-field table (see KArgs::rbf)
     static constexpr bool FLUCT = FLUCT_;
+    // a lane's FP32 projection sums run on through the blocks of CHAIN bands, one
+    // below the other: the sums of a shape with CHAIN times the rows per lane
+    static constexpr int CHAIN = CHAIN_;
     static constexpr int NC = NF / 2;
     static constexpr int FR = 2 * R, FC = 2 * C;
     static constexpr int LPB = NC / C;            // lanes per band
@@ -112,6 +115,8 @@ struct Shape {
     static_assert(C % 2 == 0 || (C == 1 && R <= 2), "cell pairs are worked on two at a time");
     static_assert(LPB <= 32 && (LPB & (LPB - 1)) == 0, "a band must be a power-of-two warp segment");
     static_assert(NC % C == 0 && NC % R == 0, "lane blocks must tile the coarse grid");
+    static_assert(CHAIN == 1 || (CHAIN == 2 && !WARP && CL == 1 && 32 % (2 * LPB) == 0),
+                  "chained bands share a warp");
     static_assert(WARP || (THREADS % 32 == 0 && THREADS <= 1024 && NB % CL == 0), "bad CTA shape");
     static_assert(WARP || CL == 1 || (LPS / CL) % LPB == 0, "bands may not straddle CTAs");
     static constexpr size_t fixed_smem() {
@@ -646,24 +651,37 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB) level_kernel(const KArgs 
             for (int k = 0; k < kMaxObs; ++k) {
                 float sf = 0.f, sc = 0.f;
                 if (k < a.n_obs) {
+                    const auto project = [&]() {
 #pragma unroll
-                    for (int r = 0; r < FR; ++r) {
-                        int32_t qb[FC];
-                        float ph[FC];
-                        load_row<FC>(qb, a.qbf + (size_t)(row0 + r) * NF + col0);
-                        load_row_f<FC>(ph, a.phif + (size_t)k * NF * NF + (size_t)(row0 + r) * NF + col0);
+                        for (int r = 0; r < FR; ++r) {
+                            int32_t qb[FC];
+                            float ph[FC];
+                            load_row<FC>(qb, a.qbf + (size_t)(row0 + r) * NF + col0);
+                            load_row_f<FC>(ph, a.phif + (size_t)k * NF * NF + (size_t)(row0 + r) * NF + col0);
 #pragma unroll
-                        for (int c = 0; c < FC; ++c) sf = fmaf(__int2float_rn(q[r][c] - qb[c]), ph[c], sf);
-                    }
-                    if constexpr (CPL) {
+                            for (int c = 0; c < FC; ++c) sf = fmaf(__int2float_rn(q[r][c] - qb[c]), ph[c], sf);
+                        }
+                        if constexpr (CPL) {
 #pragma unroll
-                        for (int i = 0; i < R; ++i) {
-                            int32_t qb[C];
-                            float ph[C];
-                            load_row<C>(qb, a.qbc + (size_t)(crow0 + i) * NC + ccol0);
-                            load_row_f<C>(ph, a.phic + (size_t)k * NC * NC + (size_t)(crow0 + i) * NC + ccol0);
+                            for (int i = 0; i < R; ++i) {
+                                int32_t qb[C];
+                                float ph[C];
+                                load_row<C>(qb, a.qbc + (size_t)(crow0 + i) * NC + ccol0);
+                                load_row_f<C>(ph, a.phic + (size_t)k * NC * NC + (size_t)(crow0 + i) * NC + ccol0);
 #pragma unroll
-                            for (int j = 0; j < C; ++j) sc = fmaf(__int2float_rn(qc[i][j] - qb[j]), ph[j], sc);
+                                for (int j = 0; j < C; ++j) sc = fmaf(__int2float_rn(qc[i][j] - qb[j]), ph[j], sc);
+                            }
+                        }
+                    };
+                    project();
+                    if constexpr (S::CHAIN == 2) {
+                        // odd bands continue the sum of the band above, in the same warp
+                        const float uf = __shfl_up_sync(kFull, sf, LPB), uc = __shfl_up_sync(kFull, sc, LPB);
+                        sf = sc = 0.f;
+                        if (band & 1) {
+                            sf = uf;
+                            sc = uc;
+                            project();
                         }
                     }
                 }
@@ -945,14 +963,46 @@ struct VariantEntry {
     cudaError_t (*launch)(bool coupled, const KArgs& a, int n_ctas, cudaStream_t st, int priority);
 };
 
+// Few samples: the same level on twice the lanes, half the rows each.  Below about
+// a warp per scheduler the time of a batch is that of one sample's chain of steps,
+// and half the cells per lane shorten it; the sums keep the full shape's order
+// (CHAIN).  Measured, us, full shape / twice the lanes: 16^2 x 52 steps, 256 samples
+// 43.6 / 25.1, 912 57.8 / 44.1, 1216 56.9 / 65.4; 32^2 x 208 coupled, 152 samples 193 /
+// 122, 456 297 / 248, 608 300 / 391; 32^2 plain, 456 282 / 231, 608 283 / 362.  At
+// 64^2 the full shape fills an SM's schedulers with one sample and wins (152: 312 / 347).
+template <int NF, int C, int R, int CL, bool FL>
+struct Split {
+    static constexpr bool ON = !FL && CL == 1 && ((NF == 16 && C == 1 && R == 2) || (NF == 32 && C == 2 && R == 2));
+    static constexpr long long MAX_COUNT = NF == 16 ? 912 : 456;
+    template <bool CPL>
+    using shape = Shape<NF, C, ON ? R / 2 : R, CL, CPL, FL, ON ? 2 : 1>;
+};
+
 template <int NF, int C, int R, int CL, bool FL>
 cudaError_t variant_info_fn(bool coupled, int stride, VariantInfo* vi) {
+    using SP = Split<NF, C, R, CL, FL>;
+    if constexpr (SP::ON) {
+        // the few-sample shape's launch attributes (its slots are the full shape's)
+        VariantInfo few{};
+        const cudaError_t e = coupled ? Kern<typename SP::template shape<true>>::info(stride, &few)
+                                      : Kern<typename SP::template shape<false>>::info(stride, &few);
+        if (e != cudaSuccess) return e;
+    }
     return coupled ? Kern<Shape<NF, C, R, CL, true, FL>>::info(stride, vi)
                    : Kern<Shape<NF, C, R, CL, false, FL>>::info(stride, vi);
 }
 
 template <int NF, int C, int R, int CL, bool FL>
 cudaError_t variant_launch_fn(bool coupled, const KArgs& a, int n_ctas, cudaStream_t st, int priority) {
+    using SP = Split<NF, C, R, CL, FL>;
+    if constexpr (SP::ON) {
+        // one CTA per sample slot, the same slots
+        if (a.count <= SP::MAX_COUNT) {
+            const int n_slots = n_ctas * Shape<NF, C, R, CL, true, FL>::SLOTS_PER_CTA;
+            return coupled ? Kern<typename SP::template shape<true>>::launch(a, n_slots, st, priority)
+                           : Kern<typename SP::template shape<false>>::launch(a, n_slots, st, priority);
+        }
+    }
     return coupled ? Kern<Shape<NF, C, R, CL, true, FL>>::launch(a, n_ctas, st, priority)
                    : Kern<Shape<NF, C, R, CL, false, FL>>::launch(a, n_ctas, st, priority);
 }
