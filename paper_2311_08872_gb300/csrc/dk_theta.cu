@@ -287,7 +287,7 @@ __device__ __forceinline__ void neighbours(f32x2 (&a)[R][C], Exchange<S>& x, F&&
 
 // One theta step of an R x C block of a periodic grid of LPR C columns (the
 // fine grid, or the coarse one with COARSE: the four neighbours are added in
-// another order there).
+// another order there, and in one CTA the recurrence rounds its other product).
 template <int R, int C, bool COARSE, class S>
 __device__ __forceinline__ void theta_step(int32_t (&q)[R][C], const int32_t (&G1)[R][C], const int32_t (&G2)[R][C],
                                            long long A, const TArgs& t, unsigned& bad, Exchange<S>& x) {
@@ -361,7 +361,8 @@ __device__ __forceinline__ void theta_step(int32_t (&q)[R][C], const int32_t (&G
 #pragma unroll
                 for (int c = 0; c < C; ++c) {
                     u[r][c] = add2(u[r][c], d[r][c]);
-                    d[r][c] = fma2(ca, d[r][c], mul2(cb, res[r][c]));
+                    if constexpr (COARSE && S::CL == 1) d[r][c] = fma2(cb, res[r][c], mul2(ca, d[r][c]));
+                    else d[r][c] = fma2(ca, d[r][c], mul2(cb, res[r][c]));
                 }
         }
 #pragma unroll
