@@ -26,7 +26,7 @@
 // per-step tables (fine: step m; coarse: coarse step m / 9).
 //
 // Work decomposition.  One CTA per sample.  A thread holds a block of 2 x 6
-// fine cells (two rows of 3 Philox cell pairs), their transfers and their
+// fine cells (two rows of 3 Philox cell pairs; one row at 6^2), their transfers and their
 // summed normals in registers; its two rows of state and G1 and the end columns
 // of G2 pass through shared memory, double buffered by the step's parity, so a
 // fine step has one barrier.  Every 9 steps the summed normals go to shared
@@ -35,7 +35,7 @@
 //
 // Bound by instruction issue and its latencies (issue slots 47% busy with 16 warps;
 // fixed-latency waits, the special functions and shared memory lead).  54^2, 607
-// samples x 648 steps: 4.25 ms; 5.20 with a 1 x 6 segment of cells per thread, whose
+// samples x 648 steps: 4.08 ms; 5.20 with a 1 x 6 segment of cells per thread, whose
 // shared-memory traffic (12 words a cell, here 5, with the summed normals there as
 // well) and one-point restriction (two loads per FMA) were half of the time.
 #include "dk_device.cuh"
@@ -47,10 +47,10 @@ namespace {
 constexpr unsigned kFullMaskF = 0xffffffffu;
 constexpr int kRedF = 2 * kMaxObs + 2;
 
-template <int N_>
+template <int N_, int R_>
 struct FShape {
     static constexpr int N = N_, NC = N / 3;
-    static constexpr int R = 2, C = 6;                  // fine cells per thread
+    static constexpr int R = R_, C = 6;                 // fine cells per thread
     static constexpr int BRW = N / R, BCL = N / C;      // rows / columns of blocks
     static constexpr int FT = BRW * BCL;                // threads that hold fine cells
     static constexpr int THREADS = (FT + 31) / 32 * 32;
@@ -87,9 +87,10 @@ __device__ __forceinline__ void explicit_update(const int32_t* q, const int32_t*
     }
 }
 
-template <int N, bool CPL, bool FL>
-__global__ void __launch_bounds__(FShape<N>::THREADS, FShape<N>::MINB) fourier_kernel(const KArgs a, const FArgs f) {
-    using S = FShape<N>;
+template <int N, int ROWS, bool CPL, bool FL>
+__global__ void __launch_bounds__(FShape<N, ROWS>::THREADS, FShape<N, ROWS>::MINB)
+    fourier_kernel(const KArgs a, const FArgs f) {
+    using S = FShape<N, ROWS>;
     constexpr int NC = S::NC, THREADS = S::THREADS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tid = threadIdx.x;
@@ -225,25 +226,28 @@ __global__ void __launch_bounds__(FShape<N>::THREADS, FShape<N>::MINB) fourier_k
             if constexpr (CPL) {
                 if (m9 == 8) {
                     // ---- coarse noise P1 S P1^T (S = summed fine normals, published by the barrier above):
-                    // T = S P1^T, a thread the rows 2 br, 2 br + 1 and the coarse columns 2 bc, 2 bc + 1
+                    // T = S P1^T, a thread its block's rows and the coarse columns 2 bc, 2 bc + 1
                     if (fine_thread) {
-                        const ulonglong2* const z0 = reinterpret_cast<const ulonglong2*>(Zs + 2 * br * N);
-                        const ulonglong2* const z1 = reinterpret_cast<const ulonglong2*>(Zs + (2 * br + 1) * N);
+                        const ulonglong2* const z = reinterpret_cast<const ulonglong2*>(Zs + br * R * N);
                         const float2* const w0 = reinterpret_cast<const float2*>(P1 + 2 * bc * N);
                         const float2* const w1 = reinterpret_cast<const float2*>(P1 + (2 * bc + 1) * N);
-                        f32x2 s00 = pack2(0.f, 0.f), s01 = s00, s10 = s00, s11 = s00;
+                        f32x2 s0[R], s1[R];
+#pragma unroll
+                        for (int r = 0; r < R; ++r) s0[r] = s1[r] = pack2(0.f, 0.f);
 #pragma unroll 3
                         for (int x = 0; x < N / 2; ++x) {
-                            const ulonglong2 u = z0[x], v = z1[x];
                             const float2 p = w0[x], w = w1[x];
                             const f32x2 px = pack2(p.x, p.x), py = pack2(p.y, p.y), wx = pack2(w.x, w.x), wy = pack2(w.y, w.y);
-                            s00 = fma2(u.y, py, fma2(u.x, px, s00));
-                            s01 = fma2(u.y, wy, fma2(u.x, wx, s01));
-                            s10 = fma2(v.y, py, fma2(v.x, px, s10));
-                            s11 = fma2(v.y, wy, fma2(v.x, wx, s11));
+#pragma unroll
+                            for (int r = 0; r < R; ++r) {
+                                const ulonglong2 u = z[r * (N / 2) + x];
+                                s0[r] = fma2(u.y, py, fma2(u.x, px, s0[r]));
+                                s1[r] = fma2(u.y, wy, fma2(u.x, wx, s1[r]));
+                            }
                         }
-                        reinterpret_cast<ulonglong2*>(Tm)[br * NC + bc] = make_ulonglong2(s00, s01);
-                        reinterpret_cast<ulonglong2*>(Tm)[br * NC + NC / 2 + bc] = make_ulonglong2(s10, s11);
+#pragma unroll
+                        for (int r = 0; r < R; ++r)
+                            reinterpret_cast<ulonglong2*>(Tm)[(br * R + r) * (NC / 2) + bc] = make_ulonglong2(s0[r], s1[r]);
                     }
                     __syncthreads();
                     const int32_t* qc = ccur ? qcB : qcA;
@@ -285,22 +289,35 @@ __global__ void __launch_bounds__(FShape<N>::THREADS, FShape<N>::MINB) fourier_k
 #pragma unroll
         for (int i = 0; i < kRedF; ++i) v[i] = 0.0;
         if (fine_thread) {
+            long long mass = 0;
+            int32_t d[R][C];
 #pragma unroll
             for (int r = 0; r < R; ++r)
 #pragma unroll
                 for (int c = 0; c < C; ++c) {
-                    const int x = fx0 + r * N + c;
-                    v[2 * kMaxObs] += static_cast<double>(q[r][c]);
-                    const double d = static_cast<double>(q[r][c] - a.qbf[x]);
-                    for (int k = 0; k < a.n_obs; ++k) v[k] += d * f.phif64[(size_t)k * N * N + x];
+                    mass += q[r][c];
+                    d[r][c] = q[r][c] - a.qbf[fx0 + r * N + c];
                 }
+            v[2 * kMaxObs] = static_cast<double>(mass);
+#pragma unroll
+            for (int k = 0; k < kMaxObs; ++k) {
+                if (k < a.n_obs) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+#pragma unroll
+                        for (int c = 0; c < C; ++c)
+                            v[k] += static_cast<double>(d[r][c]) * f.phif64[(size_t)k * N * N + fx0 + r * N + c];
+                }
+            }
         }
         if constexpr (CPL) {
             const int32_t* qc = ccur ? qcB : qcA;
             for (int y = tid; y < NC * NC; y += THREADS) {
                 v[2 * kMaxObs + 1] += static_cast<double>(qc[y]);
                 const double d = static_cast<double>(qc[y] - a.qbc[y]);
-                for (int k = 0; k < a.n_obs; ++k) v[kMaxObs + k] += d * f.phic64[(size_t)k * NC * NC + y];
+#pragma unroll
+                for (int k = 0; k < kMaxObs; ++k)
+                    if (k < a.n_obs) v[kMaxObs + k] += d * f.phic64[(size_t)k * NC * NC + y];
             }
         }
 #pragma unroll
@@ -355,16 +372,29 @@ __global__ void __launch_bounds__(FShape<N>::THREADS, FShape<N>::MINB) fourier_k
     for (int i = tid; i < a.slot_stride; i += THREADS) a.partials[(size_t)i * n_slots + slot] = acc[i];
 }
 
+// Two builds at 18^2: few samples run on 1 x 6 cells per thread (two warps per
+// sample), which is the faster one for a sample, many on 2 x 6 (one warp).
+// 18^2 x 72 steps, us, one row / two rows: 3 samples 62 / 113, 1216 116 / 172; 20000
+// samples 2310 (one row, normals in shared memory) / 1680.
+template <int N>
+constexpr long long kFewF = N == 18 ? 1216 : 0;
+template <int N>
+constexpr int kRows = N == 6 ? 1 : 2;
+
 template <int N, bool CPL, bool FL>
 cudaError_t fprepare(int slot_stride, VariantInfo* out) {
-    using S = FShape<N>;
+    using S = FShape<N, kRows<N>>;
     const size_t smem = S::smem(slot_stride);
-    cudaError_t e = cudaFuncSetAttribute(fourier_kernel<N, CPL, FL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const auto kernel = fourier_kernel<N, kRows<N>, CPL, FL>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if constexpr (kFewF<N> > 0) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(fourier_kernel<N, 1, CPL, FL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)FShape<N, 1>::smem(slot_stride));
+    }
     if (e != cudaSuccess) return e;
     int per_sm = 0, dev = 0, sms = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fourier_kernel<N, CPL, FL>, S::THREADS, smem)) !=
-        cudaSuccess)
-        return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, S::THREADS, smem)) != cudaSuccess) return e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     *out = VariantInfo{};
@@ -377,9 +407,9 @@ cudaError_t fprepare(int slot_stride, VariantInfo* out) {
     return cudaSuccess;
 }
 
-template <int N, bool CPL, bool FL>
-cudaError_t flaunch(const KArgs& a, const FArgs& f, int n_ctas, cudaStream_t st, int priority) {
-    using S = FShape<N>;
+template <int N, int ROWS, bool CPL, bool FL>
+cudaError_t flaunch_rows(const KArgs& a, const FArgs& f, int n_ctas, cudaStream_t st, int priority) {
+    using S = FShape<N, ROWS>;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(n_ctas);
     cfg.blockDim = dim3(S::THREADS);
@@ -394,7 +424,15 @@ cudaError_t flaunch(const KArgs& a, const FArgs& f, int n_ctas, cudaStream_t st,
     }
     cfg.attrs = attr;
     cfg.numAttrs = na;
-    return cudaLaunchKernelEx(&cfg, fourier_kernel<N, CPL, FL>, a, f);
+    return cudaLaunchKernelEx(&cfg, fourier_kernel<N, ROWS, CPL, FL>, a, f);
+}
+
+template <int N, bool CPL, bool FL>
+cudaError_t flaunch(const KArgs& a, const FArgs& f, int n_ctas, cudaStream_t st, int priority) {
+    if constexpr (kFewF<N> > 0) {
+        if (a.count <= kFewF<N>) return flaunch_rows<N, 1, CPL, FL>(a, f, n_ctas, st, priority);
+    }
+    return flaunch_rows<N, kRows<N>, CPL, FL>(a, f, n_ctas, st, priority);
 }
 
 template <bool FL>
