@@ -58,7 +58,7 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kRedW = 2 * kMaxObs + 2;     // reduced values per sample
 constexpr int kMaxStride = 2 + kNSum * 10;  // largest slot stride (4 obs with products)
 
-template <int NF_, int C_, int R_, int CL_, bool COUPLED_, bool FLUCT_ = false, int CHAIN_ = 1>
+template <int NF_, int C_, int R_, int CL_, bool COUPLED_, bool FLUCT_ = false, int CHAIN_ = 1, bool FEW_ = false>
 struct Shape {
     static constexpr int NF = NF_, C = C_, R = R_, CL = CL_;
     static constexpr bool COUPLED = COUPLED_;
@@ -91,17 +91,19 @@ struct Shape {
     //   REDRAW the sample's Philox counter word is opaque to the compiler, which
     //          then does not keep the step-independent parts of the first rounds in
     //          registers, where those would spill (128^2: 22.7 with, 23.7 without,
-    //          25.1 before; 256^2: 19.8 with, 23.0 without).
+    //          25.1 before; 256^2: 19.8 with, 23.0 without).  Fine-only 128^2 does not
+    //          spill (40 samples x 384: 1.32 with, 1.27 without, 1.31 before).
     //   The fluctuation state needs its mean-field rows in registers as well and
     //   is fastest with neither (128^2, 311 x 1024: 18.6, before 20.2; 64^2, 997 x
     //   256: 2.89, with PIPE 3.28, before 3.13; loading the next step's rows
     //   early: 20.3 at 128^2).
     static constexpr bool PIPE = !FLUCT && (CL == 1 ? !WARP : FR * FC >= 32);
-    static constexpr bool REDRAW = !FLUCT && CL > 1;
+    static constexpr bool REDRAW = !FLUCT && CL > 1 && (COUPLED || FR * FC >= 32);
     // Resident warps per SM asked for (a bound on the registers per thread).
     // 32^2 fine-only, 1000 x 103: 8 warps 0.288 ms, 12 warps 0.282; 16^2 in one
     // warp, 9250 x 52: 16 warps 0.316, 24 warps 0.306 (before 0.337).
-    static constexpr int WARPS_MIN = FLUCT ? 16 : FR * FC >= 32 ? 8 : PIPE ? (COUPLED && FR * FC >= 16 ? 8 : 12)
+    // Few samples with the fluctuation state want the registers of 8 warps.
+    static constexpr int WARPS_MIN = FLUCT ? (FEW_ ? 8 : 16) : FR * FC >= 32 ? 8 : PIPE ? (COUPLED && FR * FC >= 16 ? 8 : 12)
                                    : FR * FC >= 16 || FR * FC < 8 ? 16 : 24;
     static constexpr int MINB = WARPS_MIN * 32 / THREADS > 0 ? WARPS_MIN * 32 / THREADS : 1;
     static constexpr int SLOTS_PER_CTA = WARP ? (THREADS / 32) * SPW : 1;
@@ -972,22 +974,34 @@ struct VariantEntry {
 // 64^2 the full shape fills an SM's schedulers with one sample and wins (152: 312 / 347).
 template <int NF, int C, int R, int CL, bool FL>
 struct Split {
-    static constexpr bool ON = !FL && CL == 1 && ((NF == 16 && C == 1 && R == 2) || (NF == 32 && C == 2 && R == 2));
-    static constexpr long long MAX_COUNT = NF == 16 ? 912 : 456;
+    static constexpr bool HALVE = CL == 1 && ((NF == 16 && C == 1 && R == 2) || (NF == 32 && C == 2 && R == 2));
+    static constexpr long long HALF_MAX = !HALVE ? 0 : FL ? (NF == 16 ? 456 : 304) : (NF == 16 ? 912 : 456);
     template <bool CPL>
-    using shape = Shape<NF, C, ON ? R / 2 : R, CL, CPL, FL, ON ? 2 : 1>;
+    using half = Shape<NF, C, HALVE ? R / 2 : R, CL, CPL, FL, HALVE ? 2 : 1, true>;
+    // The fluctuation state has a build of the full shape with the registers of 8
+    // warps between the two, for as many samples as those are: us, with 16 warps /
+    // with 8: 64^2 x 256 steps coupled, 100 samples 549 / 434; 32^2 x 64, 457 138 / 116.
+    static constexpr long long FEW_MAX = !FL ? 0 : NF == 64 ? 152 : NF == 32 ? 608 : 0;
+    template <bool CPL>
+    using few = Shape<NF, C, R, CL, CPL, FL, 1, true>;
 };
 
 template <int NF, int C, int R, int CL, bool FL>
 cudaError_t variant_info_fn(bool coupled, int stride, VariantInfo* vi) {
     using SP = Split<NF, C, R, CL, FL>;
-    if constexpr (SP::ON) {
-        // the few-sample shape's launch attributes (its slots are the full shape's)
-        VariantInfo few{};
-        const cudaError_t e = coupled ? Kern<typename SP::template shape<true>>::info(stride, &few)
-                                      : Kern<typename SP::template shape<false>>::info(stride, &few);
-        if (e != cudaSuccess) return e;
+    // the launch attributes of the few-sample shapes (their slots are the full shape's)
+    VariantInfo other{};
+    cudaError_t e = cudaSuccess;
+    if constexpr (SP::HALF_MAX > 0) {
+        e = coupled ? Kern<typename SP::template half<true>>::info(stride, &other)
+                    : Kern<typename SP::template half<false>>::info(stride, &other);
     }
+    if constexpr (SP::FEW_MAX > 0) {
+        if (e == cudaSuccess)
+            e = coupled ? Kern<typename SP::template few<true>>::info(stride, &other)
+                        : Kern<typename SP::template few<false>>::info(stride, &other);
+    }
+    if (e != cudaSuccess) return e;
     return coupled ? Kern<Shape<NF, C, R, CL, true, FL>>::info(stride, vi)
                    : Kern<Shape<NF, C, R, CL, false, FL>>::info(stride, vi);
 }
@@ -995,13 +1009,18 @@ cudaError_t variant_info_fn(bool coupled, int stride, VariantInfo* vi) {
 template <int NF, int C, int R, int CL, bool FL>
 cudaError_t variant_launch_fn(bool coupled, const KArgs& a, int n_ctas, cudaStream_t st, int priority) {
     using SP = Split<NF, C, R, CL, FL>;
-    if constexpr (SP::ON) {
+    if constexpr (SP::HALF_MAX > 0) {
         // one CTA per sample slot, the same slots
-        if (a.count <= SP::MAX_COUNT) {
+        if (a.count <= SP::HALF_MAX) {
             const int n_slots = n_ctas * Shape<NF, C, R, CL, true, FL>::SLOTS_PER_CTA;
-            return coupled ? Kern<typename SP::template shape<true>>::launch(a, n_slots, st, priority)
-                           : Kern<typename SP::template shape<false>>::launch(a, n_slots, st, priority);
+            return coupled ? Kern<typename SP::template half<true>>::launch(a, n_slots, st, priority)
+                           : Kern<typename SP::template half<false>>::launch(a, n_slots, st, priority);
         }
+    }
+    if constexpr (SP::FEW_MAX > 0) {
+        if (a.count <= SP::FEW_MAX)
+            return coupled ? Kern<typename SP::template few<true>>::launch(a, n_ctas, st, priority)
+                           : Kern<typename SP::template few<false>>::launch(a, n_ctas, st, priority);
     }
     return coupled ? Kern<Shape<NF, C, R, CL, true, FL>>::launch(a, n_ctas, st, priority)
                    : Kern<Shape<NF, C, R, CL, false, FL>>::launch(a, n_ctas, st, priority);

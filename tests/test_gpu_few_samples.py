@@ -51,6 +51,23 @@ def test_few_sample_shape_gives_the_same_samples(dk, n0, level, mc, most, four):
             np.testing.assert_allclose(sums[2], dp.sum(), rtol=1e-9, atol=1e-9 * np.abs(dp).sum())
 
 
+@pytest.mark.parametrize("level,mosts", [(2, (456,)), (3, (304, 608)), (4, (152,))])
+@pytest.mark.parametrize("mc", [False, True])
+def test_few_samples_of_the_fluctuation_state(dk, level, mosts, mc):
+    """16^2, 32^2 and 64^2 about the noise-free path: the shapes for few samples on
+    both sides of each size where one ends, by the same measure."""
+    wl = W.get("paper_reg").with_(L_max=level)
+    with dk.Context.from_workload(wl) as ctx:
+        assert ctx.level_info(level).n == 4 << level
+        _, big = _run(ctx, dk, level, mc, 700)
+        scale = np.sqrt(np.mean(big ** 2, axis=0))
+        for most in mosts:
+            for count in (most, most + 1):
+                sums, samp = _run(ctx, dk, level, mc, count)
+                assert np.max(np.abs(samp - big[:count]) / np.maximum(scale, 1e-300)) <= 1e3 * 7 * 2.0 ** -53
+                assert int(sums[0]) == count and sums[1] == 0.0
+
+
 @pytest.mark.parametrize("name,mc", [("fourier6_54", False), ("fourier6_54", True), ("paper_reg_fourier", False)])
 def test_few_samples_of_the_18_grid(dk, name, mc):
     """18^2 Fourier level, absolute and fluctuation state: one and two rows of cells
