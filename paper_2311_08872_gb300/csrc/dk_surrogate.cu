@@ -116,6 +116,8 @@ __global__ void direct_feature_kernel(const FeatArgs a) {
 // Output layer forward: y[b][o] = H3[b] . w4[o] + b4[o], o < KO (one warp per row).
 __global__ void out_forward_kernel(const __nv_bfloat16* H, const float* w, const float* b, int B, int K, int KO,
                                    float* y) {
+    launch_dependents();
+    wait_previous_grid();
     const int row = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row >= B) return;
@@ -194,6 +196,8 @@ __device__ __forceinline__ void unpack8(const uint4& u, float (&v)[8]) {
 __global__ void __launch_bounds__(256) out_backward_kernel(const float* y, const float* t, const __nv_bfloat16* H,
                                                            const float* w, int B, int K, int KO, __nv_bfloat16* dH,
                                                            float* dw, float* db, double* loss) {
+    launch_dependents();
+    wait_previous_grid();
     const int tid = threadIdx.x, groups = K / 8;
     const float scale = static_cast<float>(B);
     const int n_el = static_cast<int>(((long long)B * groups + 255) / 256);
@@ -263,6 +267,8 @@ struct PrepArgs {
     int B, N;
 };
 __global__ void __launch_bounds__(256) layer_prep_kernel(const PrepArgs a) {
+    launch_dependents();
+    wait_previous_grid();
     __shared__ __nv_bfloat16 sh[32][33];
     int blk = blockIdx.x;
 #pragma unroll
@@ -300,6 +306,8 @@ __global__ void __launch_bounds__(256) layer_prep_kernel(const PrepArgs a) {
 
 // FP32 to BF16, round to nearest even.
 __global__ void to_bf16_kernel(const float* x, long long n, __nv_bfloat16* y) {
+    launch_dependents();
+    wait_previous_grid();
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i < n) y[i] = __float2bfloat16_rn(x[i]);
 }
@@ -407,16 +415,14 @@ cudaError_t launch_direct_features(const FeatArgs& a, cudaStream_t st) {
 
 cudaError_t launch_out_forward(const __nv_bfloat16* H, const float* w, const float* b, int B, int K, int KO, float* y,
                                cudaStream_t st) {
-    out_forward_kernel<<<(B + 7) / 8, 256, 0, st>>>(H, w, b, B, K, KO, y);
-    return cudaGetLastError();
+    return launch_chained(out_forward_kernel, (B + 7) / 8, 256, 0, st, H, w, b, B, K, KO, y);
 }
 
 cudaError_t launch_out_backward(const float* y, const float* t, const __nv_bfloat16* H, const float* w, int B, int K,
                                 int KO, __nv_bfloat16* dH, float* dw, float* db, double* loss, cudaStream_t st) {
     if (K % 8) return cudaErrorInvalidValue;
     const long long blocks = ((long long)B * (K / 8) + 255) / 256 + KO * (K / 8) + KO + (loss ? 1 : 0);
-    out_backward_kernel<<<(unsigned)blocks, 256, 0, st>>>(y, t, H, w, B, K, KO, dH, dw, db, loss);
-    return cudaGetLastError();
+    return launch_chained(out_backward_kernel, (unsigned)blocks, 256, 0, st, y, t, H, w, B, K, KO, dH, dw, db, loss);
 }
 
 cudaError_t launch_layer_prep(const __nv_bfloat16* dH, __nv_bfloat16* dHt, const __nv_bfloat16* Hin, __nv_bfloat16* Hint,
@@ -429,13 +435,11 @@ cudaError_t launch_layer_prep(const __nv_bfloat16* dH, __nv_bfloat16* dHt, const
     a.t[1] = {Hin, Hint, B, K, ldt, tiles(B, K)};
     if (W) a.t[2] = {W, Wt, N, K, N, tiles(N, K)};
     a.X = dH; a.colsum = colsum; a.B = B; a.N = N;
-    layer_prep_kernel<<<a.t[0].tiles + a.t[1].tiles + a.t[2].tiles + N / 8, 256, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(layer_prep_kernel, a.t[0].tiles + a.t[1].tiles + a.t[2].tiles + N / 8, 256, 0, st, a);
 }
 
 cudaError_t launch_to_bf16(const float* x, long long n, __nv_bfloat16* y, cudaStream_t st) {
-    to_bf16_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x, n, y);
-    return cudaGetLastError();
+    return launch_chained(to_bf16_kernel, (unsigned)((n + 255) / 256), 256, 0, st, x, n, y);
 }
 
 cudaError_t launch_adam(float* theta, const float* grad, float* m1, float* m2, int P, float lr, float b1, float b2,

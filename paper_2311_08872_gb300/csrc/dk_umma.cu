@@ -25,6 +25,7 @@
 #include <cstdint>
 #include <mutex>
 
+#include "dk_device.cuh"
 #include "dk_kernels.h"
 
 namespace dk {
@@ -152,6 +153,7 @@ __global__ void __launch_bounds__(128, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = tile % p.tiles_m * kTM;
     const int ktiles = (g.K + kTK - 1) / kTK;
+    launch_dependents();
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -172,6 +174,7 @@ __global__ void __launch_bounds__(128, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
+    wait_previous_grid();   // barriers and tensor memory are set up while the kernel before ends
 
     if (warp == 0 && lane == 0) {
         // producer: TMA loads of the K tiles into the stage ring
@@ -341,8 +344,8 @@ cudaError_t umma_launch(const GemmArgs* g, int count, unsigned* err, cudaStream_
             !encode_kmajor(&p[i].B, g[i].B, g[i].N, g[i].K, g[i].sbn, BN))
             return cudaErrorInvalidValue;
     }
-    umma_gemm_kernel<BN, STAGES><<<p[0].tiles + p[1].tiles, 128, umma_smem_bytes<BN, STAGES>(), st>>>(p[0], p[1], err);
-    return cudaGetLastError();
+    return launch_chained(umma_gemm_kernel<BN, STAGES>, p[0].tiles + p[1].tiles, 128, umma_smem_bytes<BN, STAGES>(), st,
+                          p[0], p[1], err);
 }
 
 }  // namespace
@@ -368,7 +371,7 @@ cudaError_t launch_gemm_tc(const GemmArgs* g, int count, unsigned* err, cudaStre
     // one wave is full: all columns of a row tile in one CTA read A once, two
     // stages (99 KB) let two CTAs share an SM.  256-column tiles with two stages
     // for every size, and one product a launch: part of the 520 us that a gradient
-    // of 1024 rows took, 138 now.
+    // of 1024 rows took, 127 now.
     if (n > 64 && tiles_m * 4 <= 152) return umma_launch<64, 8>(g, count, err, st);
     return n <= 32 ? umma_launch<32, 8>(g, count, err, st) : n <= 64 ? umma_launch<64, 8>(g, count, err, st)
          : n <= 128 ? umma_launch<128, 2>(g, count, err, st) : umma_launch<256, 2>(g, count, err, st);
