@@ -56,22 +56,22 @@ BAND_SOURCES = ("dk_band.cu", "dk_device.cuh")
 # Theta-scheme kernel (implicit diffusion weight b0 > 0): thread instructions
 # per fine cell-step (coupled, coarse work included) of the 64^2 coupled
 # launch at b0 = 1/2, tau/h^2 = 0.85 (14 Chebyshev steps per solve), from its
-# ncu --set full capture (smsp__inst_executed x 32 / fine cell-steps); valid
+# ncu capture (smsp__inst_executed x 32 / fine cell-steps); valid
 # under the recorded hash of its sources.  Bound by instruction issue.
 THETA_KERNEL_INSTR = {"kernel": "theta_kernel n=64 coupled=True b0=0.5 chebyshev_steps=14",
-                      "instructions_per_fine_cell_step": 580.6, "sources_sha256_16": "e8dc915d7d236c06"}
+                      "instructions_per_fine_cell_step": 323.4, "sources_sha256_16": "cf31327dc492abb0"}
 THETA_SOURCES = ("dk_theta.cu", "dk_device.cuh")
 # Fourier-coupled kernel: thread instructions per cell-step (fine and coarse
-# cell-steps) of the 54^2 coupled launch, from its ncu --set full capture;
+# cell-steps) of the 54^2 coupled launch, from its ncu capture;
 # valid under the recorded hash of its sources.
 FOURIER_KERNEL_INSTR = {"kernel": "fourier_kernel n=54 coupled=True",
-                        "instructions_per_cell_step": 94.6, "sources_sha256_16": "f3dd0738e5d2295f"}
+                        "instructions_per_cell_step": 69.4, "sources_sha256_16": "8affd0c0e50322dd"}
 FOURIER_SOURCES = ("dk_fourier.cu", "dk_device.cuh")
 # The 162^2 Fourier level on 6-CTA clusters: thread instructions per cell-step
-# (fine and coarse cell-steps) of the coupled launch of 144 samples, from its
+# (fine and coarse cell-steps) of the coupled launch of 24 samples, from its
 # ncu capture; valid under the recorded hash of its sources.
 FOURIER_CLUSTER_KERNEL_INSTR = {"kernel": "fourier_cluster_kernel n=162 coupled=True",
-                                "instructions_per_cell_step": 106.7, "sources_sha256_16": "9d8da938f719df45"}
+                                "instructions_per_cell_step": 76.4, "sources_sha256_16": "f87888717840f1c7"}
 FOURIER_CLUSTER_SOURCES = ("dk_fourier_cluster.cu", "dk_device.cuh")
 
 
@@ -161,8 +161,8 @@ def streamed_stencil(stream):
 
 def theta_scheme(stream):
     """The theta-scheme kernel on the finest level of the Crank--Nicolson
-    workload (64^2 coupled with 32^2, b0 = 1/2, tau/h^2 = 0.85): 32 waves of one
-    sample per SM, CUDA events on the launching stream, against the
+    workload (64^2 coupled with 32^2, b0 = 1/2, tau/h^2 = 0.85): 16 waves of two
+    samples per SM, CUDA events on the launching stream, against the
     instruction-issue roofline."""
     import torch
     from paper_2311_08872_gb300 import mlmc_dk, workloads
@@ -196,7 +196,7 @@ def theta_scheme(stream):
 
 def fourier_coupling(stream):
     """The Fourier-coupled kernel on the finest level of fourier6_54 (54^2
-    coupled with 18^2, ratio 3): 32 waves of one sample per SM, CUDA events;
+    coupled with 18^2, ratio 3): 16 waves of two samples per SM, CUDA events;
     and the 162^2 level of fourier6_162 (coupled with 54^2) on its cluster
     kernel, 144 samples."""
     import torch
