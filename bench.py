@@ -59,7 +59,7 @@ BAND_SOURCES = ("dk_band.cu", "dk_device.cuh")
 # ncu capture (smsp__inst_executed x 32 / fine cell-steps); valid
 # under the recorded hash of its sources.  Bound by instruction issue.
 THETA_KERNEL_INSTR = {"kernel": "theta_kernel n=64 coupled=True b0=0.5 chebyshev_steps=14",
-                      "instructions_per_fine_cell_step": 323.4, "sources_sha256_16": "cf31327dc492abb0"}
+                      "instructions_per_fine_cell_step": 323.4, "sources_sha256_16": "70be40720f6160da"}
 THETA_SOURCES = ("dk_theta.cu", "dk_device.cuh")
 # Fourier-coupled kernel: thread instructions per cell-step (fine and coarse
 # cell-steps) of the 54^2 coupled launch, from its ncu capture;

@@ -44,7 +44,8 @@
 // message n + 3, which that warp sent after the CTA barriers of its exchanges
 // n + 1 and n + 2, before which it read message n.  (Two slots are not enough:
 // message n + 1 need not depend on message n, as between the coarse and the next
-// fine step, and nothing else orders that read before it.)  Every wait is bounded: after kMbarPolls polls it records kErrTimeout, and the CTA waits no
+// fine step, and nothing else orders that read before it.)  Every wait is
+// bounded: after kMbarPolls polls it records kErrTimeout, and the thread waits no
 // more.
 //
 // Bound by instruction issue and latency: 9 packed operations per cell and iteration
