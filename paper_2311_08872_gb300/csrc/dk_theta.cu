@@ -13,7 +13,9 @@
 // transfers G_r(x) + G_r(x + e_r) of the central difference), and H commutes
 // with every periodic difference operator, so the increment is the backward
 // difference of H F_r = F_r + u_r with (I + alpha L) u_r = -alpha L F_r.
-// F_r is exact in 32/64-bit fixed point as in the explicit kernels; only the
+// F_r is exact in fixed point as in the explicit kernels, in 32 bits on the fine
+// grid (a flux beyond is a range error) and in 64 on the coarse one, where it may
+// leave 32 bits as long as the corrected flux does not; only the
 // correction u_r is computed in FP32, by K steps of Chebyshev iteration on the
 // spectrum [1, 1 + 8 alpha] of I + alpha L (K fixed on the host from the
 // Chebyshev error bound), and rounded once.  Adding the integer face fluxes
@@ -288,12 +290,14 @@ __device__ __forceinline__ void neighbours(f32x2 (&a)[R][C], Exchange<S>& x, F&&
 
 // One theta step of an R x C block of a periodic grid of LPR C columns (the
 // fine grid, or the coarse one with COARSE: the four neighbours are added in
-// another order there, and in one CTA the recurrence rounds its other product).
+// another order there, in one CTA the recurrence rounds its other product, and
+// the face fluxes have 64 bits).
 template <int R, int C, bool COARSE, class S>
 __device__ __forceinline__ void theta_step(int32_t (&q)[R][C], const int32_t (&G1)[R][C], const int32_t (&G2)[R][C],
                                            long long A, const TArgs& t, unsigned& bad, Exchange<S>& x) {
     // ---- exact face fluxes across the lower and the right edge of every cell
-    int32_t F1[R][C], F2[R][C];
+    using Flux = std::conditional_t<COARSE, long long, int32_t>;
+    Flux F1[R][C], F2[R][C];
     {
         f32x2 top[C], bot[C], up[C], dn[C];
 #pragma unroll
@@ -305,8 +309,8 @@ __device__ __forceinline__ void theta_step(int32_t (&q)[R][C], const int32_t (&G
         x.template collect<C>(up, dn);
         const auto face = [&](int32_t near, int32_t far, int32_t gn, int32_t gf) {
             const long long f = (long long)edge_flux64(A, far - near) + gn + gf;
-            bad |= (unsigned)(f != (long long)(int32_t)f);
-            return static_cast<int32_t>(f);
+            if constexpr (!COARSE) bad |= (unsigned)(f != (long long)(int32_t)f);
+            return static_cast<Flux>(f);
         };
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -333,7 +337,24 @@ __device__ __forceinline__ void theta_step(int32_t (&q)[R][C], const int32_t (&G
         for (int r = 0; r < R; ++r)
 #pragma unroll
             for (int c = 0; c < C; ++c)
-                d[r][c] = pack2(static_cast<float>(F1[r][c]), static_cast<float>(F2[r][c]));
+                d[r][c] = pack2(static_cast<float>(static_cast<int32_t>(F1[r][c])),
+                                static_cast<float>(static_cast<int32_t>(F2[r][c])));
+        if constexpr (COARSE) {
+            // (the conversion from 64 bits, like the one to 64 bits below, is the slow one)
+            bool wide = false;
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < C; ++c)
+                    wide |= (F1[r][c] != (int32_t)F1[r][c]) | (F2[r][c] != (int32_t)F2[r][c]);
+            if (wide) {
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int c = 0; c < C; ++c)
+                        d[r][c] = pack2(static_cast<float>(F1[r][c]), static_cast<float>(F2[r][c]));
+            }
+        }
         neighbours<R, C, S>(d, x, [&](int r, int c, f32x2 up, f32x2 dn, f32x2 l, f32x2 rt) {
             f32x2 v = mul2(pack2(4.f, 4.f), d[r][c]);
             if constexpr (COARSE) v = fma2(rt, minus1, fma2(l, minus1, fma2(dn, minus1, fma2(up, minus1, v))));
@@ -380,6 +401,7 @@ __device__ __forceinline__ void theta_step(int32_t (&q)[R][C], const int32_t (&G
     for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int c = 0; c < C; ++c) big = fmaxf(big, fmaxf(fabsf(lo2(u[r][c])), fabsf(hi2(u[r][c]))));
+    int32_t H1[R][C], H2[R][C];
     const auto correct = [&](auto round) {
 #pragma unroll
         for (int r = 0; r < R; ++r)
@@ -388,8 +410,8 @@ __device__ __forceinline__ void theta_step(int32_t (&q)[R][C], const int32_t (&G
                 const long long h1 = (long long)F1[r][c] + round(lo2(u[r][c]));
                 const long long h2 = (long long)F2[r][c] + round(hi2(u[r][c]));
                 bad |= (unsigned)((h1 != (long long)(int32_t)h1) | (h2 != (long long)(int32_t)h2));
-                F1[r][c] = static_cast<int32_t>(h1);
-                F2[r][c] = static_cast<int32_t>(h2);
+                H1[r][c] = static_cast<int32_t>(h1);
+                H2[r][c] = static_cast<int32_t>(h2);
             }
     };
     if (big < 2147483648.f) correct([](float v) { return (long long)__float2int_rn(v); });
@@ -397,18 +419,18 @@ __device__ __forceinline__ void theta_step(int32_t (&q)[R][C], const int32_t (&G
     f32x2 top[C], bot[C], up[C], dn[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-        top[c] = pack2i(F1[0][c], 0);
-        bot[c] = pack2i(F1[R - 1][c], 0);
+        top[c] = pack2i(H1[0][c], 0);
+        bot[c] = pack2i(H1[R - 1][c], 0);
     }
     x.template publish<C>(top, bot);
     x.template collect<C>(up, dn);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int32_t hl = x.left(F2[r][C - 1]);
+        const int32_t hl = x.left(H2[r][C - 1]);
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-            const int32_t ha = r > 0 ? F1[r > 0 ? r - 1 : 0][c] : lo2i(up[c]), hb = c > 0 ? F2[r][c > 0 ? c - 1 : 0] : hl;
-            const long long v = (long long)q[r][c] + ((long long)F1[r][c] - ha) + ((long long)F2[r][c] - hb);
+            const int32_t ha = r > 0 ? H1[r > 0 ? r - 1 : 0][c] : lo2i(up[c]), hb = c > 0 ? H2[r][c > 0 ? c - 1 : 0] : hl;
+            const long long v = (long long)q[r][c] + ((long long)H1[r][c] - ha) + ((long long)H2[r][c] - hb);
             bad |= (unsigned)((v >= (1LL << 30)) | (v <= -(1LL << 30)));
             q[r][c] = static_cast<int32_t>(v);
         }
