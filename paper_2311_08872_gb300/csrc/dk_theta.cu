@@ -115,6 +115,13 @@ __device__ __forceinline__ f32x2 pack2i(int32_t lo, int32_t hi) { return pack2(a
 __device__ __forceinline__ int32_t lo2i(f32x2 v) { return as_i(lo2(v)); }
 __device__ __forceinline__ int32_t hi2i(f32x2 v) { return as_i(hi2(v)); }
 
+// The larger of two values, NaN if one is (fmaxf drops it).
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
 constexpr unsigned kMbarPolls = 1u << 22;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -395,12 +402,12 @@ __device__ __forceinline__ void theta_step(int32_t (&q)[R][C], const int32_t (&G
     // ---- corrected fluxes, rounded once; the update adds integer face fluxes.
     // Corrections fit 32 bits in every sane state: the conversion to 64 bits, which
     // runs on the FP64 pipe (two per cell were a seventh of the step), is kept for a
-    // block that has one beyond.
+    // block that has one beyond, or a NaN, which that conversion makes a range error.
     float big = 0.f;
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int c = 0; c < C; ++c) big = fmaxf(big, fmaxf(fabsf(lo2(u[r][c])), fabsf(hi2(u[r][c]))));
+        for (int c = 0; c < C; ++c) big = max_nan(big, max_nan(fabsf(lo2(u[r][c])), fabsf(hi2(u[r][c]))));
     int32_t H1[R][C], H2[R][C];
     const auto correct = [&](auto round) {
 #pragma unroll
