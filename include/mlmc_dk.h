@@ -78,7 +78,7 @@ extern "C" {
 #define MLMC_DK_ERR_RANGE (-3)       /* |rho| reached 2^(30-S_l): the level's fixed-point range */
 #define MLMC_DK_ERR_UNSUPPORTED (-4) /* grid size without a kernel variant */
 #define MLMC_DK_ERR_STATE (-5)       /* checkpoint buffer does not match */
-#define MLMC_DK_ERR_TIMEOUT (-6)     /* a kernel's bounded wait for another CTA's progress gave up (band, persistent streamed and tensor-core GEMM kernels) */
+#define MLMC_DK_ERR_TIMEOUT (-6)     /* a kernel's bounded wait for another CTA's progress gave up (band, persistent streamed, theta-scheme cluster and tensor-core GEMM kernels) */
 
 #define MLMC_DK_MAX_LEVELS 16
 #define MLMC_DK_MAX_OBS 4
@@ -327,7 +327,8 @@ int mlmc_dk_run_batch(mlmc_dk_ctx* ctx, const int64_t* counts, uint64_t seed, ml
  *     keep fewer samples in flight than mlmc_dk_run_level_dev.  Per-sample
  *     values are identical; the sums agree up to FP64 summation order.
  *   - err_dev: NULL, or a caller-owned device word that receives the range
- *     error bit (1) by atomic OR; with NULL, range errors are not reported.
+ *     error bit (1) and, on theta-scheme cluster levels, the timeout bit (2) by
+ *     atomic OR; with NULL, they are not reported.
  * Outputs and alignment as mlmc_dk_run_level_dev; asynchronous on cuda_stream
  * (NULL: the context's stream); the context is not modified. */
 int mlmc_dk_run_level_static(const mlmc_dk_ctx* ctx, int32_t level, int32_t stream_tag, int64_t first_sample,
@@ -351,6 +352,16 @@ int mlmc_dk_band_wait_test(mlmc_dk_ctx* ctx, int32_t level, uint32_t polls, int3
  * at its next item, and the call returns MLMC_DK_ERR_TIMEOUT; the context
  * stays usable.  MLMC_DK_ERR_UNSUPPORTED when the level is not streamed. */
 int mlmc_dk_stream_wait_test(mlmc_dk_ctx* ctx, int32_t level, uint32_t polls, int32_t stall_tile);
+
+/* Failure-detection test of the theta-scheme cluster kernel's bounded waits (the
+ * paper has no counterpart): `n_samples` coupled samples of `level` over at most
+ * 16 fine steps, with every wait limited to `polls` polls and the first CTA of
+ * every cluster stopping before fine step `stall_step`, so that its neighbours'
+ * waits run out.  The kernel records the timeout, every CTA stops stepping, and
+ * the call returns MLMC_DK_ERR_TIMEOUT; the context stays usable.
+ * MLMC_DK_ERR_UNSUPPORTED when the level's samples do not run on clusters. */
+int mlmc_dk_theta_wait_test(mlmc_dk_ctx* ctx, int32_t level, int64_t n_samples, uint32_t polls,
+                            int32_t stall_step);
 
 /* Algorithm 1 (Section 7.1): start at L = L_start with `pilot` samples on
  * levels 0..L; repeat {run the missing samples (all levels of a round at once

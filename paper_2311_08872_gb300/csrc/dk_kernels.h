@@ -178,6 +178,10 @@ struct TArgs {
     long long Af64, Ac64;      // round(tau / (2 h^2) 2^32) of the fine / coarse grid (64-bit: tau/h^2 may exceed 1)
     const double* phif64;      // FP64 test functions [n_obs][n^2] / [n_obs][(n/2)^2]
     const double* phic64;
+    // failure-detection test of the clusters only: poll limit of every wait for a
+    // neighbour's message, and the fine step before which CTA 0 of every cluster stops
+    unsigned wait_polls;
+    int stall_step;
 };
 bool theta_supported(int n);
 cudaError_t theta_variant_info(int n, bool coupled, int slot_stride, VariantInfo* out);
@@ -185,6 +189,8 @@ cudaError_t theta_variant_info(int n, bool coupled, int slot_stride, VariantInfo
 // n_ctas * slots_per_cta * slot_stride doubles.
 cudaError_t launch_theta(int n, bool coupled, const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t stream,
                          int priority = 0);
+// Failure-detection test: a coupled 128 x 128 batch with t.wait_polls and t.stall_step.
+cudaError_t launch_theta_wait_test(const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t stream);
 
 // ---- Fourier coupling (Section 3.1): grids 6, 18, 54 (h ratio 3, tau ratio 9)
 struct FArgs {

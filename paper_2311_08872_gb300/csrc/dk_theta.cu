@@ -47,8 +47,11 @@
 // n + 1 and n + 2, before which it read message n.  (Two slots are not enough:
 // message n + 1 need not depend on message n, as between the coarse and the next
 // fine step, and nothing else orders that read before it.)  Every wait is
-// bounded: after kMbarPolls polls it records kErrTimeout, and the thread waits no
-// more.
+// bounded: a thread whose message does not come within kMbarPolls polls records
+// kErrTimeout and waits no more, arms no slot any more (an arrival on a slot whose
+// last message is still out would be one too many), and the CTA stops stepping at
+// the next fine step, for all its samples; the neighbours' waits for it run out in
+// turn.  It ends only when what they sent in that last step has had time to land.
 //
 // Bound by instruction issue and latency: 9 packed operations per cell and iteration
 // take two cycles each on the FP32 pipe, and an iteration ends in a barrier.
@@ -72,11 +75,14 @@ namespace cg = cooperative_groups;
 constexpr unsigned kFullMask = 0xffffffffu;
 constexpr int kRed = 2 * kMaxObs + 2;   // reduced values per sample
 
-// Shapes: fine block R x C per thread, CL CTAs per sample.
-template <int N_, bool DENSE_>
+// Shapes: fine block R x C per thread, CL CTAs per sample.  (A poll limit and a
+// stopping step read at run time cost the 128^2 build 100 to 400 bytes of spills and
+// a tenth to a quarter of its speed: only the test's build has them.)
+template <int N_, bool DENSE_, bool TEST_ = false>
 struct TShape {
     static constexpr int N = N_, NC = N / 2;
     static constexpr bool DENSE = DENSE_;
+    static constexpr bool TEST = TEST_;                    // build of the failure-detection test (TArgs)
     static constexpr bool SMALL = N < 32 || (N == 32 && !DENSE);
     static constexpr int R = SMALL ? 2 : 4, C = N >= 16 && !(N == 32 && !DENSE) ? 4 : 2;
     static constexpr int CL = N >= 128 ? 4 : 1;
@@ -93,11 +99,11 @@ struct TShape {
     static_assert(LPR <= 32 && (SPB == 1 || TPS <= 32) && (CL == 1 || LPR == 32), "block layout");
     // per sample: two buffers of the blocks' top and bottom rows, two words a cell;
     // in a cluster also four message slots for the rows above and below the band,
-    // and their mbarriers
+    // their mbarriers, and two words that tell of a wait that ran out
     static constexpr int BUF = 4 * N * NBR;                // words of one buffer
     static constexpr int SLOT = 4 * N;                     // words of one message slot (both sides)
     static constexpr int WORDS = 2 * BUF + (CL > 1 ? 4 * SLOT : 0);
-    static constexpr size_t SAMPLE_BYTES = sizeof(int32_t) * WORDS + (CL > 1 ? 8 * sizeof(uint64_t) : 0);
+    static constexpr size_t SAMPLE_BYTES = sizeof(int32_t) * WORDS + (CL > 1 ? 10 * sizeof(uint64_t) : 0);
     static size_t smem(int slot_stride) {
         return SAMPLE_BYTES * SPB + sizeof(double) * ((THREADS + 31) / 32) * kRed + sizeof(double) * kRed +
                sizeof(double) * SPB * slot_stride;
@@ -122,7 +128,7 @@ __device__ __forceinline__ float max_nan(float a, float b) {
     return r;
 }
 
-constexpr unsigned kMbarPolls = 1u << 22;
+constexpr unsigned kMbarPolls = 1u << 22;   // polls of one wait before it gives up
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -138,11 +144,12 @@ struct Exchange {
     uint64_t* bars = nullptr;              // [up, dn][4]
     uint32_t rup = 0, rdn = 0;             // shared::cluster address of `buf` in the CTA above / below
     unsigned* err;
+    unsigned polls;                        // limit of every wait (TEST)
     int br, bc;
     unsigned n = 0;
     bool dead = false;
-    __device__ __forceinline__ Exchange(float* b, int br_, int bc_, int rank, unsigned* err_)
-        : buf(b), err(err_), br(br_), bc(bc_) {
+    __device__ __forceinline__ Exchange(float* b, int br_, int bc_, int rank, unsigned* err_, unsigned polls_)
+        : buf(b), err(err_), polls(polls_), br(br_), bc(bc_) {
         if constexpr (S::CL > 1) {
             bars = reinterpret_cast<uint64_t*>(b + S::WORDS);
             rup = mapa(smem_u32(b), (rank + S::CL - 1) % S::CL);
@@ -150,6 +157,7 @@ struct Exchange {
             if (threadIdx.x == 0) {
                 for (int i = 0; i < 8; ++i)
                     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bars + i)) : "memory");
+                gone()[0] = gone()[1] = 0;
                 asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             }
         }
@@ -207,15 +215,21 @@ struct Exchange {
             }
         }
     }
+    // Words that a thread whose wait ran out sets, word e % 2 at exchange e.
+    __device__ __forceinline__ volatile int* gone() const { return reinterpret_cast<volatile int*>(bars + 8); }
+    // Whether to stop before exchange n, the same for the whole CTA: word n % 2 was last
+    // set at exchange n - 2 or before, ahead of the barrier of exchange n - 1, and is
+    // not set again before that of exchange n.
+    __device__ __forceinline__ bool stopped() const { return S::CL > 1 && gone()[n & 1]; }
     // The message of this exchange on side `side` (all lanes of the warp).
     template <int W>
     __device__ __forceinline__ void receive(int side) {
         const uint32_t bar = smem_u32(bars + 4 * side + (n & 3));
-        if (bc == 0)
+        if (bc == 0 && !dead)
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(S::LPR * W * 8)
                          : "memory");
         const uint32_t parity = (n >> 2) & 1;
-        for (unsigned i = 0; i < kMbarPolls && !dead; ++i) {
+        for (unsigned i = 0; i < (S::TEST ? polls : kMbarPolls) && !dead; ++i) {
             uint32_t ok;
             asm volatile(
                 "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
@@ -224,8 +238,9 @@ struct Exchange {
                 : "memory");
             if (ok) return;
         }
+        if (!dead) atomicOr(err, kErrTimeout);
         dead = true;
-        atomicOr(err, kErrTimeout);
+        gone()[n & 1] = 1;
     }
     // Hand out the block's first and last row ...
     template <int W>
@@ -451,10 +466,10 @@ __device__ __forceinline__ void sample_barrier() {
     else __syncthreads();
 }
 
-template <int N, bool CPL, bool DENSE>
+template <int N, bool CPL, bool DENSE, bool TEST = false>
 __global__ void __launch_bounds__(TShape<N, DENSE>::THREADS, TShape<N, DENSE>::MIN_CTAS)
     theta_kernel(const KArgs a, const TArgs t) {
-    using S = TShape<N, DENSE>;
+    using S = TShape<N, DENSE, TEST>;
     constexpr int NC = S::NC, TPS = S::TPS, SPB = S::SPB, THREADS = S::THREADS, R = S::R, C = S::C, CL = S::CL;
     constexpr int RC = R / 2, CC = C / 2;       // coarse block
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -469,7 +484,7 @@ __global__ void __launch_bounds__(TShape<N, DENSE>::THREADS, TShape<N, DENSE>::M
 
     const int br = lt / S::LPR, bc = lt % S::LPR;
     const int i0 = (rank * S::NBR + br) * R, j0 = bc * C;   // the block's first fine cell
-    Exchange<S> x(reinterpret_cast<float*>(smem_raw + S::SAMPLE_BYTES * sl), br, bc, rank, a.err);
+    Exchange<S> x(reinterpret_cast<float*>(smem_raw + S::SAMPLE_BYTES * sl), br, bc, rank, a.err, t.wait_polls);
 
     const long long n_slots = (long long)gridDim.x * SPB / CL;
     const long long cta_slot0 = (long long)(blockIdx.x / CL) * SPB;
@@ -499,7 +514,8 @@ __global__ void __launch_bounds__(TShape<N, DENSE>::THREADS, TShape<N, DENSE>::M
                 qc[r][c] = CPL ? a.q0c[(i0 / 2 + r) * NC + j0 / 2 + c] : 0;
             }
 
-        for (int m = 0; m < a.M; ++m) {
+        const auto step = [&](int m) { return x.stopped() || (S::TEST && m == t.stall_step && rank == 0) ? a.M : m; };
+        for (int m = step(0); m < a.M; m = step(m + 1)) {
             {
                 // ---- noise of the fine block: Philox4x32-10 per horizontal cell pair, Box--Muller
                 int32_t G1[R][C], G2[R][C];
@@ -656,6 +672,13 @@ __global__ void __launch_bounds__(TShape<N, DENSE>::THREADS, TShape<N, DENSE>::M
         sample_barrier<S>();   // the reduction scratch is reused by the next sample
     }
     if (bad) atomicOr(a.err, kErrRange);
+    if constexpr (CL > 1) {
+        // after a timeout, in some CTA of the cluster: messages that nobody waited for may be
+        // on their way to this CTA (all sent before the cluster barrier above; about a
+        // microsecond): stay for a millisecond
+        if (ld_volatile(a.err) & kErrTimeout)
+            for (int i = 0; i < 1000; ++i) __nanosleep(1000);
+    }
 
     // ---- per-slot partial sums to global scratch, entry-major [stride][n_slots]
     __syncthreads();
@@ -734,14 +757,14 @@ cudaError_t prepare(int slot_stride, VariantInfo* out) {
     return cudaSuccess;
 }
 
-template <int N, bool CPL, bool DENSE>
+template <int N, bool CPL, bool DENSE, bool TEST = false>
 cudaError_t launch_build(const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t st, int priority) {
     using S = TShape<N, DENSE>;
     if (n_ctas % S::CL != 0) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     launch_config<S>(cfg, attr, n_ctas, a.slot_stride, st, priority);
-    return cudaLaunchKernelEx(&cfg, theta_kernel<N, CPL, DENSE>, a, t);
+    return cudaLaunchKernelEx(&cfg, theta_kernel<N, CPL, DENSE, TEST>, a, t);
 }
 
 template <int N, bool CPL>
@@ -777,6 +800,14 @@ cudaError_t theta_variant_info(int n, bool coupled, int slot_stride, VariantInfo
     cudaError_t e = cudaSuccess;
     for_grid(n, [&](auto N) { e = coupled ? prepare<N.value, true>(slot_stride, out) : prepare<N.value, false>(slot_stride, out); });
     return e;
+}
+
+cudaError_t launch_theta_wait_test(const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t st) {
+    if (t.K < 0 || t.K > kMaxCheb) return cudaErrorInvalidValue;
+    constexpr int N = 128;
+    static_assert(TShape<N, true>::SAMPLE_BYTES < 45000, "no shared-memory attribute needed");
+    return a.count > kFew<N> ? launch_build<N, true, true, true>(a, t, n_ctas, st, 0)
+                             : launch_build<N, true, false, true>(a, t, n_ctas, st, 0);
 }
 
 cudaError_t launch_theta(int n, bool coupled, const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t st,

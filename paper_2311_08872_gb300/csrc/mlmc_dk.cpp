@@ -415,6 +415,16 @@ int launch_band(mlmc_dk_ctx* c, int level, int stream_tag, int64_t first, int64_
     return MLMC_DK_OK;
 }
 
+dk::TArgs theta_args(const mlmc_dk_ctx* c, int level, bool coupled) {
+    const LevelTab& t = c->lv[level];
+    dk::TArgs ta = c->targs;
+    ta.Af64 = t.A64;
+    ta.Ac64 = coupled ? c->lv[level - 1].A64 : 0;
+    ta.phif64 = t.d_phi64;
+    ta.phic64 = coupled ? c->lv[level - 1].d_phi64 : nullptr;
+    return ta;
+}
+
 // The level's sample kernel: the theta-scheme kernel on a theta context, the
 // register-resident kernel variant in use otherwise.
 cudaError_t launch_main(const mlmc_dk_ctx* c, int level, bool coupled, const dk::KArgs& a, int n_ctas,
@@ -429,14 +439,7 @@ cudaError_t launch_main(const mlmc_dk_ctx* c, int level, bool coupled, const dk:
             return dk::launch_fourier_cluster(t.n, coupled, a, fa, n_ctas, st, priority);
         return dk::launch_fourier(t.n, coupled, a, fa, n_ctas, st, priority, c->fluct != 0);
     }
-    if (c->theta) {
-        dk::TArgs ta = c->targs;
-        ta.Af64 = t.A64;
-        ta.Ac64 = coupled ? c->lv[level - 1].A64 : 0;
-        ta.phif64 = t.d_phi64;
-        ta.phic64 = coupled ? c->lv[level - 1].d_phi64 : nullptr;
-        return dk::launch_theta(t.n, coupled, a, ta, n_ctas, st, priority);
-    }
+    if (c->theta) return dk::launch_theta(t.n, coupled, a, theta_args(c, level, coupled), n_ctas, st, priority);
     return dk::launch_level(t.n, coupled, t.sel[coupled ? 1 : 0], a, n_ctas, st, priority, c->fluct != 0);
 }
 
@@ -1219,6 +1222,27 @@ int mlmc_dk_band_wait_test(mlmc_dk_ctx* ctx, int32_t level, uint32_t polls, int3
     if (rc != MLMC_DK_OK) return rc;
     const cudaError_t e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "band_wait_test");
+    return check_device_error(ctx);
+}
+
+int mlmc_dk_theta_wait_test(mlmc_dk_ctx* ctx, int32_t level, int64_t n_samples, uint32_t polls, int32_t stall_step) {
+    if (!ctx) return fail(nullptr, MLMC_DK_ERR_INVALID, "null context");
+    if (level < 1 || level > ctx->L_max || n_samples < 1 || polls == 0 || stall_step < 0)
+        return fail(ctx, MLMC_DK_ERR_INVALID, "theta_wait_test: bad arguments");
+    const LevelTab& t = ctx->lv[level];
+    const dk::VariantInfo& vi = t.vi(true);
+    if (!ctx->theta || t.n != 128 || vi.cluster < 2)
+        return fail(ctx, MLMC_DK_ERR_UNSUPPORTED, "theta_wait_test: the level's samples do not run on clusters");
+    const int64_t groups = std::min<int64_t>(n_samples, vi.max_ctas / vi.cluster);
+    dk::KArgs a = make_args(ctx, level, 0, true, 0, n_samples, 0x7465, nullptr);
+    a.partials = ctx->d_partials;
+    a.M = std::min(a.M, 16);
+    dk::TArgs ta = theta_args(ctx, level, true);
+    ta.wait_polls = polls;
+    ta.stall_step = stall_step;
+    cudaError_t e = dk::launch_theta_wait_test(a, ta, (int)(groups * vi.cluster), ctx->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "theta_wait_test");
     return check_device_error(ctx);
 }
 

@@ -141,6 +141,7 @@ def lib() -> ctypes.CDLL:
                                          ctypes.c_int32, ROUND_FN, REDUCE_FN, vp, ctypes.POINTER(Result)]
         L.mlmc_dk_band_wait_test.argtypes = [vp, ctypes.c_int32, ctypes.c_uint32, ctypes.c_int32]
         L.mlmc_dk_stream_wait_test.argtypes = [vp, ctypes.c_int32, ctypes.c_uint32, ctypes.c_int32]
+        L.mlmc_dk_theta_wait_test.argtypes = [vp, ctypes.c_int32, ctypes.c_int64, ctypes.c_uint32, ctypes.c_int32]
         L.mlmc_dk_run_batch_dev.argtypes = [vp, ctypes.POINTER(ctypes.c_int64), ctypes.c_int64, ctypes.c_uint64,
                                             vp, vp]
         L.mlmc_dk_run_batch.argtypes = [vp, ctypes.POINTER(ctypes.c_int64), ctypes.c_uint64, ctypes.POINTER(LevelSums)]
@@ -365,6 +366,10 @@ class Context:
     def stream_wait_test(self, level: int, polls: int, stall_tile: int) -> int:
         """Failure-detection test of the persistent streamed kernel's bounded waits; returns the status code."""
         return lib().mlmc_dk_stream_wait_test(self._ctx, level, polls, stall_tile)
+
+    def theta_wait_test(self, level: int, n_samples: int, polls: int, stall_step: int) -> int:
+        """Failure-detection test of the theta-scheme cluster kernel's bounded waits; returns the status code."""
+        return lib().mlmc_dk_theta_wait_test(self._ctx, level, n_samples, polls, stall_step)
 
     def run_batch_dev(self, counts, first: int, seed: int, sums_ptr: int, stream: int = 0):
         """All levels concurrently (CUDA graph); sums_ptr: device double[L_max+1][sums_len]."""
