@@ -19,6 +19,10 @@ LIB = os.path.join(PKG, "libmlmc_dk.so")
 BUILD_DIR = os.path.join(ROOT, "_build")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
+# nvcc compresses a device image from about 10 MB on, which the level kernels
+# exceed; unpacking it took 11 ms of a process's first context (13.8 ms for one
+# 16^2 level, 2.5 without)
+FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--no-compress", "-Xcompiler", "-fPIC"]
 SOURCES = ["dk_kernels.cu", "dk_band.cu", "dk_stream.cu", "dk_surrogate.cu", "dk_umma.cu", "dk_theta.cu", "dk_fourier.cu", "dk_fourier_cluster.cu", "mlmc_dk.cpp"]
 HEADERS = ["dk_kernels.h", "dk_device.cuh"]
 
@@ -34,7 +38,7 @@ def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in SOURCES + HEADERS] + [os.path.join(INCLUDE, "mlmc_dk.h")]
+    deps = [os.path.join(CSRC, f) for f in SOURCES + HEADERS] + [os.path.join(INCLUDE, "mlmc_dk.h"), os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
@@ -43,7 +47,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         return LIB
     os.makedirs(BUILD_DIR, exist_ok=True)
     cc = nvcc()
-    common = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
+    common = ARCH + FLAGS + ["-I", INCLUDE, "-I", CSRC]
     if verbose:
         common += ["-Xptxas", "-v"]
     procs, objs = [], []
