@@ -653,7 +653,11 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB) level_kernel(const KArgs 
             for (int k = 0; k < kMaxObs; ++k) {
                 float sf = 0.f, sc = 0.f;
                 if (k < a.n_obs) {
-                    const auto project = [&]() {
+                    if constexpr (!CPL && CL == 1 && !S::WARP && FR * FC >= 16) {
+                        // (in place: within the lambda below, the registers of these shapes' step
+                        // loop are allocated worse: 32^2, 1000 x 103 steps 288 us so, 281 in place;
+                        // 64^2, 1151 x 208 2397 and 2345.  Coupled, cluster and small blocks are
+                        // the other way round, 64^2 coupled fluctuation state 434 and 480.)
 #pragma unroll
                         for (int r = 0; r < FR; ++r) {
                             int32_t qb[FC];
@@ -663,27 +667,39 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB) level_kernel(const KArgs 
 #pragma unroll
                             for (int c = 0; c < FC; ++c) sf = fmaf(__int2float_rn(q[r][c] - qb[c]), ph[c], sf);
                         }
-                        if constexpr (CPL) {
+                    } else {
+                        const auto project = [&]() {
 #pragma unroll
-                            for (int i = 0; i < R; ++i) {
-                                int32_t qb[C];
-                                float ph[C];
-                                load_row<C>(qb, a.qbc + (size_t)(crow0 + i) * NC + ccol0);
-                                load_row_f<C>(ph, a.phic + (size_t)k * NC * NC + (size_t)(crow0 + i) * NC + ccol0);
+                            for (int r = 0; r < FR; ++r) {
+                                int32_t qb[FC];
+                                float ph[FC];
+                                load_row<FC>(qb, a.qbf + (size_t)(row0 + r) * NF + col0);
+                                load_row_f<FC>(ph, a.phif + (size_t)k * NF * NF + (size_t)(row0 + r) * NF + col0);
 #pragma unroll
-                                for (int j = 0; j < C; ++j) sc = fmaf(__int2float_rn(qc[i][j] - qb[j]), ph[j], sc);
+                                for (int c = 0; c < FC; ++c) sf = fmaf(__int2float_rn(q[r][c] - qb[c]), ph[c], sf);
                             }
-                        }
-                    };
-                    project();
-                    if constexpr (S::CHAIN == 2) {
-                        // odd bands continue the sum of the band above, in the same warp
-                        const float uf = __shfl_up_sync(kFull, sf, LPB), uc = __shfl_up_sync(kFull, sc, LPB);
-                        sf = sc = 0.f;
-                        if (band & 1) {
-                            sf = uf;
-                            sc = uc;
-                            project();
+                            if constexpr (CPL) {
+#pragma unroll
+                                for (int i = 0; i < R; ++i) {
+                                    int32_t qb[C];
+                                    float ph[C];
+                                    load_row<C>(qb, a.qbc + (size_t)(crow0 + i) * NC + ccol0);
+                                    load_row_f<C>(ph, a.phic + (size_t)k * NC * NC + (size_t)(crow0 + i) * NC + ccol0);
+#pragma unroll
+                                    for (int j = 0; j < C; ++j) sc = fmaf(__int2float_rn(qc[i][j] - qb[j]), ph[j], sc);
+                                }
+                            }
+                        };
+                        project();
+                        if constexpr (S::CHAIN == 2) {
+                            // odd bands continue the sum of the band above, in the same warp
+                            const float uf = __shfl_up_sync(kFull, sf, LPB), uc = __shfl_up_sync(kFull, sc, LPB);
+                            sf = sc = 0.f;
+                            if (band & 1) {
+                                sf = uf;
+                                sc = uc;
+                                project();
+                            }
                         }
                     }
                 }
