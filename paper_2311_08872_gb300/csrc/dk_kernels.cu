@@ -409,6 +409,20 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB) level_kernel(const KArgs 
             // ---- rows of the block in order: noise, transfers, and the row's part of the update
             const bool cstep = CPL && ((m & 3) == 3);
             const int par = m & 1;
+            // the coarse path's noise-free row.  A sample in one warp loads it here, ahead of
+            // the noise: few samples wait for every load (8^2 x 640 steps, 256 samples: 291 us
+            // with scalar noise, whose loads the compiler moved up; packed 325 where it is
+            // used, 300 here; 20000 samples 2554, 2331, 2298).  The larger shapes need the
+            // registers: 64^2 x 256, 152 samples 435 there, 480 here.
+            constexpr bool kEarly = S::FLUCT && CPL && S::WARP;
+            float rbc[S::FLUCT && CPL ? R : 1][S::FLUCT && CPL ? C : 1];
+            if constexpr (kEarly) {
+                if (cstep) {
+#pragma unroll
+                    for (int i = 0; i < R; ++i)
+                        load_row_f<C>(rbc[i], a.rbc + (size_t)(m >> 2) * NC * NC + (size_t)(crow0 + i) * NC + ccol0);
+                }
+            }
             const f32x2 gf2 = pack2(a.gf, a.gf);
             int32_t G1[FR][FC], G2[FR][FC];
             int32_t pend[2][FC];      // change of the row in hand still to be added (parity of the row)
@@ -500,8 +514,7 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB) level_kernel(const KArgs 
             int32_t Gc1[R][C], Gc2[R][C];
             if constexpr (CPL) {
                 if (cstep) {
-                    float rbc[S::FLUCT ? R : 1][S::FLUCT ? C : 1];
-                    if constexpr (S::FLUCT) {
+                    if constexpr (S::FLUCT && !kEarly) {
 #pragma unroll
                         for (int i = 0; i < R; ++i)
                             load_row_f<C>(rbc[i], a.rbc + (size_t)(m >> 2) * NC * NC + (size_t)(crow0 + i) * NC + ccol0);
