@@ -58,7 +58,7 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kRedW = 2 * kMaxObs + 2;     // reduced values per sample
 constexpr int kMaxStride = 2 + kNSum * 10;  // largest slot stride (4 obs with products)
 
-template <int NF_, int C_, int R_, int CL_, bool COUPLED_, bool FLUCT_ = false, int CHAIN_ = 1, bool FEW_ = false>
+template <int NF_, int C_, int R_, int CL_, bool COUPLED_, bool FLUCT_ = false, int CHAIN_ = 1, bool SECOND_ = false>
 struct Shape {
     static constexpr int NF = NF_, C = C_, R = R_, CL = CL_;
     static constexpr bool COUPLED = COUPLED_;
@@ -68,6 +68,8 @@ struct Shape {
     // a lane's FP32 projection sums run on through the blocks of CHAIN bands, one
     // below the other: the sums of a shape with CHAIN times the rows per lane
     static constexpr int CHAIN = CHAIN_;
+    // the second build of a shape that has two (see Split)
+    static constexpr bool SECOND = SECOND_;
     static constexpr int NC = NF / 2;
     static constexpr int FR = 2 * R, FC = 2 * C;
     static constexpr int LPB = NC / C;            // lanes per band
@@ -79,32 +81,50 @@ struct Shape {
     static constexpr int BPC = WARP ? 1 : NB / CL;   // bands per CTA
     // How a step is laid out in the instruction stream (the arithmetic is the
     // same), by block size and registers per thread; measured, ms at the sizes
-    // given (coupled unless said otherwise):
+    // given (coupled unless said otherwise; "before": scalar FP32 noise, no bound on
+    // the registers):
     //   PIPE   the Philox rounds of the next two cell pairs run between the
     //          Box--Muller stages of the current two (FMA and ALU pipes under the
     //          XU pipe), and a row is updated as soon as its transfers are known.
-    //          It wants the registers of 8 to 12 warps per SM: one-CTA samples of
+    //          It wants the registers of 8 to 16 warps per SM: one-CTA samples of
     //          several warps (64^2, 1151 samples x 832 steps: 9.6, without 10.5,
-    //          scalar FP32 before 11.1; 32^2, 4630 x 208: 2.31, 2.52, 2.57) and
-    //          blocks of 32 cells (256^2, 59 x 1536: 19.8, 23.5, 22.8).  At 128
-    //          registers it spills and loses (128^2, 304 x 1664: 25.0, without 23.7).
+    //          before 11.1; 32^2, 4630 x 208: 2.31, 2.52, 2.57), of one warp with 16
+    //          cells a lane or a coupled path (16^2, 2 x 2 coarse cells a lane, 1000 x 52
+    //          plain: 0.055, without 0.068, before 0.068; 1 x 2 coupled, 10000 x 52:
+    //          0.35, 0.37, 0.37), and in clusters blocks of 32 cells (256^2, 59 x 1536:
+    //          19.8, 23.5, 22.8) or of one coarse row (128^2 by 4 CTAs, 304 x 64: 3.24,
+    //          without 3.83, before 3.54).  With 2 x 2 coarse cells at 128 registers it
+    //          spills and loses (128^2, 304 x 1664: 25.0, without 23.7).
     //   REDRAW the sample's Philox counter word is opaque to the compiler, which
     //          then does not keep the step-independent parts of the first rounds in
     //          registers, where those would spill (128^2: 22.7 with, 23.7 without,
     //          25.1 before; 256^2: 19.8 with, 23.0 without).  Fine-only 128^2 does not
-    //          spill (40 samples x 384: 1.32 with, 1.27 without, 1.31 before).
+    //          spill (40 samples x 384: 1.32 with, 1.27 without, 1.31 before).  One
+    //          coarse row: only plain with 4 columns (256^2, 59 x 102: 3.13 with, 3.49
+    //          without, 3.72 before).
     //   The fluctuation state needs its mean-field rows in registers as well and
     //   is fastest with neither (128^2, 311 x 1024: 18.6, before 20.2; 64^2, 997 x
     //   256: 2.89, with PIPE 3.28, before 3.13; loading the next step's rows
-    //   early: 20.3 at 128^2).
-    static constexpr bool PIPE = !FLUCT && (CL == 1 ? !WARP : FR * FC >= 32);
-    static constexpr bool REDRAW = !FLUCT && CL > 1 && (COUPLED || FR * FC >= 32);
-    // Resident warps per SM asked for (a bound on the registers per thread).
-    // 32^2 fine-only, 1000 x 103: 8 warps 0.288 ms, 12 warps 0.282; 16^2 in one
-    // warp, 9250 x 52: 16 warps 0.316, 24 warps 0.306 (before 0.337).
-    // Few samples with the fluctuation state want the registers of 8 warps.
-    static constexpr int WARPS_MIN = FLUCT ? (FEW_ ? 8 : 16) : FR * FC >= 32 ? 8 : PIPE ? (COUPLED && FR * FC >= 16 ? 8 : 12)
-                                   : FR * FC >= 16 || FR * FC < 8 ? 16 : 24;
+    //   early: 20.3 at 128^2), but for the plain 32^2 level (1824 x 64: 0.269 with,
+    //   0.328 without, before 0.302).
+    static constexpr bool PIPE = FLUCT    ? NF == 32 && !COUPLED && SECOND && CHAIN == 1
+                                 : CL > 1 ? R == 1 || FR * FC >= 32
+                                 : WARP   ? R == 2 && (COUPLED || C == 2)
+                                          : !(NF == 16 && C == 1 && R == 1 && !SECOND && CHAIN == 1);
+    static constexpr bool REDRAW = !FLUCT && CL > 1 && (R == 1 ? C == 4 && !COUPLED : COUPLED || FR * FC >= 32);
+    // Resident warps per SM asked for (a bound on the registers per thread); the
+    // figures of the shapes with two builds are at Split.  32^2 fine-only, 1000 x 103:
+    // 8 warps 0.288 ms, 12 warps 0.281; 16^2 in one warp, plain, 9250 x 52: 16 warps
+    // 0.316, 24 warps 0.306 (before 0.337), coupled, 1000 x 52: 16 warps with PIPE
+    // 0.059, 24 warps 0.072 (before 0.062).
+    static constexpr int WARPS_MIN =
+        FLUCT               ? (NF == 8 ? (SECOND ? 16 : 20) : !SECOND ? 16 : PIPE ? 12 : 8)
+        : FR * FC >= 32     ? 8
+        : WARP              ? (FR * FC >= 16 ? 8 : FR * FC >= 8 && !COUPLED ? 24 : 16)
+        : FR * FC < 8       ? (PIPE ? 12 : 24)
+        : PIPE && FR * FC < 16 && NF == 32 && CHAIN == 1 ? (SECOND ? 12 : 16)
+        : PIPE              ? (COUPLED && FR * FC >= 16 ? 8 : 12)
+                            : 16;
     static constexpr int MINB = WARPS_MIN * 32 / THREADS > 0 ? WARPS_MIN * 32 / THREADS : 1;
     static constexpr int SLOTS_PER_CTA = WARP ? (THREADS / 32) * SPW : 1;
     // Two cell pairs (Philox calls) are worked on together, packed: neighbours
@@ -897,15 +917,18 @@ template <class S>
 struct Kern {
     static size_t smem_bytes(int stride) { return S::fixed_smem() + sizeof(double) * S::SLOTS_PER_CTA * stride; }
 
-    static cudaError_t info(int stride, VariantInfo* vi) {
+    static cudaError_t prepare() {
         auto fn = level_kernel<S>;
         const size_t smax = smem_bytes(kMaxStride);
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smax);
+        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smax);
+        if (e != cudaSuccess || S::CL == 1) return e;
+        return cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    }
+
+    static cudaError_t info(int stride, VariantInfo* vi) {
+        auto fn = level_kernel<S>;
+        cudaError_t e = prepare();
         if (e != cudaSuccess) return e;
-        if (S::CL > 1) {
-            e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-            if (e != cudaSuccess) return e;
-        }
         int dev = 0, sms = 0;
         if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -991,7 +1014,7 @@ namespace {
 struct VariantEntry {
     int n, C, R, CL;
     cudaError_t (*info)(bool coupled, int stride, VariantInfo* vi);
-    cudaError_t (*launch)(bool coupled, const KArgs& a, int n_ctas, cudaStream_t st, int priority);
+    cudaError_t (*launch)(bool coupled, const VariantInfo& vi, const KArgs& a, int* n_ctas, cudaStream_t st, int priority);
 };
 
 // Few samples: the same level on twice the lanes, half the rows each.  Below about
@@ -1001,58 +1024,93 @@ struct VariantEntry {
 // 43.6 / 25.1, 912 57.8 / 44.1, 1216 56.9 / 65.4; 32^2 x 208 coupled, 152 samples 193 /
 // 122, 456 297 / 248, 608 300 / 391; 32^2 plain, 456 282 / 231, 608 283 / 362.  At
 // 64^2 the full shape fills an SM's schedulers with one sample and wins (152: 312 / 347).
+//
+// Two builds of a shape, of which the first holds more samples at once and the
+// second has more registers: which is the faster one depends on how full the
+// passes over the resident samples are.  Measured, us, first / second build (in
+// brackets before the packed noise, with no bound on the registers):
+//   fluctuation state, 64^2 x 256 coupled, resident 304 / 152: 152 samples 548 / 436
+//     (455), 400 1285 / 1288 (1347), 456 1717 / 1290 (1348), 712 2040 / 2140 (2240), 760
+//     2565 / 2145 (2243); plain, 152 samples 461 / 430 (488), 304 794 / 851 (818)
+//   fluctuation state, 32^2 x 64 coupled, resident 1216 / 608: 608 samples 139 / 115
+//     (115), 912 173 / 215 (217), 1672 318 / 322 (323), 1824 367 / 323 (323), 4256 749 /
+//     741 (740); plain, 1216 / 912: 608 113 / 100 (119), 1216 196 / 222 (255), 1824 328 /
+//     269 (302), 2432 380 / 396 (445), 20000 3048 / 2846 (3208)
+//   fluctuation state, 8^2 x 64 coupled, 6080 / 4864: 2000 samples 55 / 50 (51), 5000
+//     87 / 90 (92), 100000 1185 / 1182 (1318)
+//   16^2 x 52 on two warps, 1824 / 912: 256 samples 28.8 / 24.7 (28.8), 1200 57 / 65
+//     (57), 1824 76 / 76 (78), 5000 202 / 185 (189), 20000 712 / 712 (712)
+//   32^2 x 103 on four warps, coupled, 608 / 456: 456 samples 138 / 131 (144), 608 176 /
+//     206 (182), 912 290 / 249 (302), 4630 1261 / 1229 (1300)
 template <int NF, int C, int R, int CL, bool FL>
 struct Split {
     static constexpr bool HALVE = CL == 1 && ((NF == 16 && C == 1 && R == 2) || (NF == 32 && C == 2 && R == 2));
     static constexpr long long HALF_MAX = !HALVE ? 0 : FL ? (NF == 16 ? 456 : 304) : (NF == 16 ? 912 : 456);
     template <bool CPL>
     using half = Shape<NF, C, HALVE ? R / 2 : R, CL, CPL, FL, HALVE ? 2 : 1, true>;
-    // The fluctuation state has a build of the full shape with the registers of 8
-    // warps between the two, for as many samples as those are: us, with 16 warps /
-    // with 8: 64^2 x 256 steps coupled, 100 samples 549 / 434; 32^2 x 64, 457 138 / 116.
-    static constexpr long long FEW_MAX = !FL ? 0 : NF == 64 ? 152 : NF == 32 ? 608 : 0;
     template <bool CPL>
-    using few = Shape<NF, C, R, CL, CPL, FL, 1, true>;
+    using first = Shape<NF, C, R, CL, CPL, FL>;
+    template <bool CPL>
+    using second = Shape<NF, C, R, CL, CPL, FL, 1, true>;
+    static constexpr bool TWO = FL ? NF == 8 || NF == 32 || NF == 64
+                                   : CL == 1 && ((NF == 16 && C == 1 && R == 1) || (NF == 32 && C * R == 2));
+    // Whether `count` samples run on the second build: `most` and `few` are the
+    // samples that the first and the second build hold at once, `rest` the samples of
+    // the first build's last pass (one that is at most three quarters of `few` runs
+    // alone on its SMs at once, a fuller one two samples to an SM).
+    static bool use_second(bool coupled, long long count, long long most, long long few) {
+        const long long rest = (count - 1) % most + 1;
+        if constexpr (!FL) return count <= few || count > (NF == 32 ? most : 2 * most);
+        if constexpr (NF == 8) return count <= few;
+        if (!coupled) return NF == 64 ? count <= few : rest <= few || count > 2 * most;
+        return count <= few || (rest <= few && 4 * rest > 3 * few && (NF == 64 || count <= 4 * most));
+    }
 };
 
 template <int NF, int C, int R, int CL, bool FL>
 cudaError_t variant_info_fn(bool coupled, int stride, VariantInfo* vi) {
     using SP = Split<NF, C, R, CL, FL>;
-    // the launch attributes of the few-sample shapes (their slots are the full shape's)
-    VariantInfo other{};
     cudaError_t e = cudaSuccess;
-    if constexpr (SP::HALF_MAX > 0) {
-        e = coupled ? Kern<typename SP::template half<true>>::info(stride, &other)
-                    : Kern<typename SP::template half<false>>::info(stride, &other);
+    if constexpr (SP::HALVE) {
+        // its slots are those of the first build; only the launch attribute (and its code loaded)
+        e = coupled ? Kern<typename SP::template half<true>>::prepare() : Kern<typename SP::template half<false>>::prepare();
+        if (e != cudaSuccess) return e;
     }
-    if constexpr (SP::FEW_MAX > 0) {
-        if (e == cudaSuccess)
-            e = coupled ? Kern<typename SP::template few<true>>::info(stride, &other)
-                        : Kern<typename SP::template few<false>>::info(stride, &other);
+    VariantInfo second{};
+    if constexpr (SP::TWO) {
+        e = coupled ? Kern<typename SP::template second<true>>::info(stride, &second)
+                    : Kern<typename SP::template second<false>>::info(stride, &second);
+        if (e != cudaSuccess) return e;
     }
-    if (e != cudaSuccess) return e;
-    return coupled ? Kern<Shape<NF, C, R, CL, true, FL>>::info(stride, vi)
-                   : Kern<Shape<NF, C, R, CL, false, FL>>::info(stride, vi);
+    e = coupled ? Kern<typename SP::template first<true>>::info(stride, vi)
+                : Kern<typename SP::template first<false>>::info(stride, vi);
+    vi->second_ctas = second.max_ctas;
+    return e;
 }
 
 template <int NF, int C, int R, int CL, bool FL>
-cudaError_t variant_launch_fn(bool coupled, const KArgs& a, int n_ctas, cudaStream_t st, int priority) {
+cudaError_t variant_launch_fn(bool coupled, const VariantInfo& vi, const KArgs& a, int* n_ctas, cudaStream_t st,
+                              int priority) {
     using SP = Split<NF, C, R, CL, FL>;
-    if constexpr (SP::HALF_MAX > 0) {
+    if constexpr (SP::HALVE) {
         // one CTA per sample slot, the same slots
         if (a.count <= SP::HALF_MAX) {
-            const int n_slots = n_ctas * Shape<NF, C, R, CL, true, FL>::SLOTS_PER_CTA;
+            const int n_slots = *n_ctas * SP::template first<true>::SLOTS_PER_CTA;
             return coupled ? Kern<typename SP::template half<true>>::launch(a, n_slots, st, priority)
                            : Kern<typename SP::template half<false>>::launch(a, n_slots, st, priority);
         }
     }
-    if constexpr (SP::FEW_MAX > 0) {
-        if (a.count <= SP::FEW_MAX)
-            return coupled ? Kern<typename SP::template few<true>>::launch(a, n_ctas, st, priority)
-                           : Kern<typename SP::template few<false>>::launch(a, n_ctas, st, priority);
+    if constexpr (SP::TWO) {
+        static_assert(CL == 1, "CTAs hold whole samples");
+        constexpr int slots = SP::template first<true>::SLOTS_PER_CTA;
+        if (SP::use_second(coupled, a.count, (long long)vi.max_ctas * slots, (long long)vi.second_ctas * slots)) {
+            *n_ctas = std::min(*n_ctas, vi.second_ctas);
+            return coupled ? Kern<typename SP::template second<true>>::launch(a, *n_ctas, st, priority)
+                           : Kern<typename SP::template second<false>>::launch(a, *n_ctas, st, priority);
+        }
     }
-    return coupled ? Kern<Shape<NF, C, R, CL, true, FL>>::launch(a, n_ctas, st, priority)
-                   : Kern<Shape<NF, C, R, CL, false, FL>>::launch(a, n_ctas, st, priority);
+    return coupled ? Kern<typename SP::template first<true>>::launch(a, *n_ctas, st, priority)
+                   : Kern<typename SP::template first<false>>::launch(a, *n_ctas, st, priority);
 }
 
 #define DK_ENTRY(NF, C, R, CL) \
@@ -1100,11 +1158,11 @@ cudaError_t variant_info(int n, bool coupled, int stride, int idx, VariantInfo* 
     return e;
 }
 
-cudaError_t launch_level(int n, bool coupled, int idx, const KArgs& a, int n_ctas, cudaStream_t st, int priority,
-                         bool fluct) {
+cudaError_t launch_level(int n, bool coupled, int idx, const VariantInfo& vi, const KArgs& a, int* n_ctas,
+                         cudaStream_t st, int priority, bool fluct) {
     const VariantEntry* v = find_variant(n, idx, fluct);
     if (!v) return cudaErrorInvalidValue;
-    return v->launch(coupled, a, n_ctas, st, priority);
+    return v->launch(coupled, vi, a, n_ctas, st, priority);
 }
 
 cudaError_t launch_reduce(const double* partials, int n_slots, int slot_stride, double* out, cudaStream_t st) {

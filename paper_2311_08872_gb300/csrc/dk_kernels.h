@@ -56,6 +56,7 @@ struct VariantInfo {
     int slots_per_cta;      // samples in flight per CTA (1/cluster for clusters)
     size_t smem;            // dynamic shared memory per CTA
     int max_ctas;           // resident CTAs on the whole GPU
+    int second_ctas;        // the same of the register kernel's second build (0: there is one build)
     int C, R;               // lane block: C x R coarse cells (2R x 2C fine)
     int tile_rows;          // streamed kernels: fine rows per CTA tile (0 for the register kernels)
     int persistent;         // streamed kernels: 1 = one launch per wave (work items from a counter)
@@ -72,12 +73,14 @@ int variant_count(int n, bool fluct = false);
 // supported = 0 when it does not exist.
 cudaError_t variant_info(int n, bool coupled, int slot_stride, int idx, VariantInfo* out, bool fluct = false);
 
-// Launch one batch with variant `idx` on n_ctas CTAs; partials must hold
-// (n_ctas / cluster) * slots_per_cta * slot_stride doubles.
+// Launch one batch with variant `idx` (vi: its variant_info) on *n_ctas CTAs, or
+// fewer where a.count runs on a build that keeps fewer resident: *n_ctas is then
+// lowered to the CTAs launched.  partials must hold
+// (*n_ctas / cluster) * slots_per_cta * slot_stride doubles.
 // `priority` (0: none) is passed as the launch's scheduling priority (lower
 // numbers are more urgent, as for streams).
-cudaError_t launch_level(int n, bool coupled, int idx, const KArgs& a, int n_ctas, cudaStream_t stream,
-                         int priority = 0, bool fluct = false);
+cudaError_t launch_level(int n, bool coupled, int idx, const VariantInfo& vi, const KArgs& a, int* n_ctas,
+                         cudaStream_t stream, int priority = 0, bool fluct = false);
 
 // Deterministic fixed-order reduction of the per-slot partials into
 // out[slot_stride]: entry 1 is a max, all others sums.

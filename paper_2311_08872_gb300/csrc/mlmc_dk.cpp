@@ -426,8 +426,9 @@ dk::TArgs theta_args(const mlmc_dk_ctx* c, int level, bool coupled) {
 }
 
 // The level's sample kernel: the theta-scheme kernel on a theta context, the
-// register-resident kernel variant in use otherwise.
-cudaError_t launch_main(const mlmc_dk_ctx* c, int level, bool coupled, const dk::KArgs& a, int n_ctas,
+// register-resident kernel variant in use otherwise, on *n_ctas CTAs or fewer
+// (*n_ctas: the CTAs launched).
+cudaError_t launch_main(const mlmc_dk_ctx* c, int level, bool coupled, const dk::KArgs& a, int* n_ctas,
                         cudaStream_t st, int priority) {
     const LevelTab& t = c->lv[level];
     if (c->coupling == 1) {
@@ -436,11 +437,11 @@ cudaError_t launch_main(const mlmc_dk_ctx* c, int level, bool coupled, const dk:
         fa.phif64 = t.d_phi64;
         fa.phic64 = coupled ? c->lv[level - 1].d_phi64 : nullptr;
         if (dk::fourier_cluster_supported(t.n))
-            return dk::launch_fourier_cluster(t.n, coupled, a, fa, n_ctas, st, priority);
-        return dk::launch_fourier(t.n, coupled, a, fa, n_ctas, st, priority, c->fluct != 0);
+            return dk::launch_fourier_cluster(t.n, coupled, a, fa, *n_ctas, st, priority);
+        return dk::launch_fourier(t.n, coupled, a, fa, *n_ctas, st, priority, c->fluct != 0);
     }
-    if (c->theta) return dk::launch_theta(t.n, coupled, a, theta_args(c, level, coupled), n_ctas, st, priority);
-    return dk::launch_level(t.n, coupled, t.sel[coupled ? 1 : 0], a, n_ctas, st, priority, c->fluct != 0);
+    if (c->theta) return dk::launch_theta(t.n, coupled, a, theta_args(c, level, coupled), *n_ctas, st, priority);
+    return dk::launch_level(t.n, coupled, t.sel[coupled ? 1 : 0], t.vi(coupled), a, n_ctas, st, priority, c->fluct != 0);
 }
 
 int launch_batch_into(mlmc_dk_ctx* c, int level, int stream_tag, int64_t first, int64_t count, uint64_t seed,
@@ -463,13 +464,13 @@ int launch_batch_into(mlmc_dk_ctx* c, int level, int stream_tag, int64_t first, 
     const int64_t want_groups = (count + per_cluster - 1) / per_cluster;
     const int64_t max_groups = vi.max_ctas / vi.cluster;
     const int64_t groups = std::min(want_groups, max_groups);
-    const int n_ctas = (int)(groups * vi.cluster);
-    const int n_slots = (int)(groups * per_cluster);
-    if ((size_t)n_slots * c->stride > cap) return fail(c, MLMC_DK_ERR_INVALID, "scratch too small");
+    int n_ctas = (int)(groups * vi.cluster);
+    if ((size_t)(groups * per_cluster) * c->stride > cap) return fail(c, MLMC_DK_ERR_INVALID, "scratch too small");
     dk::KArgs a = make_args(c, level, stream_tag, coupled, first, count, seed, samples_dev);
     a.partials = partials;
-    if ((e = launch_main(c, level, coupled, a, n_ctas, st, priority)) != cudaSuccess)
+    if ((e = launch_main(c, level, coupled, a, &n_ctas, st, priority)) != cudaSuccess)
         return cuda_fail(c, e, "level kernel launch");
+    const int n_slots = (int)(n_ctas / vi.cluster * per_cluster);
     if ((e = dk::launch_reduce(partials, n_slots, c->stride, sums_dev, st)) != cudaSuccess)
         return cuda_fail(c, e, "reduce kernel launch");
     return MLMC_DK_OK;
@@ -1197,13 +1198,13 @@ int mlmc_dk_run_level_static(const mlmc_dk_ctx* ctx, int32_t level, int32_t stre
                     std::to_string(usable) + " doubles");
     const int64_t groups = std::min({(n_samples + per_group - 1) / per_group, (int64_t)(vi.max_ctas / vi.cluster),
                                      fit_groups});
-    const int n_ctas = (int)(groups * vi.cluster);
-    const int n_slots = (int)(groups * per_group);
+    int n_ctas = (int)(groups * vi.cluster);
     dk::KArgs a = make_args(c, level, stream_tag, coupled, first_sample, n_samples, seed, samples_dev);
     a.partials = scratch;        // fully overwritten by the level kernel: nothing to clear
     a.err = err_dev ? err_dev : reinterpret_cast<unsigned*>(scratch + (capacity - 1));
-    if ((e = launch_main(ctx, level, coupled, a, n_ctas, st, 0)) != cudaSuccess)
+    if ((e = launch_main(ctx, level, coupled, a, &n_ctas, st, 0)) != cudaSuccess)
         return cuda_fail(c, e, "level kernel launch");
+    const int n_slots = (int)(n_ctas / vi.cluster * per_group);
     if ((e = dk::launch_reduce(scratch, n_slots, ctx->stride, sums_dev, st)) != cudaSuccess)
         return cuda_fail(c, e, "reduce kernel launch");
     return MLMC_DK_OK;

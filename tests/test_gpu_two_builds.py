@@ -1,0 +1,74 @@
+"""Register shapes with two builds (registers per thread) run the same arithmetic:
+the same samples from batches on both sides of every size where the build changes,
+and sums over the slots that were launched, also where a build keeps fewer samples
+resident than the other (several passes of a smaller grid) and where the static
+scratch limits the grid further."""
+import numpy as np
+import pytest
+
+from paper_2311_08872_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dk():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2311_08872_gb300 import build as libbuild
+    libbuild.build()
+    from paper_2311_08872_gb300 import mlmc_dk
+    return mlmc_dk
+
+
+def _run(ctx, dk, level, mc, count, static=False):
+    import torch
+    st = torch.cuda.current_stream().cuda_stream
+    sums = torch.full((dk.sums_len(ctx.n_quant),), float("nan"), dtype=torch.float64, device="cuda")
+    samp = torch.full((count, dk.sample_stride(ctx.n_obs)), float("nan"), dtype=torch.float64, device="cuda")
+    if static:
+        ctx.run_level_static(level, int(mc), 7, count, 5, sums.data_ptr(), samp.data_ptr(), 0, st)
+    else:
+        ctx.run_level_dev(level, int(mc), 7, count, 5, sums.data_ptr(), samp.data_ptr(), st)
+    torch.cuda.synchronize()
+    return sums.cpu().numpy(), samp.cpu().numpy()
+
+
+FL = "paper_reg"        # N = 2e9: fluctuation state
+
+
+@pytest.mark.parametrize("name,n0,level,variant,mc,counts", [
+    (FL, 4, 4, 0, False, (152, 153, 305, 418, 419, 456, 457, 760)),
+    (FL, 4, 4, 0, True, (152, 153, 456)),
+    (FL, 4, 3, 0, False, (608, 609, 1216, 1672, 1673, 1824, 1825, 4256, 5472)),
+    (FL, 4, 3, 0, True, (912, 913, 1216, 1217, 2128, 2129, 2432, 2433)),
+    (FL, 4, 1, 0, False, (4864, 4865, 6081)),
+    (FL, 4, 1, 0, True, (4864, 4865, 6081)),
+    ("mlmc16_256", 16, 0, 2, True, (912, 913, 1824, 3648, 3649)),
+    ("mlmc16_256", 8, 1, 2, False, (912, 913, 1824, 3648, 3649)),
+    ("mlmc16_256", 16, 1, 1, False, (456, 457, 608, 609)),
+    ("mlmc16_256", 16, 1, 1, True, (456, 457, 608, 609)),
+    ("mlmc16_256", 16, 1, 2, False, (456, 457, 608, 609)),
+    ("mlmc16_256", 16, 1, 2, True, (456, 457, 608, 609)),
+])
+def test_both_builds_give_the_same_samples(dk, name, n0, level, variant, mc, counts):
+    """Integer paths and per-lane FP32 sums are the same; only FP64 sums over lanes and
+    slots run in another order (at most 2^13 terms: 13 roundings of 2^-53 of the partial
+    sums' size, which is at most 10^3 of their total's)."""
+    wl = W.get(name)
+    wl = wl.with_(L_max=max(level, 1)) if name == FL else wl.with_(n0=n0, L_max=max(level, 1), T=0.004)
+    with dk.Context.from_workload(wl) as ctx:
+        assert ctx.level_info(level).n == wl.n0 << level
+        ctx.set_variant(level, level > 0 and not mc, variant)
+        _, big = _run(ctx, dk, level, mc, max(counts))
+        assert np.isfinite(big).all()
+        scale = np.maximum(np.sqrt(np.mean(big ** 2, axis=0)), 1e-300)
+        for count in counts:
+            for static in (False, True):
+                sums, samp = _run(ctx, dk, level, mc, count, static)
+                assert np.max(np.abs(samp - big[:count]) / scale) <= 1e3 * 13 * 2.0 ** -53
+                assert int(sums[0]) == count and sums[1] == 0.0
+                coarse = samp[:, ctx.n_obs] if level > 0 and not mc else 0.0
+                dp = wl.N * (samp[:, 0] ** 2 - coarse ** 2)
+                np.testing.assert_allclose(sums[2], dp.sum(), rtol=1e-9, atol=1e-9 * np.abs(dp).sum())
