@@ -23,7 +23,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # exceed; unpacking it took 11 ms of a process's first context (13.8 ms for one
 # 16^2 level, 2.5 without)
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--no-compress", "-Xcompiler", "-fPIC"]
-SOURCES = ["dk_kernels.cu", "dk_band.cu", "dk_stream.cu", "dk_surrogate.cu", "dk_umma.cu", "dk_theta.cu", "dk_fourier.cu", "dk_fourier_cluster.cu", "mlmc_dk.cpp"]
+SOURCES = ["dk_kernels.cu", "dk_kernels_fluct.cu", "dk_common.cu", "dk_band.cu", "dk_stream.cu", "dk_surrogate.cu", "dk_umma.cu", "dk_theta.cu", "dk_fourier.cu", "dk_fourier_cluster.cu", "mlmc_dk.cpp"]
 HEADERS = ["dk_kernels.h", "dk_device.cuh"]
 
 

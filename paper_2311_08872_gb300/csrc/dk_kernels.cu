@@ -44,8 +44,7 @@
 // before; 32^2 fine only, 1000 x 103: 0.280 ms, 0.316 before.
 #include <cooperative_groups.h>
 
-#include <atomic>
-#include <mutex>
+#include <algorithm>
 
 #include "dk_device.cuh"
 #include "dk_kernels.h"
@@ -827,91 +826,6 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB) level_kernel(const KArgs 
     if constexpr (CL > 1) cg::this_cluster().sync();   // peers may still read our shared memory
 }
 
-// Fixed-order reduction over slots: one block per entry.
-__global__ void __launch_bounds__(256) reduce_kernel(const double* part, int n_slots, double* out) {
-    const int e = blockIdx.x;
-    const bool is_max = (e == 1);
-    const double* row = part + (size_t)e * n_slots;
-    double v = 0.0;
-    for (int s = threadIdx.x; s < n_slots; s += 256) v = is_max ? fmax(v, row[s]) : v + row[s];
-    __shared__ double sh[256];
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-            const double o = sh[threadIdx.x + w];
-            sh[threadIdx.x] = is_max ? fmax(sh[threadIdx.x], o) : sh[threadIdx.x] + o;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[e] = sh[0];
-}
-
-// out[e] += in[e] (entry 1, the max mass error: max): merges the sums of two
-// disjoint sample ranges of one level.
-__global__ void add_sums_kernel(double* out, const double* in, int stride) {
-    for (int e = threadIdx.x; e < stride; e += blockDim.x) out[e] = e == 1 ? fmax(out[e], in[e]) : out[e] + in[e];
-}
-
-// Normals of one fine step, written out (the level kernel keeps them in
-// registers); same device functions as the level kernel.
-__global__ void noise_kernel(int n, uint32_t m, uint32_t c2, uint32_t c3, uint32_t k0, uint32_t k1,
-                             float* z, uint32_t* raw) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n * n / 2) return;
-    const uint4 x = philox10(make_uint4(static_cast<uint32_t>(p), m, c2, c3), k0, k1);
-    if (raw) reinterpret_cast<uint4*>(raw)[p] = x;
-    if (z) {
-        float a1, a2, b1, b2;
-        box_muller(x.x, x.y, a1, a2);
-        box_muller(x.z, x.w, b1, b2);
-        reinterpret_cast<float4*>(z)[p] = make_float4(a1, a2, b1, b2);
-    }
-}
-
-cudaError_t launch_noise(int n, uint32_t m, uint32_t c2, uint32_t c3, uint32_t k0, uint32_t k1, float* z,
-                         uint32_t* raw, cudaStream_t st) {
-    const int pairs = n * n / 2;
-    noise_kernel<<<(pairs + 255) / 256, 256, 0, st>>>(n, m, c2, c3, k0, k1, z, raw);
-    return cudaGetLastError();
-}
-
-// -------------------------------------------- statically allocated scratch
-// Scratch for the per-slot partial sums of mlmc_dk_run_level_static, whose
-// callers cannot allocate device memory.  Every GPU that loads the library
-// holds this array until the process exits; all calls share it.
-static __device__ __align__(256) double g_static_partials[kStaticScratchDoubles];
-
-namespace {
-constexpr int kMaxDevices = 64;
-double* g_static_ptr[kMaxDevices] = {};
-std::atomic<int> g_static_ready[kMaxDevices];
-std::mutex g_static_mutex;
-}  // namespace
-
-cudaError_t static_scratch(double** out, size_t* capacity) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    if (!g_static_ready[dev].load(std::memory_order_acquire)) {
-        // Set-up, once per device, with that device current: in host code the
-        // array's name is only a host-side stand-in, so the kernels get the
-        // device address from the runtime.
-        std::lock_guard<std::mutex> lock(g_static_mutex);
-        if (!g_static_ready[dev].load(std::memory_order_relaxed)) {
-            void* p = nullptr;
-            e = cudaGetSymbolAddress(&p, g_static_partials);
-            if (e != cudaSuccess) return e;
-            g_static_ptr[dev] = static_cast<double*>(p);
-            g_static_ready[dev].store(1, std::memory_order_release);
-        }
-    }
-    *out = g_static_ptr[dev];
-    *capacity = kStaticScratchDoubles;
-    return cudaSuccess;
-}
-
 // ------------------------------------------------------------------ dispatch
 template <class S>
 struct Kern {
@@ -1010,13 +924,15 @@ struct Kern {
     X(256, 4, 2, 8)    \
     X(256, 4, 1, 8)
 
-namespace {
 struct VariantEntry {
     int n, C, R, CL;
     cudaError_t (*info)(bool coupled, int stride, VariantInfo* vi);
     cudaError_t (*launch)(bool coupled, const VariantInfo& vi, const KArgs& a, int* n_ctas, cudaStream_t st, int priority);
 };
+// The fluctuation-state builds' table.
+const VariantEntry* fluct_variants(int* count);
 
+namespace {
 // Few samples: the same level on twice the lanes, half the rows each.  Below about
 // a warp per scheduler the time of a batch is that of one sample's chain of steps,
 // and half the cells per lane shorten it; the sums keep the full shape's order
@@ -1113,10 +1029,7 @@ cudaError_t variant_launch_fn(bool coupled, const VariantInfo& vi, const KArgs& 
                    : Kern<typename SP::template first<false>>::launch(a, *n_ctas, st, priority);
 }
 
-#define DK_ENTRY(NF, C, R, CL) \
-    {NF, C, R, CL, variant_info_fn<NF, C, R, CL, false>, variant_launch_fn<NF, C, R, CL, false>},
-const VariantEntry kVariants[] = {DK_VARIANTS(DK_ENTRY)};
-#undef DK_ENTRY
+#ifdef DK_FLUCT_BUILD
 // Fluctuation-state builds: one lane-block shape per grid size up to 128^2
 // (the grids of the high-particle-number hierarchies that need them).
 #define DK_FLUCT_VARIANTS(X) \
@@ -1130,12 +1043,21 @@ const VariantEntry kVariants[] = {DK_VARIANTS(DK_ENTRY)};
     {NF, C, R, CL, variant_info_fn<NF, C, R, CL, true>, variant_launch_fn<NF, C, R, CL, true>},
 const VariantEntry kFluctVariants[] = {DK_FLUCT_VARIANTS(DK_ENTRY)};
 #undef DK_ENTRY
+}  // namespace
+
+const VariantEntry* fluct_variants(int* count) {
+    *count = (int)(sizeof(kFluctVariants) / sizeof(kFluctVariants[0]));
+    return kFluctVariants;
+}
+#else
+#define DK_ENTRY(NF, C, R, CL) \
+    {NF, C, R, CL, variant_info_fn<NF, C, R, CL, false>, variant_launch_fn<NF, C, R, CL, false>},
+const VariantEntry kVariants[] = {DK_VARIANTS(DK_ENTRY)};
+#undef DK_ENTRY
 
 const VariantEntry* find_variant(int n, int idx, bool fluct) {
-    const VariantEntry* tab = fluct ? kFluctVariants : kVariants;
-    const int count = fluct ? (int)(sizeof(kFluctVariants) / sizeof(kFluctVariants[0]))
-                            : (int)(sizeof(kVariants) / sizeof(kVariants[0]));
-    int k = 0;
+    int count = (int)(sizeof(kVariants) / sizeof(kVariants[0])), k = 0;
+    const VariantEntry* tab = fluct ? fluct_variants(&count) : kVariants;
     for (int i = 0; i < count; ++i)
         if (tab[i].n == n && k++ == idx) return &tab[i];
     return nullptr;
@@ -1164,15 +1086,6 @@ cudaError_t launch_level(int n, bool coupled, int idx, const VariantInfo& vi, co
     if (!v) return cudaErrorInvalidValue;
     return v->launch(coupled, vi, a, n_ctas, st, priority);
 }
-
-cudaError_t launch_reduce(const double* partials, int n_slots, int slot_stride, double* out, cudaStream_t st) {
-    reduce_kernel<<<slot_stride, 256, 0, st>>>(partials, n_slots, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_add_sums(double* out, const double* in, int slot_stride, cudaStream_t st) {
-    add_sums_kernel<<<1, 256, 0, st>>>(out, in, slot_stride);
-    return cudaGetLastError();
-}
+#endif  // DK_FLUCT_BUILD
 
 }  // namespace dk

@@ -82,6 +82,9 @@ cudaError_t variant_info(int n, bool coupled, int slot_stride, int idx, VariantI
 cudaError_t launch_level(int n, bool coupled, int idx, const VariantInfo& vi, const KArgs& a, int* n_ctas,
                          cudaStream_t stream, int priority = 0, bool fluct = false);
 
+// Load the code and the static scratch that every context uses (at its creation and
+// not in its first call).
+cudaError_t load_common();
 // Deterministic fixed-order reduction of the per-slot partials into
 // out[slot_stride]: entry 1 is a max, all others sums.
 cudaError_t launch_reduce(const double* partials, int n_slots, int slot_stride, double* out,

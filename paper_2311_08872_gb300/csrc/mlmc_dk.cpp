@@ -1034,7 +1034,8 @@ int mlmc_dk_init(const mlmc_dk_config* cfg, mlmc_dk_ctx** out) {
             t.split_ok = 1;
         }
     }
-    if ((e = cudaMalloc(&c->d_partials, sizeof(double) * std::max<size_t>(partials_need, 1))) != cudaSuccess ||
+    if ((e = dk::load_common()) != cudaSuccess ||
+        (e = cudaMalloc(&c->d_partials, sizeof(double) * std::max<size_t>(partials_need, 1))) != cudaSuccess ||
         (e = cudaMalloc(&c->d_sums, sizeof(double) * c->stride)) != cudaSuccess ||
         (e = cudaMalloc(&c->d_err, sizeof(unsigned))) != cudaSuccess ||
         (e = cudaMemset(c->d_err, 0, sizeof(unsigned))) != cudaSuccess ||
