@@ -94,15 +94,18 @@ struct TShape {
     // Registers per thread: up to 255 (8 warps on an SM), 128 for the 2 x 2 blocks at
     // 32^2 and where DENSE (16 warps; the fluxes and the coarse state of 4 x 4 blocks
     // then spill outside the iteration).  16^2 wants the first: 256 samples 34.0 us
-    // with 155 registers, 40.0 with 128.
-    static constexpr int MIN_CTAS = (DENSE || N == 32 ? 512 : 256) / THREADS;
+    // with 155 registers, 40.0 with 128.  4^2 has 128: 100000 samples x 5 steps 171 us
+    // with 150, 164 with 128, 193 with 96.
+    static constexpr int MIN_CTAS = (N == 4 || DENSE || N == 32 ? 512 : 256) / THREADS;
     static_assert(LPR <= 32 && (SPB == 1 || TPS <= 32) && (CL == 1 || LPR == 32), "block layout");
     // per sample: two buffers of the blocks' top and bottom rows, two words a cell;
     // in a cluster also four message slots for the rows above and below the band,
     // their mbarriers, and two words that tell of a wait that ran out
     static constexpr int BUF = 4 * N * NBR;                // words of one buffer
     static constexpr int SLOT = 4 * N;                     // words of one message slot (both sides)
-    static constexpr int WORDS = 2 * BUF + (CL > 1 ? 4 * SLOT : 0);
+    // (4 x 4: 16 words of padding, so that the two samples of a quarter warp use different
+    // banks; 100000 samples x 5 steps 230 us without, 171 with, 209 before these blocks)
+    static constexpr int WORDS = 2 * BUF + (CL > 1 ? 4 * SLOT : 0) + (N == 4 ? 16 : 0);
     static constexpr size_t SAMPLE_BYTES = sizeof(int32_t) * WORDS + (CL > 1 ? 10 * sizeof(uint64_t) : 0);
     static size_t smem(int slot_stride) {
         return SAMPLE_BYTES * SPB + sizeof(double) * ((THREADS + 31) / 32) * kRed + sizeof(double) * kRed +
