@@ -56,7 +56,7 @@ struct VariantInfo {
     int slots_per_cta;      // samples in flight per CTA (1/cluster for clusters)
     size_t smem;            // dynamic shared memory per CTA
     int max_ctas;           // resident CTAs on the whole GPU
-    int second_ctas;        // the same of the register kernel's second build (0: there is one build)
+    int second_ctas;        // the same of the kernel's other build, which some counts run on (0: there is none)
     int C, R;               // lane block: C x R coarse cells (2R x 2C fine)
     int tile_rows;          // streamed kernels: fine rows per CTA tile (0 for the register kernels)
     int persistent;         // streamed kernels: 1 = one launch per wave (work items from a counter)
@@ -191,10 +191,10 @@ struct TArgs {
 };
 bool theta_supported(int n);
 cudaError_t theta_variant_info(int n, bool coupled, int slot_stride, VariantInfo* out);
-// Launch one batch of the theta-scheme kernel on n_ctas CTAs; partials must hold
-// n_ctas * slots_per_cta * slot_stride doubles.
-cudaError_t launch_theta(int n, bool coupled, const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t stream,
-                         int priority = 0);
+// Launch one batch of the theta-scheme kernel on *n_ctas CTAs or fewer (as
+// launch_level); partials must hold *n_ctas * slots_per_cta * slot_stride doubles.
+cudaError_t launch_theta(int n, bool coupled, const VariantInfo& vi, const KArgs& a, const TArgs& t, int* n_ctas,
+                         cudaStream_t stream, int priority = 0);
 // Failure-detection test: a coupled 128 x 128 batch with t.wait_polls and t.stall_step.
 cudaError_t launch_theta_wait_test(const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t stream);
 

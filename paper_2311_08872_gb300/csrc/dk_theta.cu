@@ -93,10 +93,9 @@ struct TShape {
     static constexpr int SPB = THREADS / TPS;              // samples per CTA
     // Registers per thread: up to 255 (8 warps on an SM), 128 for the 2 x 2 blocks at
     // 32^2 and where DENSE (16 warps; the fluxes and the coarse state of 4 x 4 blocks
-    // then spill outside the iteration).  16^2 wants the first: 256 samples 34.0 us
-    // with 155 registers, 40.0 with 128.  4^2 has 128: 100000 samples x 5 steps 171 us
-    // with 150, 164 with 128, 193 with 96.
-    static constexpr int MIN_CTAS = (N == 4 || DENSE || N == 32 ? 512 : 256) / THREADS;
+    // then spill outside the iteration).  16^2 has 155, or 96 where DENSE (20 warps).
+    // 4^2 has 128: 100000 samples x 5 steps 171 us with 150, 164 with 128, 193 with 96.
+    static constexpr int MIN_CTAS = N == 16 && DENSE ? 5 : (N == 4 || DENSE || N == 32 ? 512 : 256) / THREADS;
     static_assert(LPR <= 32 && (SPB == 1 || TPS <= 32) && (CL == 1 || LPR == 32), "block layout");
     // per sample: two buffers of the blocks' top and bottom rows, two words a cell;
     // in a cluster also four message slots for the rows above and below the band,
@@ -717,22 +716,32 @@ void launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int 
     cfg.numAttrs = na;
 }
 
-// From 32 x 32 on there are two builds, chosen by the number of samples: one for
+// From 16 x 16 on there are two builds, chosen by the number of samples: one for
 // few, which is the faster one for a sample, and a DENSE one for the GPU's
 // throughput.  FEW is the number of samples that the first holds at once.
 // Measured, ms, first build / DENSE: 128^2 x 384 steps, 36 samples 5.1 / 6.7, 150
 // samples 25.3 / 22.6; 64^2 x 96, 152 samples 1.03 / 1.15, 304 2.2 / 1.8, 1000 7.7 /
 // 6.2; 32^2 x 24 (2 x 2 blocks / 4 x 4), 3 samples 0.10 / 0.22, 304 0.160 / 0.25.
+// 16^2 holds 1824 samples at once in the first build, 3040 in the DENSE one; the
+// first keeps the sizes that it finishes in as many passes, or in a short one more
+// (coupled, 77 steps, us; in brackets one warp per 2 x 2 blocks and no bound, 2128 at
+// once): 256 samples 364 / 370 (386), 2000 970 / 1010 (934), 2432 1212 / 1010 (1123),
+// 3648 1495 / 1690 (1690), 5000 2232 / 2180 (2180), 20000 8140 / 8030 (8720).
 template <int N>
 constexpr long long kFew = N == 32 ? 304 : N == 64 ? 152 : N == 128 ? 36 : 0;
+template <int N>
+constexpr bool first_build(long long count) {
+    if (N == 16) return count <= 2128 || (count > 3040 && count <= 3648);
+    return N < 16 || count <= kFew<N>;
+}
 
 template <int N, bool CPL>
 cudaError_t prepare(int slot_stride, VariantInfo* out) {
-    using S = TShape<N, (N >= 32)>;
+    using S = TShape<N, (N >= 16)>;
     const size_t smem = S::smem(slot_stride);
-    const auto kernel = theta_kernel<N, CPL, (N >= 32)>;
+    const auto kernel = theta_kernel<N, CPL, (N >= 16)>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess && N >= 32)
+    if (e == cudaSuccess && N >= 16)
         e = cudaFuncSetAttribute(theta_kernel<N, CPL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)TShape<N, false>::smem(slot_stride));
     if (e != cudaSuccess) return e;
@@ -755,6 +764,13 @@ cudaError_t prepare(int slot_stride, VariantInfo* out) {
             (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
             return e;
         out->max_ctas = per_sm * sms;
+        if constexpr (N == 16) {
+            // the first build also runs batches of several passes, on its own residency
+            const auto few = theta_kernel<N, CPL, false>;
+            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, few, TShape<N, false>::THREADS, smem)) != cudaSuccess)
+                return e;
+            out->second_ctas = per_sm * sms;
+        }
     }
     out->supported = out->max_ctas > 0;
     return cudaSuccess;
@@ -771,11 +787,13 @@ cudaError_t launch_build(const KArgs& a, const TArgs& t, int n_ctas, cudaStream_
 }
 
 template <int N, bool CPL>
-cudaError_t launch_n(const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t st, int priority) {
-    // (both builds have one sample slot per CTA or cluster from 32 x 32 on)
-    if constexpr (N >= 32)
-        if (a.count > kFew<N>) return launch_build<N, CPL, true>(a, t, n_ctas, st, priority);
-    return launch_build<N, CPL, false>(a, t, n_ctas, st, priority);
+cudaError_t launch_n(const VariantInfo& vi, const KArgs& a, const TArgs& t, int* n_ctas, cudaStream_t st, int priority) {
+    // (both builds have the same sample slots per CTA or cluster)
+    static_assert(TShape<N, false>::SPB == TShape<N, (N >= 16)>::SPB, "slots");
+    if constexpr (N >= 16)
+        if (!first_build<N>(a.count)) return launch_build<N, CPL, true>(a, t, *n_ctas, st, priority);
+    if (vi.second_ctas > 0 && vi.second_ctas < *n_ctas) *n_ctas = vi.second_ctas;
+    return launch_build<N, CPL, false>(a, t, *n_ctas, st, priority);
 }
 
 // f(std::integral_constant<int, N>) for the grid sizes with a kernel.
@@ -809,16 +827,17 @@ cudaError_t launch_theta_wait_test(const KArgs& a, const TArgs& t, int n_ctas, c
     if (t.K < 0 || t.K > kMaxCheb) return cudaErrorInvalidValue;
     constexpr int N = 128;
     static_assert(TShape<N, true>::SAMPLE_BYTES < 45000, "no shared-memory attribute needed");
-    return a.count > kFew<N> ? launch_build<N, true, true, true>(a, t, n_ctas, st, 0)
-                             : launch_build<N, true, false, true>(a, t, n_ctas, st, 0);
+    return first_build<N>(a.count) ? launch_build<N, true, false, true>(a, t, n_ctas, st, 0)
+                                   : launch_build<N, true, true, true>(a, t, n_ctas, st, 0);
 }
 
-cudaError_t launch_theta(int n, bool coupled, const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t st,
-                         int priority) {
+cudaError_t launch_theta(int n, bool coupled, const VariantInfo& vi, const KArgs& a, const TArgs& t, int* n_ctas,
+                         cudaStream_t st, int priority) {
     if (t.K < 0 || t.K > kMaxCheb) return cudaErrorInvalidValue;
     cudaError_t e = cudaErrorInvalidValue;
     for_grid(n, [&](auto N) {
-        e = coupled ? launch_n<N.value, true>(a, t, n_ctas, st, priority) : launch_n<N.value, false>(a, t, n_ctas, st, priority);
+        e = coupled ? launch_n<N.value, true>(vi, a, t, n_ctas, st, priority)
+                    : launch_n<N.value, false>(vi, a, t, n_ctas, st, priority);
     });
     return e;
 }

@@ -440,7 +440,7 @@ cudaError_t launch_main(const mlmc_dk_ctx* c, int level, bool coupled, const dk:
             return dk::launch_fourier_cluster(t.n, coupled, a, fa, *n_ctas, st, priority);
         return dk::launch_fourier(t.n, coupled, a, fa, *n_ctas, st, priority, c->fluct != 0);
     }
-    if (c->theta) return dk::launch_theta(t.n, coupled, a, theta_args(c, level, coupled), *n_ctas, st, priority);
+    if (c->theta) return dk::launch_theta(t.n, coupled, t.vi(coupled), a, theta_args(c, level, coupled), n_ctas, st, priority);
     return dk::launch_level(t.n, coupled, t.sel[coupled ? 1 : 0], t.vi(coupled), a, n_ctas, st, priority, c->fluct != 0);
 }
 

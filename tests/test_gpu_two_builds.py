@@ -72,3 +72,20 @@ def test_both_builds_give_the_same_samples(dk, name, n0, level, variant, mc, cou
                 coarse = samp[:, ctx.n_obs] if level > 0 and not mc else 0.0
                 dp = wl.N * (samp[:, 0] ** 2 - coarse ** 2)
                 np.testing.assert_allclose(sums[2], dp.sum(), rtol=1e-9, atol=1e-9 * np.abs(dp).sum())
+
+
+@pytest.mark.parametrize("mc", [False, True])
+def test_both_builds_of_the_16_grid_theta_level(dk, mc):
+    """16^2 theta level: both builds run the same operations on every cell; the FP64
+    sums over lanes too."""
+    wl = W.get("theta16_128").with_(n0=8, L_max=1, T=0.02)
+    with dk.Context.from_workload(wl) as ctx:
+        assert ctx.level_info(1).n == 16 and ctx.level_info(1).theta == 1
+        _, big = _run(ctx, dk, 1, mc, 4000)
+        for count in (1, 1825, 2128, 2129, 3040, 3041, 3648, 3649, 4000):
+            for static in (False, True):
+                sums, samp = _run(ctx, dk, 1, mc, count, static)
+                np.testing.assert_array_equal(samp, big[:count])
+                assert int(sums[0]) == count and sums[1] == 0.0
+                dp = wl.N * (samp[:, 0] ** 2 - (0.0 if mc else samp[:, 1] ** 2))
+                np.testing.assert_allclose(sums[2], dp.sum(), rtol=1e-9, atol=1e-9 * np.abs(dp).sum())
