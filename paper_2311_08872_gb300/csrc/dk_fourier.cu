@@ -375,9 +375,12 @@ __global__ void __launch_bounds__(FShape<N, ROWS>::THREADS, FShape<N, ROWS>::MIN
 // Two builds at 18^2: few samples run on 1 x 6 cells per thread (two warps per
 // sample), which is the faster one for a sample, many on 2 x 6 (one warp).
 // 18^2 x 72 steps, us, one row / two rows: 3 samples 62 / 113, 1216 116 / 172; 20000
-// samples 2310 (one row, normals in shared memory) / 1680.
-template <int N>
-constexpr long long kFewF = N == 18 ? 1216 : 0;
+// samples 2310 (one row, normals in shared memory) / 1680.  At 54^2 with the
+// fluctuation state, whose mean-field loads a sample alone on its SM waits for, the
+// same: x 243 steps, plain, 152 samples 366 / 437 (before the 2 x 6 blocks 411), coupled
+// 500 / 570 (606); without it there is little between them (coupled 332 / 330).
+template <int N, bool FL>
+constexpr long long kFewF = N == 18 ? 1216 : N == 54 && FL ? 152 : 0;
 template <int N>
 constexpr int kRows = N == 6 ? 1 : 2;
 
@@ -387,7 +390,7 @@ cudaError_t fprepare(int slot_stride, VariantInfo* out) {
     const size_t smem = S::smem(slot_stride);
     const auto kernel = fourier_kernel<N, kRows<N>, CPL, FL>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if constexpr (kFewF<N> > 0) {
+    if constexpr (kFewF<N, FL> > 0) {
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(fourier_kernel<N, 1, CPL, FL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)FShape<N, 1>::smem(slot_stride));
@@ -429,8 +432,8 @@ cudaError_t flaunch_rows(const KArgs& a, const FArgs& f, int n_ctas, cudaStream_
 
 template <int N, bool CPL, bool FL>
 cudaError_t flaunch(const KArgs& a, const FArgs& f, int n_ctas, cudaStream_t st, int priority) {
-    if constexpr (kFewF<N> > 0) {
-        if (a.count <= kFewF<N>) return flaunch_rows<N, 1, CPL, FL>(a, f, n_ctas, st, priority);
+    if constexpr (kFewF<N, FL> > 0) {
+        if (a.count <= kFewF<N, FL>) return flaunch_rows<N, 1, CPL, FL>(a, f, n_ctas, st, priority);
     }
     return flaunch_rows<N, kRows<N>, CPL, FL>(a, f, n_ctas, st, priority);
 }

@@ -89,3 +89,20 @@ def test_both_builds_of_the_16_grid_theta_level(dk, mc):
                 assert int(sums[0]) == count and sums[1] == 0.0
                 dp = wl.N * (samp[:, 0] ** 2 - (0.0 if mc else samp[:, 1] ** 2))
                 np.testing.assert_allclose(sums[2], dp.sum(), rtol=1e-9, atol=1e-9 * np.abs(dp).sum())
+
+
+@pytest.mark.parametrize("mc", [False, True])
+def test_both_builds_of_the_54_grid_fourier_level(dk, mc):
+    """54^2 Fourier level with the fluctuation state: few samples run on one row of
+    cells per thread.  Integer paths are the same; the FP64 sums over threads (486 of
+    them: 9 levels, partial sums at most 10^3 of their total) run in another order."""
+    wl = W.get("paper_reg_fourier")
+    with dk.Context.from_workload(wl) as ctx:
+        assert ctx.level_info(2).n == 54 and ctx.level_info(2).fluct == 1
+        _, big = _run(ctx, dk, 2, mc, 305)
+        scale = np.maximum(np.sqrt(np.mean(big ** 2, axis=0)), 1e-300)
+        for count in (1, 152, 153, 305):
+            for static in (False, True):
+                sums, samp = _run(ctx, dk, 2, mc, count, static)
+                assert np.max(np.abs(samp - big[:count]) / scale) <= 1e3 * 9 * 2.0 ** -53
+                assert int(sums[0]) == count and sums[1] == 0.0
