@@ -78,12 +78,13 @@ constexpr int kRed = 2 * kMaxObs + 2;   // reduced values per sample
 // Shapes: fine block R x C per thread, CL CTAs per sample.  (A poll limit and a
 // stopping step read at run time cost the 128^2 build 100 to 400 bytes of spills and
 // a tenth to a quarter of its speed: only the test's build has them.)
-template <int N_, bool DENSE_, bool TEST_ = false>
+enum Build { kFirst, kDense, kMid };   // see first_build
+template <int N_, Build B, bool TEST_ = false>
 struct TShape {
     static constexpr int N = N_, NC = N / 2;
-    static constexpr bool DENSE = DENSE_;
+    static constexpr bool DENSE = B == kDense;
     static constexpr bool TEST = TEST_;                    // build of the failure-detection test (TArgs)
-    static constexpr bool SMALL = N < 32 || (N == 32 && !DENSE);
+    static constexpr bool SMALL = N < 32 || (N == 32 && B == kFirst);
     static constexpr int R = SMALL ? 2 : 4, C = N >= 16 && !(N == 32 && !DENSE) ? 4 : 2;
     static constexpr int CL = N >= 128 ? 4 : 1;
     static constexpr int LPR = N / C;                      // lanes per row of blocks
@@ -92,7 +93,7 @@ struct TShape {
     static constexpr int THREADS = TPS >= 64 ? TPS : 128;
     static constexpr int SPB = THREADS / TPS;              // samples per CTA
     // Registers per thread: up to 255 (8 warps on an SM), 128 for the 2 x 2 blocks at
-    // 32^2 and where DENSE (16 warps; the fluxes and the coarse state of 4 x 4 blocks
+    // 32^2, 4 x 2 ones and where DENSE (16 warps; the fluxes and the coarse state of 4 x 4 blocks
     // then spill outside the iteration).  16^2 has 155, or 96 where DENSE (20 warps).
     // 4^2 has 128: 100000 samples x 5 steps 171 us with 150, 164 with 128, 193 with 96.
     static constexpr int MIN_CTAS = N == 16 && DENSE ? 5 : (N == 4 || DENSE || N == 32 ? 512 : 256) / THREADS;
@@ -468,10 +469,10 @@ __device__ __forceinline__ void sample_barrier() {
     else __syncthreads();
 }
 
-template <int N, bool CPL, bool DENSE, bool TEST = false>
-__global__ void __launch_bounds__(TShape<N, DENSE>::THREADS, TShape<N, DENSE>::MIN_CTAS)
+template <int N, bool CPL, Build B, bool TEST = false>
+__global__ void __launch_bounds__(TShape<N, B>::THREADS, TShape<N, B>::MIN_CTAS)
     theta_kernel(const KArgs a, const TArgs t) {
-    using S = TShape<N, DENSE, TEST>;
+    using S = TShape<N, B, TEST>;
     constexpr int NC = S::NC, TPS = S::TPS, SPB = S::SPB, THREADS = S::THREADS, R = S::R, C = S::C, CL = S::CL;
     constexpr int RC = R / 2, CC = C / 2;       // coarse block
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -716,12 +717,16 @@ void launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int 
     cfg.numAttrs = na;
 }
 
-// From 16 x 16 on there are two builds, chosen by the number of samples: one for
+// From 16 x 16 on there are two builds (32 x 32: three), chosen by the number of samples: one for
 // few, which is the faster one for a sample, and a DENSE one for the GPU's
 // throughput.  FEW is the number of samples that the first holds at once.
 // Measured, ms, first build / DENSE: 128^2 x 384 steps, 36 samples 5.1 / 6.7, 150
 // samples 25.3 / 22.6; 64^2 x 96, 152 samples 1.03 / 1.15, 304 2.2 / 1.8, 1000 7.7 /
 // 6.2; 32^2 x 24 (2 x 2 blocks / 4 x 4), 3 samples 0.10 / 0.22, 304 0.160 / 0.25.
+// 32^2 has 4 x 2 blocks between the two, for as many samples as those hold (608; two
+// to four samples to an SM are too few warps of 4 x 4 blocks): 83 steps, plain, 2 x 2 /
+// 4 x 2 / 4 x 4, 304 samples 145 / 165 / 229, 456 250 / 171 / 231 (206 before these
+// blocks), 912 - / 363 / 317; coupled, 456 - / 190 / 254 (325).
 // 16^2 holds 1824 samples at once in the first build, 3040 in the DENSE one; the
 // first keeps the sizes that it finishes in as many passes, or in a short one more
 // (coupled, 77 steps, us; in brackets one warp per 2 x 2 blocks and no bound, 2128 at
@@ -729,6 +734,7 @@ void launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int 
 // 3648 1495 / 1690 (1690), 5000 2232 / 2180 (2180), 20000 8140 / 8030 (8720).
 template <int N>
 constexpr long long kFew = N == 32 ? 304 : N == 64 ? 152 : N == 128 ? 36 : 0;
+constexpr long long kMid32 = 608;
 template <int N>
 constexpr bool first_build(long long count) {
     if (N == 16) return count <= 2128 || (count > 3040 && count <= 3648);
@@ -737,13 +743,18 @@ constexpr bool first_build(long long count) {
 
 template <int N, bool CPL>
 cudaError_t prepare(int slot_stride, VariantInfo* out) {
-    using S = TShape<N, (N >= 16)>;
+    constexpr Build B = N >= 16 ? kDense : kFirst;   // the build that holds the most samples
+    using S = TShape<N, B>;
     const size_t smem = S::smem(slot_stride);
-    const auto kernel = theta_kernel<N, CPL, (N >= 16)>;
+    const auto kernel = theta_kernel<N, CPL, B>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess && N >= 16)
-        e = cudaFuncSetAttribute(theta_kernel<N, CPL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)TShape<N, false>::smem(slot_stride));
+        e = cudaFuncSetAttribute(theta_kernel<N, CPL, kFirst>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)TShape<N, kFirst>::smem(slot_stride));
+    if constexpr (N == 32)
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(theta_kernel<N, CPL, kMid>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)TShape<N, kMid>::smem(slot_stride));
     if (e != cudaSuccess) return e;
     *out = VariantInfo{};
     out->threads = S::THREADS;
@@ -766,8 +777,8 @@ cudaError_t prepare(int slot_stride, VariantInfo* out) {
         out->max_ctas = per_sm * sms;
         if constexpr (N == 16) {
             // the first build also runs batches of several passes, on its own residency
-            const auto few = theta_kernel<N, CPL, false>;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, few, TShape<N, false>::THREADS, smem)) != cudaSuccess)
+            const auto few = theta_kernel<N, CPL, kFirst>;
+            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, few, TShape<N, kFirst>::THREADS, smem)) != cudaSuccess)
                 return e;
             out->second_ctas = per_sm * sms;
         }
@@ -776,24 +787,27 @@ cudaError_t prepare(int slot_stride, VariantInfo* out) {
     return cudaSuccess;
 }
 
-template <int N, bool CPL, bool DENSE, bool TEST = false>
+template <int N, bool CPL, Build B, bool TEST = false>
 cudaError_t launch_build(const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t st, int priority) {
-    using S = TShape<N, DENSE>;
+    using S = TShape<N, B>;
     if (n_ctas % S::CL != 0) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     launch_config<S>(cfg, attr, n_ctas, a.slot_stride, st, priority);
-    return cudaLaunchKernelEx(&cfg, theta_kernel<N, CPL, DENSE, TEST>, a, t);
+    return cudaLaunchKernelEx(&cfg, theta_kernel<N, CPL, B, TEST>, a, t);
 }
 
 template <int N, bool CPL>
 cudaError_t launch_n(const VariantInfo& vi, const KArgs& a, const TArgs& t, int* n_ctas, cudaStream_t st, int priority) {
-    // (both builds have the same sample slots per CTA or cluster)
-    static_assert(TShape<N, false>::SPB == TShape<N, (N >= 16)>::SPB, "slots");
+    // (the builds of a grid size have the same sample slots per CTA or cluster)
+    static_assert(TShape<N, kFirst>::SPB == TShape<N, (N >= 16 ? kDense : kFirst)>::SPB &&
+                      (N != 32 || TShape<32, kMid>::SPB == 1), "slots");
+    if constexpr (N == 32)
+        if (a.count > kFew<N> && a.count <= kMid32) return launch_build<N, CPL, kMid>(a, t, *n_ctas, st, priority);
     if constexpr (N >= 16)
-        if (!first_build<N>(a.count)) return launch_build<N, CPL, true>(a, t, *n_ctas, st, priority);
+        if (!first_build<N>(a.count)) return launch_build<N, CPL, kDense>(a, t, *n_ctas, st, priority);
     if (vi.second_ctas > 0 && vi.second_ctas < *n_ctas) *n_ctas = vi.second_ctas;
-    return launch_build<N, CPL, false>(a, t, *n_ctas, st, priority);
+    return launch_build<N, CPL, kFirst>(a, t, *n_ctas, st, priority);
 }
 
 // f(std::integral_constant<int, N>) for the grid sizes with a kernel.
@@ -826,9 +840,9 @@ cudaError_t theta_variant_info(int n, bool coupled, int slot_stride, VariantInfo
 cudaError_t launch_theta_wait_test(const KArgs& a, const TArgs& t, int n_ctas, cudaStream_t st) {
     if (t.K < 0 || t.K > kMaxCheb) return cudaErrorInvalidValue;
     constexpr int N = 128;
-    static_assert(TShape<N, true>::SAMPLE_BYTES < 45000, "no shared-memory attribute needed");
-    return first_build<N>(a.count) ? launch_build<N, true, false, true>(a, t, n_ctas, st, 0)
-                                   : launch_build<N, true, true, true>(a, t, n_ctas, st, 0);
+    static_assert(TShape<N, kDense>::SAMPLE_BYTES < 45000, "no shared-memory attribute needed");
+    return first_build<N>(a.count) ? launch_build<N, true, kFirst, true>(a, t, n_ctas, st, 0)
+                                   : launch_build<N, true, kDense, true>(a, t, n_ctas, st, 0);
 }
 
 cudaError_t launch_theta(int n, bool coupled, const VariantInfo& vi, const KArgs& a, const TArgs& t, int* n_ctas,

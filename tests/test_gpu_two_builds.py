@@ -106,3 +106,19 @@ def test_both_builds_of_the_54_grid_fourier_level(dk, mc):
                 sums, samp = _run(ctx, dk, 2, mc, count, static)
                 assert np.max(np.abs(samp - big[:count]) / scale) <= 1e3 * 9 * 2.0 ** -53
                 assert int(sums[0]) == count and sums[1] == 0.0
+
+
+@pytest.mark.parametrize("mc", [False, True])
+def test_three_builds_of_the_32_grid_theta_level(dk, mc):
+    """32^2 theta level: 2 x 2, 4 x 2 and 4 x 4 blocks per thread run the same operations
+    on every cell, up to the order of the FP64 sums over threads (256: 8 levels)."""
+    wl = W.get("theta16_128").with_(L_max=1, T=0.005)
+    with dk.Context.from_workload(wl) as ctx:
+        assert ctx.level_info(1).n == 32 and ctx.level_info(1).theta == 1
+        _, big = _run(ctx, dk, 1, mc, 900)
+        scale = np.maximum(np.sqrt(np.mean(big ** 2, axis=0)), 1e-300)
+        for count in (1, 304, 305, 608, 609, 900):
+            for static in (False, True):
+                sums, samp = _run(ctx, dk, 1, mc, count, static)
+                assert np.max(np.abs(samp - big[:count]) / scale) <= 1e3 * 8 * 2.0 ** -53
+                assert int(sums[0]) == count and sums[1] == 0.0
