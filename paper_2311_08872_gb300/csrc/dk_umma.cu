@@ -372,9 +372,7 @@ cudaError_t launch_gemm_tc(const GemmArgs* g, int count, unsigned* err, cudaStre
     // stages (99 KB) let two CTAs share an SM.  256-column tiles with two stages
     // for every size, and one product a launch: part of the 520 us that a gradient
     // of 1024 rows took, 127 now.
-    if (n > 64 && tiles_m * 4 <= 152) return umma_launch<64, 8>(g, count, err, st);
-    return n <= 32 ? umma_launch<32, 8>(g, count, err, st) : n <= 64 ? umma_launch<64, 8>(g, count, err, st)
-         : n <= 128 ? umma_launch<128, 2>(g, count, err, st) : umma_launch<256, 2>(g, count, err, st);
+    return n <= 64 || tiles_m * 4 <= 152 ? umma_launch<64, 8>(g, count, err, st) : umma_launch<256, 2>(g, count, err, st);
 }
 
 }  // namespace dk
