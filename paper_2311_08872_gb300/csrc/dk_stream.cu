@@ -426,7 +426,9 @@ __global__ void __launch_bounds__(kThreads) stream_coarse_kernel(const SArgs a, 
 // from are done, which are always earlier items: a fine tile at step m needs
 // itself and its four neighbours at step m (their step m-1 done: q^m written
 // and q^{m-1}, which step m overwrites, read); at m = 4cn+4 also the coarse
-// tiles whose halo reads its coupled sums done with step cn.  A coarse tile at
+// tiles whose halo reads its coupled sums done with step cn (the sums that step m
+// overwrites, two buffers in turn, are those of coarse step cn-1, so waiting for
+// that one would do).  A coarse tile at
 // step cn needs the fine tiles under it and its halo done with fine step
 // 4cn+3, and itself and its four neighbours done with coarse step cn-1.
 // Every earlier item is held by a running CTA, so the waits end; each is
