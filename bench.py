@@ -59,13 +59,13 @@ BAND_SOURCES = ("dk_band.cu", "dk_device.cuh")
 # ncu capture (smsp__inst_executed x 32 / fine cell-steps); valid
 # under the recorded hash of its sources.  Bound by instruction issue.
 THETA_KERNEL_INSTR = {"kernel": "theta_kernel n=64 coupled=True b0=0.5 chebyshev_steps=14",
-                      "instructions_per_fine_cell_step": 323.4, "sources_sha256_16": "70be40720f6160da"}
+                      "instructions_per_fine_cell_step": 323.6, "sources_sha256_16": "6de38d14192fc076"}
 THETA_SOURCES = ("dk_theta.cu", "dk_device.cuh")
 # Fourier-coupled kernel: thread instructions per cell-step (fine and coarse
 # cell-steps) of the 54^2 coupled launch, from its ncu capture;
 # valid under the recorded hash of its sources.
 FOURIER_KERNEL_INSTR = {"kernel": "fourier_kernel n=54 coupled=True",
-                        "instructions_per_cell_step": 69.4, "sources_sha256_16": "8affd0c0e50322dd"}
+                        "instructions_per_cell_step": 69.4, "sources_sha256_16": "2f93e298649c39aa"}
 FOURIER_SOURCES = ("dk_fourier.cu", "dk_device.cuh")
 # The 162^2 Fourier level on 6-CTA clusters: thread instructions per cell-step
 # (fine and coarse cell-steps) of the coupled launch of 24 samples, from its
@@ -82,11 +82,12 @@ FOURIER_CLUSTER_SOURCES = ("dk_fourier_cluster.cu", "dk_device.cuh")
 # (smsp__inst_executed x 32 / fine cell-steps); keyed by kernel function.
 KERNEL_PROFILE = {
     "stream_fine_kernel": {
-        "sources": ("dk_stream.cu", "dk_device.cuh"), "sources_sha256_16": "4a364a9befb1c264",
-        "per_n": {1024: {"dram_bytes_per_fine_cell_step": 0.92, "instructions_per_fine_cell_step": 82.8},
-                  512: {"dram_bytes_per_fine_cell_step": 0.016, "instructions_per_fine_cell_step": 82.8}},
-        "capture": "ncu --cache-control none, 3 consecutive launches of the 1024^2 (5 samples) and 512^2 "
-                   "(8 samples) fine step (profiles/stream_fine_kernel_1024_pdl_full.md, _512_pdl_full.md)",
+        "sources": ("dk_stream.cu", "dk_device.cuh"), "sources_sha256_16": "f7208955e2a9a8ba",
+        "per_n": {1024: {"dram_bytes_per_fine_cell_step": 1.75, "instructions_per_fine_cell_step": 82.5},
+                  512: {"dram_bytes_per_fine_cell_step": 0.033, "instructions_per_fine_cell_step": 82.4}},
+        "capture": "ncu --cache-control none, 4 consecutive launches (one of them with a coarse step's tiles) of the "
+                   "1024^2 (5 samples) and 512^2 (8 samples) fine step, the coarse step's work included "
+                   "(profiles/stream_fine_kernel_1024_pdl_full.md, _512_pdl_full.md)",
     },
 }
 
@@ -218,7 +219,7 @@ def fourier_coupling(stream):
     out = {"workload": wl.name, "level": level, "n": info.n, "coarse_n": info.n // 3, "fine_steps": info.M,
            "samples": count, "s": sec, "cell_steps_per_s": count * info.cost / sec,
            "coupled_sample_steps_per_s": count * info.M / sec,
-           "bound": "alu (instruction issue; shared-memory queue stalls lead)"}
+           "bound": "alu (instruction issue; fixed-latency and short-scoreboard waits lead)"}
     if kernel_sources_hash(FOURIER_SOURCES) == FOURIER_KERNEL_INSTR["sources_sha256_16"]:
         ipc = FOURIER_KERNEL_INSTR["instructions_per_cell_step"]
         warp_inst = count * info.cost * ipc / 32.0 / sec
@@ -242,7 +243,7 @@ def fourier_coupling(stream):
     cl = {"workload": wl.name, "level": level, "n": info.n, "coarse_n": info.n // 3, "fine_steps": info.M,
           "cluster": info.cluster, "samples": count, "s": sec, "cell_steps_per_s": count * info.cost / sec,
           "fine_cell_steps_per_s": count * info.cost_mc / sec, "coupled_sample_steps_per_s": count * info.M / sec,
-          "bound": "alu (instruction issue; shared-memory queue and scoreboard stalls lead)"}
+          "bound": "alu (instruction latency: fixed-latency waits with 8 warps per SM lead)"}
     if kernel_sources_hash(FOURIER_CLUSTER_SOURCES) == FOURIER_CLUSTER_KERNEL_INSTR["sources_sha256_16"]:
         ipc = FOURIER_CLUSTER_KERNEL_INSTR["instructions_per_cell_step"]
         warp_inst = count * info.cost * ipc / 32.0 / sec

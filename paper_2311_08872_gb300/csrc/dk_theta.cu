@@ -56,9 +56,9 @@
 // Bound by instruction issue and latency: 9 packed operations per cell and iteration
 // take two cycles each on the FP32 pipe, and an iteration ends in a barrier.
 // Crank--Nicolson (14 iterations), ms, in brackets with 2 x 2 blocks per thread and a
-// cluster barrier per iteration: 128^2, 75 samples x 384 steps, 14.2 (29.7), 36
-// samples 4.95 (9.90); 64^2, 1000 x 96, 6.15 (8.98), 152 samples 1.03 (1.29); 32^2,
-// 20000 x 24, 7.14 (10.4).  With the inner rows of a block after the barrier instead
+// cluster barrier per iteration: 128^2, 75 samples x 384 steps, 14.0 (29.7), 36
+// samples 4.95 (9.90); 64^2, 1000 x 96, 6.2 (8.98), 152 samples 1.03 (1.29); 32^2,
+// 20000 x 24, 7.17 (10.4).  With the inner rows of a block after the barrier instead
 // of before it, 64^2 took 1.11 (152 samples) and 6.61 (1000).
 #include <cooperative_groups.h>
 
